@@ -8,10 +8,19 @@
 // and the constructed loss whose incoming gradient is the error itself (h = r).  Six statistics per
 // trial (see bsp_lsm_stat_id), then mean, standard error over trials and z.
 //
-// lsm_prep_kernel: l and p once per row.  lsm_trial_kernel: one block per trial walks the rows; a
-// thread owns groups of four classes (one generator block per group and stream), the row's sum of
-// errors is a block reduction of sign counts, the backward is evaluated as the operator defines it.
-// lsm_reduce_kernel: per-column sums over trials in double.  Generator-bound; no tensor cores.
+// What a class contributes depends on its error's sign alone: with A = (exp(l + r) - p) / p and
+// B = (exp(l + r) / cosh(eps) - p) / p the six terms are A, A' (of the copy's sign), -A sum_r, -A' sum_r,
+// B and -B sum_r, because h itself cancels between g and g* and sum_r = 1^T h of the constructed loss
+// is common to the row.  So lsm_prep_kernel forms A and B for both signs once per row and class, and a
+// trial adds up the entries its signs select.
+//
+// lsm_trial_kernel: a thread is a trial and walks the classes of its rows, so a row's sums stay in one
+// thread: no shuffle, no barrier, and a warp reads one table entry at one address.  Per four classes
+// two generator blocks and about 36 instructions of selection and addition: generator-bound.  The block
+// per trial it replaces, which evaluated the exponentials per trial and reduced every row over the
+// block, took 293 us for 64 x 128, 4096 trials; this one takes 57 us (two words per entry and trial
+// at the generator's 1690 G words/s are 40 us).
+// lsm_collect_kernel: sums over row chunks per trial, then the column sums over trials in double.
 #include "common.cuh"
 
 namespace bsp {
@@ -20,7 +29,7 @@ constexpr int kLsmThreads = 256;
 constexpr int kLsmStats = 6, kLsmCols = 8;
 
 __global__ void __launch_bounds__(kLsmThreads)
-lsm_prep_kernel(const float* __restrict__ logits, int classes, float* __restrict__ l, float* __restrict__ p) {
+lsm_prep_kernel(const float* __restrict__ logits, int classes, float eps, float4* __restrict__ table) {
   __shared__ float red[kLsmThreads / 32];
   __shared__ float bc;
   const size_t row = blockIdx.x;
@@ -50,107 +59,119 @@ lsm_prep_kernel(const float* __restrict__ logits, int classes, float* __restrict
   }
   __syncthreads();
   const float lz = bc;
+  const float inv_c = 1.0f / coshf(eps);
   for (int j = threadIdx.x; j < classes; j += kLsmThreads) {
-    const float v = (x[j] - m) - lz;
-    l[row * classes + j] = v;
-    p[row * classes + j] = expf(v);
+    const float l = (x[j] - m) - lz, p = expf(l), up = expf(l + eps), dn = expf(l - eps);
+    table[row * classes + j] = make_float4((up - p) / p, (dn - p) / p, (up * inv_c - p) / p, (dn * inv_c - p) / p);
   }
 }
 
+// Block (x, y): trials x * blockDim.x .., rows of chunk y; partial[y][statistic][trial].
 __global__ void __launch_bounds__(kLsmThreads)
-lsm_trial_kernel(const float* __restrict__ l, const float* __restrict__ p, const int32_t* __restrict__ target, int rows,
-                 int classes, float eps, PhiloxKey key_reuse, PhiloxKey key_copy, float* __restrict__ per_trial) {
-  __shared__ int cnt_s[2][kLsmThreads / 32];
-  __shared__ float acc_s[kLsmThreads / 32][kLsmStats];
-  const uint32_t trial = blockIdx.x;
-  const int groups = classes / 4;
-  const float inv_c = 1.0f / coshf(eps);
+lsm_trial_kernel(const float4* __restrict__ table, int rows, int rows_per_chunk, int classes, float eps, PhiloxKey key_reuse,
+                 PhiloxKey key_copy, int trials, float* __restrict__ partial) {
+  const int trial = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  const int row0 = (int)blockIdx.y * rows_per_chunk;
+  const int row1 = row0 + rows_per_chunk < rows ? row0 + rows_per_chunk : rows;
+  const int groups = classes / 4;                                   // classes % 4 == 0: groups never straddle rows
   float acc[kLsmStats] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (int row = 0; row < rows; ++row) {
-    // signs of this thread's classes (bit e of `sg`: class 4 * group + e of the thread's n-th group)
-    uint32_t sg = 0, sg2 = 0;
-    int cnt = 0, nb = 0;
-    for (int gq = threadIdx.x; gq < groups; gq += kLsmThreads, nb += 4) {
-      const uint64_t q = ((uint64_t)row * classes) / 4 + gq;      // classes % 4 == 0: groups never straddle rows
-      const uint4 w = philox_block(key_reuse, q, trial), w2 = philox_block(key_copy, q, trial);
-      const uint32_t b = (w.x >> 31) | ((w.y >> 31) << 1) | ((w.z >> 31) << 2) | ((w.w >> 31) << 3);
-      const uint32_t b2 = (w2.x >> 31) | ((w2.y >> 31) << 1) | ((w2.z >> 31) << 2) | ((w2.w >> 31) << 3);
-      sg |= b << nb; sg2 |= b2 << nb;
-      cnt += __popc(b);
-    }
-    // 1^T h of the constructed loss: the sum of the consumed errors over the row
-    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-    const int buf = row & 1;
-    if ((threadIdx.x & 31) == 0) cnt_s[buf][threadIdx.x >> 5] = cnt;
-    __syncthreads();
-    int total = 0;
-#pragma unroll
-    for (int w = 0; w < kLsmThreads / 32; ++w) total += cnt_s[buf][w];
-    const float sum_r = eps * (float)(2 * total - classes);
-    const int y = __ldg(target + row);
-    nb = 0;
-    for (int gq = threadIdx.x; gq < groups; gq += kLsmThreads, nb += 4) {
-      const size_t i0 = (size_t)row * classes + 4 * (size_t)gq;
-      const float4 lv = __ldg(reinterpret_cast<const float4*>(l + i0)), pv = __ldg(reinterpret_cast<const float4*>(p + i0));
-      const float ls[4] = {lv.x, lv.y, lv.z, lv.w}, ps[4] = {pv.x, pv.y, pv.z, pv.w};
+  for (int row = row0; row < row1; ++row) {
+    const float4* __restrict__ t = table + (size_t)row * classes;
+    const uint64_t q0 = ((uint64_t)row * classes) / 4;
+    float a1 = 0.f, a2 = 0.f, b1 = 0.f;
+    int cnt = 0;
+#pragma unroll 2
+    for (int g = 0; g < groups; ++g) {
+      const uint4 w1 = philox_block(key_reuse, q0 + g, (uint32_t)trial), w2 = philox_block(key_copy, q0 + g, (uint32_t)trial);
+      const uint32_t u1[4] = {w1.x, w1.y, w1.z, w1.w}, u2[4] = {w2.x, w2.y, w2.z, w2.w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const float r = (sg >> (nb + e)) & 1u ? eps : -eps, r2 = (sg2 >> (nb + e)) & 1u ? eps : -eps;
-        const float eS = expf(ls[e] + r), eS2 = expf(ls[e] + r2), pj = ps[e], ipj = 1.0f / pj;
-        const float h_lik = (4 * gq + e) == y ? -1.0f : 0.f;
-        // the operator: g = h - exp(S) * (1^T h); likelihood: 1^T h = -1; constructed: h = r, 1^T h = sum_r
-        const float gs_lik = h_lik + pj, gs_con = r - pj * sum_r;
-        acc[0] += ((h_lik + eS) - gs_lik) * ipj;
-        acc[1] += ((h_lik + eS2) - gs_lik) * ipj;
-        acc[2] += ((r - eS * sum_r) - gs_con) * ipj;
-        acc[3] += ((r - eS2 * sum_r) - gs_con) * ipj;
-        acc[4] += ((h_lik + eS * inv_c) - gs_lik) * ipj;
-        acc[5] += ((r - eS * inv_c * sum_r) - gs_con) * ipj;
+        const float4 v = __ldg(t + 4 * g + e);
+        a1 += (int)u1[e] < 0 ? v.x : v.y;                           // the top bit set: +eps
+        b1 += (int)u1[e] < 0 ? v.z : v.w;
+        a2 += (int)u2[e] < 0 ? v.x : v.y;
+        cnt += (int)(u1[e] >> 31);
       }
     }
+    const float sum_r = eps * (float)(2 * cnt - classes);           // 1^T h of the constructed loss
+    acc[0] += a1;
+    acc[1] += a2;
+    acc[2] -= a1 * sum_r;
+    acc[3] -= a2 * sum_r;
+    acc[4] += b1;
+    acc[5] -= b1 * sum_r;
   }
+  if (trial < trials)
 #pragma unroll
-  for (int i = 0; i < kLsmStats; ++i) acc[i] = warp_sum(acc[i]);
-  if ((threadIdx.x & 31) == 0)
-    for (int i = 0; i < kLsmStats; ++i) acc_s[threadIdx.x >> 5][i] = acc[i];
-  __syncthreads();
-  if (threadIdx.x < kLsmStats) {
-    double t = 0.0;
-    for (int w = 0; w < kLsmThreads / 32; ++w) t += (double)acc_s[w][threadIdx.x];
-    per_trial[(size_t)trial * kLsmStats + threadIdx.x] = (float)(t / ((double)rows * classes));
-  }
+    for (int i = 0; i < kLsmStats; ++i) partial[((size_t)blockIdx.y * kLsmStats + i) * trials + trial] = acc[i];
 }
 
-// Column c < 6: the statistic itself; 6 and 7: the paired contrasts reuse - independent (likelihood,
-// constructed).  out[2c], out[2c + 1] = sum and sum of squares over trials, in double.
+// Per trial the statistics as means over rows and classes (FP32 out), and per block the sums over its
+// trials: column c < 6 the statistic itself, 6 and 7 the paired contrasts reuse - independent
+// (likelihood, constructed); out[block][2c], [2c + 1] = sum and sum of squares in double.  A block takes
+// 32 trials at a time, eight threads sharing a trial's row chunks; fixed order throughout.
 __global__ void __launch_bounds__(256)
-lsm_reduce_kernel(const float* __restrict__ per_trial, int trials, double* __restrict__ out) {
-  // thread t sums the trials t, t + 256, ... of every column; the 256 partial sums are then added
-  // pairwise in a fixed tree, so the result does not depend on scheduling
-  __shared__ double sh[2 * kLsmCols][256];
+lsm_collect_kernel(const float* __restrict__ partial, int nchunks, int trials, double inv_n, float* __restrict__ per_trial,
+                   double* __restrict__ out) {
+  __shared__ double part[8][kLsmStats][33];
+  __shared__ double sh[2 * kLsmCols][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double s1[kLsmCols], s2[kLsmCols];
 #pragma unroll
   for (int c = 0; c < kLsmCols; ++c) s1[c] = s2[c] = 0.0;
-  for (int t = threadIdx.x; t < trials; t += 256) {
-    const float* v = per_trial + (size_t)t * kLsmStats;
-    double x[kLsmCols];
+  for (int t0 = (int)blockIdx.x * 32; t0 < trials; t0 += (int)gridDim.x * 32) {
+    const int t = t0 + lane;
+    double a[kLsmStats] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    if (t < trials)
+      for (int y = w; y < nchunks; y += 8)
 #pragma unroll
-    for (int c = 0; c < kLsmStats; ++c) x[c] = (double)v[c];
-    x[6] = x[0] - x[1];
-    x[7] = x[2] - x[3];
+        for (int i = 0; i < kLsmStats; ++i) a[i] += (double)__ldg(partial + ((size_t)y * kLsmStats + i) * trials + t);
 #pragma unroll
-    for (int c = 0; c < kLsmCols; ++c) { s1[c] += x[c]; s2[c] += x[c] * x[c]; }
-  }
+    for (int i = 0; i < kLsmStats; ++i) part[w][i][lane] = a[i];
+    __syncthreads();
+    if (w == 0 && t < trials) {
+      double x[kLsmCols];
 #pragma unroll
-  for (int c = 0; c < kLsmCols; ++c) { sh[2 * c][threadIdx.x] = s1[c]; sh[2 * c + 1][threadIdx.x] = s2[c]; }
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o)
-      for (int c = 0; c < 2 * kLsmCols; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + o];
+      for (int i = 0; i < kLsmStats; ++i) {
+        double v = 0.0;
+        for (int k = 0; k < 8; ++k) v += part[k][i][lane];
+        const float f = (float)(v * inv_n);
+        per_trial[(size_t)t * kLsmStats + i] = f;
+        x[i] = (double)f;
+      }
+      x[6] = x[0] - x[1];
+      x[7] = x[2] - x[3];
+#pragma unroll
+      for (int c = 0; c < kLsmCols; ++c) { s1[c] += x[c]; s2[c] += x[c] * x[c]; }
+    }
     __syncthreads();
   }
-  if (threadIdx.x < 2 * kLsmCols) out[threadIdx.x] = sh[threadIdx.x][0];
+  if (w == 0)
+#pragma unroll
+    for (int c = 0; c < kLsmCols; ++c) { sh[2 * c][lane] = s1[c]; sh[2 * c + 1][lane] = s2[c]; }
+  __syncthreads();
+  if (threadIdx.x < 2 * kLsmCols) {
+    double v = 0.0;
+    for (int k = 0; k < 32; ++k) v += sh[threadIdx.x][k];
+    out[(size_t)blockIdx.x * 2 * kLsmCols + threadIdx.x] = v;
+  }
 }
+
+// How a call is cut: blocks of up to 256 trials by chunks of rows, about seven blocks per SM (one wave
+// of the eight that fit) where the rows allow it.
+struct LsmPlan {
+  int threads, tblocks, rows_per_chunk, nchunks, cblocks;
+  LsmPlan(int rows, int trials) {
+    threads = trials >= kLsmThreads ? kLsmThreads : (trials + 31) / 32 * 32;
+    tblocks = (trials + threads - 1) / threads;
+    int want = (kNumSMs * 7 + tblocks - 1) / tblocks;
+    if (want > rows) want = rows;
+    rows_per_chunk = (rows + want - 1) / want;
+    nchunks = (rows + rows_per_chunk - 1) / rows_per_chunk;
+    cblocks = (trials + 31) / 32;
+    if (cblocks > kNumSMs) cblocks = kNumSMs;
+  }
+};
 
 }  // namespace bsp
 
@@ -160,8 +181,10 @@ extern "C" {
 
 size_t bsp_lsm_check_workspace_bytes(int rows, int classes, int trials) {
   if (rows <= 0 || classes <= 0 || trials <= 0) return 0;
-  const size_t n = (size_t)rows * classes;
-  return 2 * round_up(n * 4, 256) + round_up((size_t)trials * kLsmStats * 4, 256) + 256;
+  const LsmPlan plan(rows, trials);
+  return round_up((size_t)rows * classes * sizeof(float4), 256) +
+         round_up((size_t)plan.nchunks * trials * kLsmStats * sizeof(float), 256) +
+         round_up((size_t)trials * kLsmStats * sizeof(float), 256) + (size_t)kNumSMs * 2 * kLsmCols * sizeof(double);
 }
 
 int bsp_lsm_check(const float* logits, const int32_t* target, int rows, int classes, float eps, int trials, uint64_t seed,
@@ -174,27 +197,36 @@ int bsp_lsm_check(const float* logits, const int32_t* target, int rows, int clas
     return BSP_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t n = (size_t)rows * classes;
+  const LsmPlan plan(rows, trials);
   char* base = reinterpret_cast<char*>(ws);
-  float* l = reinterpret_cast<float*>(base);
-  float* p = reinterpret_cast<float*>(base + round_up(n * 4, 256));
-  float* pt = reinterpret_cast<float*>(base + 2 * round_up(n * 4, 256));
-  double* sums = reinterpret_cast<double*>(base + 2 * round_up(n * 4, 256) + round_up((size_t)trials * kLsmStats * 4, 256));
-  if (per_trial) pt = per_trial;
+  float4* table = reinterpret_cast<float4*>(base);
+  base += round_up(n * sizeof(float4), 256);
+  float* partial = reinterpret_cast<float*>(base);
+  base += round_up((size_t)plan.nchunks * trials * kLsmStats * sizeof(float), 256);
+  float* pt = per_trial ? per_trial : reinterpret_cast<float*>(base);
+  base += round_up((size_t)trials * kLsmStats * sizeof(float), 256);
+  double* sums = reinterpret_cast<double*>(base);
   bsp_key_t k;
   k.seed = seed; k.tensor_id = tensor_id; k.stream = BSP_STREAM_FORWARD; k.draw = 0; k.reserved = 0;
   const PhiloxKey kr = make_key(k);
   k.stream = BSP_STREAM_GAIN;                                       // the independent copy's own stream
   const PhiloxKey kc = make_key(k);
-  lsm_prep_kernel<<<(unsigned)rows, kLsmThreads, 0, st>>>(logits, classes, l, p);
+  lsm_prep_kernel<<<(unsigned)rows, kLsmThreads, 0, st>>>(logits, classes, eps, table);
   BSP_LAUNCH_CHECK();
-  lsm_trial_kernel<<<(unsigned)trials, kLsmThreads, 0, st>>>(l, p, target, rows, classes, eps, kr, kc, pt);
+  lsm_trial_kernel<<<dim3((unsigned)plan.tblocks, (unsigned)plan.nchunks), plan.threads, 0, st>>>(
+      table, rows, plan.rows_per_chunk, classes, eps, kr, kc, trials, partial);
   BSP_LAUNCH_CHECK();
-  lsm_reduce_kernel<<<1, 256, 0, st>>>(pt, trials, sums);
+  lsm_collect_kernel<<<(unsigned)plan.cblocks, 256, 0, st>>>(partial, plan.nchunks, trials, 1.0 / ((double)rows * classes), pt, sums);
   BSP_LAUNCH_CHECK();
-  double host[2 * kLsmCols];
-  BSP_CHECK_CUDA(cudaMemcpyAsync(host, sums, sizeof(host), cudaMemcpyDeviceToHost, st));
-  count_d2h(sizeof(host));
+  double parts[kNumSMs * 2 * kLsmCols], host[2 * kLsmCols];
+  const size_t bytes = (size_t)plan.cblocks * 2 * kLsmCols * sizeof(double);
+  BSP_CHECK_CUDA(cudaMemcpyAsync(parts, sums, bytes, cudaMemcpyDeviceToHost, st));
+  count_d2h(bytes);
   BSP_CHECK_CUDA(cudaStreamSynchronize(st));
+  for (int c = 0; c < 2 * kLsmCols; ++c) {
+    host[c] = 0.0;
+    for (int k = 0; k < plan.cblocks; ++k) host[c] += parts[k * 2 * kLsmCols + c];
+  }
   for (int c = 0; c < kLsmCols; ++c) {
     const double mean = host[2 * c] / trials;
     double var = (host[2 * c + 1] - host[2 * c] * mean) / (trials - 1);

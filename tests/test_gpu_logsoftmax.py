@@ -101,3 +101,20 @@ def test_argument_errors(b):
         b.bsp_lsm_check(x, y, 6, 8, 0.1, 1, 0, 3, None, ws)               # fewer than two trials
     with pytest.raises(b.BspError):
         b.bsp_lsm_check(x, y, 6, 8, 0.1, 1 << 20, 0, 3, None, ws)         # workspace too small
+
+
+# one thread per trial: trials that do not fill a warp, a block, two blocks; rows cut into chunks or not
+@pytest.mark.parametrize("rows,classes,trials", [(1, 4, 2), (40, 8, 33), (9, 36, 257), (300, 32, 513)])
+def test_cuts_by_trials_and_row_chunks(b, rows, classes, trials):
+    eps = 0.25
+    logits, target = _inputs(rows, classes, 5)
+    pt = torch.full((trials * 6,), float("nan"), device="cuda")
+    ws = b.workspace(b.bsp_lsm_check_workspace_bytes(rows, classes, trials))
+    stats = b.bsp_lsm_check(torch.from_numpy(logits).cuda(), torch.from_numpy(target).cuda(), rows, classes, eps, trials,
+                            3, ls.TENSOR_S, pt, ws)
+    want, (mean, se, z) = ls.run(logits, target, eps, 3, trials)
+    scale = np.maximum(np.abs(want[:, :6]), eps * eps)
+    assert np.max(np.abs(pt.cpu().numpy().reshape(trials, 6) - want[:, :6]) / scale) <= 2e-4      # as above
+    for c in range(8):
+        assert abs(stats[c].mean - mean[c]) <= 2e-4 * max(abs(mean[c]), eps * eps)
+        assert abs(stats[c].se - se[c]) <= 1e-3 * se[c] + 1e-9
