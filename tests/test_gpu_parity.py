@@ -234,6 +234,23 @@ def test_gain_use_monte_carlo_sums(b, case):
     assert rel_l2(mean_gpu, gk.mean(0)) <= TOL_FP32
 
 
+# edges of the 64 x 64 tiles and of a thread's 4 x 4 block, draws that do not divide over grid.z
+@pytest.mark.parametrize("T,C,draws", [(1, 16, 1), (77, 80, 37), (130, 64, 5), (64, 208, 9)])
+@pytest.mark.parametrize("make", [workloads.config2, workloads.config4])
+def test_fresh_draws_equal_single_roundings(b, make, T, C, draws):
+    inp = make(T=T, C=C, O=16, K=4, seed=5)
+    g = NormLinearGpu(inp)
+    q = b.quant(inp.store_fmt, b.ROUND_STOCHASTIC, 1.0, g.scale)
+    got = torch.full((draws, C, g.ld_t), 0xAA, dtype=torch.uint8, device="cuda")
+    b.bsp_norm_fwd_draws(g.kind, g.x, T, C, g.gamma, g.beta, g.rstd, g.mean, q,
+                         b.key(inp.seed, g.tensor_id, b.STREAM_WGRAD, 0), 3, draws, got, g.ld_t)
+    one = torch.zeros(C, g.ld_t, dtype=torch.uint8, device="cuda")
+    for k in range(draws):
+        b.bsp_norm_fwd(g.kind, g.x, T, C, g.gamma, g.beta, g.rstd, g.mean, q,
+                       b.key(inp.seed, g.tensor_id, b.STREAM_WGRAD, 3 + k), None, one, g.ld_t)
+        assert torch.equal(got[k], one), k              # the padded tokens are zero in both
+
+
 # ------------------------------------------------------------------------------ contractions
 
 
