@@ -213,7 +213,7 @@ static size_t carve(const bsp_norm_linear_desc_t* op, int K, char* base, CheckBu
   c.dx = (float*)b.take(T * C * 4);
   c.dW_ref = (float*)b.take(O * C * 4); c.dW_pol = (float*)b.take(O * C * 4); c.S2w = (float*)b.take(O * C * 4);
   c.b_bwd = bsp_norm_bwd_workspace_bytes(op->T, op->C);
-  c.b_gain = norm_gain_mc_workspace(op->T, op->C, K > 0 ? K : 1, true);   // room for either kernel variant
+  c.b_gain = norm_gain_mc_workspace(op->T, op->C, K > 0 ? K : 1);
   c.b_wgrad = bsp_linear_wgrad_workspace_bytes(op->T, op->O, op->C, BSP_READ_ORIGINAL);
   c.b_dgrad = bsp_linear_dgrad_workspace_bytes(op->T, op->O, op->C);
   c.b_stats = kMaxPendingStats * kStatSlotBytes;
@@ -409,9 +409,8 @@ int bsp_mc_check(const bsp_norm_linear_desc_t* op, int K, const bsp_verdict_rule
   };
 
   // When both uses ask for the fresh read and the caller gave a side stream, the K-draw gain kernel
-  // runs there beside the first K-draw contraction of the weight use: one is bound by the integer
-  // pipes, the other by the tensor pipes, and the thin variant of the gain kernel fits next to the
-  // contraction's CTA.
+  // runs there beside the first K-draw contraction of the weight use (in practice in the SMs that the
+  // contraction's last wave leaves idle).
   const bool overlap_gain = op->side_stream && (op->policy_mask & 4u) && ((op->policy_mask >> 3) & 4u);
   SideWork sw;
   bsp_use_result_t* gain_n_result = nullptr;
@@ -495,7 +494,7 @@ int bsp_mc_check(const bsp_norm_linear_desc_t* op, int K, const bsp_verdict_rule
           // the contraction is queued first, so its CTAs take the SMs first; the gain blocks fill in
           BSP_CHECK_CUDA(cudaStreamWaitEvent(sw.side, sw.fork, 0));
           sw.launched = true;
-          BSP_TRY(norm_gain_mc_run(true, op->norm_kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt,
+          BSP_TRY(norm_gain_mc_run(op->norm_kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt,
                                    qu, gain_key, 0, K, b.dg_ref, b.S1g, b.S2g, b.ws_gain, b.b_gain, diag, sw.side));
           BSP_CHECK_CUDA(cudaEventRecord(sw.join, sw.side));
         }

@@ -200,120 +200,162 @@ column_reduce_kernel(const float* __restrict__ part0, float* __restrict__ out0, 
 
 // ------------------------------------------------------------------------------- gain-use Monte Carlo
 
-constexpr int kMcRows = 8;             // rows per thread
-constexpr int kMcSlab = 8 * kMcRows;    // rows per block (8 warps)
-constexpr int kMcCols = 128;            // columns per block (32 lanes x 4)
-constexpr int kMcChunk = 64;            // draws per launch
-constexpr size_t kMcSmemBytes = (size_t)2 * kMcRows * 256 * sizeof(float4);   // values + weights of a slab
-constexpr int kMcThinWarps = 4, kMcThinRows = 4;     // the thin variant: 4 warps x 4 rows per thread
-constexpr size_t kMcThinSmemBytes = (size_t)2 * kMcThinRows * kMcThinWarps * 32 * sizeof(float4);
+constexpr int kMcWarps = 8, kMcRows = 4;            // a sub-slab: 8 warps x 4 rows per thread
+constexpr int kMcSub = kMcWarps * kMcRows;
+constexpr int kMcCols = 128;                        // columns per block (32 lanes x 4)
+constexpr int kMcBlockDraws = 64;                   // draws per block: one row of sums in shared memory each
 
-template <int DT, int DU_DT, int FMT, int NW, int ROWS>
-__global__ void __launch_bounds__(NW * 32, NW == 8 ? 3 : 4)
+// How a call is cut: blocks of kMcCols columns x slabs of `subs` sub-slabs x `draws_per_z` draws.  A
+// block keeps the sums of its draws in shared memory over its sub-slabs, so the more sub-slabs the
+// fewer partial sums go through memory; slabs are taken as long as leaves about twelve blocks per SM
+// (six rounds of the two that fit).  Draws are split over grid.z where that leaves fewer, in shares of
+// at least eight, and beyond kMcBlockDraws.
+struct GainPlan {
+  int subs, nslabs, draws_per_z;
+  GainPlan(int64_t T, int64_t C, int K) {
+    const int64_t cols = (C + kMcCols - 1) / kMcCols, nsub = (T + kMcSub - 1) / kMcSub, want = (int64_t)kNumSMs * 12;
+    int64_t nz = (K + kMcBlockDraws - 1) / kMcBlockDraws;
+    subs = (int)(cols * nsub * nz / want);
+    if (subs < 1) subs = 1;
+    if (subs > 16) subs = 16;
+    nslabs = (int)((nsub + subs - 1) / subs);
+    const int64_t most = (K + 7) / 8, more = (want / 2) / (cols * (nslabs > 0 ? nslabs : 1));
+    if (nz < more) nz = more < most ? more : most;
+    if (nz < 1) nz = 1;
+    draws_per_z = (int)((K + nz - 1) / nz);
+  }
+};
+// Draws per launch: the partial sums of a launch stay within 64 MiB, at least kMcBlockDraws draws.
+static int gain_chunk(int64_t T, int64_t C, int K) {
+  const GainPlan plan(T, C, K);
+  const int64_t per = (int64_t)(plan.nslabs > 0 ? plan.nslabs : 1) * C * (int64_t)sizeof(float);
+  int64_t fit = ((int64_t)64 << 20) / (per > 0 ? per : 1);
+  if (fit < kMcBlockDraws) fit = kMcBlockDraws;
+  return (int)(fit < K ? fit : K);
+}
+
+template <int DT, int DU_DT, int FMT>
+__global__ void __launch_bounds__(kMcWarps * 32, 2)
 gain_mc_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
                const float* __restrict__ beta, const float* __restrict__ rstd, const float* __restrict__ mean,
                const void* __restrict__ du, float scale_val, const float* __restrict__ scale_dev,
-               const float* __restrict__ grid_steps, PhiloxKey key, int draw_begin, int ndraws,
+               const float* __restrict__ grid_steps, PhiloxKey key, int draw_begin, int ndraws, int draws_per_z, int subs,
                float* __restrict__ partial /* [ndraws][nslabs][C] */, bsp_diag_t* __restrict__ diag) {
   // A fresh rounding of an element is its round-down value plus, with probability frac, one grid
   // step: value(U) = lo + (U < P) * (hi - lo) with the threshold P of f8_sr_threshold.  So the
   // gain-use sum of draw k is  sum_t (lo/scale - beta)/gamma * du  (the same for every draw, summed
   // once) plus  sum_t [U_k,t < P_t] * (hi - lo)/scale/gamma * du : per element and draw one generator
-  // word, one comparison and one conditional add.  The slab's thresholds and step weights live in
-  // shared memory (each thread reads back only what it wrote), which keeps the register count low
-  // enough for three blocks per SM: the draw loop is a chain of dependent integer multiplies, and it
-  // is occupancy that hides their latency.
+  // word, one comparison and one conditional add.
   // grid_steps != NULL selects the b-bit per-token store instead of the FP8 store: the element sits at
   // t = u / s on the uniform grid of its token's step s, lo = s floor(t), the step weight is s and the
   // threshold floor(frac(t) 2^32).  Everything after the prologue is the same.
-  extern __shared__ __align__(16) float4 mc_smem[];
-  uint4* sp = reinterpret_cast<uint4*>(mc_smem);   // [kMcRows][256] thresholds
-  constexpr int NT = NW * 32;
-  float4* sw = mc_smem + ROWS * NT;                // [ROWS][NT] step weights
-  __shared__ __align__(16) float red[2][NW][kMcCols];
+  //
+  // Bound by the generator's integer multiplies (the heavy half of the FMA pipe), behind chains of
+  // dependent multiplies: two draws of four rows give a thread eight independent chains, with the
+  // thresholds and step weights in registers.  4096 x 1024, 64 draws: 214 us = 1.25 T draws/s (one draw at
+  // a time with both in shared memory, three blocks per SM: 255 us); 64 x 128, 256 draws, which were one
+  // block: 290 -> 9 us.
+  extern __shared__ __align__(16) float mc_sum[];        // [draws of this block][kMcCols]
+  constexpr int NT = kMcWarps * 32;
+  __shared__ __align__(16) float red[2][2][kMcWarps][kMcCols];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t c = (int64_t)blockIdx.x * kMcCols + lane * 4;
   const int64_t slab = blockIdx.y, nslabs = gridDim.y;
   const float scale = grid_steps ? 1.0f : (scale_dev ? __ldg(scale_dev) : scale_val);
   const float inv_scale = __fdiv_rn(1.0f, scale);
   const bool col_ok = c < C;
+  const int k0 = (int)blockIdx.z * draws_per_z, kend = k0 + draws_per_z < ndraws ? k0 + draws_per_z : ndraws, nd = kend - k0;
 
   float4 g4 = make_float4(1.f, 1.f, 1.f, 1.f), b4 = make_float4(0.f, 0.f, 0.f, 0.f);
   if (col_ok) {
     g4 = __ldg(reinterpret_cast<const float4*>(gamma + c));
     if (kind == BSP_LAYERNORM) b4 = __ldg(reinterpret_cast<const float4*>(beta + c));
   }
-  // generator block index of this thread's four columns in row (slab*NW*ROWS + warp + NW*i) is
-  // q0 + i*qstep; rows beyond T keep v = wgt = 0 and contribute nothing whatever word they draw
-  const uint64_t q0 = (uint64_t)((slab * (NW * ROWS) + warp) * C + (col_ok ? c : 0)) >> 2;
-  const uint64_t qstep = (uint64_t)(NW * C) / 4;
-  float base[4] = {0.f, 0.f, 0.f, 0.f};                 // the draw-independent part of this thread's sums
+  const float gg[4] = {g4.x, g4.y, g4.z, g4.w};
+  const float bb[4] = {b4.x, b4.y, b4.z, b4.w};
   DiagCounters dc;                                       // non-finite x or du, counted once per element
-#pragma unroll 1
-  for (int i = 0; i < ROWS; ++i) {
-    const int64_t r = slab * (NW * ROWS) + warp + NW * i;
-    uint32_t thr[4] = {0u, 0u, 0u, 0u};
-    float wgt[4] = {0.f, 0.f, 0.f, 0.f};
-    if (r < T && col_ok) {
-      const size_t i0 = (size_t)r * C + c;
-      const float4 xv = load4<DT>(x, i0);
-      const float4 dv = load4<DU_DT>(du, i0);
-      const float rs = __ldg(rstd + r);
-      const float mu = kind == BSP_LAYERNORM ? __ldg(mean + r) : 0.f;
-      const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
-      const float ds[4] = {dv.x, dv.y, dv.z, dv.w};
-      const float gg[4] = {g4.x, g4.y, g4.z, g4.w};
-      const float bb[4] = {b4.x, b4.y, b4.z, b4.w};
+  int buf = 0;
+  for (int sub = 0; sub < subs; ++sub) {
+    const int64_t row0 = (slab * subs + sub) * kMcSub + warp;
+    if (row0 - warp >= T) break;
+    // generator block index of this thread's four columns in row row0 + kMcWarps * i is q0 + i * qstep;
+    // rows beyond T keep a zero weight and contribute nothing whatever word they draw
+    const uint64_t q0 = (uint64_t)(row0 * C + (col_ok ? c : 0)) >> 2, qstep = (uint64_t)(kMcWarps * C) / 4;
+    uint32_t thr[kMcRows][4];
+    float wgt[kMcRows][4], base[4] = {0.f, 0.f, 0.f, 0.f};   // base: the draw-independent part of this thread's sums
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        float u;
-        if (kind == BSP_RMSNORM) u = __fmul_rn(__fmul_rn(xs[e], rs), gg[e]);
-        else u = __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(xs[e], mu), rs), gg[e]), bb[e]);
-        const float w = __fdiv_rn(ds[e], gg[e]);
-        if (!isfinite(xs[e]) || !isfinite(ds[e])) dc.nonfinite++;
-        if (grid_steps) {
-          const float st = __ldg(grid_steps + r);
-          const float t = __fdiv_rn(u, st);
-          const float n0 = floorf(t);
-          thr[e] = __float2uint_rd(__fsub_rn(t, n0) * 4294967296.0f);
-          base[e] = fmaf(fmaf(st, n0, -bb[e]), w, base[e]);
-          wgt[e] = thr[e] ? st * w : 0.f;
-          continue;
+    for (int i = 0; i < kMcRows; ++i) {
+      const int64_t r = row0 + kMcWarps * i;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) { thr[i][e] = 0u; wgt[i][e] = 0.f; }
+      if (r < T && col_ok) {
+        const size_t i0 = (size_t)r * C + c;
+        const float4 xv = load4<DT>(x, i0);
+        const float4 dv = load4<DU_DT>(du, i0);
+        const float rs = __ldg(rstd + r);
+        const float mu = kind == BSP_LAYERNORM ? __ldg(mean + r) : 0.f;
+        const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
+        const float ds[4] = {dv.x, dv.y, dv.z, dv.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          float u;
+          if (kind == BSP_RMSNORM) u = __fmul_rn(__fmul_rn(xs[e], rs), gg[e]);
+          else u = __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(xs[e], mu), rs), gg[e]), bb[e]);
+          const float w = __fdiv_rn(ds[e], gg[e]);
+          if (blockIdx.z == 0 && (!isfinite(xs[e]) || !isfinite(ds[e]))) dc.nonfinite++;
+          if (grid_steps) {
+            const float st = __ldg(grid_steps + r);
+            const float t = __fdiv_rn(u, st);
+            const float n0 = floorf(t);
+            thr[i][e] = __float2uint_rd(__fsub_rn(t, n0) * 4294967296.0f);
+            base[e] = fmaf(fmaf(st, n0, -bb[e]), w, base[e]);
+            wgt[i][e] = thr[i][e] ? st * w : 0.f;
+            continue;
+          }
+          const float v = __fmul_rn(u, scale);
+          const float lo = sr_value<FMT>(v, 0xFFFFFFFFu), hi = sr_value<FMT>(v, 0u);   // never up / up whenever possible
+          thr[i][e] = f8_sr_threshold<FMT>(v);
+          base[e] = fmaf(fmaf(lo, inv_scale, -bb[e]), w, base[e]);
+          wgt[i][e] = thr[i][e] ? (hi - lo) * inv_scale * w : 0.f;    // (NaN has threshold 0: it stays in base)
         }
-        const float v = __fmul_rn(u, scale);
-        const float lo = sr_value<FMT>(v, 0xFFFFFFFFu), hi = sr_value<FMT>(v, 0u);   // never up / up whenever possible
-        thr[e] = f8_sr_threshold<FMT>(v);
-        base[e] = fmaf(fmaf(lo, inv_scale, -bb[e]), w, base[e]);
-        wgt[e] = thr[e] ? (hi - lo) * inv_scale * w : 0.f;      // (NaN has threshold 0: it stays in base)
       }
     }
-    sp[i * NT + tid] = make_uint4(thr[0], thr[1], thr[2], thr[3]);
-    sw[i * NT + tid] = make_float4(wgt[0], wgt[1], wgt[2], wgt[3]);
-  }
-  diag_flush_warp(diag, dc);                             // (the host hands diag to the first chunk of draws only)
-  for (int k = 0; k < ndraws; ++k) {
-    const uint32_t draw = (uint32_t)(draw_begin + k);
-    float acc[4] = {base[0], base[1], base[2], base[3]};
-#pragma unroll 2
-    for (int i = 0; i < ROWS; ++i) {
-      const uint4 w = philox_block(key, q0 + (uint64_t)i * qstep, draw);
-      const uint4 p4 = sp[i * NT + tid];
-      const float4 w4 = sw[i * NT + tid];
-      acc[0] += w.x < p4.x ? w4.x : 0.f;
-      acc[1] += w.y < p4.y ? w4.y : 0.f;
-      acc[2] += w.z < p4.z ? w4.z : 0.f;
-      acc[3] += w.w < p4.w ? w4.w : 0.f;
-    }
-    const int buf = k & 1;
-    *reinterpret_cast<float4*>(&red[buf][warp][lane * 4]) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    __syncthreads();
-    if (tid < kMcCols) {
+    for (int k = 0; k < nd; k += 2) {                    // an odd count ends with a draw nobody stores
+      float acc[2][4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[h][e] = base[e];
+#pragma unroll
+      for (int i = 0; i < kMcRows; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const uint4 w = philox_block(key, q0 + (uint64_t)i * qstep, (uint32_t)(draw_begin + k0 + k + h));
+          acc[h][0] += w.x < thr[i][0] ? wgt[i][0] : 0.f;
+          acc[h][1] += w.y < thr[i][1] ? wgt[i][1] : 0.f;
+          acc[h][2] += w.z < thr[i][2] ? wgt[i][2] : 0.f;
+          acc[h][3] += w.w < thr[i][3] ? wgt[i][3] : 0.f;
+        }
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        *reinterpret_cast<float4*>(&red[buf][h][warp][lane * 4]) = make_float4(acc[h][0], acc[h][1], acc[h][2], acc[h][3]);
+      __syncthreads();
+      static_assert(NT == 2 * kMcCols, "one thread per column and draw");
+      const int h = tid / kMcCols, cl = tid % kMcCols;
       float s = 0.f;
 #pragma unroll
-      for (int w8 = 0; w8 < NW; ++w8) s += red[buf][w8][tid];
-      const int64_t cc = (int64_t)blockIdx.x * kMcCols + tid;
-      if (cc < C) partial[((size_t)k * nslabs + slab) * C + cc] = s;
+      for (int w8 = 0; w8 < kMcWarps; ++w8) s += red[buf][h][w8][cl];
+      if (k + h < nd) {
+        float* slot = mc_sum + (k + h) * kMcCols + cl;   // always this thread's own
+        *slot = sub == 0 ? s : *slot + s;
+      }
+      buf ^= 1;
     }
+  }
+  diag_flush_warp(diag, dc);                             // (the host hands diag to the first chunk of draws only)
+  for (int k = tid / kMcCols; k < nd; k += 2) {
+    const int64_t cc = (int64_t)blockIdx.x * kMcCols + tid % kMcCols;
+    if (cc < C) partial[((size_t)(k0 + k) * nslabs + slab) * C + cc] = mc_sum[k * kMcCols + tid % kMcCols];
   }
 }
 
@@ -337,21 +379,34 @@ gain_mc_slab_reduce_kernel(const float* __restrict__ partial, int nslabs, int64_
   }
 }
 
-// S1[c] += sum_k (gk - ref), S2[c] += sum_k (gk - ref)^2.
-__global__ void gain_mc_accumulate_kernel(const float* __restrict__ gk, int ndraws, int64_t C,
-                                          const float* __restrict__ ref, float* __restrict__ S1,
-                                          float* __restrict__ S2) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C) return;
-  const float g0 = ref[c];
+// S1[c] += sum_k (gk - ref), S2[c] += sum_k (gk - ref)^2: 32 columns by eight draws per block, the
+// eight partial sums added in order.
+__global__ void __launch_bounds__(256)
+gain_mc_accumulate_kernel(const float* __restrict__ gk, int ndraws, int64_t C, const float* __restrict__ ref,
+                          float* __restrict__ S1, float* __restrict__ S2) {
+  __shared__ float sm[2][8][33];
+  const int cl = threadIdx.x & 31, pl = threadIdx.x >> 5;
+  const int64_t c = (int64_t)blockIdx.x * 32 + cl;
   float s1 = 0.f, s2 = 0.f;
-  for (int k = 0; k < ndraws; ++k) {
-    const float d = gk[(size_t)k * C + c] - g0;
-    s1 += d;
-    s2 = fmaf(d, d, s2);
+  if (c < C) {
+    const float g0 = ref[c];
+#pragma unroll 4
+    for (int k = pl; k < ndraws; k += 8) {
+      const float d = gk[(size_t)k * C + c] - g0;
+      s1 += d;
+      s2 = fmaf(d, d, s2);
+    }
   }
-  S1[c] += s1;
-  S2[c] += s2;
+  sm[0][pl][cl] = s1;
+  sm[1][pl][cl] = s2;
+  __syncthreads();
+  if (pl < 2 && c < C) {
+    float* out = pl ? S2 : S1;
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += sm[pl][w][cl];
+    out[c] += t;
+  }
 }
 
 static int bwd_grid(int64_t T) {
@@ -460,14 +515,14 @@ int bsp_norm_bwd(int kind, const void* x, int dt, int64_t T, int64_t C, const fl
 }
 
 size_t bsp_norm_gain_mc_workspace_bytes(int64_t T, int64_t C, int K) {
-  return bsp::norm_gain_mc_workspace(T, C, K, false);
+  return bsp::norm_gain_mc_workspace(T, C, K);
 }
 
 int bsp_norm_gain_mc(int kind, const void* x, int dt, int64_t T, int64_t C, const float* gamma, const float* beta,
                      const float* rstd, const float* mean, const void* du, int du_dt, bsp_quant_t q, bsp_key_t key,
                      int draw0, int K, const float* g_ref, float* S1, float* S2, void* ws, size_t ws_bytes,
                      bsp_diag_t* diag, void* stream) {
-  return bsp::norm_gain_mc_run(false, kind, x, dt, T, C, gamma, beta, rstd, mean, du, du_dt, q, key, draw0, K, g_ref, S1,
+  return bsp::norm_gain_mc_run(kind, x, dt, T, C, gamma, beta, rstd, mean, du, du_dt, q, key, draw0, K, g_ref, S1,
                                S2, ws, ws_bytes, diag, stream);
 }
 
@@ -475,17 +530,13 @@ int bsp_norm_gain_mc(int kind, const void* x, int dt, int64_t T, int64_t C, cons
 
 namespace bsp {
 
-size_t norm_gain_mc_workspace(int64_t T, int64_t C, int K, bool thin) {
+size_t norm_gain_mc_workspace(int64_t T, int64_t C, int K) {
   if (T <= 0 || C <= 0 || K <= 0) return 0;
-  const int slab_rows = thin ? kMcThinWarps * kMcThinRows : kMcSlab;
-  const size_t nslabs = (size_t)((T + slab_rows - 1) / slab_rows);
-  const size_t kc = (size_t)(K < kMcChunk ? K : kMcChunk);
+  const size_t nslabs = (size_t)GainPlan(T, C, K).nslabs, kc = (size_t)gain_chunk(T, C, K);
   return round_up(kc * nslabs * (size_t)C * sizeof(float), 256) + round_up(kc * (size_t)C * sizeof(float), 256);
 }
 
-// thin: the variant of the kernel made to run beside a kernel that fills the SMs (128 threads, 16 KB
-// of shared memory, 64 registers: one block fits next to a CTA of the Monte-Carlo contraction).
-int norm_gain_mc_run(bool thin, int kind, const void* x, int dt, int64_t T, int64_t C, const float* gamma,
+int norm_gain_mc_run(int kind, const void* x, int dt, int64_t T, int64_t C, const float* gamma,
                      const float* beta, const float* rstd, const float* mean, const void* du, int du_dt, bsp_quant_t q,
                      bsp_key_t key, int draw0, int K, const float* g_ref, float* S1, float* S2, void* ws, size_t ws_bytes,
                      bsp_diag_t* diag, void* stream, const float* grid_steps) {
@@ -497,32 +548,29 @@ int norm_gain_mc_run(bool thin, int kind, const void* x, int dt, int64_t T, int6
   if (T > 0 && (!x || !gamma || !rstd || !du || (kind == BSP_LAYERNORM && (!beta || !mean)))) return BSP_ERR_ARG;
   if (C % 4 != 0) return BSP_ERR_UNSUPPORTED;
   if (!aligned16(x) || !aligned16(du) || !aligned16(gamma) || !aligned16(beta)) return BSP_ERR_ALIGN;
-  if (!ws || ws_bytes < norm_gain_mc_workspace(T, C, K, thin) || (reinterpret_cast<uintptr_t>(ws) & 255u))
+  if (!ws || ws_bytes < norm_gain_mc_workspace(T, C, K) || (reinterpret_cast<uintptr_t>(ws) & 255u))
     return BSP_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
-  const int slab_rows = thin ? kMcThinWarps * kMcThinRows : kMcSlab;
-  const int nslabs = (int)((T + slab_rows - 1) / slab_rows);
-  const int kc_max = K < kMcChunk ? K : kMcChunk;
+  const GainPlan plan(T, C, K);
+  const int nslabs = T > 0 ? plan.nslabs : 0, kc_max = gain_chunk(T, C, K);
   float* partial = reinterpret_cast<float*>(ws);
   float* gk = reinterpret_cast<float*>(reinterpret_cast<char*>(ws) +
                                        round_up((size_t)kc_max * (nslabs > 0 ? nslabs : 1) * C * sizeof(float), 256));
   const PhiloxKey pk = make_key(key);
-  for (int kb = 0; kb < K; kb += kMcChunk) {
-    const int nd = (K - kb) < kMcChunk ? (K - kb) : kMcChunk;
+  for (int kb = 0; kb < K; kb += kc_max) {
+    const int nd = (K - kb) < kc_max ? (K - kb) : kc_max;
+    const int per_z = plan.draws_per_z < nd ? plan.draws_per_z : nd;
     if (nslabs > 0) {
-      dim3 grid((unsigned)((C + kMcCols - 1) / kMcCols), (unsigned)nslabs);
+      dim3 grid((unsigned)((C + kMcCols - 1) / kMcCols), (unsigned)nslabs, (unsigned)((nd + per_z - 1) / per_z));
+      const size_t smem = (size_t)per_z * kMcCols * sizeof(float);
 #define BSP_GM(DT, DU, FMT)                                                                                     \
   do {                                                                                                          \
-    if (thin) {                                                                                                 \
-      gain_mc_kernel<DT, DU, FMT, kMcThinWarps, kMcThinRows><<<grid, kMcThinWarps * 32, kMcThinSmemBytes, st>>>(kind, x, T, C, gamma, beta, rstd, mean, du, \
-                                                                 q.scale, q.scale_dev, grid_steps, pk, draw0 + kb, nd, partial, kb == 0 ? diag : nullptr); \
-      break;                                                                                                    \
-    }                                                                                                           \
-    BSP_CHECK_CUDA(cudaFuncSetAttribute(gain_mc_kernel<DT, DU, FMT, 8, kMcRows>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                        (int)kMcSmemBytes));                                                    \
-    gain_mc_kernel<DT, DU, FMT, 8, kMcRows><<<grid, 256, kMcSmemBytes, st>>>(kind, x, T, C, gamma, beta, rstd, mean, du,    \
+    BSP_CHECK_CUDA(cudaFuncSetAttribute(gain_mc_kernel<DT, DU, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                        (int)(kMcBlockDraws * kMcCols * sizeof(float))));                       \
+    gain_mc_kernel<DT, DU, FMT><<<grid, kMcWarps * 32, smem, st>>>(kind, x, T, C, gamma, beta, rstd, mean, du,  \
                                                                  q.scale, q.scale_dev, grid_steps, pk,           \
-                                                                 draw0 + kb, nd, partial, kb == 0 ? diag : nullptr); \
+                                                                 draw0 + kb, nd, per_z, plan.subs, partial,      \
+                                                                 kb == 0 ? diag : nullptr);                      \
   } while (0)
       if (q.fmt == BSP_E4M3) {
         if (dt == BSP_F32 && du_dt == BSP_F32) BSP_GM(BSP_F32, BSP_F32, BSP_E4M3);
@@ -538,10 +586,12 @@ int norm_gain_mc_run(bool thin, int kind, const void* x, int dt, int64_t T, int6
 #undef BSP_GM
       BSP_LAUNCH_CHECK();
     }
-    dim3 rgrid((unsigned)((C + 31) / 32), (unsigned)nd);
-    gain_mc_slab_reduce_kernel<<<rgrid, 256, 0, st>>>(partial, nslabs, C, gk);
-    BSP_LAUNCH_CHECK();
-    gain_mc_accumulate_kernel<<<(unsigned)((C + 255) / 256), 256, 0, st>>>(gk, nd, C, g_ref, S1, S2);
+    if (nslabs != 1) {                                   // (a single slab's sums are the draw's)
+      dim3 rgrid((unsigned)((C + 31) / 32), (unsigned)nd);
+      gain_mc_slab_reduce_kernel<<<rgrid, 256, 0, st>>>(partial, nslabs, C, gk);
+      BSP_LAUNCH_CHECK();
+    }
+    gain_mc_accumulate_kernel<<<(unsigned)((C + 31) / 32), 256, 0, st>>>(nslabs == 1 ? partial : gk, nd, C, g_ref, S1, S2);
     BSP_LAUNCH_CHECK();
   }
   return BSP_OK;

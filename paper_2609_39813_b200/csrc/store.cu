@@ -356,7 +356,7 @@ static size_t store_carve(const bsp_store_desc_t* op, int K, char* base, StoreBu
   c.dW_ref = (float*)take(O * C * 4); c.dW_pol = (float*)take(O * C * 4);
   c.S1w = (float*)take(O * C * 4); c.S2w = (float*)take(O * C * 4);
   c.b_bwd = bsp_norm_bwd_workspace_bytes(op->T, op->C);
-  c.b_gain = norm_gain_mc_workspace(op->T, op->C, K > 0 ? K : 1, false);
+  c.b_gain = norm_gain_mc_workspace(op->T, op->C, K > 0 ? K : 1);
   c.b_dgrad = bsp_linear_dgrad_workspace_bytes(op->T, op->O, op->C);
   c.b_stats = kMaxPendingStats * kStatSlotBytes;
   c.ws_bwd = take(c.b_bwd); c.ws_gain = take(c.b_gain); c.ws_dgrad = take(c.b_dgrad); c.ws_stats = take(c.b_stats);
@@ -506,7 +506,7 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
       BSP_CHECK_CUDA(cudaMemsetAsync(b.zero_c, 0, C * sizeof(float), st));
       BSP_CHECK_CUDA(cudaMemsetAsync(b.dg_pol, 0, C * sizeof(float), st));
       BSP_CHECK_CUDA(cudaMemsetAsync(b.S2g, 0, C * sizeof(float), st));
-      BSP_TRY(norm_gain_mc_run(false, kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt, qnone, key, 0, 1,
+      BSP_TRY(norm_gain_mc_run(kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt, qnone, key, 0, 1,
                                b.zero_c, b.dg_pol, b.S2g, b.ws_gain, b.b_gain, diag, st, b.steps));
       BSP_TRY(pend.add(b.dg_ref, b.dg_pol, nullptr, C, 1, 0, emit(BSP_STREAM_GAIN, BSP_OUT_DGAMMA, BSP_READ_FORWARD)));
     }
@@ -515,7 +515,7 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
       BSP_CHECK_CUDA(cudaMemsetAsync(b.S2g, 0, C * sizeof(float), st));
       bsp_key_t gk = key;
       gk.stream = BSP_STREAM_GAIN;
-      BSP_TRY(norm_gain_mc_run(false, kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt, qnone, gk, 0, K,
+      BSP_TRY(norm_gain_mc_run(kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt, qnone, gk, 0, K,
                                b.dg_ref, b.S1g, b.S2g, b.ws_gain, b.b_gain, diag, st, b.steps));
       BSP_TRY(pend.add(b.dg_ref, b.S1g, b.S2g, C, K, 1, emit(BSP_STREAM_GAIN, BSP_OUT_DGAMMA, BSP_READ_FRESH)));
     }

@@ -251,6 +251,36 @@ def test_fresh_draws_equal_single_roundings(b, make, T, C, draws):
         assert torch.equal(got[k], one), k              # the padded tokens are zero in both
 
 
+# blocks of several sub-slabs with a ragged last one, draws over grid.z, more draws than a block takes,
+# an odd count, one slab only; bsp_norm_bwd under a fresh read forms the same draws one at a time
+@pytest.mark.parametrize("T,C,K", [(8013, 4096, 5), (70, 48, 131), (32, 132, 64), (1, 16, 4), (513, 260, 9)])
+def test_gain_draws_equal_single_backwards(b, T, C, K):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(T + C)
+    x, du = (torch.randn(T, C, generator=gen, device="cuda") for _ in range(2))
+    gamma = 1.0 + 0.1 * torch.randn(C, generator=gen, device="cuda")
+    rstd, mean, amax, scale = (torch.zeros(n, device="cuda") for n in (T, T, 1, 1))
+    b.bsp_norm_stats(b.RMSNORM, x, T, C, gamma, None, 1e-6, rstd, mean, amax)
+    b.bsp_scale_from_amax(amax, 1, b.E4M3, scale)
+    q = b.quant(b.E4M3, b.ROUND_STOCHASTIC, 1.0, scale)
+    ref, one = torch.zeros(C, device="cuda"), torch.zeros(C, device="cuda")
+    ws = b.workspace(b.bsp_norm_bwd_workspace_bytes(T, C))
+    want = []
+    for k in range(K):
+        b.bsp_norm_bwd(b.RMSNORM, x, T, C, gamma, None, rstd, mean, du, 2, None, q, b.key(9, 1, b.STREAM_GAIN, k), one,
+                       None, None, ws)
+        want.append(one.double().cpu())
+    want = torch.stack(want)
+    ref.copy_(want.mean(0))
+    S1, S2 = torch.zeros(C, device="cuda"), torch.zeros(C, device="cuda")
+    ws = b.workspace(b.bsp_norm_gain_mc_workspace_bytes(T, C, K))
+    b.bsp_norm_gain_mc(b.RMSNORM, x, T, C, gamma, None, rstd, mean, du, q, b.key(9, 1, b.STREAM_GAIN, 0), 0, K, ref, S1, S2, ws)
+    d = want - ref.double().cpu()
+    # per draw both are FP32 sums over the tokens: TOL_FP32 of the gradient's size
+    assert (S1.double().cpu() - d.sum(0)).norm() <= TOL_FP32 * K * want.mean(0).norm()
+    assert rel_l2(down(S2), (d * d).sum(0).numpy()) <= 1e-3
+
+
 # ------------------------------------------------------------------------------ contractions
 
 
