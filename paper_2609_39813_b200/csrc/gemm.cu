@@ -256,28 +256,50 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 
 // ------------------------------------------------------------------------------- Monte-Carlo contraction
 
-// FP8 contraction over nb draws of B with the per-element shifted sums kept in tensor memory:
-// for every output tile the CTA walks all draws b and accumulates
+// Contraction over nb draws of B with the per-element shifted sums kept on chip: for every output tile
+// the CTA walks the draws b and accumulates
 //   S1 += alpha*acc_b - ref,   S2 += (alpha*acc_b - ref)^2
-// without ever writing a per-draw gradient.  Tile 128 x 128; TMEM columns: two accumulator stages
-// [0,128) and [128,256), S1 in [256,384), S2 in [384,512).  The reference tile sits in the
-// epilogue threads' registers for the whole tile; S1/S2 are read from global memory once per tile
-// (so calls can be chained over draw ranges) and written back once.
-// 320 threads: warp 0 TMA, warp 1 MMA, warps 2..9 epilogue (two warps per TMEM lane quarter, each
-// owning 64 of the 128 columns).
+// without ever writing a per-draw gradient.  Tile 128 x 128, draws two at a time: a stage of the ring
+// holds the A tile and the B tiles of both draws, so one 128 x 256 product per K slice fills both
+// accumulators and the A tile is fetched (from L2 and from shared memory) once for two draws.
+//
+// 384 threads: warp 0 TMA, warp 1 MMA, warps 4..11 epilogue (two warps per TMEM lane quarter, each
+// owning 64 of the 128 columns).  The reference and both sums of a tile sit in the epilogue threads'
+// registers (3 x 64), to which the producer's warpgroup gives up its share; that leaves all 512 columns
+// of tensor memory to two pairs of accumulators, so the products of a pair run under the epilogue of
+// the pair before.  With the sums in tensor memory (one pair of accumulators) every pair ended in an
+// epilogue the tensor pipe waited for: 4096 x 1024 x 4096, 64 draws (with the split below): 847 -> 767 us.
+//
+// The walk is over units (tile, range of draws).  Whole waves of tiles take all their draws; the tiles
+// of a last, partial wave (or of a problem with fewer tiles than SMs) are cut into nseg ranges, range
+// by range over the tiles, so that CTAs which run together read the same draws.  Range 0 adds to S1 and
+// S2, range s > 0 writes its sums to slot (s - 1) of the split workspace, and gemm_mc_merge_kernel adds
+// the slots in order: every sum has one order, whatever the scheduling.
 constexpr int MC_BN = 128;
-// Draws are taken two at a time: a stage holds the A tile and the B tiles of both draws, one
-// after the other, so a single 128 x 256 product per K slice fills both accumulators and the A tile
-// is fetched (from L2 and from shared memory) once for two draws.
 constexpr int kMcStages = 4;
 constexpr int kMcABytes = BM * BKB, kMcBBytes = MC_BN * BKB, kMcStageBytes = kMcABytes + 2 * kMcBBytes;
-constexpr int kMcThreads = 320;
+constexpr int kMcThreads = 384;
+constexpr int kMcRegsProducer = 40, kMcRegsEpilogue = 232;   // 40 + 2 * 232 = 3 * 168: the launch's registers
 constexpr size_t kMcSmem = (size_t)kMcStages * kMcStageBytes + 1024 + 256;
+constexpr size_t kMcSplitTileFloats = (size_t)2 * BM * MC_BN;   // S1 and S2 of one tile in a split slot
 
+// Units of the walk: tiles [0, whole) with all draws, then nseg ranges over the other tiles.
+struct McSplit {
+  int whole, rest, nseg, pairs_per_seg;
+};
+__device__ __forceinline__ void mc_unit(const McSplit& sp, int u, int npairs, int& tile, int& seg, int& p0, int& p1) {
+  if (u < sp.whole) { tile = u; seg = 0; p0 = 0; p1 = npairs; return; }
+  const int v = u - sp.whole;
+  seg = v / sp.rest;
+  tile = sp.whole + v - seg * sp.rest;
+  p0 = seg * sp.pairs_per_seg;
+  p1 = p0 + sp.pairs_per_seg < npairs ? p0 + sp.pairs_per_seg : npairs;
+}
 
 template <bool FP8>
 __global__ void __launch_bounds__(kMcThreads, 1)
-gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p) {
+gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p,
+               McSplit sp, float* __restrict__ split_ws) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;
@@ -289,7 +311,7 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tiles_m = (p.M + BM - 1) / BM, tiles_n = (p.N + MC_BN - 1) / MC_BN;
-  const int ntiles = tiles_m * tiles_n;
+  const int nunits = sp.whole + sp.rest * sp.nseg, npairs = (p.nb + 1) / 2;
   constexpr int kElemsPerStage = FP8 ? BKB : BKB / 2;   // K extent of one 128-byte stage in elements
   const int kblocks = (p.K + kElemsPerStage - 1) / kElemsPerStage;
 
@@ -306,8 +328,9 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 0) {
-    if (lane == 0) {
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMcRegsProducer));
+    if (warp == 0 && lane == 0) {
       tma_prefetch_desc(&tmap_a);
       tma_prefetch_desc(&tmap_b);
       // the dY panel of a tile row is read again by every pass over a pair of draws (and by the
@@ -315,10 +338,12 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       const uint64_t keep = l2_policy_evict_last();
       uint32_t it = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        int tm, tn;
-      tile_coords(t, tiles_m, tiles_n, tm, tn);
-        for (int b = 0; b < p.nb && ok; b += 2) {
+      for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+        int t, seg, p0, p1, tm, tn;
+        mc_unit(sp, u, npairs, t, seg, p0, p1);
+        tile_coords(t, tiles_m, tiles_n, tm, tn);
+        for (int pr = p0; pr < p1 && ok; ++pr) {
+          const int b = 2 * pr;
           const bool two = b + 1 < p.nb;                       // an odd count ends with a single draw
           for (int kb = 0; kb < kblocks; ++kb, ++it) {
             const uint32_t s = it % kMcStages, ph = (it / kMcStages) & 1u;
@@ -334,19 +359,18 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       if (!ok) {
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
       }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
+    } else if (warp == 1 && lane == 0) {
       uint32_t it = 0, tc = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        for (int b = 0; b < p.nb && ok; b += 2, ++tc) {
-          const bool two = b + 1 < p.nb;
-          // both accumulators (columns 0..127 and 128..255) belong to this pair of draws; the
-          // epilogue of the pair before must be through with them
-          if (!mbar_wait(tempty0, (tc & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+      for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+        int t, seg, p0, p1;
+        mc_unit(sp, u, npairs, t, seg, p0, p1);
+        for (int pr = p0; pr < p1 && ok; ++pr, ++tc) {
+          const uint32_t as = tc & 1u, aph = (tc >> 1) & 1u;
+          // the epilogue of the pair before last must be through with this pair of accumulators
+          if (!mbar_wait(tempty0 + 8 * as, aph ^ 1u, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t idesc = two ? p.idesc2 : p.idesc;
+          const uint32_t idesc = 2 * pr + 1 < p.nb ? p.idesc2 : p.idesc, tmem_d = tmem_base + as * 2 * MC_BN;
           for (int kb = 0; kb < kblocks; ++kb, ++it) {
             const uint32_t s = it % kMcStages, ph = (it / kMcStages) & 1u;
             if (!mbar_wait(full0 + 8 * s, ph, abort_flag)) { ok = false; break; }
@@ -355,104 +379,93 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             const uint64_t adesc = make_smem_desc(sa), bdesc = make_smem_desc(sb);   // B: 128 or 256 rows
 #pragma unroll
             for (int k = 0; k < BKB / 32; ++k)
-              tc_mma<FP8>(tmem_base, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
+              tc_mma<FP8>(tmem_d, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
             tc_commit(empty0 + 8 * s);
           }
-          if (ok) tc_commit(tfull0);
+          if (ok) tc_commit(tfull0 + 8 * as);
         }
       }
     }
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kMcRegsEpilogue));
     const int q = warp & 3;                  // TMEM lane quarter
-    const int h = (warp - 2) >> 2;           // column half
+    const int h = (warp - 4) >> 2;           // column half
     const float inv_a = __fdiv_rn(1.0f, p.sa_dev ? __ldg(p.sa_dev) : p.sa);
     const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? __ldg(p.sb_dev) : p.sb);
-    const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
-    const uint32_t s1_base = lane_base + 2 * MC_BN + h * 64, s2_base = lane_base + 3 * MC_BN + h * 64;
+    const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16) + h * 64;
     uint32_t tc = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      int tm, tn;
+    for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+      int t, seg, p0, p1, tm, tn;
+      mc_unit(sp, u, npairs, t, seg, p0, p1);
       tile_coords(t, tiles_m, tiles_n, tm, tn);
       const int row = tm * BM + q * 32 + lane;
       const int colbase = tn * MC_BN + h * 64;
-      float refv[64];
-      // ---- tile start: reference into registers, running sums into tensor memory
+      float refv[64], s1[64], s2[64];
+      // ---- unit start: the reference, and the sums so far when this unit continues them
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int col = colbase + c * 16;
-        uint32_t a1[16], a2[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) { a1[j] = 0u; a2[j] = 0u; refv[c * 16 + j] = 0.f; }
-        if (row < p.M && col < p.N) {
-          const size_t off = (size_t)row * p.ldc + col;
-#pragma unroll
-          for (int j = 0; j < 16; j += 4) {
-            // no reference: the products are differences to the reference already
-            const float4 g0 = p.ref ? *reinterpret_cast<const float4*>(p.ref + off + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-            const uint4 v1 = *reinterpret_cast<const uint4*>(p.S1 + off + j);
-            const uint4 v2 = *reinterpret_cast<const uint4*>(p.S2 + off + j);
-            refv[c * 16 + j] = g0.x; refv[c * 16 + j + 1] = g0.y; refv[c * 16 + j + 2] = g0.z; refv[c * 16 + j + 3] = g0.w;
-            a1[j] = v1.x; a1[j + 1] = v1.y; a1[j + 2] = v1.z; a1[j + 3] = v1.w;
-            a2[j] = v2.x; a2[j + 1] = v2.y; a2[j + 2] = v2.z; a2[j + 3] = v2.w;
+      for (int c = 0; c < 64; c += 4) {
+        float4 g0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = g0, v2 = g0;
+        if (row < p.M && colbase + c < p.N) {
+          const size_t off = (size_t)row * p.ldc + colbase + c;
+          // no reference: the products are differences to the reference already
+          if (p.ref) g0 = *reinterpret_cast<const float4*>(p.ref + off);
+          if (seg == 0) {
+            v1 = *reinterpret_cast<const float4*>(p.S1 + off);
+            v2 = *reinterpret_cast<const float4*>(p.S2 + off);
           }
         }
-        tmem_st16(s1_base + c * 16, a1);
-        tmem_st16(s2_base + c * 16, a2);
+        refv[c] = g0.x; refv[c + 1] = g0.y; refv[c + 2] = g0.z; refv[c + 3] = g0.w;
+        s1[c] = v1.x; s1[c + 1] = v1.y; s1[c + 2] = v1.z; s1[c + 3] = v1.w;
+        s2[c] = v2.x; s2[c + 1] = v2.y; s2[c + 2] = v2.z; s2[c + 3] = v2.w;
       }
-      tmem_wait_st();
-      // ---- every draw of this tile
-      for (int b = 0; b < p.nb && ok; b += 2, ++tc) {
-        const bool two = b + 1 < p.nb;
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(tfull0, tc & 1u, abort_flag));
+      // ---- the unit's draws
+      for (int pr = p0; pr < p1 && ok; ++pr, ++tc) {
+        const uint32_t as = tc & 1u, aph = (tc >> 1) & 1u;
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(tfull0 + 8 * as, aph, abort_flag));
         if (!ok) break;
         tc_fence_after();
-        const uint32_t acc_base = lane_base + h * 64;         // draw b; draw b + 1 is MC_BN columns further
+        const uint32_t acc_base = lane_base + as * 2 * MC_BN;  // draw 2 pr; draw 2 pr + 1 is MC_BN columns further
+        // the sums take the draws in order, as a one-draw-at-a-time pass would
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          uint32_t acc[16], acc2[16], a1[16], a2[16];
-          tmem_ld16(acc_base + c * 16, acc);
-          if (two) tmem_ld16(acc_base + MC_BN + c * 16, acc2);
-          tmem_ld16(s1_base + c * 16, a1);
-          tmem_ld16(s2_base + c * 16, a2);
-          tmem_wait_ld();
+        for (int d = 0; d < 2; ++d) {
+          if (d == 0 || 2 * pr + 1 < p.nb) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            // the sums take the draws in order, as a one-draw-at-a-time pass would
-            const float d = __uint_as_float(acc[j]) * inv_a * inv_b - refv[c * 16 + j];
-            float t1 = __uint_as_float(a1[j]) + d, t2 = fmaf(d, d, __uint_as_float(a2[j]));
-            if (two) {
-              const float e = __uint_as_float(acc2[j]) * inv_a * inv_b - refv[c * 16 + j];
-              t1 += e;
-              t2 = fmaf(e, e, t2);
+            for (int c = 0; c < 64; c += 16) {
+              uint32_t acc[16];
+              tmem_ld16(acc_base + d * MC_BN + c, acc);
+              tmem_wait_ld();
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const float e = __uint_as_float(acc[j]) * inv_a * inv_b - refv[c + j];
+                s1[c + j] += e;
+                s2[c + j] = fmaf(e, e, s2[c + j]);
+              }
             }
-            a1[j] = __float_as_uint(t1);
-            a2[j] = __float_as_uint(t2);
           }
-          tmem_st16(s1_base + c * 16, a1);
-          tmem_st16(s2_base + c * 16, a2);
         }
-        tmem_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(tempty0);
+        if (lane == 0) mbar_arrive(tempty0 + 8 * as);
       }
       if (!ok) break;
-      // ---- tile end: running sums back to global memory
+      // ---- unit end: the sums back to S1 and S2, or to the unit's split slot
+      if (seg == 0) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int col = colbase + c * 16;
-        uint32_t a1[16], a2[16];
-        tmem_ld16(s1_base + c * 16, a1);
-        tmem_ld16(s2_base + c * 16, a2);
-        tmem_wait_ld();
-        if (row < p.M && col < p.N) {
-          const size_t off = (size_t)row * p.ldc + col;
-#pragma unroll
-          for (int j = 0; j < 16; j += 4) {
-            *reinterpret_cast<uint4*>(p.S1 + off + j) = make_uint4(a1[j], a1[j + 1], a1[j + 2], a1[j + 3]);
-            *reinterpret_cast<uint4*>(p.S2 + off + j) = make_uint4(a2[j], a2[j + 1], a2[j + 2], a2[j + 3]);
+        for (int c = 0; c < 64; c += 4)
+          if (row < p.M && colbase + c < p.N) {
+            const size_t off = (size_t)row * p.ldc + colbase + c;
+            *reinterpret_cast<float4*>(p.S1 + off) = make_float4(s1[c], s1[c + 1], s1[c + 2], s1[c + 3]);
+            *reinterpret_cast<float4*>(p.S2 + off) = make_float4(s2[c], s2[c + 1], s2[c + 2], s2[c + 3]);
           }
+      } else {
+        // [S1 | S2][column / 4][row] as groups of four columns: a warp writes 512 consecutive bytes
+        float4* slot = reinterpret_cast<float4*>(split_ws + ((size_t)(seg - 1) * sp.rest + (t - sp.whole)) * kMcSplitTileFloats) +
+                       (h * 16) * BM + q * 32 + lane;
+#pragma unroll
+        for (int c = 0; c < 64; c += 4) {
+          slot[(c / 4) * BM] = make_float4(s1[c], s1[c + 1], s1[c + 2], s1[c + 3]);
+          slot[(MC_BN / 4 + c / 4) * BM] = make_float4(s2[c], s2[c + 1], s2[c + 2], s2[c + 3]);
         }
       }
     }
@@ -466,6 +479,28 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
+}
+
+// S1 += slot sums, S2 likewise, of the tiles whose draws were split.  Block (t, y): tile whole + t, a
+// thread takes four columns of one row; slots are added in the order of their draws.
+__global__ void __launch_bounds__(256)
+gemm_mc_merge_kernel(const float* __restrict__ split_ws, McSplit sp, int M, int N, int64_t ldc, float* __restrict__ S1,
+                     float* __restrict__ S2) {
+  const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + MC_BN - 1) / MC_BN;
+  int tm, tn;
+  tile_coords(sp.whole + (int)blockIdx.x, tiles_m, tiles_n, tm, tn);
+  const int i = (int)blockIdx.y * 256 + threadIdx.x, second = i >= BM * MC_BN / 4, k = i - second * (BM * MC_BN / 4);
+  const int row = tm * BM + (k & (BM - 1)), col = tn * MC_BN + 4 * (k / BM);
+  if (row >= M || col >= N) return;
+  float4* dst = reinterpret_cast<float4*>((second ? S2 : S1) + (size_t)row * ldc + col);
+  float4 s = *dst;
+  const float4* src = reinterpret_cast<const float4*>(split_ws + (size_t)blockIdx.x * kMcSplitTileFloats) + i;
+#pragma unroll 4
+  for (int g = 1; g < sp.nseg; ++g, src += (size_t)sp.rest * (kMcSplitTileFloats / 4)) {
+    const float4 v = __ldg(src);
+    s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+  }
+  *dst = s;
 }
 
 // ------------------------------------------------------------------------------- diagnostic SIMT path
@@ -556,6 +591,44 @@ static bool simt_forced() {
   return e && e[0] == '1';
 }
 
+static int device_sms() {
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+    return v;
+  return kNumSMs;
+}
+
+// How the draws of a Monte-Carlo contraction are cut.  Costs are in pairs of draws per CTA: a pair's
+// products take kblocks ring stages of about 0.27 us, and a cut adds the merge launch (about 3 us) and
+// 128 KB written and read per slot.  Cuts are of at least four pairs, so that a range's start (the
+// reference from memory) stays small beside its products.
+static McSplit mc_split_plan(int64_t M, int64_t N, int64_t k_bytes, int nb, int nsm) {
+  const int ntiles = (int)(((M + BM - 1) / BM) * ((N + MC_BN - 1) / MC_BN)), npairs = (nb + 1) / 2;
+  McSplit sp;
+  sp.whole = ntiles / nsm * nsm;
+  sp.rest = ntiles - sp.whole;
+  sp.nseg = 1;
+  sp.pairs_per_seg = npairs;
+  if (sp.rest == 0) return sp;
+  const double pair_us = 1.0 + 0.27 * (double)((k_bytes + BKB - 1) / BKB);
+  double best = npairs * pair_us;
+  for (int s = 2; s <= 32 && npairs >= 4 * s; ++s) {
+    const int per = (npairs + s - 1) / s, nseg = (npairs + per - 1) / per;
+    const int rounds = (sp.rest * nseg + nsm - 1) / nsm;
+    const double cost = (double)rounds * per * pair_us + 3.0 + 0.05 * sp.rest * (nseg - 1) + 1.0 * (rounds - 1);
+    if (cost < 0.97 * best) { best = cost; sp.nseg = nseg; sp.pairs_per_seg = per; }
+  }
+  return sp;
+}
+static size_t mc_split_bytes(const McSplit& sp) {
+  return (size_t)(sp.nseg - 1) * (size_t)sp.rest * kMcSplitTileFloats * sizeof(float);
+}
+size_t gemm_mc_split_bytes(int64_t M, int64_t N, int64_t K, bool fp8, int nb) {
+  if (M <= 0 || N <= 0 || K <= 0 || nb <= 0) return 0;
+  return mc_split_bytes(mc_split_plan(M, N, K * (fp8 ? 1 : 2), nb, device_sms()));
+}
+
 int gemm_run(const GemmArgs& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.nb <= 0) return BSP_OK;
   if (g.K <= 0) return BSP_ERR_ARG;
@@ -592,19 +665,13 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
     return BSP_OK;
   }
 
-  int nsm = kNumSMs;
-  {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-      nsm = v;
-  }
+  const int nsm = device_sms();
   CUtensorMap ma, mb;
   int rc = make_operand_map(&ma, g.A, eb, g.K, g.M, g.lda, 0, 0, BM, g.a_mn);
   if (rc != BSP_OK) return rc;
 
   if (g.mode == EPI_MC) {
-    // shifted sums resident in tensor memory over all draws of a tile
+    // shifted sums on chip over all draws of a tile
     if (g.N % 16 != 0 || !g.S1 || !g.S2) return BSP_ERR_ARG;
     rc = make_operand_map(&mb, g.B, eb, g.K, g.N, g.ldb, g.nb, g.b_batch_stride, MC_BN);
     if (rc != BSP_OK) return rc;
@@ -618,11 +685,21 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
       else BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_mc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMcSmem));
       mc_attr_set.store(true, std::memory_order_release);
     }
-    const int ntiles_mc = (int)(((g.M + BM - 1) / BM) * ((g.N + MC_BN - 1) / MC_BN));
-    const int grid_mc = ntiles_mc < nsm ? ntiles_mc : nsm;
-    if (g.fp8) gemm_mc_kernel<true><<<grid_mc, kMcThreads, kMcSmem, st>>>(ma, mb, p);
-    else gemm_mc_kernel<false><<<grid_mc, kMcThreads, kMcSmem, st>>>(ma, mb, p);
+    McSplit sp = mc_split_plan(g.M, g.N, g.K * eb, g.nb, nsm);
+    if (!g.split_ws || g.split_ws_bytes < mc_split_bytes(sp)) {      // no room: every tile takes all its draws
+      sp.whole += sp.rest;
+      sp.rest = 0;
+      sp.nseg = 1;
+    }
+    const int nunits = sp.whole + sp.rest * sp.nseg, grid_mc = nunits < nsm ? nunits : nsm;
+    if (g.fp8) gemm_mc_kernel<true><<<grid_mc, kMcThreads, kMcSmem, st>>>(ma, mb, p, sp, g.split_ws);
+    else gemm_mc_kernel<false><<<grid_mc, kMcThreads, kMcSmem, st>>>(ma, mb, p, sp, g.split_ws);
     BSP_LAUNCH_CHECK();
+    if (sp.nseg > 1) {
+      gemm_mc_merge_kernel<<<dim3((unsigned)sp.rest, 2 * BM * MC_BN / 4 / 256), 256, 0, st>>>(g.split_ws, sp, p.M, p.N, p.ldc,
+                                                                                              p.S1, p.S2);
+      BSP_LAUNCH_CHECK();
+    }
     return BSP_OK;
   }
 
@@ -759,6 +836,16 @@ int bsp_gemm(int64_t M, int64_t N, int64_t K, int elem, const void* A, int64_t l
 int bsp_linear_wgrad_mc(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t, bsp_quant_t q_dy,
                         const uint8_t* x_t_draws, bsp_quant_t q_x, int64_t ld_t, int n_draws, const float* g_ref,
                         float* S1, float* S2, bsp_diag_t* diag, void* stream) {
+  return bsp::linear_wgrad_mc_run(T, O, C, dy_codes_t, q_dy, x_t_draws, q_x, ld_t, n_draws, g_ref, S1, S2, nullptr, 0,
+                                  diag, stream);
+}
+
+}  // extern "C"
+
+// The same with room for split ranges of draws (gemm_mc_split_bytes).
+int bsp::linear_wgrad_mc_run(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t, bsp_quant_t q_dy,
+                             const uint8_t* x_t_draws, bsp_quant_t q_x, int64_t ld_t, int n_draws, const float* g_ref,
+                             float* S1, float* S2, float* split_ws, size_t split_ws_bytes, bsp_diag_t* diag, void* stream) {
   if (T < 0 || O < 0 || C < 0 || n_draws < 0 || !valid_enum(q_dy.fmt, 1) || !valid_enum(q_x.fmt, 1)) return BSP_ERR_ARG;
   if (O == 0 || C == 0 || n_draws == 0) return BSP_OK;
   if (!g_ref || !S1 || !S2) return BSP_ERR_ARG;
@@ -771,8 +858,11 @@ int bsp_linear_wgrad_mc(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes
   g.lda = ld_t; g.ldb = ld_t; g.b_batch_stride = (int64_t)C * ld_t;
   g.sa = q_dy.scale; g.sa_dev = q_dy.scale_dev; g.sb = q_x.scale; g.sb_dev = q_x.scale_dev;
   g.mode = EPI_MC; g.C = nullptr; g.ldc = C; g.ref = g_ref; g.S1 = S1; g.S2 = S2; g.diag = diag;
+  g.split_ws = split_ws; g.split_ws_bytes = split_ws_bytes;
   return gemm_run(g, (cudaStream_t)stream);
 }
+
+extern "C" {
 
 size_t bsp_linear_dgrad_workspace_bytes(int64_t T, int64_t O, int64_t C) {
   if (T <= 0 || O <= 0 || C <= 0) return 0;

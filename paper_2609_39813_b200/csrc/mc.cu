@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "gemm.cuh"
 #include "mc_stats.cuh"
 #include "tc.cuh"
 
@@ -188,7 +189,8 @@ struct CheckBuffers {
   float *dg_ref, *db_ref, *dg_pol, *S1g, *S2g, *dx;
   float *dW_ref, *dW_pol, *S2w;
   void *ws_bwd, *ws_gain, *ws_wgrad, *ws_dgrad, *ws_stats;
-  size_t b_bwd, b_gain, b_wgrad, b_dgrad, b_stats;
+  size_t b_bwd, b_gain, b_wgrad, b_dgrad, b_stats, b_split;
+  float* ws_split;
   int64_t ld_t;
 };
 
@@ -219,6 +221,14 @@ static size_t carve(const bsp_norm_linear_desc_t* op, int K, char* base, CheckBu
   c.b_stats = kMaxPendingStats * kStatSlotBytes;
   c.ws_bwd = b.take(c.b_bwd); c.ws_gain = b.take(c.b_gain); c.ws_wgrad = b.take(c.b_wgrad);
   c.ws_dgrad = b.take(c.b_dgrad); c.ws_stats = b.take(c.b_stats);
+  // split ranges of draws: the whole chunks and a last, shorter one may be cut differently
+  const int chunk = draw_chunk((int64_t)C, (int64_t)ld_t, K > 0 ? K : 1, op->draw_buffer_bytes);
+  c.b_split = gemm_mc_split_bytes(op->O, op->C, op->T, true, chunk);
+  if (K % chunk) {
+    const size_t last = gemm_mc_split_bytes(op->O, op->C, op->T, true, K % chunk);
+    if (last > c.b_split) c.b_split = last;
+  }
+  c.ws_split = (float*)b.take(c.b_split);
   if (cb) *cb = c;
   return b.off;
 }
@@ -488,8 +498,8 @@ int bsp_mc_check(const bsp_norm_linear_desc_t* op, int K, const bsp_verdict_rule
           BSP_CHECK_CUDA(cudaEventCreateWithFlags(&sw.join, cudaEventDisableTiming));
           BSP_CHECK_CUDA(cudaEventRecord(sw.fork, st));
         }
-        BSP_TRY(bsp_linear_wgrad_mc(T, O, C, b.dy_codes_t, qdy, b.fresh_t, qf, b.ld_t, nd, b.dW_ref, S1w, b.S2w, diag,
-                                    st));
+        BSP_TRY(linear_wgrad_mc_run(T, O, C, b.dy_codes_t, qdy, b.fresh_t, qf, b.ld_t, nd, b.dW_ref, S1w, b.S2w,
+                                    b.ws_split, b.b_split, diag, st));
         if (overlap_gain && k0 == 0) {
           // the contraction is queued first, so its CTAs take the SMs first; the gain blocks fill in
           BSP_CHECK_CUDA(cudaStreamWaitEvent(sw.side, sw.fork, 0));

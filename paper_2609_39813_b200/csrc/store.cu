@@ -317,7 +317,8 @@ struct StoreBuffers {
   float *dg_ref, *db_ref, *dg_pol, *S1g, *S2g, *dx, *zero_c;
   float *dW_ref, *dW_pol, *S1w, *S2w;
   void *ws_bwd, *ws_gain, *ws_dgrad, *ws_stats;
-  size_t b_bwd, b_gain, b_dgrad, b_stats;
+  size_t b_bwd, b_gain, b_dgrad, b_stats, b_split;
+  float* ws_split;
   int64_t ld_t;
 };
 
@@ -360,6 +361,13 @@ static size_t store_carve(const bsp_store_desc_t* op, int K, char* base, StoreBu
   c.b_dgrad = bsp_linear_dgrad_workspace_bytes(op->T, op->O, op->C);
   c.b_stats = kMaxPendingStats * kStatSlotBytes;
   c.ws_bwd = take(c.b_bwd); c.ws_gain = take(c.b_gain); c.ws_dgrad = take(c.b_dgrad); c.ws_stats = take(c.b_stats);
+  // split ranges of draws: the whole chunks and a last, shorter one may be cut differently
+  c.b_split = gemm_mc_split_bytes(op->O, op->C, op->T, false, c.chunk);
+  if (K > 0 && K % c.chunk) {
+    const size_t last = gemm_mc_split_bytes(op->O, op->C, op->T, false, K % c.chunk);
+    if (last > c.b_split) c.b_split = last;
+  }
+  c.ws_split = (float*)take(c.b_split);
   if (out) *out = c;
   return off;
 }
@@ -575,6 +583,7 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
         g.A = b.dys_t; g.B = b.diff_t; g.lda = b.ld_t; g.ldb = b.ld_t; g.b_batch_stride = (int64_t)C * b.ld_t;
         g.sa = 1.f; g.sa_dev = b.scale_dy; g.sb = 1.f; g.sb_dev = nullptr;
         g.mode = EPI_MC; g.ldc = C; g.ref = nullptr; g.S1 = b.S1w; g.S2 = b.S2w; g.diag = diag;
+        g.split_ws = b.ws_split; g.split_ws_bytes = b.b_split;
         BSP_TRY(gemm_run(g, st));
       }
       BSP_TRY(pend.add(b.dW_ref, b.S1w, b.S2w, O * C, K, 1,

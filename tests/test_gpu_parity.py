@@ -309,6 +309,31 @@ def test_weight_gradient_three_reads(b, case, policy):
     assert rel_l2(down(dW).reshape(O, C), want) <= TOL_TC
 
 
+# the check may cut a contraction's draws into ranges (few tiles, or a last partial wave of them) and
+# merge the ranges' sums; bsp_linear_wgrad_mc, which has no workspace, walks them in one go
+@pytest.mark.parametrize("T,C,O,K", [(64, 128, 128, 41), (80, 272, 400, 32), (48, 128, 272, 9), (33, 2064, 1168, 20)])
+def test_split_draws_equal_one_walk(b, T, C, O, K):
+    inp = workloads.config1(T=T, C=C, O=O, K=K, seed=6)
+    g = NormLinearGpu(inp)
+    desc = g.desc(0x30)                                  # weight use: the forward's read and fresh reads
+    ws = b.workspace(b.bsp_mc_check_workspace_bytes(desc, K))
+    diag = b.new_diag()
+    b.bsp_mc_check(desc, K, ws, diag)
+    assert b.read_diag(diag)["status"] == 0
+    lay = b.bsp_mc_check_layout(desc, K)
+    ref, S1, S2 = (b.ws_view(ws, off, O * C).clone() for off in (lay.dW_ref, lay.dW_S1, lay.dW_S2))
+    q = b.quant(inp.store_fmt, b.ROUND_STOCHASTIC, 1.0, g.scale)
+    fresh = torch.zeros(K * C * g.ld_t, dtype=torch.uint8, device="cuda")
+    b.bsp_norm_fwd_draws(g.kind, g.x, T, C, g.gamma, g.beta, g.rstd, g.mean, q,
+                         b.key(inp.seed, g.tensor_id, b.STREAM_WGRAD, 0), 0, K, fresh, g.ld_t)
+    one1, one2 = torch.zeros_like(S1), torch.zeros_like(S2)
+    b.bsp_linear_wgrad_mc(T, O, C, g.dy_codes_t, g.q_dy, fresh, q, g.ld_t, K, ref, one1, one2, diag)
+    # the same FP32 terms, added in another order: K roundings of the sums of their magnitudes
+    tol = K * 2.0 ** -24
+    assert float((S2 - one2).abs().max()) <= tol * float(one2.max())
+    assert float((S1 - one1).abs().max()) <= tol * float((K * one2).sqrt().max())
+
+
 def test_weight_gradient_fused_monte_carlo_epilogue(b, case):
     inp, g, kind, prep = case
     T, C, O, K = inp.T, inp.C, inp.O, 6
