@@ -2,10 +2,12 @@
 // both operands K-major (K contiguous), FP8 (kind::f8f6f4, E5M2/E4M3 in any combination) or BF16
 // (kind::f16) operands and FP32 accumulation in tensor memory.
 //
-// One persistent CTA per SM, 192 threads:
+// One persistent CTA per SM, 320 threads:
 //   warp 0      TMA producer   (cp.async.bulk.tensor, 128-byte swizzle, kStages-deep mbarrier ring)
 //   warp 1      MMA issuer     (one elected lane issues tcgen05.mma 128 x 256 x 32B; owns TMEM alloc)
-//   warps 2..5  epilogue       (tcgen05.ld 32 lanes x 32 columns -> registers -> global)
+//   warps 2..9  epilogue       (tcgen05.ld 32 lanes x 32 columns -> registers -> global; two warps per
+//               lane quarter take every other 32 columns: with one, a tile of a short contraction (K of
+//               1024 and below) spent longer in its epilogue than in its products)
 // Two accumulator stages (2 x 256 TMEM columns) let the epilogue of one tile overlap the main loop
 // of the next.  Work items are (tile, batch): a CTA owns its tiles and walks all batches of a tile
 // in order, so the Monte-Carlo epilogue's read-modify-write of the shifted sums is race-free and
@@ -26,15 +28,15 @@ namespace bsp {
 constexpr int BM = 128, BN = 256, BKB = 128;      // tile; BKB = K extent of one stage in bytes
 constexpr int kStages = 4;
 constexpr int kABytes = BM * BKB, kBBytes = BN * BKB, kStageBytes = kABytes + kBBytes;
-constexpr int kGemmThreads = 192;
+constexpr int kGemmThreads = 320;
 constexpr int kTmemCols = 512;
-constexpr int kEpiStage = 4 * 4096;              // one 32-row x 128-byte staging block per epilogue warp
+constexpr int kEpiStage = 8 * 4096;              // one 32-row x 128-byte staging block per epilogue warp
 constexpr size_t kGemmSmem = (size_t)kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kEpiStage;
 
 struct GemmParams {
   int M, N, K;            // K in elements
+  int bn;                 // gemm_tc_kernel: tile columns (see tile_columns)
   int nb;                 // batches of B (and of C in plain mode)
-  int elem_bytes;         // 1 (FP8) or 2 (BF16)
   int a_mn, b_mn;         // operand stored [K][M] / [K][N] (MN-major) instead of [M][K] / [N][K]
   uint32_t idesc;
   uint32_t idesc2;               // gemm_mc_kernel: the 128 x 256 product over a pair of draws
@@ -47,6 +49,10 @@ struct GemmParams {
   const float* ref;       // EPI_MC
   float* S1;
   float* S2;
+  uint16_t* split;        // EPI_SPLIT
+  uint16_t* diff;
+  float moment_scale;     // EPI_MOMENTS
+  int moment_first;
   bsp_diag_t* diag;
 };
 
@@ -65,9 +71,18 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
   tn = c0 + idx - tm * wb;
 }
 
-template <bool FP8>
+// Four values as two bf16 terms each, packed in pairs: v = hi + lo to 16 bits.
+__device__ __forceinline__ void split4(const float4& v, uint2& hi, uint2& lo) {
+  const uint32_t h0 = float_to_bf16_bits(v.x), h1 = float_to_bf16_bits(v.y), h2 = float_to_bf16_bits(v.z), h3 = float_to_bf16_bits(v.w);
+  hi = make_uint2(h0 | (h1 << 16), h2 | (h3 << 16));
+  lo = make_uint2(float_to_bf16_bits(v.x - bf16_bits_to_float(h0)) | (float_to_bf16_bits(v.y - bf16_bits_to_float(h1)) << 16),
+                  float_to_bf16_bits(v.z - bf16_bits_to_float(h2)) | (float_to_bf16_bits(v.w - bf16_bits_to_float(h3)) << 16));
+}
+
+template <bool FP8, int MODE>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p) {
+  constexpr int kElem = FP8 ? 1 : 2, bk_elems = BKB / kElem, kAtom = 128 / kElem;   // elements per 128 bytes
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;                    // 1024-byte aligned operand ring
@@ -80,14 +95,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 16 * kStages + 36);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tiles_m = (p.M + BM - 1) / BM, tiles_n = (p.N + BN - 1) / BN;
+  const int tiles_m = (p.M + BM - 1) / BM, tiles_n = (p.N + p.bn - 1) / p.bn;
   const int ntiles = tiles_m * tiles_n;
-  const int kblocks = (p.K * p.elem_bytes + BKB - 1) / BKB;
-  const int bk_elems = BKB / p.elem_bytes;
+  const int kblocks = (p.K * kElem + BKB - 1) / BKB;
+  // an MN-major B comes in atoms of 128 bytes of N: the last one may reach past the tile's columns
+  const int b_atoms = (p.bn * kElem + 127) / 128, b_bytes = p.b_mn ? b_atoms * bk_elems * 128 : p.bn * BKB;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, 4); }
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, 8); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -113,20 +129,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             const uint32_t s = it % kStages, ph = (it / kStages) & 1u;
             if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
             const uint32_t sa = tiles + s * kStageBytes, sb = sa + kABytes;
-            mbar_expect_tx(full0 + 8 * s, kStageBytes);
+            mbar_expect_tx(full0 + 8 * s, kABytes + b_bytes);
             if (!p.a_mn) {
               tma_load_2d(sa, &tmap_a, full0 + 8 * s, kb * bk_elems, tm * BM);
             } else {
               // one box per 128 bytes of M: [bk_elems k rows][128 B]
-              for (int a = 0; a < BM * p.elem_bytes / 128; ++a)
-                tma_load_2d(sa + a * bk_elems * 128, &tmap_a, full0 + 8 * s, tm * BM + a * (128 / p.elem_bytes),
+              #pragma unroll
+              for (int a = 0; a < BM / kAtom; ++a)
+                tma_load_2d(sa + a * bk_elems * 128, &tmap_a, full0 + 8 * s, tm * BM + a * kAtom,
                             kb * bk_elems);
             }
             if (!p.b_mn) {
-              tma_load_3d(sb, &tmap_b, full0 + 8 * s, kb * bk_elems, tn * BN, b);
+              tma_load_3d(sb, &tmap_b, full0 + 8 * s, kb * bk_elems, tn * p.bn, b);
             } else {
-              for (int a = 0; a < BN * p.elem_bytes / 128; ++a)
-                tma_load_3d(sb + a * bk_elems * 128, &tmap_b, full0 + 8 * s, tn * BN + a * (128 / p.elem_bytes),
+              #pragma unroll
+              for (int a = 0; a < BN / kAtom; ++a)
+                if (a < b_atoms)
+                tma_load_3d(sb + a * bk_elems * 128, &tmap_b, full0 + 8 * s, tn * p.bn + a * kAtom,
                             kb * bk_elems, b);
             }
           }
@@ -156,7 +175,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             // K-major: one MMA advances 32 bytes along K inside the swizzle atom (+2 in 16-byte
             // units).  MN-major: it advances 32/elem_bytes k rows of 128 bytes.
             const uint32_t atom_bytes = (uint32_t)bk_elems * 128u;
-            const uint32_t mn_step = (32u / (uint32_t)p.elem_bytes) * 128u >> 4;
+            const uint32_t mn_step = (32u / (uint32_t)kElem) * 128u >> 4;
             const uint64_t adesc = p.a_mn ? make_smem_desc_mn(sa, atom_bytes) : make_smem_desc(sa);
             const uint64_t bdesc = p.b_mn ? make_smem_desc_mn(sb, atom_bytes) : make_smem_desc(sb);
             const uint32_t astep = p.a_mn ? mn_step : 2u, bstep = p.b_mn ? mn_step : 2u;
@@ -170,7 +189,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       }
     }
   } else {
-    // ------------------------------------------------ epilogue (warps 2..5)
+    // ------------------------------------------------ epilogue (warps 2..9)
     const int q = warp & 3;                      // TMEM lane quarter this warp may access
     const float inv_a = __fdiv_rn(1.0f, p.sa_dev ? __ldg(p.sa_dev) : p.sa);
     const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? __ldg(p.sb_dev) : p.sb);
@@ -180,20 +199,36 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       int tm, tn;
       tile_coords(t, tiles_m, tiles_n, tm, tn);
       const int row = tm * BM + q * 32 + lane;
+      const int nlim = p.N < (tn + 1) * p.bn ? p.N : (tn + 1) * p.bn;   // columns from here on are not this tile's
       for (int b = 0; b < p.nb && ok; ++b, ++tc) {
         const uint32_t as = tc & 1u, aph = (tc >> 1) & 1u;
         // every lane polls; the outcome is made warp-uniform before any .aligned instruction
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(tfull0 + 8 * as, aph, abort_flag));
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait_suspend(tfull0 + 8 * as, aph, abort_flag));
         if (!ok) break;
         tc_fence_after();
         const uint32_t taddr = tmem_base + as * BN + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
-        for (int ch = 0; ch < BN / 32; ++ch) {
-          const int col0 = tn * BN + ch * 32;
-          if (col0 >= p.N) break;                // warp-uniform
+        for (int ch = (warp - 2) >> 2; ch < BN / 32; ch += 2) {
+          const int col0 = tn * p.bn + ch * 32;
+          if (col0 >= nlim) break;               // warp-uniform
           uint32_t r[32];
+          // what the warp will write goes row by row (row 4 t + lane / 8, four columns from 4 (lane % 8)); the
+          // values that an epilogue reads back there are fetched before the accumulator
+          constexpr bool by_rows = MODE != EPI_STORE_BF16;
+          const int row8 = tm * BM + q * 32 + (lane >> 3), col4 = col0 + 4 * (lane & 7);
+          float4 old1[8], old2[8];
+          const bool reads1 = (MODE == EPI_SPLIT && p.ref) || (MODE == EPI_MOMENTS && !p.moment_first);
+          if (reads1) {
+            const float* src = MODE == EPI_SPLIT ? p.ref : p.S1;
+#pragma unroll
+            for (int t8 = 0; t8 < 8; ++t8)
+              if (row8 + 4 * t8 < p.M && col4 < nlim) {
+                old1[t8] = *reinterpret_cast<const float4*>(src + (size_t)(row8 + 4 * t8) * p.ldc + col4);
+                if (MODE == EPI_MOMENTS) old2[t8] = *reinterpret_cast<const float4*>(p.S2 + (size_t)(row8 + 4 * t8) * p.ldc + col4);
+              }
+          }
           tmem_ld32(taddr + ch * 32, r);
-          if (p.mode == EPI_STORE_F32) {
+          if (by_rows) {
             // A lane holds 128 bytes of its own row; written as they are, a warp's store touches 32
             // rows with 16 bytes each.  Through the warp's 4 KB staging block the warp instead writes
             // four rows of 128 contiguous bytes per instruction (row 4 t + lane / 8, chunk lane % 8).
@@ -214,19 +249,45 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                            : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w)
                            : "r"(wb + (uint32_t)rl * 128u + ((uint32_t)(c4 ^ (rl & 7)) << 4)));
               const int orow = tm * BM + q * 32 + rl, ocol = col0 + 4 * c4;
-              if (orow < p.M && ocol < p.N) *reinterpret_cast<float4*>(cbase + (size_t)orow * p.ldc + ocol) = o;
+              if (orow < p.M && ocol < nlim) {
+                const size_t off = (size_t)orow * p.ldc + ocol;
+                if (MODE == EPI_STORE_F32) {
+                  *reinterpret_cast<float4*>(cbase + off) = o;
+                } else if (MODE == EPI_SPLIT) {
+                  if (p.C) *reinterpret_cast<float4*>(cbase + off) = o;
+                  uint2 hi, lo;
+                  split4(o, hi, lo);
+                  uint16_t* sp = p.split + (size_t)orow * 2 * p.N + ocol;
+                  *reinterpret_cast<uint2*>(sp) = hi;
+                  *reinterpret_cast<uint2*>(sp + p.N) = lo;
+                  if (p.ref) {
+                    const float4 a = old1[t8];
+                    split4(make_float4(a.x - o.x, a.y - o.y, a.z - o.z, a.w - o.w), hi, lo);
+                    uint16_t* df = p.diff + (size_t)orow * p.N + ocol;
+                    *reinterpret_cast<uint2*>(df) = hi;
+                    *reinterpret_cast<uint2*>(df + (size_t)p.M * p.N) = lo;
+                  }
+                } else {
+                  const float f = p.moment_scale;
+                  float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b2 = a;
+                  if (!p.moment_first) { a = old1[t8]; b2 = old2[t8]; }
+                  a.x = fmaf(f, o.x, a.x); a.y = fmaf(f, o.y, a.y); a.z = fmaf(f, o.z, a.z); a.w = fmaf(f, o.w, a.w);
+                  b2.x = fmaf(f * o.x, o.x, b2.x); b2.y = fmaf(f * o.y, o.y, b2.y);
+                  b2.z = fmaf(f * o.z, o.z, b2.z); b2.w = fmaf(f * o.w, o.w, b2.w);
+                  *reinterpret_cast<float4*>(p.S1 + off) = a;
+                  *reinterpret_cast<float4*>(p.S2 + off) = b2;
+                }
+              }
             }
             __syncwarp();
           }
           if (row < p.M) {
             const size_t off = (size_t)row * p.ldc + col0;
-            if (p.mode == EPI_STORE_F32) {
-              // (stored above, by the warp together)
-            } else if (p.mode == EPI_STORE_BF16) {
+            if (!by_rows) {
               uint16_t* dst = reinterpret_cast<uint16_t*>(p.C) + (size_t)b * p.M * p.ldc + off;
 #pragma unroll
               for (int j = 0; j < 32; j += 4) {
-                if (col0 + j < p.N) {
+                if (col0 + j < nlim) {
                   const uint32_t lo = float_to_bf16_bits(__uint_as_float(r[j]) * inv_a * inv_b) |
                                       (float_to_bf16_bits(__uint_as_float(r[j + 1]) * inv_a * inv_b) << 16);
                   const uint32_t hi = float_to_bf16_bits(__uint_as_float(r[j + 2]) * inv_a * inv_b) |
@@ -422,7 +483,7 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       // ---- the unit's draws
       for (int pr = p0; pr < p1 && ok; ++pr, ++tc) {
         const uint32_t as = tc & 1u, aph = (tc >> 1) & 1u;
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(tfull0 + 8 * as, aph, abort_flag));
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait_suspend(tfull0 + 8 * as, aph, abort_flag));
         if (!ok) break;
         tc_fence_after();
         const uint32_t acc_base = lane_base + as * 2 * MC_BN;  // draw 2 pr; draw 2 pr + 1 is MC_BN columns further
@@ -524,14 +585,14 @@ gemm_simt_kernel(const void* __restrict__ A, const void* __restrict__ B, int a_f
     const int mr = blockIdx.y * 16 + ty, nr = blockIdx.x * 16 + ty;
     if (mr < p.M && ka < p.K) {
       if (FP8) {
-        const uint32_t c = reinterpret_cast<const uint8_t*>(A)[(size_t)mr * lda + ka];
+        const uint32_t c = reinterpret_cast<const uint8_t*>(A)[p.a_mn ? (size_t)ka * lda + mr : (size_t)mr * lda + ka];
         av = a_fmt == BSP_E4M3 ? f8_decode<BSP_E4M3>(c) : f8_decode<BSP_E5M2>(c);
       } else {
-        av = bf16_bits_to_float(reinterpret_cast<const uint16_t*>(A)[(size_t)mr * lda + ka]);
+        av = bf16_bits_to_float(reinterpret_cast<const uint16_t*>(A)[p.a_mn ? (size_t)ka * lda + mr : (size_t)mr * lda + ka]);
       }
     }
     if (nr < p.N && ka < p.K) {
-      const size_t idx = (size_t)b * b_batch_stride + (size_t)nr * ldb + ka;
+      const size_t idx = (size_t)b * b_batch_stride + (p.b_mn ? (size_t)ka * ldb + nr : (size_t)nr * ldb + ka);
       if (FP8) {
         const uint32_t c = reinterpret_cast<const uint8_t*>(B)[idx];
         bv = b_fmt == BSP_E4M3 ? f8_decode<BSP_E4M3>(c) : f8_decode<BSP_E5M2>(c);
@@ -553,6 +614,21 @@ gemm_simt_kernel(const void* __restrict__ A, const void* __restrict__ B, int a_f
       reinterpret_cast<float*>(p.C)[(size_t)b * p.M * p.ldc + off] = v;
     } else if (p.mode == EPI_STORE_BF16) {
       reinterpret_cast<uint16_t*>(p.C)[(size_t)b * p.M * p.ldc + off] = (uint16_t)float_to_bf16_bits(v);
+    } else if (p.mode == EPI_SPLIT) {
+      if (p.C) reinterpret_cast<float*>(p.C)[off] = v;
+      const uint32_t hi = float_to_bf16_bits(v);
+      p.split[(size_t)m * 2 * p.N + n] = (uint16_t)hi;
+      p.split[(size_t)m * 2 * p.N + p.N + n] = (uint16_t)float_to_bf16_bits(v - bf16_bits_to_float(hi));
+      if (p.ref) {
+        const float e = p.ref[off] - v;
+        const uint32_t eh = float_to_bf16_bits(e);
+        p.diff[(size_t)m * p.N + n] = (uint16_t)eh;
+        p.diff[(size_t)(p.M + m) * p.N + n] = (uint16_t)float_to_bf16_bits(e - bf16_bits_to_float(eh));
+      }
+    } else if (p.mode == EPI_MOMENTS) {
+      const float f = p.moment_scale;
+      p.S1[off] = fmaf(f, v, p.moment_first ? 0.f : p.S1[off]);
+      p.S2[off] = fmaf(f * v, v, p.moment_first ? 0.f : p.S2[off]);
     } else {
       const float d = v - (p.ref ? p.ref[off] : 0.f);
       p.S1[off] += d;
@@ -599,6 +675,25 @@ static int device_sms() {
   return kNumSMs;
 }
 
+// Columns of a plain contraction's tile, 64 .. 256 in steps of 16.  The time goes with the number of rounds
+// the tiles take over the SMs times what a tile costs: per 32 bytes of K the product's bn / 2 cycles or, with
+// every SM loading, the (128 + bn) * 32 bytes of its operands at the 80 bytes per cycle and SM that L2 was
+// seen to give (256 columns reach 0.83 of the tensor rate, 128 columns 0.6), and the epilogue of the last
+// tile (about 12 cycles a column).  256 columns unless fewer save a twentieth (3001 x 1552 x 4112 bf16: 144 columns, 66 -> 54 us).
+static int tile_columns(int64_t M, int64_t N, int64_t k_bytes, int nsm) {
+  const int64_t tm = (M + BM - 1) / BM, slices = (k_bytes + 31) / 32;
+  int best = BN;
+  double best_cost = 0.0;
+  for (int bn = BN; bn >= 64; bn -= 16) {
+    const int64_t rounds = (tm * ((N + bn - 1) / bn) + nsm - 1) / nsm;
+    const double slice = bn / 2.0 > 0.4 * (128 + bn) ? bn / 2.0 : 0.4 * (128 + bn);
+    const double cost = (double)rounds * (double)slices * slice + 12.0 * bn;
+    if (bn == BN) best_cost = cost;
+    else if (cost < 0.95 * best_cost) { best_cost = cost; best = bn; }
+  }
+  return best;
+}
+
 // How the draws of a Monte-Carlo contraction are cut.  Costs are in pairs of draws per CTA: a pair's
 // products take kblocks ring stages of about 0.27 us, and a cut adds the merge launch (about 3 us) and
 // 128 KB written and read per slot.  Cuts are of at least four pairs, so that a range's start (the
@@ -629,6 +724,20 @@ size_t gemm_mc_split_bytes(int64_t M, int64_t N, int64_t K, bool fp8, int nb) {
   return mc_split_bytes(mc_split_plan(M, N, K * (fp8 ? 1 : 2), nb, device_sms()));
 }
 
+template <bool FP8, int MODE>
+static int gemm_tc_launch(const CUtensorMap& ma, const CUtensorMap& mb, const GemmParams& p, int nsm, cudaStream_t st) {
+  static std::atomic<bool> attr_set_dev[kMaxDevices];
+  std::atomic<bool>& attr_set = attr_set_dev[device_slot()];
+  if (!attr_set.load(std::memory_order_acquire)) {
+    BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<FP8, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
+    attr_set.store(true, std::memory_order_release);
+  }
+  const int ntiles = ((p.M + BM - 1) / BM) * ((p.N + p.bn - 1) / p.bn);
+  gemm_tc_kernel<FP8, MODE><<<ntiles < nsm ? ntiles : nsm, kGemmThreads, kGemmSmem, st>>>(ma, mb, p);
+  BSP_LAUNCH_CHECK();
+  return BSP_OK;
+}
+
 int gemm_run(const GemmArgs& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.nb <= 0) return BSP_OK;
   if (g.K <= 0) return BSP_ERR_ARG;
@@ -638,14 +747,14 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
     return BSP_ERR_ALIGN;
   if ((g.b_batch_stride * eb) % 16 != 0) return BSP_ERR_ALIGN;
   GemmParams p;
-  p.M = (int)g.M; p.N = (int)g.N; p.K = (int)g.K; p.nb = g.nb; p.elem_bytes = eb;
+  p.M = (int)g.M; p.N = (int)g.N; p.K = (int)g.K; p.nb = g.nb;
   p.a_mn = g.a_mn ? 1 : 0; p.b_mn = g.b_mn ? 1 : 0;
-  p.idesc = g.fp8 ? make_idesc(g.a_fmt == BSP_E5M2 ? 1u : 0u, g.b_fmt == BSP_E5M2 ? 1u : 0u, BM, BN)
-                  : make_idesc(1u, 1u, BM, BN);
-  p.idesc |= (g.a_mn ? 1u << 15 : 0u) | (g.b_mn ? 1u << 16 : 0u);     // operand major bits
-  if ((g.a_mn || g.b_mn) && (g.mode == EPI_MC || simt_forced())) return BSP_ERR_UNSUPPORTED;
+  p.idesc = 0u; p.idesc2 = 0u; p.bn = BN;
+  if ((g.a_mn || g.b_mn) && g.mode == EPI_MC) return BSP_ERR_UNSUPPORTED;
+  if (g.mode >= EPI_SPLIT && g.nb != 1) return BSP_ERR_UNSUPPORTED;
   p.sa = g.sa; p.sb = g.sb; p.sa_dev = g.sa_dev; p.sb_dev = g.sb_dev;
   p.mode = g.mode; p.C = g.C; p.ldc = g.ldc; p.ref = g.ref; p.S1 = g.S1; p.S2 = g.S2; p.diag = g.diag;
+  p.split = g.split; p.diff = g.diff; p.moment_scale = g.moment_scale; p.moment_first = g.moment_first ? 1 : 0;
 
   if (simt_forced()) {
     dim3 grid((unsigned)((g.N + 15) / 16), (unsigned)((g.M + 15) / 16), (unsigned)g.nb);
@@ -703,21 +812,19 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
     return BSP_OK;
   }
 
-  rc = make_operand_map(&mb, g.B, eb, g.K, g.N, g.ldb, g.nb, g.b_batch_stride, BN, g.b_mn);
+  p.bn = tile_columns(g.M, g.N, g.K * eb, nsm);
+  const uint32_t fa = g.fp8 ? (g.a_fmt == BSP_E5M2 ? 1u : 0u) : 1u, fb = g.fp8 ? (g.b_fmt == BSP_E5M2 ? 1u : 0u) : 1u;
+  p.idesc = make_idesc(fa, fb, BM, (uint32_t)p.bn) | (g.a_mn ? 1u << 15 : 0u) | (g.b_mn ? 1u << 16 : 0u);   // operand major bits
+  rc = make_operand_map(&mb, g.B, eb, g.K, g.N, g.ldb, g.nb, g.b_batch_stride, p.bn, g.b_mn);
   if (rc != BSP_OK) return rc;
-  static std::atomic<bool> attr_set_dev[kMaxDevices][2];
-  std::atomic<bool>* attr_set = attr_set_dev[device_slot()];
-  if (!attr_set[g.fp8 ? 1 : 0].load(std::memory_order_acquire)) {
-    if (g.fp8) BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
-    else BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
-    attr_set[g.fp8 ? 1 : 0].store(true, std::memory_order_release);
+  if (g.fp8) return g.mode == EPI_STORE_F32 ? gemm_tc_launch<true, EPI_STORE_F32>(ma, mb, p, nsm, st) : BSP_ERR_UNSUPPORTED;
+  switch (g.mode) {
+    case EPI_STORE_F32: return gemm_tc_launch<false, EPI_STORE_F32>(ma, mb, p, nsm, st);
+    case EPI_STORE_BF16: return gemm_tc_launch<false, EPI_STORE_BF16>(ma, mb, p, nsm, st);
+    case EPI_SPLIT: return gemm_tc_launch<false, EPI_SPLIT>(ma, mb, p, nsm, st);
+    case EPI_MOMENTS: return gemm_tc_launch<false, EPI_MOMENTS>(ma, mb, p, nsm, st);
+    default: return BSP_ERR_UNSUPPORTED;
   }
-  const int ntiles = (int)(((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN));
-  const int grid = ntiles < nsm ? ntiles : nsm;
-  if (g.fp8) gemm_tc_kernel<true><<<grid, kGemmThreads, kGemmSmem, st>>>(ma, mb, p);
-  else gemm_tc_kernel<false><<<grid, kGemmThreads, kGemmSmem, st>>>(ma, mb, p);
-  BSP_LAUNCH_CHECK();
-  return BSP_OK;
 }
 
 // ------------------------------------------------------------------------------- operand preparation

@@ -9,10 +9,13 @@
 
 namespace bsp {
 
-enum { EPI_STORE_F32 = 0, EPI_STORE_BF16 = 1, EPI_MC = 2 };
+enum { EPI_STORE_F32 = 0, EPI_STORE_BF16 = 1, EPI_MC = 2, EPI_SPLIT = 3, EPI_MOMENTS = 4 };
 
 // C[b][M][ldc] = alpha * A[M][K] * B[b][N][K]^T, alpha = (1/sa) * (1/sb); operands K-major.
 // EPI_MC: S1 += C - ref, S2 += (C - ref)^2 for every batch in order (single [M][ldc] buffers).
+// EPI_SPLIT: the result as two bf16 terms side by side, split[M][2 N] = hi | lo, besides C when given;
+// with ref also the terms of ref - C below each other, diff[2 M][N].
+// EPI_MOMENTS: S1 += f C, S2 += f C^2 with f = moment_scale, or without the sums so far (moment_first).
 struct GemmArgs {
   int64_t M = 0, N = 0, K = 0;
   int nb = 1;
@@ -32,6 +35,10 @@ struct GemmArgs {
   const float* ref = nullptr;
   float* S1 = nullptr;
   float* S2 = nullptr;
+  uint16_t* split = nullptr;
+  uint16_t* diff = nullptr;
+  float moment_scale = 1.f;
+  bool moment_first = false;
   float* split_ws = nullptr;           // EPI_MC: room for split ranges of draws (gemm_mc_split_bytes), or none
   size_t split_ws_bytes = 0;
   bsp_diag_t* diag = nullptr;
