@@ -274,6 +274,15 @@ __device__ __forceinline__ void f8_decode4(uint32_t packed, float (&out)[4]) {
   out[0] = a.x; out[1] = a.y; out[2] = b.x; out[3] = b.y;
 }
 
+// Four codes to four bf16 values (exact: every FP8 value is a bf16 value, the upper half of its FP32).
+template <int FMT>
+__device__ __forceinline__ uint2 f8_to_bf16x4(uint32_t packed) {
+  float v[4];
+  f8_decode4<FMT>(packed, v);
+  return make_uint2(__byte_perm(__float_as_uint(v[0]), __float_as_uint(v[1]), 0x7632),
+                    __byte_perm(__float_as_uint(v[2]), __float_as_uint(v[3]), 0x7632));
+}
+
 __device__ __forceinline__ void diag_flush(bsp_diag_t* diag, const DiagCounters& dc) {
   if (diag == nullptr) return;
   if (dc.sat) atomicAdd(&diag->n_saturated, (unsigned long long)dc.sat);

@@ -829,26 +829,29 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
 
 // ------------------------------------------------------------------------------- operand preparation
 
-// codes -> bf16 (exact: every FP8 value is a bf16 value), same layout.
+// codes -> bf16 (exact), same layout; sixteen codes per thread through the hardware conversions
+// (bound by its 3 B per code; field by field it was bound by instructions; 180 M codes: 146 -> 95 us).
 template <int FMT>
-__global__ void decode_to_bf16_kernel(const uint8_t* __restrict__ codes, size_t n16, uint16_t* __restrict__ out) {
+__global__ void __launch_bounds__(256)
+decode_to_bf16_kernel(const uint8_t* __restrict__ codes, size_t n16, uint16_t* __restrict__ out) {
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n16) return;
   const uint4 c = __ldg(reinterpret_cast<const uint4*>(codes) + t);
-  const uint32_t w[4] = {c.x, c.y, c.z, c.w};
-  uint32_t o[8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t b0 = __float_as_uint(f8_decode<FMT>(w[i] & 0xFFu)) >> 16;
-    const uint32_t b1 = __float_as_uint(f8_decode<FMT>((w[i] >> 8) & 0xFFu)) >> 16;
-    const uint32_t b2 = __float_as_uint(f8_decode<FMT>((w[i] >> 16) & 0xFFu)) >> 16;
-    const uint32_t b3 = __float_as_uint(f8_decode<FMT>(w[i] >> 24)) >> 16;
-    o[2 * i] = b0 | (b1 << 16);
-    o[2 * i + 1] = b2 | (b3 << 16);
-  }
+  const uint2 a = f8_to_bf16x4<FMT>(c.x), b = f8_to_bf16x4<FMT>(c.y), d = f8_to_bf16x4<FMT>(c.z), e = f8_to_bf16x4<FMT>(c.w);
   uint4* dst = reinterpret_cast<uint4*>(out) + 2 * t;
-  dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-  dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+  dst[0] = make_uint4(a.x, a.y, b.x, b.y);
+  dst[1] = make_uint4(d.x, d.y, e.x, e.y);
+}
+
+// FP32 -> bf16, same layout.
+__global__ void __launch_bounds__(256)
+to_bf16_kernel(const float* __restrict__ in, size_t n8, uint16_t* __restrict__ out) {
+  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n8) return;
+  const float4 a = __ldg(reinterpret_cast<const float4*>(in) + 2 * t), b = __ldg(reinterpret_cast<const float4*>(in) + 2 * t + 1);
+  reinterpret_cast<uint4*>(out)[t] =
+      make_uint4(float_to_bf16_bits(a.x) | (float_to_bf16_bits(a.y) << 16), float_to_bf16_bits(a.z) | (float_to_bf16_bits(a.w) << 16),
+                 float_to_bf16_bits(b.x) | (float_to_bf16_bits(b.y) << 16), float_to_bf16_bits(b.z) | (float_to_bf16_bits(b.w) << 16));
 }
 
 // out[c*ld_out + r] = bf16(in[r*cols + c]); 32 x 32 tiles.
@@ -995,11 +998,15 @@ int bsp_linear_dgrad(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes, b
   else
     decode_to_bf16_kernel<BSP_E4M3><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes, n16, dyb);
   BSP_LAUNCH_CHECK();
-  // W [O][C] is the B operand with the contraction index outermost: a bf16 W is read in place as
-  // an MN-major operand; an FP32 W (or a C that breaks the 16-byte pitch) goes through a bf16
-  // transposed copy
-  const bool w_in_place = w_dt == BSP_BF16 && C % 8 == 0 && aligned16(W) && !simt_forced();
-  if (!w_in_place) {
+  // W [O][C] is the B operand with the contraction index outermost and is read as it lies (MN-major): a
+  // bf16 W in place, an FP32 W from a bf16 copy of the same layout (a transposed copy, a quarter of the
+  // speed at 4112 x 1552: 21 us against 7, is left for a C that breaks the 16-byte pitch)
+  const bool pitch_ok = C % 8 == 0 && aligned16(W), w_in_place = pitch_ok && w_dt == BSP_BF16;
+  if (pitch_ok && !w_in_place) {
+    const size_t n8 = (size_t)O * C / 8;
+    to_bf16_kernel<<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>(reinterpret_cast<const float*>(W), n8, wt);
+    BSP_LAUNCH_CHECK();
+  } else if (!pitch_ok) {
     dim3 tg((unsigned)((C + 31) / 32), (unsigned)((O + 31) / 32));
     if (w_dt == BSP_F32) to_bf16_transpose_kernel<BSP_F32><<<tg, 256, 0, st>>>(W, O, C, wt, O);
     else to_bf16_transpose_kernel<BSP_BF16><<<tg, 256, 0, st>>>(W, O, C, wt, O);
@@ -1008,7 +1015,7 @@ int bsp_linear_dgrad(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes, b
   GemmArgs g;
   g.M = T; g.N = C; g.K = O; g.nb = 1; g.fp8 = false; g.a_fmt = 0; g.b_fmt = 0;
   g.A = dyb; g.lda = O;
-  if (w_in_place) { g.B = W; g.b_mn = true; g.ldb = C; g.b_batch_stride = (int64_t)O * C; }
+  if (pitch_ok) { g.B = w_in_place ? W : wt; g.b_mn = true; g.ldb = C; g.b_batch_stride = (int64_t)O * C; }
   else { g.B = wt; g.ldb = O; g.b_batch_stride = (int64_t)C * O; }
   g.sa = q_dy.scale; g.sa_dev = q_dy.scale_dev; g.sb = 1.0f; g.sb_dev = nullptr;
   g.mode = du_dt == BSP_F32 ? EPI_STORE_F32 : EPI_STORE_BF16;

