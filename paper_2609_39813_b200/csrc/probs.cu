@@ -14,6 +14,7 @@
 // streams), 4 n d multiply-adds, five block-wide dot products, three block barriers.  CUDA cores
 // only: bound by the FP32 multiply-add rate (4 n d per row and draw).
 #include "common.cuh"
+#include "probs_tc.cuh"
 
 namespace bsp {
 
@@ -413,6 +414,22 @@ int bsp_probs_mc(const float* p, const float* V, int64_t rows, int n, int d, int
   k.stream = 0; const PhiloxKey kq = make_key(k);
   k.stream = 1; const PhiloxKey ka = make_key(k);
   k.stream = 2; const PhiloxKey kb = make_key(k);
+  // The tensor-core kernel's tile costs the same whatever part of its 128 slots is drawn, which the kernels below
+  // undercut for few draws: 4096 rows of 128 x 64, 8 draws 348 us here and 350 there, 16 draws 455 and 350; of
+  // 64 x 64, 8 draws 336 and 322; of 32 x 32, 24 draws 261 and 298, 32 draws 329 and 299; of 16 x 16 likewise.  It
+  // wants whole generator blocks per row and 16-byte stores of the gradient rows.
+  if (n <= kPtN && n % 4 == 0 && K >= (n >= 64 ? 8 : 32) && (d % 4 != 0 || aligned16(dV_sum))) {
+    int dev = 0, nsm = kNumSMs;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int g = K <= 64 ? 64 : 128;                           // slots per row: two rows' draws share a tile up to 64
+    const int64_t ngroups = (rows + kPtSlots / g - 1) / (kPtSlots / g);
+    auto kern = law == 1 ? probs_mc_tc_kernel<1> : probs_mc_tc_kernel<0>;
+    BSP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPtSmemBytes));
+    kern<<<(unsigned)(ngroups < nsm ? ngroups : nsm), kPtThreads, kPtSmemBytes, (cudaStream_t)stream>>>(
+        p, V, n, d, param, kq, draw0, K, g, ds_sum, ds_sq, dV_sum, (size_t)rows);
+    BSP_LAUNCH_CHECK();
+    return BSP_OK;
+  }
   if (n == kPfN && d == kPfD && (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (reinterpret_cast<uintptr_t>(dV_sum) & 15u) == 0) {
     const size_t smem_f = kPfSmemFloats * sizeof(float);
     BSP_CHECK_CUDA(cudaFuncSetAttribute(probs_mc_128x64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f));

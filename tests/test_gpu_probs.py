@@ -62,6 +62,26 @@ def test_sums_match_the_oracle_draw_for_draw(b, R, n, d, law, param):
         assert np.max(np.abs(dV[i] - want_dV[i])) <= 2e-5 * scale
 
 
+# the tensor-core form (16 draws up, whole generator blocks per row): both cuts of a tile (up to 64 draws two
+# rows share one), partly filled tiles and slot groups, draws beyond a segment of 256, entries and columns
+# that are not whole products, an odd row count, more groups than SMs
+@pytest.mark.parametrize("R,n,d,law,param,K", [
+    (3, 128, 64, 0, 1.0 / 64, 16), (3, 128, 64, 1, 1.0 / 512, 64), (2, 128, 64, 0, 1.0 / 64, 65),
+    (1, 128, 64, 0, 1.0 / 128, 257), (5, 4, 1, 0, 0.125, 31), (4, 16, 3, 1, 1.0 / 64, 33), (3, 36, 33, 0, 1.0 / 64, 129),
+    (2, 124, 62, 0, 1.0 / 128, 100), (301, 20, 16, 0, 1.0 / 32, 17), (2, 100, 64, 1, 1.0 / 256, 128)])
+def test_tensor_core_form_matches_the_oracle(b, R, n, d, law, param, K):
+    p, V = _rows(R, n, d, 7 + n)
+    ds, sq, dV = _run(b, p, V, law, param, 43, 2, K)
+    want_ds, want_sq, want_dV = probs.mc_sums(p, V, law, param, 43, K, 2)
+    # FP32 sums of K errors: sqrt(K / 9) times the bound for nine draws above covers their growth
+    f = max(1.0, np.sqrt(K / 9))
+    for i in range(5):
+        assert np.max(np.abs(ds[i] - want_ds[i])) <= 2e-5 * f * (np.max(np.abs(want_ds[i])) + 1e-30), i
+        assert np.max(np.abs(sq[i] - want_sq[i])) <= 1e-4 * (np.max(np.abs(want_sq[i])) + 1e-30), i
+    for i in range(2):
+        assert np.max(np.abs(dV[i] - want_dV[i])) <= 2e-5 * f * (np.max(np.abs(want_dV[i])) + 1e-30), i
+
+
 def test_bench_size_on_sampled_rows(b):
     """The size `bench.py` times (16384 rows of 128 probabilities, d = 64, grid 1/64, 256 draws; rows
     drawn by the same recipe): blocks of rows from the start, the middle and the end of the tensor
