@@ -313,10 +313,12 @@ quant_tile_kernel(Producer prod, const void* __restrict__ x, int64_t rows, int64
 // column, four consecutive rows), and those go straight to memory: sixteen neighbouring lanes cover
 // the 64 rows of a column.  Bound by the generator (integer multiplies, 1.69 T words/s measured for the
 // bare loop); no shared memory and no barrier in the draw loop (transposed through shared memory byte
-// by byte, 16384 x 4096 bf16, 16 draws: 1048 us; this form 904 us = 1.19 T draws/s).  grid.z splits the
+// by byte, 16384 x 4096 bf16, 16 draws: 1048 us; here 888; 8192 x 2048 FP32, 64 draws: 1004 and 745).  Two draws at a time give a thread
+// eight independent generator chains, which is worth more than the warps its registers cost (two blocks per
+// SM: 1.54 T draws/s in the bare loop, one draw and four blocks 1.39).  grid.z splits the
 // draws of a small tensor (64 x 128, 256 draws: two blocks, 162 us; now 7 us).
 template <int DT, int FMT>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(256, 2)
 reround_draws_kernel(NormProducer prod, const void* __restrict__ x, int64_t rows, int64_t cols, float scale_val,
                      const float* __restrict__ scale_dev, PhiloxKey key, int draw0, int ndraws, int draws_per_z,
                      uint8_t* __restrict__ codes_t, int64_t ld_t) {
@@ -352,7 +354,7 @@ reround_draws_kernel(NormProducer prod, const void* __restrict__ x, int64_t rows
   const int d1 = d0 + draws_per_z < ndraws ? d0 + draws_per_z : ndraws;
   const uint64_t q0 = (uint64_t)(r * cols + c) >> 2, qstep = (uint64_t)cols >> 2;   // cols % 16 == 0
   uint8_t* out = codes_t + ((size_t)d0 * cols + c) * ld_t + r;
-  for (int d = d0; d < d1; ++d, out += (size_t)cols * ld_t) {
+  auto draw = [&](int d) {
     uint32_t w4[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -370,7 +372,11 @@ reround_draws_kernel(NormProducer prod, const void* __restrict__ x, int64_t rows
                            __byte_perm(t2, t3, 0x5410), __byte_perm(t2, t3, 0x7632)};
 #pragma unroll
     for (int j = 0; j < 4; ++j) *reinterpret_cast<uint32_t*>(out + (size_t)j * ld_t) = o[j];
-  }
+    out += (size_t)cols * ld_t;
+  };
+  int d = d0;
+  for (; d + 1 < d1; d += 2) { draw(d); draw(d + 1); }
+  if (d < d1) draw(d);
 }
 
 // ------------------------------------------------------------------------------- norm statistics
@@ -684,8 +690,8 @@ int bsp_norm_fwd_draws(int kind, const void* x, int dt, int64_t T, int64_t C, co
   prod.kind = kind; prod.gamma = gamma; prod.beta = beta; prod.rstd = rstd; prod.mean = mean;
   prod.r_ = 0.f; prod.m_ = 0.f;
   dim3 grid((unsigned)((C + kTile - 1) / kTile), (unsigned)((T + kTile - 1) / kTile));
-  // few tiles: the draws are split over grid.z until there are about eight blocks per SM (two rounds of
-  // the four that fit), but never below four draws a block, which pay for finding the grid positions
+  // few tiles: the draws are split over grid.z until there are about eight blocks per SM (four rounds of
+  // the two that fit), but never below four draws a block, which pay for finding the grid positions
   const int64_t tiles = (int64_t)grid.x * grid.y, want = (int64_t)kNumSMs * 8;
   int nz = tiles < want ? (int)((want + tiles - 1) / tiles) : 1;
   if (nz > (n_draws + 3) / 4) nz = (n_draws + 3) / 4;
