@@ -331,17 +331,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 // the pair before.  With the sums in tensor memory (one pair of accumulators) every pair ended in an
 // epilogue the tensor pipe waited for: 4096 x 1024 x 4096, 64 draws (with the split below): 847 -> 767 us.
 //
+// PAIR: two CTAs of a cluster take two tile rows of the same columns as one product over 256 rows
+// (cta_group::2): each loads its own A rows and one of the two draws' B tiles, 32 KB per 128 bytes of K
+// instead of 48, which is what L2 has to deliver to every SM (96 bytes per cycle at the tensor rate
+// without pairs, of about 80 it gives with all SMs loading): see mc_pairs for what it measured.  The leader's (rank 0) warp 1
+// issues for both; its full barriers count both CTAs' bytes, its commits arrive in both.
+//
 // The walk is over units (tile, range of draws).  Whole waves of tiles take all their draws; the tiles
 // of a last, partial wave (or of a problem with fewer tiles than SMs) are cut into nseg ranges, range
 // by range over the tiles, so that CTAs which run together read the same draws.  Range 0 adds to S1 and
 // S2, range s > 0 writes its sums to slot (s - 1) of the split workspace, and gemm_mc_merge_kernel adds
 // the slots in order: every sum has one order, whatever the scheduling.
 constexpr int MC_BN = 128;
-constexpr int kMcStages = 4;
-constexpr int kMcABytes = BM * BKB, kMcBBytes = MC_BN * BKB, kMcStageBytes = kMcABytes + 2 * kMcBBytes;
+constexpr int kMcABytes = BM * BKB, kMcBBytes = MC_BN * BKB;
+template <bool PAIR> struct McRing {
+  static constexpr int kStages = PAIR ? 6 : 4, kStageBytes = kMcABytes + (PAIR ? 1 : 2) * kMcBBytes;
+};
+static_assert(McRing<true>::kStages * McRing<true>::kStageBytes == McRing<false>::kStages * McRing<false>::kStageBytes, "one ring size");
 constexpr int kMcThreads = 384;
 constexpr int kMcRegsProducer = 40, kMcRegsEpilogue = 232;   // 40 + 2 * 232 = 3 * 168: the launch's registers
-constexpr size_t kMcSmem = (size_t)kMcStages * kMcStageBytes + 1024 + 256;
+constexpr size_t kMcSmem = (size_t)McRing<true>::kStages * McRing<true>::kStageBytes + 1024 + 256;
 constexpr size_t kMcSplitTileFloats = (size_t)2 * BM * MC_BN;   // S1 and S2 of one tile in a split slot
 
 // Units of the walk: tiles [0, whole) with all draws, then nseg ranges over the other tiles.
@@ -357,10 +366,11 @@ __device__ __forceinline__ void mc_unit(const McSplit& sp, int u, int npairs, in
   p1 = p0 + sp.pairs_per_seg < npairs ? p0 + sp.pairs_per_seg : npairs;
 }
 
-template <bool FP8>
+template <bool FP8, bool PAIR>
 __global__ void __launch_bounds__(kMcThreads, 1)
 gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p,
                McSplit sp, float* __restrict__ split_ws) {
+  constexpr int kMcStages = McRing<PAIR>::kStages, kMcStageBytes = McRing<PAIR>::kStageBytes, kCtas = PAIR ? 2 : 1;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;
@@ -371,21 +381,26 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 16 * kMcStages + 36);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tiles_m = (p.M + BM - 1) / BM, tiles_n = (p.N + MC_BN - 1) / MC_BN;
+  const int rank = PAIR ? (int)cluster_rank() : 0;
+  const int tiles_m = (p.M + kCtas * BM - 1) / (kCtas * BM), tiles_n = (p.N + MC_BN - 1) / MC_BN;
   const int nunits = sp.whole + sp.rest * sp.nseg, npairs = (p.nb + 1) / 2;
   constexpr int kElemsPerStage = FP8 ? BKB : BKB / 2;   // K extent of one 128-byte stage in elements
   const int kblocks = (p.K + kElemsPerStage - 1) / kElemsPerStage;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kMcStages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, 8); }
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, 8 * kCtas); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+  if (warp == 1) {
+    if (PAIR) tmem_alloc2(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+    else tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+  }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();                              // both CTAs' barriers exist before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -399,7 +414,7 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       const uint64_t keep = l2_policy_evict_last();
       uint32_t it = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+      for (int u = blockIdx.x / kCtas; u < nunits && ok; u += gridDim.x / kCtas) {
         int t, seg, p0, p1, tm, tn;
         mc_unit(sp, u, npairs, t, seg, p0, p1);
         tile_coords(t, tiles_m, tiles_n, tm, tn);
@@ -410,6 +425,17 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             const uint32_t s = it % kMcStages, ph = (it / kMcStages) & 1u;
             if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
             const uint32_t sa = tiles + s * kMcStageBytes, sb = sa + kMcABytes;
+            if (PAIR) {
+              // one draw's B tile per CTA; of a single draw's tile a CTA provides half the columns (the box
+              // is whole all the same).  Bytes that arrive before the leader announces them only make
+              // its count negative for a while: the phase still waits for the leader's own arrival.
+              const uint32_t bar = leader_addr(full0 + 8 * s);
+              if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * kMcStageBytes);
+              tma_load_2d_pair(sa, &tmap_a, bar, kb * kElemsPerStage, (2 * tm + rank) * BM, keep);
+              tma_load_3d_pair(sb, &tmap_b, bar, kb * kElemsPerStage, tn * MC_BN + (two ? 0 : rank * (MC_BN / 2)),
+                               two ? b + rank : b);
+              continue;
+            }
             mbar_expect_tx(full0 + 8 * s, kMcABytes + (two ? 2 : 1) * kMcBBytes);
             tma_load_2d_hint(sa, &tmap_a, full0 + 8 * s, kb * kElemsPerStage, tm * BM, keep);
             tma_load_3d(sb, &tmap_b, full0 + 8 * s, kb * kElemsPerStage, tn * MC_BN, b);
@@ -420,10 +446,10 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       if (!ok) {
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && lane == 0 && rank == 0) {
       uint32_t it = 0, tc = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+      for (int u = blockIdx.x / kCtas; u < nunits && ok; u += gridDim.x / kCtas) {
         int t, seg, p0, p1;
         mc_unit(sp, u, npairs, t, seg, p0, p1);
         for (int pr = p0; pr < p1 && ok; ++pr, ++tc) {
@@ -439,11 +465,17 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             const uint32_t sa = tiles + s * kMcStageBytes, sb = sa + kMcABytes;
             const uint64_t adesc = make_smem_desc(sa), bdesc = make_smem_desc(sb);   // B: 128 or 256 rows
 #pragma unroll
-            for (int k = 0; k < BKB / 32; ++k)
-              tc_mma<FP8>(tmem_d, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
-            tc_commit(empty0 + 8 * s);
+            for (int k = 0; k < BKB / 32; ++k) {
+              if (PAIR) tc_mma2<FP8>(tmem_d, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
+              else tc_mma<FP8>(tmem_d, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            }
+            if (PAIR) tc_commit2(empty0 + 8 * s);
+            else tc_commit(empty0 + 8 * s);
           }
-          if (ok) tc_commit(tfull0 + 8 * as);
+          if (ok) {
+            if (PAIR) tc_commit2(tfull0 + 8 * as);
+            else tc_commit(tfull0 + 8 * as);
+          }
         }
       }
     }
@@ -456,11 +488,11 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16) + h * 64;
     uint32_t tc = 0;
     bool ok = true;
-    for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+    for (int u = blockIdx.x / kCtas; u < nunits && ok; u += gridDim.x / kCtas) {
       int t, seg, p0, p1, tm, tn;
       mc_unit(sp, u, npairs, t, seg, p0, p1);
       tile_coords(t, tiles_m, tiles_n, tm, tn);
-      const int row = tm * BM + q * 32 + lane;
+      const int row = (kCtas * tm + rank) * BM + q * 32 + lane;
       const int colbase = tn * MC_BN + h * 64;
       float refv[64], s1[64], s2[64];
       // ---- unit start: the reference, and the sums so far when this unit continues them
@@ -507,7 +539,10 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(tempty0 + 8 * as);
+        if (lane == 0) {
+          if (PAIR) mbar_arrive_cluster(leader_addr(tempty0 + 8 * as));
+          else mbar_arrive(tempty0 + 8 * as);
+        }
       }
       if (!ok) break;
       // ---- unit end: the sums back to S1 and S2, or to the unit's split slot
@@ -521,7 +556,7 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           }
       } else {
         // [S1 | S2][column / 4][row] as groups of four columns: a warp writes 512 consecutive bytes
-        float4* slot = reinterpret_cast<float4*>(split_ws + ((size_t)(seg - 1) * sp.rest + (t - sp.whole)) * kMcSplitTileFloats) +
+        float4* slot = reinterpret_cast<float4*>(split_ws + (((size_t)(seg - 1) * sp.rest + (t - sp.whole)) * kCtas + rank) * kMcSplitTileFloats) +
                        (h * 16) * BM + q * 32 + lane;
 #pragma unroll
         for (int c = 0; c < 64; c += 4) {
@@ -534,22 +569,26 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();                              // nothing of this CTA is used by the other any more
   if (threadIdx.x == 0 && *abort_flag && p.diag) atomicMax(&p.diag->status, (int)BSP_ERR_TIMEOUT);
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    if (PAIR) tmem_dealloc2(tmem_base, kTmemCols);
+    else tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
-// S1 += slot sums, S2 likewise, of the tiles whose draws were split.  Block (t, y): tile whole + t, a
+// S1 += slot sums, S2 likewise, of the tiles whose draws were split.  Block (t, y): tile whole + t / ctas
+// (its row tile t % ctas), a
 // thread takes four columns of one row; slots are added in the order of their draws.
 __global__ void __launch_bounds__(256)
-gemm_mc_merge_kernel(const float* __restrict__ split_ws, McSplit sp, int M, int N, int64_t ldc, float* __restrict__ S1,
+gemm_mc_merge_kernel(const float* __restrict__ split_ws, McSplit sp, int ctas, int M, int N, int64_t ldc, float* __restrict__ S1,
                      float* __restrict__ S2) {
-  const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + MC_BN - 1) / MC_BN;
+  const int tiles_m = (M + ctas * BM - 1) / (ctas * BM), tiles_n = (N + MC_BN - 1) / MC_BN;
   int tm, tn;
-  tile_coords(sp.whole + (int)blockIdx.x, tiles_m, tiles_n, tm, tn);
+  tile_coords(sp.whole + (int)blockIdx.x / ctas, tiles_m, tiles_n, tm, tn);
+  tm = tm * ctas + (int)blockIdx.x % ctas;
   const int i = (int)blockIdx.y * 256 + threadIdx.x, second = i >= BM * MC_BN / 4, k = i - second * (BM * MC_BN / 4);
   const int row = tm * BM + (k & (BM - 1)), col = tn * MC_BN + 4 * (k / BM);
   if (row >= M || col >= N) return;
@@ -557,7 +596,7 @@ gemm_mc_merge_kernel(const float* __restrict__ split_ws, McSplit sp, int M, int 
   float4 s = *dst;
   const float4* src = reinterpret_cast<const float4*>(split_ws + (size_t)blockIdx.x * kMcSplitTileFloats) + i;
 #pragma unroll 4
-  for (int g = 1; g < sp.nseg; ++g, src += (size_t)sp.rest * (kMcSplitTileFloats / 4)) {
+  for (int g = 1; g < sp.nseg; ++g, src += (size_t)sp.rest * ctas * (kMcSplitTileFloats / 4)) {
     const float4 v = __ldg(src);
     s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
   }
@@ -698,8 +737,17 @@ static int tile_columns(int64_t M, int64_t N, int64_t k_bytes, int nsm) {
 // products take kblocks ring stages of about 0.27 us, and a cut adds the merge launch (about 3 us) and
 // 128 KB written and read per slot.  Cuts are of at least four pairs, so that a range's start (the
 // reference from memory) stays small beside its products.
+static bool mc_pairs(int64_t M, int64_t k_bytes) {
+  // An odd count of tile rows leaves half a pair idle: worth it when that is one in nine or fewer.  Pairs win
+  // 4 to 14 % (A of 17, 34, 90 MB: 1012 -> 931 us, 1850 -> 1755, 5400 -> 4800) until A, which every pass over a
+  // pair of draws reads again, is larger than L2: 180 MB, 16 draws, 8.75 ms alone and 8.9 in pairs.
+  const int64_t tm = (M + BM - 1) / BM;
+  return (tm % 2 == 0 || tm >= 9) && M * k_bytes <= (int64_t)120 << 20;
+}
 static McSplit mc_split_plan(int64_t M, int64_t N, int64_t k_bytes, int nb, int nsm) {
-  const int ntiles = (int)(((M + BM - 1) / BM) * ((N + MC_BN - 1) / MC_BN)), npairs = (nb + 1) / 2;
+  const int ctas = mc_pairs(M, k_bytes) ? 2 : 1;         // CTAs per unit of the walk
+  const int ntiles = (int)(((M + ctas * BM - 1) / (ctas * BM)) * ((N + MC_BN - 1) / MC_BN)), npairs = (nb + 1) / 2;
+  nsm /= ctas;
   McSplit sp;
   sp.whole = ntiles / nsm * nsm;
   sp.rest = ntiles - sp.whole;
@@ -711,17 +759,38 @@ static McSplit mc_split_plan(int64_t M, int64_t N, int64_t k_bytes, int nb, int 
   for (int s = 2; s <= 32 && npairs >= 4 * s; ++s) {
     const int per = (npairs + s - 1) / s, nseg = (npairs + per - 1) / per;
     const int rounds = (sp.rest * nseg + nsm - 1) / nsm;
-    const double cost = (double)rounds * per * pair_us + 3.0 + 0.05 * sp.rest * (nseg - 1) + 1.0 * (rounds - 1);
+    const double cost = (double)rounds * per * pair_us + 3.0 + 0.05 * sp.rest * ctas * (nseg - 1) + 1.0 * (rounds - 1);
     if (cost < 0.97 * best) { best = cost; sp.nseg = nseg; sp.pairs_per_seg = per; }
   }
   return sp;
 }
-static size_t mc_split_bytes(const McSplit& sp) {
-  return (size_t)(sp.nseg - 1) * (size_t)sp.rest * kMcSplitTileFloats * sizeof(float);
+static size_t mc_split_bytes(const McSplit& sp, int64_t M, int64_t k_bytes) {
+  return (size_t)(sp.nseg - 1) * (size_t)sp.rest * (mc_pairs(M, k_bytes) ? 2 : 1) * kMcSplitTileFloats * sizeof(float);
 }
 size_t gemm_mc_split_bytes(int64_t M, int64_t N, int64_t K, bool fp8, int nb) {
   if (M <= 0 || N <= 0 || K <= 0 || nb <= 0) return 0;
-  return mc_split_bytes(mc_split_plan(M, N, K * (fp8 ? 1 : 2), nb, device_sms()));
+  const int64_t k_bytes = K * (fp8 ? 1 : 2);
+  return mc_split_bytes(mc_split_plan(M, N, k_bytes, nb, device_sms()), M, k_bytes);
+}
+
+template <bool FP8, bool PAIR>
+static int gemm_mc_launch(const CUtensorMap& ma, const CUtensorMap& mb, const GemmParams& p, const McSplit& sp, float* split_ws,
+                          int grid, cudaStream_t st) {
+  static std::atomic<bool> attr_set_dev[kMaxDevices];
+  std::atomic<bool>& attr_set = attr_set_dev[device_slot()];
+  if (!attr_set.load(std::memory_order_acquire)) {
+    BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_mc_kernel<FP8, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMcSmem));
+    attr_set.store(true, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = PAIR ? 2 : 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kMcThreads); cfg.dynamicSmemBytes = kMcSmem; cfg.stream = st;
+  cfg.attrs = attr; cfg.numAttrs = PAIR ? 1 : 0;
+  BSP_CHECK_CUDA(cudaLaunchKernelEx(&cfg, gemm_mc_kernel<FP8, PAIR>, ma, mb, p, sp, split_ws));
+  BSP_LAUNCH_CHECK();
+  return BSP_OK;
 }
 
 template <bool FP8, int MODE>
@@ -785,27 +854,22 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
     rc = make_operand_map(&mb, g.B, eb, g.K, g.N, g.ldb, g.nb, g.b_batch_stride, MC_BN);
     if (rc != BSP_OK) return rc;
     const uint32_t fa = g.fp8 ? (g.a_fmt == BSP_E5M2 ? 1u : 0u) : 1u, fb = g.fp8 ? (g.b_fmt == BSP_E5M2 ? 1u : 0u) : 1u;
-    p.idesc = make_idesc(fa, fb, BM, MC_BN);
-    p.idesc2 = make_idesc(fa, fb, BM, 2 * MC_BN);
-    static std::atomic<bool> mc_attr_set_dev[kMaxDevices][2];
-    std::atomic<bool>& mc_attr_set = mc_attr_set_dev[device_slot()][g.fp8 ? 1 : 0];
-    if (!mc_attr_set.load(std::memory_order_acquire)) {
-      if (g.fp8) BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_mc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMcSmem));
-      else BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_mc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMcSmem));
-      mc_attr_set.store(true, std::memory_order_release);
-    }
+    const bool pair = mc_pairs(g.M, g.K * eb);
+    const int ctas = pair ? 2 : 1;
+    p.idesc = make_idesc(fa, fb, ctas * BM, MC_BN);
+    p.idesc2 = make_idesc(fa, fb, ctas * BM, 2 * MC_BN);
     McSplit sp = mc_split_plan(g.M, g.N, g.K * eb, g.nb, nsm);
-    if (!g.split_ws || g.split_ws_bytes < mc_split_bytes(sp)) {      // no room: every tile takes all its draws
+    if (!g.split_ws || g.split_ws_bytes < mc_split_bytes(sp, g.M, g.K * eb)) {      // no room: every tile takes all its draws
       sp.whole += sp.rest;
       sp.rest = 0;
       sp.nseg = 1;
     }
-    const int nunits = sp.whole + sp.rest * sp.nseg, grid_mc = nunits < nsm ? nunits : nsm;
-    if (g.fp8) gemm_mc_kernel<true><<<grid_mc, kMcThreads, kMcSmem, st>>>(ma, mb, p, sp, g.split_ws);
-    else gemm_mc_kernel<false><<<grid_mc, kMcThreads, kMcSmem, st>>>(ma, mb, p, sp, g.split_ws);
-    BSP_LAUNCH_CHECK();
+    const int nunits = sp.whole + sp.rest * sp.nseg, grid_mc = ctas * (nunits < nsm / ctas ? nunits : nsm / ctas);
+    if (g.fp8) rc = pair ? gemm_mc_launch<true, true>(ma, mb, p, sp, g.split_ws, grid_mc, st) : gemm_mc_launch<true, false>(ma, mb, p, sp, g.split_ws, grid_mc, st);
+    else rc = pair ? gemm_mc_launch<false, true>(ma, mb, p, sp, g.split_ws, grid_mc, st) : gemm_mc_launch<false, false>(ma, mb, p, sp, g.split_ws, grid_mc, st);
+    if (rc != BSP_OK) return rc;
     if (sp.nseg > 1) {
-      gemm_mc_merge_kernel<<<dim3((unsigned)sp.rest, 2 * BM * MC_BN / 4 / 256), 256, 0, st>>>(g.split_ws, sp, p.M, p.N, p.ldc,
+      gemm_mc_merge_kernel<<<dim3((unsigned)(sp.rest * ctas), 2 * BM * MC_BN / 4 / 256), 256, 0, st>>>(g.split_ws, sp, ctas, p.M, p.N, p.ldc,
                                                                                               p.S1, p.S2);
       BSP_LAUNCH_CHECK();
     }
