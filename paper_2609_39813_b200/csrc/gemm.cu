@@ -31,6 +31,8 @@ constexpr int kABytes = BM * BKB, kBBytes = BN * BKB, kStageBytes = kABytes + kB
 constexpr int kGemmThreads = 320;
 constexpr int kTmemCols = 512;
 constexpr int kEpiStage = 8 * 4096;              // one 32-row x 128-byte staging block per epilogue warp
+constexpr int kPairStages = 6, kPairStageBytes = kABytes + kBBytes / 2;   // a CTA of a pair holds half of B's tile
+static_assert(kPairStages * kPairStageBytes == kStages * kStageBytes, "one ring size");
 constexpr size_t kGemmSmem = (size_t)kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kEpiStage;
 
 struct GemmParams {
@@ -79,9 +81,13 @@ __device__ __forceinline__ void split4(const float4& v, uint2& hi, uint2& lo) {
                   float_to_bf16_bits(v.z - bf16_bits_to_float(h2)) | (float_to_bf16_bits(v.w - bf16_bits_to_float(h3)) << 16));
 }
 
-template <bool FP8, int MODE>
+// PAIR: two CTAs of a cluster take two tile rows of the same columns as one product over 256 rows
+// (cta_group::2), each with its own A rows and half of B's columns: (128 + bn / 2) instead of (128 + bn)
+// rows through L2 and shared memory per CTA.  The leader (rank 0) issues for both.
+template <bool FP8, int MODE, bool PAIR>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p) {
+  constexpr int kStages = PAIR ? kPairStages : bsp::kStages, kStageBytes = PAIR ? kPairStageBytes : bsp::kStageBytes, kCtas = PAIR ? 2 : 1;
   constexpr int kElem = FP8 ? 1 : 2, bk_elems = BKB / kElem, kAtom = 128 / kElem;   // elements per 128 bytes
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -95,22 +101,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 16 * kStages + 36);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tiles_m = (p.M + BM - 1) / BM, tiles_n = (p.N + p.bn - 1) / p.bn;
+  const int rank = PAIR ? (int)cluster_rank() : 0, bn_cta = p.bn / kCtas;   // columns of B this CTA loads
+  const int tiles_m = (p.M + kCtas * BM - 1) / (kCtas * BM), tiles_n = (p.N + p.bn - 1) / p.bn;
   const int ntiles = tiles_m * tiles_n;
   const int kblocks = (p.K * kElem + BKB - 1) / BKB;
   // an MN-major B comes in atoms of 128 bytes of N: the last one may reach past the tile's columns
-  const int b_atoms = (p.bn * kElem + 127) / 128, b_bytes = p.b_mn ? b_atoms * bk_elems * 128 : p.bn * BKB;
+  const int b_atoms = (bn_cta * kElem + 127) / 128, b_bytes = p.b_mn ? b_atoms * bk_elems * 128 : bn_cta * BKB;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, 8); }
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, 8 * kCtas); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+  if (warp == 1) {
+    if (PAIR) tmem_alloc2(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+    else tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+  }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();                              // both CTAs' barriers exist before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -121,7 +132,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       tma_prefetch_desc(&tmap_b);
       uint32_t it = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      for (int t = blockIdx.x / kCtas; t < ntiles && ok; t += gridDim.x / kCtas) {
         int tm, tn;
       tile_coords(t, tiles_m, tiles_n, tm, tn);
         for (int b = 0; b < p.nb && ok; ++b) {
@@ -129,24 +140,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             const uint32_t s = it % kStages, ph = (it / kStages) & 1u;
             if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
             const uint32_t sa = tiles + s * kStageBytes, sb = sa + kABytes;
-            mbar_expect_tx(full0 + 8 * s, kABytes + b_bytes);
+            // the leader's barrier counts both CTAs' bytes
+            const uint32_t bar = PAIR ? leader_addr(full0 + 8 * s) : full0 + 8 * s;
+            if (rank == 0) mbar_expect_tx(full0 + 8 * s, kCtas * (kABytes + b_bytes));
+            const int row0 = (kCtas * tm + rank) * BM, col0 = tn * p.bn + rank * bn_cta;
             if (!p.a_mn) {
-              tma_load_2d(sa, &tmap_a, full0 + 8 * s, kb * bk_elems, tm * BM);
+              tma_load_2d_c<PAIR>(sa, &tmap_a, bar, kb * bk_elems, row0);
             } else {
               // one box per 128 bytes of M: [bk_elems k rows][128 B]
-              #pragma unroll
+#pragma unroll
               for (int a = 0; a < BM / kAtom; ++a)
-                tma_load_2d(sa + a * bk_elems * 128, &tmap_a, full0 + 8 * s, tm * BM + a * kAtom,
-                            kb * bk_elems);
+                tma_load_2d_c<PAIR>(sa + a * bk_elems * 128, &tmap_a, bar, row0 + a * kAtom, kb * bk_elems);
             }
             if (!p.b_mn) {
-              tma_load_3d(sb, &tmap_b, full0 + 8 * s, kb * bk_elems, tn * p.bn, b);
+              tma_load_3d_c<PAIR>(sb, &tmap_b, bar, kb * bk_elems, col0, b);
             } else {
-              #pragma unroll
-              for (int a = 0; a < BN / kAtom; ++a)
+#pragma unroll
+              for (int a = 0; a < BN / kCtas / kAtom; ++a)
                 if (a < b_atoms)
-                tma_load_3d(sb + a * bk_elems * 128, &tmap_b, full0 + 8 * s, tn * p.bn + a * kAtom,
-                            kb * bk_elems, b);
+                  tma_load_3d_c<PAIR>(sb + a * bk_elems * 128, &tmap_b, bar, col0 + a * kAtom, kb * bk_elems, b);
             }
           }
         }
@@ -158,10 +170,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (lane == 0 && rank == 0) {
       uint32_t it = 0, tc = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      for (int t = blockIdx.x / kCtas; t < ntiles && ok; t += gridDim.x / kCtas) {
         for (int b = 0; b < p.nb && ok; ++b, ++tc) {
           const uint32_t as = tc & 1u, aph = (tc >> 1) & 1u;
           if (!mbar_wait(tempty0 + 8 * as, aph ^ 1u, abort_flag)) { ok = false; break; }
@@ -181,10 +193,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             const uint32_t astep = p.a_mn ? mn_step : 2u, bstep = p.b_mn ? mn_step : 2u;
 #pragma unroll
             for (int k = 0; k < BKB / 32; ++k)
-              tc_mma<FP8>(tmem_d, adesc + astep * k, bdesc + bstep * k, p.idesc, (kb | k) != 0 ? 1u : 0u);
-            tc_commit(empty0 + 8 * s);          // frees the stage when these MMAs have read it
+              if (PAIR) tc_mma2<FP8>(tmem_d, adesc + astep * k, bdesc + bstep * k, p.idesc, (kb | k) != 0 ? 1u : 0u);
+              else tc_mma<FP8>(tmem_d, adesc + astep * k, bdesc + bstep * k, p.idesc, (kb | k) != 0 ? 1u : 0u);
+            if (PAIR) tc_commit2(empty0 + 8 * s);   // frees the stage when these MMAs have read it
+            else tc_commit(empty0 + 8 * s);
           }
-          if (ok) tc_commit(tfull0 + 8 * as);   // accumulator complete
+          if (ok) {                                 // accumulator complete
+            if (PAIR) tc_commit2(tfull0 + 8 * as);
+            else tc_commit(tfull0 + 8 * as);
+          }
         }
       }
     }
@@ -195,10 +212,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? __ldg(p.sb_dev) : p.sb);
     uint32_t tc = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+    for (int t = blockIdx.x / kCtas; t < ntiles && ok; t += gridDim.x / kCtas) {
       int tm, tn;
       tile_coords(t, tiles_m, tiles_n, tm, tn);
-      const int row = tm * BM + q * 32 + lane;
+      const int row0 = (kCtas * tm + rank) * BM, row = row0 + q * 32 + lane;
       const int nlim = p.N < (tn + 1) * p.bn ? p.N : (tn + 1) * p.bn;   // columns from here on are not this tile's
       for (int b = 0; b < p.nb && ok; ++b, ++tc) {
         const uint32_t as = tc & 1u, aph = (tc >> 1) & 1u;
@@ -215,7 +232,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           // what the warp will write goes row by row (row 4 t + lane / 8, four columns from 4 (lane % 8)); the
           // values that an epilogue reads back there are fetched before the accumulator
           constexpr bool by_rows = MODE != EPI_STORE_BF16;
-          const int row8 = tm * BM + q * 32 + (lane >> 3), col4 = col0 + 4 * (lane & 7);
+          const int row8 = row0 + q * 32 + (lane >> 3), col4 = col0 + 4 * (lane & 7);
           float4 old1[8], old2[8];
           const bool reads1 = (MODE == EPI_SPLIT && p.ref) || (MODE == EPI_MOMENTS && !p.moment_first);
           if (reads1) {
@@ -248,7 +265,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
               asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                            : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w)
                            : "r"(wb + (uint32_t)rl * 128u + ((uint32_t)(c4 ^ (rl & 7)) << 4)));
-              const int orow = tm * BM + q * 32 + rl, ocol = col0 + 4 * c4;
+              const int orow = row0 + q * 32 + rl, ocol = col0 + 4 * c4;
               if (orow < p.M && ocol < nlim) {
                 const size_t off = (size_t)orow * p.ldc + ocol;
                 if (MODE == EPI_STORE_F32) {
@@ -300,18 +317,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(tempty0 + 8 * as);
+        if (lane == 0) {
+          if (PAIR) mbar_arrive_cluster(leader_addr(tempty0 + 8 * as));
+          else mbar_arrive(tempty0 + 8 * as);
+        }
       }
     }
   }
 
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();                              // nothing of this CTA is used by the other any more
   if (threadIdx.x == 0 && *abort_flag && p.diag) atomicMax(&p.diag->status, (int)BSP_ERR_TIMEOUT);
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    if (PAIR) tmem_dealloc2(tmem_base, kTmemCols);
+    else tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
@@ -714,21 +736,33 @@ static int device_sms() {
   return kNumSMs;
 }
 
-// Columns of a plain contraction's tile, 64 .. 256 in steps of 16.  The time goes with the number of rounds
-// the tiles take over the SMs times what a tile costs: per 32 bytes of K the product's bn / 2 cycles or, with
-// every SM loading, the (128 + bn) * 32 bytes of its operands at the 80 bytes per cycle and SM that L2 was
-// seen to give (256 columns reach 0.83 of the tensor rate, 128 columns 0.6), and the epilogue of the last
-// tile (about 12 cycles a column).  256 columns unless fewer save a twentieth (3001 x 1552 x 4112 bf16: 144 columns, 66 -> 54 us).
-static int tile_columns(int64_t M, int64_t N, int64_t k_bytes, int nsm) {
-  const int64_t tm = (M + BM - 1) / BM, slices = (k_bytes + 31) / 32;
-  int best = BN;
-  double best_cost = 0.0;
-  for (int bn = BN; bn >= 64; bn -= 16) {
-    const int64_t rounds = (tm * ((N + bn - 1) / bn) + nsm - 1) / nsm;
-    const double slice = bn / 2.0 > 0.4 * (128 + bn) ? bn / 2.0 : 0.4 * (128 + bn);
-    const double cost = (double)rounds * (double)slices * slice + 12.0 * bn;
-    if (bn == BN) best_cost = cost;
-    else if (cost < 0.95 * best_cost) { best_cost = cost; best = bn; }
+// How a plain contraction is tiled: columns of a tile, 64 .. 256 in steps of 16 (of 32 for a pair of CTAs),
+// and whether pairs take two tile rows together.  The time goes with the number of rounds the tiles take
+// over the SMs times what a tile costs: per 32 bytes of K the product's bn / 2 cycles or, with every SM
+// loading, the 32 bytes of each operand row at the 80 bytes per cycle and SM that L2 was seen to give
+// (alone, 256 columns reach 0.83 of the tensor rate, 128 columns 0.6), and the epilogue of the last tile
+// (about 12 cycles a column).  Fewer columns only where they save a twentieth (3001 x 1552 x 4112 bf16, 144 columns: 66 -> 54 us); pairs wherever they
+// cost no more (16384 x 4096 x 11008 bf16: 1070 -> 954 us; 4096 x 1024 x 8192: 63 -> 55).
+struct TilePlan {
+  int bn;
+  bool pair;
+};
+static TilePlan plan_tiles(int64_t M, int64_t N, int64_t k_bytes, int nsm) {
+  const int64_t slices = (k_bytes + 31) / 32;
+  TilePlan best = {BN, false};
+  double least = 0.0;
+  for (int ctas = 1; ctas <= 2; ++ctas) {
+    if (ctas == 2 && M <= BM) break;
+    const int64_t tm = (M + ctas * BM - 1) / (ctas * BM);
+    TilePlan mine = {BN, ctas == 2};
+    double cost_mine = 0.0;
+    for (int bn = BN; bn >= 64; bn -= 16 * ctas) {
+      const int64_t rounds = (tm * ((N + bn - 1) / bn) + nsm / ctas - 1) / (nsm / ctas);
+      const double feed = 0.4 * (128 + bn / ctas), slice = bn / 2.0 > feed ? bn / 2.0 : feed;
+      const double cost = (double)rounds * (double)slices * slice + 12.0 * bn;
+      if (bn == BN || cost < 0.95 * cost_mine) { cost_mine = cost; mine.bn = bn; }
+    }
+    if (ctas == 1 || cost_mine <= least) { least = cost_mine; best = mine; }
   }
   return best;
 }
@@ -793,18 +827,30 @@ static int gemm_mc_launch(const CUtensorMap& ma, const CUtensorMap& mb, const Ge
   return BSP_OK;
 }
 
-template <bool FP8, int MODE>
-static int gemm_tc_launch(const CUtensorMap& ma, const CUtensorMap& mb, const GemmParams& p, int nsm, cudaStream_t st) {
+template <bool FP8, int MODE, bool PAIR>
+static int gemm_tc_launch_as(const CUtensorMap& ma, const CUtensorMap& mb, const GemmParams& p, int nsm, cudaStream_t st) {
   static std::atomic<bool> attr_set_dev[kMaxDevices];
   std::atomic<bool>& attr_set = attr_set_dev[device_slot()];
   if (!attr_set.load(std::memory_order_acquire)) {
-    BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<FP8, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
+    BSP_CHECK_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<FP8, MODE, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
     attr_set.store(true, std::memory_order_release);
   }
-  const int ntiles = ((p.M + BM - 1) / BM) * ((p.N + p.bn - 1) / p.bn);
-  gemm_tc_kernel<FP8, MODE><<<ntiles < nsm ? ntiles : nsm, kGemmThreads, kGemmSmem, st>>>(ma, mb, p);
+  constexpr int ctas = PAIR ? 2 : 1;
+  const int ntiles = ((p.M + ctas * BM - 1) / (ctas * BM)) * ((p.N + p.bn - 1) / p.bn);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(ctas * (ntiles < nsm / ctas ? ntiles : nsm / ctas)));
+  cfg.blockDim = dim3(kGemmThreads); cfg.dynamicSmemBytes = kGemmSmem; cfg.stream = st;
+  cfg.attrs = attr; cfg.numAttrs = PAIR ? 1 : 0;
+  BSP_CHECK_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<FP8, MODE, PAIR>, ma, mb, p));
   BSP_LAUNCH_CHECK();
   return BSP_OK;
+}
+template <bool FP8, int MODE>
+static int gemm_tc_launch(const CUtensorMap& ma, const CUtensorMap& mb, const GemmParams& p, bool pair, int nsm, cudaStream_t st) {
+  return pair ? gemm_tc_launch_as<FP8, MODE, true>(ma, mb, p, nsm, st) : gemm_tc_launch_as<FP8, MODE, false>(ma, mb, p, nsm, st);
 }
 
 int gemm_run(const GemmArgs& g, cudaStream_t st) {
@@ -876,17 +922,19 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
     return BSP_OK;
   }
 
-  p.bn = tile_columns(g.M, g.N, g.K * eb, nsm);
+  const TilePlan plan = plan_tiles(g.M, g.N, g.K * eb, nsm);
+  const int ctas = plan.pair ? 2 : 1;
+  p.bn = plan.bn;
   const uint32_t fa = g.fp8 ? (g.a_fmt == BSP_E5M2 ? 1u : 0u) : 1u, fb = g.fp8 ? (g.b_fmt == BSP_E5M2 ? 1u : 0u) : 1u;
-  p.idesc = make_idesc(fa, fb, BM, (uint32_t)p.bn) | (g.a_mn ? 1u << 15 : 0u) | (g.b_mn ? 1u << 16 : 0u);   // operand major bits
-  rc = make_operand_map(&mb, g.B, eb, g.K, g.N, g.ldb, g.nb, g.b_batch_stride, p.bn, g.b_mn);
+  p.idesc = make_idesc(fa, fb, ctas * BM, (uint32_t)p.bn) | (g.a_mn ? 1u << 15 : 0u) | (g.b_mn ? 1u << 16 : 0u);   // operand major bits
+  rc = make_operand_map(&mb, g.B, eb, g.K, g.N, g.ldb, g.nb, g.b_batch_stride, p.bn / ctas, g.b_mn);
   if (rc != BSP_OK) return rc;
-  if (g.fp8) return g.mode == EPI_STORE_F32 ? gemm_tc_launch<true, EPI_STORE_F32>(ma, mb, p, nsm, st) : BSP_ERR_UNSUPPORTED;
+  if (g.fp8) return g.mode == EPI_STORE_F32 ? gemm_tc_launch<true, EPI_STORE_F32>(ma, mb, p, plan.pair, nsm, st) : BSP_ERR_UNSUPPORTED;
   switch (g.mode) {
-    case EPI_STORE_F32: return gemm_tc_launch<false, EPI_STORE_F32>(ma, mb, p, nsm, st);
-    case EPI_STORE_BF16: return gemm_tc_launch<false, EPI_STORE_BF16>(ma, mb, p, nsm, st);
-    case EPI_SPLIT: return gemm_tc_launch<false, EPI_SPLIT>(ma, mb, p, nsm, st);
-    case EPI_MOMENTS: return gemm_tc_launch<false, EPI_MOMENTS>(ma, mb, p, nsm, st);
+    case EPI_STORE_F32: return gemm_tc_launch<false, EPI_STORE_F32>(ma, mb, p, plan.pair, nsm, st);
+    case EPI_STORE_BF16: return gemm_tc_launch<false, EPI_STORE_BF16>(ma, mb, p, plan.pair, nsm, st);
+    case EPI_SPLIT: return gemm_tc_launch<false, EPI_SPLIT>(ma, mb, p, plan.pair, nsm, st);
+    case EPI_MOMENTS: return gemm_tc_launch<false, EPI_MOMENTS>(ma, mb, p, plan.pair, nsm, st);
     default: return BSP_ERR_UNSUPPORTED;
   }
 }

@@ -231,6 +231,22 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       : "memory");
 }
 
+// Loads of a kernel that exists for one CTA and for a pair.
+template <bool PAIR>
+__device__ __forceinline__ void tma_load_2d_c(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
+  if (PAIR)
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y)
+        : "memory");
+  else tma_load_2d(dst, map, bar, x, y);
+}
+template <bool PAIR>
+__device__ __forceinline__ void tma_load_3d_c(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z) {
+  if (PAIR) tma_load_3d_pair(dst, map, bar, x, y, z);
+  else tma_load_3d(dst, map, bar, x, y, z);
+}
+
 template <bool FP8>
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
   if (FP8) {
