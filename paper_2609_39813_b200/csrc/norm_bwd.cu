@@ -478,7 +478,10 @@ int bsp_norm_bwd(int kind, const void* x, int dt, int64_t T, int64_t C, const fl
   // (an input gradient that reads a copy is outside the reference and takes the plain kernel too)
   StreamPlan plan = plan_stream(T, C, dt, du_dt, gain_read, x, du, u_codes);
   if (dx_read != BSP_READ_ORIGINAL) plan.ok = false;
-  const int grid = plan.ok ? plan.grid : bwd_grid(T);
+  // the plain kernel: one wave of the blocks that fit (1024 threads per SM), so that a block's start and its
+  // column partials are spread over as many rows as there are (3001 x 1552 FP32: 26 -> 24 us, its column sums 6.5 -> 4)
+  const int fit = kNumSMs * (C <= 1024 ? 4 : C <= 2048 ? 2 : 1);
+  const int grid = plan.ok ? plan.grid : bwd_grid(T) < fit ? bwd_grid(T) : fit;
   float* part_g = reinterpret_cast<float*>(ws);
   float* part_b = dbeta ? reinterpret_cast<float*>(reinterpret_cast<char*>(ws) +
                                                    round_up((size_t)grid * C * sizeof(float), 256))
