@@ -103,6 +103,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
             const __grid_constant__ CUtensorMap tm_o0, const __grid_constant__ CUtensorMap tm_o1,
             const __grid_constant__ CUtensorMap tm_o2, AttnParams p) {
+  grid_dependency();
   static_assert(!DQF || (MODE == AT_DKV && !FP8 && DV && !MC && ND == 1), "fused dQ: plain BF16 dK/dV kernel only");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -517,8 +518,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     const uint32_t t_acc0 = t_accbase + ab * 128, t_acc1 = t_acc0 + 64;
     float inv_q = 1.f, inv_k = 1.f, inv_v = 1.f, inv_do = 1.f;
     if (FP8) {
-      inv_q = __fdiv_rn(1.0f, __ldg(p.sc_q + bh)); inv_k = __fdiv_rn(1.0f, __ldg(p.sc_k + bh));
-      inv_v = __fdiv_rn(1.0f, __ldg(p.sc_v + bh)); inv_do = __fdiv_rn(1.0f, __ldg(p.sc_do + bh));
+      inv_q = __fdiv_rn(1.0f, ldg(p.sc_q + bh)); inv_k = __fdiv_rn(1.0f, ldg(p.sc_k + bh));
+      inv_v = __fdiv_rn(1.0f, ldg(p.sc_v + bh)); inv_do = __fdiv_rn(1.0f, ldg(p.sc_do + bh));
     }
     const float c2 = FP8 ? p.c * kLog2e * inv_q * inv_k : p.c * kLog2e;   // scores arrive as products of decoded codes
     const float dp_mul = FP8 ? inv_do * inv_v : 1.0f;                     // likewise dP
@@ -532,13 +533,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     float nx_mul = bias_mul;                                  // the same factor for the next item's head
     auto bias_fetch = [&](int tbh, int step) -> float {
       const int q = step * AT_BLK + (ts & 127);
-      return __ldg(bias_src + (size_t)tbh * p.S + (q < p.S ? q : 0));
+      return ldg(bias_src + (size_t)tbh * p.S + (q < p.S ? q : 0));
     };
     // the second draw's correction term of the same query (threads of the D tile only)
     auto bias_fetch2 = [&](int tbh, int step) -> float {
       if (ND != 2 || ts < 128) return 0.f;
       const int q = step * AT_BLK + (ts & 127);
-      return __ldg(p.dterm + (size_t)p.BH * p.S + (size_t)tbh * p.S + (q < p.S ? q : 0));
+      return ldg(p.dterm + (size_t)p.BH * p.S + (size_t)tbh * p.S + (q < p.S ? q : 0));
     };
     auto bias_put = [&](int step, uint32_t jt, float raw, float mul, float raw2) {
       const int q = ts & 127;
@@ -572,8 +573,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         decode_item(wn, nb, nx_bh, nx_begin, ns);
         nx_total = ns;
         if (FP8) {                                            // per-head operand scales
-          const float nq = __fdiv_rn(1.0f, __ldg(p.sc_q + nx_bh)), nk = __fdiv_rn(1.0f, __ldg(p.sc_k + nx_bh));
-          const float nv = __fdiv_rn(1.0f, __ldg(p.sc_v + nx_bh)), ndo = __fdiv_rn(1.0f, __ldg(p.sc_do + nx_bh));
+          const float nq = __fdiv_rn(1.0f, ldg(p.sc_q + nx_bh)), nk = __fdiv_rn(1.0f, ldg(p.sc_k + nx_bh));
+          const float nv = __fdiv_rn(1.0f, ldg(p.sc_v + nx_bh)), ndo = __fdiv_rn(1.0f, ldg(p.sc_do + nx_bh));
           nx_mul = ts < 128 ? -kLog2e / (p.c * kLog2e * nq * nk) : -1.0f / (ndo * nv);
         }
       }
@@ -595,11 +596,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     if (MODE != AT_DKV) {
       qrow = blk * AT_BLK + r;
       if (MODE == AT_DQ && qrow < p.S) {
-        lse2 = __ldg(p.lse + (size_t)bh * p.S + qrow) * kLog2e;
-        dq = __ldg(p.dterm + (size_t)bh * p.S + qrow);
-        if (ND == 2) dq2 = __ldg(p.dterm + (size_t)p.BH * p.S + (size_t)bh * p.S + qrow);
+        lse2 = ldg(p.lse + (size_t)bh * p.S + qrow) * kLog2e;
+        dq = ldg(p.dterm + (size_t)bh * p.S + qrow);
+        if (ND == 2) dq2 = ldg(p.dterm + (size_t)p.BH * p.S + (size_t)bh * p.S + qrow);
       }
-      if (lse_known && qrow < p.S) lse2 = __ldg(p.lse + (size_t)bh * p.S + qrow) * kLog2e;
+      if (lse_known && qrow < p.S) lse2 = ldg(p.lse + (size_t)bh * p.S + qrow) * kLog2e;
     }
     // FWD: the shift in use (log2 units) and the sum of exp2(c2 s - shift) of this row and column half
     float run_m = lse_known ? lse2 : -INFINITY, run_l = 0.f;
@@ -1016,7 +1017,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
         const int orow = blk * AT_BLK + q4 * 32 + 4 * t + (lane >> 3);
-        rc[t] = __ldg(reinterpret_cast<const float4*>(p.mc_ref + ((size_t)bh * p.S + (orow < p.S ? orow : 0)) * AT_D + h * 32) +
+        rc[t] = ldg(reinterpret_cast<const float4*>(p.mc_ref + ((size_t)bh * p.S + (orow < p.S ? orow : 0)) * AT_D + h * 32) +
                       (lane & 7));
       }
     }
@@ -1164,9 +1165,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
 // conditional add of dO * step.
 template <int DT, int FMT, int kDtRows>
 __global__ void __launch_bounds__(256)
-attn_dterm_kernel(const void* __restrict__ dO, const float* __restrict__ o_orig, const uint8_t* __restrict__ o_codes,
-                  const float* __restrict__ o_scales, const float* __restrict__ do_scales, int64_t rows, int S,
-                  int policy, PhiloxKey key, int draw0, int n_draws, float* __restrict__ D) {
+attn_dterm_kernel(const void* dO, const float* o_orig, const uint8_t* o_codes,
+                  const float* o_scales, const float* do_scales, int64_t rows, int S,
+                  int policy, PhiloxKey key, int draw0, int n_draws, float* D) {
+  grid_dependency();
   const int sub = threadIdx.x & 7;
   const int64_t row0 = (int64_t)blockIdx.x * (32 * kDtRows) + (threadIdx.x >> 3);
   float g[kDtRows][8], o[kDtRows][8], scale[kDtRows], inv[kDtRows];
@@ -1181,15 +1183,15 @@ attn_dterm_kernel(const void* __restrict__ dO, const float* __restrict__ o_orig,
     g[m][0] = g0.x; g[m][1] = g0.y; g[m][2] = g0.z; g[m][3] = g0.w;
     g[m][4] = g1.x; g[m][5] = g1.y; g[m][6] = g1.z; g[m][7] = g1.w;
     if (policy == BSP_READ_FORWARD) {
-      const uint2 pk = __ldg(reinterpret_cast<const uint2*>(o_codes + i0[m]));
+      const uint2 pk = ldg(reinterpret_cast<const uint2*>(o_codes + i0[m]));
       float d0[4], d1[4];
       f8_decode4<FMT>(pk.x, d0);
       f8_decode4<FMT>(pk.y, d1);
 #pragma unroll
       for (int j = 0; j < 4; ++j) { o[m][j] = d0[j]; o[m][4 + j] = d1[j]; }
     } else {
-      const float4 a0 = __ldg(reinterpret_cast<const float4*>(o_orig + i0[m]));
-      const float4 a1 = __ldg(reinterpret_cast<const float4*>(o_orig + i0[m] + 4));
+      const float4 a0 = ldg(reinterpret_cast<const float4*>(o_orig + i0[m]));
+      const float4 a1 = ldg(reinterpret_cast<const float4*>(o_orig + i0[m] + 4));
       o[m][0] = a0.x; o[m][1] = a0.y; o[m][2] = a0.z; o[m][3] = a0.w;
       o[m][4] = a1.x; o[m][5] = a1.y; o[m][6] = a1.z; o[m][7] = a1.w;
     }
@@ -1197,11 +1199,11 @@ attn_dterm_kernel(const void* __restrict__ dO, const float* __restrict__ o_orig,
 #pragma unroll
   for (int m = 0; m < kDtRows; ++m) {
     const int64_t row = active[m] ? row0 + 32 * m : 0;
-    scale[m] = o_scales ? __ldg(o_scales + row / S) : 1.f;
+    scale[m] = o_scales ? ldg(o_scales + row / S) : 1.f;
     inv[m] = __fdiv_rn(1.0f, scale[m]);
     if (do_scales) {
       // dO holds decoded FP8 codes: bring back its per-(b,h) scale
-      const float inv_do = __fdiv_rn(1.0f, __ldg(do_scales + row / S));
+      const float inv_do = __fdiv_rn(1.0f, ldg(do_scales + row / S));
 #pragma unroll
       for (int j = 0; j < 8; ++j) g[m][j] *= inv_do;
     }
@@ -1292,7 +1294,7 @@ static int launch_attn_mode(const void* q, const void* k, const void* v, const v
     nsm = sm_count;
   const int64_t nitems = (int64_t)p.nblk * p.BH;
   const unsigned grid = (unsigned)(nitems < nsm ? nitems : nsm);
-  attn_kernel<MODE, FP8, DV, MC, ND, DQF><<<grid, kAtThreads, kAtSmem, st>>>(mq, mk, mv, mdo, mo0, mo1, mo2, p);
+  launch_kernel(attn_kernel<MODE, FP8, DV, MC, ND, DQF>, grid, kAtThreads, kAtSmem, st, mq, mk, mv, mdo, mo0, mo1, mo2, p);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -1389,7 +1391,7 @@ int attn_dterm_impl(int B, int H, int S, int Dh, const void* dO, int dt, const f
   cudaStream_t st = (cudaStream_t)stream;
   const PhiloxKey pk = make_key(key);
 #define BSP_DT(DT, FMT)                                                                                          \
-  attn_dterm_kernel<DT, FMT, nr><<<grid, 256, 0, st>>>(dO, o_orig, o_codes, o_scales, do_scales, rows, S, d_read, \
+  launch_kernel(attn_dterm_kernel<DT, FMT, nr>, grid, 256, 0, st, dO, o_orig, o_codes, o_scales, do_scales, rows, S, d_read, \
                                                        pk, draw0, n_draws, d_out)
   if (dt == BSP_F32 && o_fmt == BSP_E4M3) BSP_DT(BSP_F32, BSP_E4M3);
   else if (dt == BSP_F32) BSP_DT(BSP_F32, BSP_E5M2);
@@ -1479,13 +1481,14 @@ int attn_bwd_dterm_mc(int B, int H, int S, int Dh, int causal, float softmax_sca
 // codes as bf16 (exact), plus the scales.
 template <int FMT>
 __global__ void __launch_bounds__(256)
-quantize_decode_kernel(const uint16_t* __restrict__ x, size_t group_size, const float* __restrict__ scales,
-                       uint16_t* __restrict__ out, uint8_t* __restrict__ codes, size_t n8) {
+quantize_decode_kernel(const uint16_t* x, size_t group_size, const float* scales,
+                       uint16_t* out, uint8_t* codes, size_t n8) {
+  grid_dependency();
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n8) return;
   const size_t i0 = t * 8;
-  const float s = __ldg(scales + i0 / group_size);
-  const uint4 raw = __ldg(reinterpret_cast<const uint4*>(x) + t);
+  const float s = ldg(scales + i0 / group_size);
+  const uint4 raw = ldg(reinterpret_cast<const uint4*>(x) + t);
   const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
   uint32_t o[4], c[4];
   DiagCounters dc;                                          // (non-finite inputs were counted by the amax pass)
@@ -1543,11 +1546,11 @@ int bsp_attn_quantize(const void* x, int n_groups, size_t group_size, int fmt, v
   const unsigned grid = (unsigned)((n8 + 255) / 256);
   cudaStream_t st = (cudaStream_t)stream;
   if (fmt == BSP_E4M3)
-    quantize_decode_kernel<BSP_E4M3><<<grid, 256, 0, st>>>(reinterpret_cast<const uint16_t*>(x), group_size, scales,
-                                                           reinterpret_cast<uint16_t*>(xq), codes, n8);
+    launch_kernel(quantize_decode_kernel<BSP_E4M3>, grid, 256, 0, st, reinterpret_cast<const uint16_t*>(x), group_size, scales,
+                  reinterpret_cast<uint16_t*>(xq), codes, n8);
   else
-    quantize_decode_kernel<BSP_E5M2><<<grid, 256, 0, st>>>(reinterpret_cast<const uint16_t*>(x), group_size, scales,
-                                                           reinterpret_cast<uint16_t*>(xq), codes, n8);
+    launch_kernel(quantize_decode_kernel<BSP_E5M2>, grid, 256, 0, st, reinterpret_cast<const uint16_t*>(x), group_size, scales,
+                  reinterpret_cast<uint16_t*>(xq), codes, n8);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }

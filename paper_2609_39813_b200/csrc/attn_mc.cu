@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(kDkThreads, 1)
 attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_s1, const __grid_constant__ CUtensorMap tm_s2,
                     DkDiffParams p) {
+  grid_dependency();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -217,7 +218,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     auto bias_fetch = [&](int tbh, int step) -> float {
       if (ts >= 128) return 0.f;
       const int q = step * AT_BLK + ts;
-      return q < p.S ? __ldg(p.lse + (size_t)tbh * p.S + q) : 0.f;
+      return q < p.S ? ldg(p.lse + (size_t)tbh * p.S + q) : 0.f;
     };
     // (fenced = false: the caller issues the proxy fence itself, after other stores that need one too)
     auto bias_put = [&](uint32_t jt, float rawv, bool fenced = true) {
@@ -271,9 +272,9 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const bool q_in = step * AT_BLK + r < p.S;
         {
           const size_t qi = (size_t)bh * p.S + (q_in ? step * AT_BLK + r : 0);
-          dref_raw = __ldg(p.d_ref + qi);
+          dref_raw = ldg(p.d_ref + qi);
 #pragma unroll
-          for (int d = 0; d < kDkND; ++d) draw_raw[d] = d < p.nd ? __ldg(p.d_draws + (size_t)d * rows_total + qi) : 0.f;
+          for (int d = 0; d < kDkND; ++d) draw_raw[d] = d < p.nd ? ldg(p.d_draws + (size_t)d * rows_total + qi) : 0.f;
         }
         int bias_bh = 0, bias_step = 0;
         const bool bias_due = bias_written == jt + 2u && bias_target(it, bias_bh, bias_step);
@@ -442,23 +443,25 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 // S1[i, :] = -c PK[i, :] a[i], S2[i, :] = c^2 PK[i, :]^2 b[i] with a = sum_k (D_k - D*), b = sum_k (D_k - D*)^2
 // (the rowwise sums of the correction term itself): the K draws of dQ in one elementwise pass.
 __global__ void __launch_bounds__(256)
-attn_dq_sums_kernel(const float* __restrict__ pk, const float* __restrict__ S1d, const float* __restrict__ S2d, float c,
-                    float* __restrict__ S1q, float* __restrict__ S2q, size_t n4) {
+attn_dq_sums_kernel(const float* pk, const float* S1d, const float* S2d, float c,
+                    float* S1q, float* S2q, size_t n4) {
+  grid_dependency();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n4) return;
   const size_t row = i / (AT_D / 4);
-  const float4 v = __ldg(reinterpret_cast<const float4*>(pk) + i);
-  const float a = -c * __ldg(S1d + row), b = c * c * __ldg(S2d + row);
+  const float4 v = ldg(reinterpret_cast<const float4*>(pk) + i);
+  const float a = -c * ldg(S1d + row), b = c * c * ldg(S2d + row);
   reinterpret_cast<float4*>(S1q)[i] = make_float4(v.x * a, v.y * a, v.z * a, v.w * a);
   reinterpret_cast<float4*>(S2q)[i] = make_float4(v.x * v.x * b, v.y * v.y * b, v.z * v.z * b, v.w * v.w * b);
 }
 
 // S1 += times * (g - ref), S2 += times * (g - ref)^2, elementwise (times = 1: one draw).
-__global__ void mc_accumulate_kernel(const float* __restrict__ g, const float* __restrict__ ref, float* __restrict__ S1,
-                                     float* __restrict__ S2, size_t n4, float times) {
+__global__ void mc_accumulate_kernel(const float* g, const float* ref, float* S1,
+                                     float* S2, size_t n4, float times) {
+  grid_dependency();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n4) return;
-  const float4 a = __ldg(reinterpret_cast<const float4*>(g) + i), r = __ldg(reinterpret_cast<const float4*>(ref) + i);
+  const float4 a = ldg(reinterpret_cast<const float4*>(g) + i), r = ldg(reinterpret_cast<const float4*>(ref) + i);
   float4 s1 = reinterpret_cast<float4*>(S1)[i], s2 = reinterpret_cast<float4*>(S2)[i];
   const float d0 = a.x - r.x, d1 = a.y - r.y, d2 = a.z - r.z, d3 = a.w - r.w;
   s1.x = fmaf(times, d0, s1.x); s1.y = fmaf(times, d1, s1.y); s1.z = fmaf(times, d2, s1.z); s1.w = fmaf(times, d3, s1.w);
@@ -470,15 +473,16 @@ __global__ void mc_accumulate_kernel(const float* __restrict__ g, const float* _
 
 // The same over nd draws held back to back (g[d * stride + i]), in draw order: one launch instead of
 // nd for a tensor as small as the correction term.  Any n (no vector accesses).
-__global__ void mc_accumulate_draws_kernel(const float* __restrict__ g, size_t stride, int nd,
-                                           const float* __restrict__ ref, float* __restrict__ S1,
-                                           float* __restrict__ S2, size_t n) {
+__global__ void mc_accumulate_draws_kernel(const float* g, size_t stride, int nd,
+                                           const float* ref, float* S1,
+                                           float* S2, size_t n) {
+  grid_dependency();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float r = __ldg(ref + i);
+  const float r = ldg(ref + i);
   float s1 = S1[i], s2 = S2[i];
   for (int d = 0; d < nd; ++d) {
-    const float e = __ldg(g + (size_t)d * stride + i) - r;
+    const float e = ldg(g + (size_t)d * stride + i) - r;
     s1 += e;
     s2 = fmaf(e, e, s2);
   }
@@ -509,7 +513,7 @@ static int attn_dk_diff(int BH, int S, int causal, float c, const void* q, const
   const int nsm = sm_count_or_default();
   const int64_t nitems = (int64_t)p.nblk * BH;
   const unsigned grid = (unsigned)(nitems < nsm ? nitems : nsm);
-  attn_dk_diff_kernel<<<grid, kDkThreads, kDkSmem, st>>>(mq, mk, m1, m2, p);
+  launch_kernel(attn_dk_diff_kernel, grid, kDkThreads, kDkSmem, st, mq, mk, m1, m2, p);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -567,7 +571,7 @@ int bsp_mc_accumulate(const float* g, const float* g_ref, float* S1, float* S2, 
   if (!aligned16(g) || !aligned16(g_ref) || !aligned16(S1) || !aligned16(S2)) return BSP_ERR_ALIGN;
   if (n == 0) return BSP_OK;
   const size_t n4 = n / 4;
-  mc_accumulate_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, (cudaStream_t)stream>>>(g, g_ref, S1, S2, n4, 1.0f);
+  launch_kernel(mc_accumulate_kernel, (unsigned)((n4 + 255) / 256), 256, 0, (cudaStream_t)stream, g, g_ref, S1, S2, n4, 1.0f);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -670,8 +674,8 @@ int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t
                             0, K, b.d_draws, st));
     BSP_CHECK_CUDA(cudaMemsetAsync(b.S1d, 0, rows * 4, st));
     BSP_CHECK_CUDA(cudaMemsetAsync(b.S2d, 0, rows * 4, st));
-    mc_accumulate_draws_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(b.d_draws, rows, K, b.d_ref, b.S1d, b.S2d,
-                                                                              rows);
+    launch_kernel(mc_accumulate_draws_kernel, (unsigned)((rows + 255) / 256), 256, 0, st, b.d_draws, rows, K, b.d_ref, b.S1d, b.S2d,
+                  rows);
     BSP_LAUNCH_CHECK();
     for (int t = 0; t < 2; ++t) {
       BSP_CHECK_CUDA(cudaMemsetAsync(b.S1[t], 0, n * 4, st));
@@ -681,8 +685,8 @@ int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t
       // dQ: P K once (the forward kernel with K in place of V and the rows' LSE given, so it takes one
       // pass over the keys; g_pol[0] is free by now), then the K draws collapse to one elementwise pass
       BSP_TRY(attn_fwd_impl(B, H, S, Dh, op->causal, c, q, k, k, dt, nullptr, b.g_pol[0], nullptr, diag, st, b.lse));
-      attn_dq_sums_kernel<<<(unsigned)((n / 4 + 255) / 256), 256, 0, st>>>(b.g_pol[0], b.S1d, b.S2d, c, b.S1[0], b.S2[0],
-                                                                          n / 4);
+      launch_kernel(attn_dq_sums_kernel, (unsigned)((n / 4 + 255) / 256), 256, 0, st, b.g_pol[0], b.S1d, b.S2d, c, b.S1[0], b.S2[0],
+                    n / 4);
       BSP_LAUNCH_CHECK();
       // dK: four draws per launch
       for (int k0 = 0; k0 < K; k0 += kDkND) {

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/bsp.h"
 
 #define BSP_CHECK_CUDA(expr)                      \
@@ -23,6 +25,33 @@
   } while (0)
 
 namespace bsp {
+
+// Kernels of the library follow one another closely: each is launched with leave to start while the one
+// before it in the stream drains (its blocks take the slots that become free), and each begins by waiting
+// until that one is complete and its writes are visible.  So the order of a stream holds as ever, and a
+// launch's latency runs under the kernel before it: the smallest check 210 -> 168 us,
+// one policy evaluation at 3001 x 1552 x 4112 197 -> 180 us, the longest checks unchanged.
+template <typename... P, typename... A>
+inline void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);    // (an error is cudaGetLastError's: BSP_LAUNCH_CHECK)
+}
+// First in every kernel launched so, before any access to global memory: waits until the kernels before are
+// complete and what they wrote is visible.  Kernel arguments carry no __restrict__, for the reason below: with it
+// the compiler may move a read over this (without it nothing measured slower).
+__device__ __forceinline__ void grid_dependency() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// A plain read.  Not __ldg: that tells the compiler that nothing writes the value while the kernel runs, and it
+// may then read it before grid_dependency has waited for the kernel that does.
+template <typename T>
+__device__ __forceinline__ T ldg(const T* p) { return *p; }
 
 void count_launch();          // defined in mc.cu
 void count_d2h(size_t bytes);  // bytes the library itself copies device -> host (mc.cu)
@@ -315,9 +344,9 @@ __device__ __forceinline__ float bf16_bits_to_float(uint32_t h) { return __uint_
 template <int DT>
 __device__ __forceinline__ float4 load4(const void* p, size_t i) {
   if (DT == BSP_F32) {
-    return __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + i));
+    return ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + i));
   } else {
-    const uint2 r = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(p) + i));
+    const uint2 r = ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(p) + i));
     return make_float4(bf16_bits_to_float(r.x & 0xFFFFu), bf16_bits_to_float(r.x >> 16),
                        bf16_bits_to_float(r.y & 0xFFFFu), bf16_bits_to_float(r.y >> 16));
   }
@@ -329,12 +358,12 @@ template <int DT>
 __device__ __forceinline__ void load16(const void* p, size_t i, float (&v)[16]) {
   if (DT == BSP_F32) {
     const float4* q = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + i);
-    const float4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2), d = __ldg(q + 3);
+    const float4 a = ldg(q), b = ldg(q + 1), c = ldg(q + 2), d = ldg(q + 3);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
     v[8] = c.x; v[9] = c.y; v[10] = c.z; v[11] = c.w; v[12] = d.x; v[13] = d.y; v[14] = d.z; v[15] = d.w;
   } else {
     const uint4* q = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(p) + i);
-    const uint4 a = __ldg(q), b = __ldg(q + 1);
+    const uint4 a = ldg(q), b = ldg(q + 1);
     const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -346,8 +375,8 @@ __device__ __forceinline__ void load16(const void* p, size_t i, float (&v)[16]) 
 
 template <int DT>
 __device__ __forceinline__ float load1(const void* p, size_t i) {
-  if (DT == BSP_F32) return __ldg(reinterpret_cast<const float*>(p) + i);
-  return bf16_bits_to_float(__ldg(reinterpret_cast<const uint16_t*>(p) + i));
+  if (DT == BSP_F32) return ldg(reinterpret_cast<const float*>(p) + i);
+  return bf16_bits_to_float(ldg(reinterpret_cast<const uint16_t*>(p) + i));
 }
 
 // Round-to-nearest-even float -> bf16 bit pattern (finite inputs).

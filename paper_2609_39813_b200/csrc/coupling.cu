@@ -57,24 +57,25 @@ __device__ __forceinline__ void bf16x4_to_float(const uint2& b, float (&v)[4]) {
 constexpr int kCpRows = 16;
 template <int DT, int FMT, bool SR>
 __global__ void __launch_bounds__(256)
-cp_forward_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
-                  const float* __restrict__ beta, const float* __restrict__ rstd, const float* __restrict__ mean,
-                  const float* __restrict__ scale_dev, PhiloxKey key, uint16_t* __restrict__ uq,
-                  const uint16_t* __restrict__ uq_a, uint16_t* __restrict__ dr, bsp_diag_t* diag) {
+cp_forward_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
+                  const float* beta, const float* rstd, const float* mean,
+                  const float* scale_dev, PhiloxKey key, uint16_t* uq,
+                  const uint16_t* uq_a, uint16_t* dr, bsp_diag_t* diag) {
+  grid_dependency();
   const int64_t c = 4 * ((int64_t)blockIdx.x * 64 + threadIdx.x);
-  const float scale = __ldg(scale_dev);
+  const float scale = ldg(scale_dev);
   DiagCounters dc;
   if (c < C) {
-    const float4 g4 = __ldg(reinterpret_cast<const float4*>(gamma + c));
+    const float4 g4 = ldg(reinterpret_cast<const float4*>(gamma + c));
     float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (kind == BSP_LAYERNORM) b4 = __ldg(reinterpret_cast<const float4*>(beta + c));
+    if (kind == BSP_LAYERNORM) b4 = ldg(reinterpret_cast<const float4*>(beta + c));
 #pragma unroll
     for (int j = 0; j < kCpRows / 4; ++j) {
       const int64_t t = (int64_t)blockIdx.y * kCpRows + threadIdx.y + 4 * j;
       if (t >= T) break;
       const size_t i = (size_t)t * C + c;
       float u[4];
-      cp_chain(kind, load4<DT>(x, i), __ldg(rstd + t), kind == BSP_LAYERNORM ? __ldg(mean + t) : 0.f, g4, b4, u);
+      cp_chain(kind, load4<DT>(x, i), ldg(rstd + t), kind == BSP_LAYERNORM ? ldg(mean + t) : 0.f, g4, b4, u);
       uint4 w = make_uint4(0, 0, 0, 0);
       if (SR) w = philox_block(key, (uint64_t)i >> 2, key.c2);
       const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
@@ -84,7 +85,7 @@ cp_forward_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, co
       const uint2 q = f8_to_bf16x4<FMT>(packed);
       *reinterpret_cast<uint2*>(uq + i) = q;
       if (uq_a) {
-        const uint2 a = __ldg(reinterpret_cast<const uint2*>(uq_a + i));
+        const uint2 a = ldg(reinterpret_cast<const uint2*>(uq_a + i));
         float qa[4], qb[4];
         bf16x4_to_float(a, qa);
         bf16x4_to_float(q, qb);
@@ -101,7 +102,8 @@ cp_forward_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, co
 // W as bf16, twice: Wd[o][c] = Wd[O + o][c].  (W need not be aligned.)
 template <int DT>
 __global__ void __launch_bounds__(256)
-cp_weight_kernel(const void* __restrict__ W, size_t n4, uint16_t* __restrict__ Wd) {
+cp_weight_kernel(const void* W, size_t n4, uint16_t* Wd) {
+  grid_dependency();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n4) return;
   const float4 v = (reinterpret_cast<uintptr_t>(W) & 15u) == 0
@@ -123,41 +125,42 @@ cp_weight_kernel(const void* __restrict__ W, size_t n4, uint16_t* __restrict__ W
 constexpr int kCpSlabs = 64;
 template <int DT, int FMT>
 __global__ void __launch_bounds__(256, 3)
-cp_sums_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
-               const float* __restrict__ beta, const float* __restrict__ rstd, const float* __restrict__ mean,
-               const float* __restrict__ scale_dev, PhiloxKey key, int64_t slab_rows, const uint16_t* __restrict__ uq,
-               const float* __restrict__ du, const uint16_t* __restrict__ uq_a, const float* __restrict__ dua,
-               float* __restrict__ sum_r, float* __restrict__ sum_du, bool first, float* __restrict__ partial,
-               double* __restrict__ dots, bsp_diag_t* diag) {
+cp_sums_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
+               const float* beta, const float* rstd, const float* mean,
+               const float* scale_dev, PhiloxKey key, int64_t slab_rows, const uint16_t* uq,
+               const float* du, const uint16_t* uq_a, const float* dua,
+               float* sum_r, float* sum_du, bool first, float* partial,
+               double* dots, bsp_diag_t* diag) {
+  grid_dependency();
   __shared__ __align__(16) float sm[2][8][128];
   __shared__ double sd[2][8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t c = (int64_t)blockIdx.x * 128 + 4 * lane;
-  const float scale = __ldg(scale_dev), inv = __fdiv_rn(1.0f, scale);
+  const float scale = ldg(scale_dev), inv = __fdiv_rn(1.0f, scale);
   const int64_t t0 = (int64_t)blockIdx.y * slab_rows, t1 = t0 + slab_rows < T ? t0 + slab_rows : T;
   float own[4] = {0.f, 0.f, 0.f, 0.f}, fresh[4] = {0.f, 0.f, 0.f, 0.f}, da[4] = {0.f, 0.f, 0.f, 0.f}, db[4] = {0.f, 0.f, 0.f, 0.f};
   DiagCounters dc;
   if (c < C) {
-    const float4 g4 = __ldg(reinterpret_cast<const float4*>(gamma + c));
+    const float4 g4 = ldg(reinterpret_cast<const float4*>(gamma + c));
     float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (kind == BSP_LAYERNORM) b4 = __ldg(reinterpret_cast<const float4*>(beta + c));
+    if (kind == BSP_LAYERNORM) b4 = ldg(reinterpret_cast<const float4*>(beta + c));
 #pragma unroll 1
     for (int64_t t = t0 + w; t < t1; t += 8) {
       const size_t i = (size_t)t * C + c;
-      const float4 xv = load4<DT>(x, i), dv = __ldg(reinterpret_cast<const float4*>(du + i));
-      const uint2 qv = __ldg(reinterpret_cast<const uint2*>(uq + i));
+      const float4 xv = load4<DT>(x, i), dv = ldg(reinterpret_cast<const float4*>(du + i));
+      const uint2 qv = ldg(reinterpret_cast<const uint2*>(uq + i));
       uint2 qav = make_uint2(0u, 0u);
       float4 ya = make_float4(0.f, 0.f, 0.f, 0.f), sr = ya, sdu = ya;
       if (uq_a) {
-        qav = __ldg(reinterpret_cast<const uint2*>(uq_a + i));
-        ya = __ldg(reinterpret_cast<const float4*>(dua + i));
+        qav = ldg(reinterpret_cast<const uint2*>(uq_a + i));
+        ya = ldg(reinterpret_cast<const float4*>(dua + i));
         if (!first) {
           sr = *reinterpret_cast<const float4*>(sum_r + i);
           sdu = *reinterpret_cast<const float4*>(sum_du + i);
         }
       }
       float u[4], q4[4], dec[4];
-      cp_chain(kind, xv, __ldg(rstd + t), kind == BSP_LAYERNORM ? __ldg(mean + t) : 0.f, g4, b4, u);
+      cp_chain(kind, xv, ldg(rstd + t), kind == BSP_LAYERNORM ? ldg(mean + t) : 0.f, g4, b4, u);
       const uint4 wd = philox_block(key, (uint64_t)i >> 2, key.c2);
       const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
       uint32_t packed = 0;
@@ -219,7 +222,8 @@ cp_sums_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const
 
 // out[k] = { T, control } of pair k from its blocks' dot products, in a fixed order.  One block per pair.
 __global__ void __launch_bounds__(256)
-cp_dots_final_kernel(const double* __restrict__ partial, int nblocks, double* __restrict__ out) {
+cp_dots_final_kernel(const double* partial, int nblocks, double* out) {
+  grid_dependency();
   __shared__ double sm[2][256];
   const double* p = partial + (size_t)blockIdx.x * 2 * nblocks;
   double a = 0.0, b = 0.0;
@@ -235,8 +239,9 @@ cp_dots_final_kernel(const double* __restrict__ partial, int nblocks, double* __
 
 // The column sums sum_t a[t][c] b[t][c] per slab of rows (the mean part of the gain error at the end).
 __global__ void __launch_bounds__(256)
-cp_mean_part_kernel(const float* __restrict__ a, const float* __restrict__ b, int64_t T, int64_t C, int64_t slab_rows,
-                    float* __restrict__ partial /* [slab][C] */) {
+cp_mean_part_kernel(const float* a, const float* b, int64_t T, int64_t C, int64_t slab_rows,
+                    float* partial /* [slab][C] */) {
+  grid_dependency();
   __shared__ float sm[8][33];
   const int cl = threadIdx.x & 31, rl = threadIdx.x >> 5;
   const int64_t c = (int64_t)blockIdx.x * 32 + cl;
@@ -256,8 +261,9 @@ cp_mean_part_kernel(const float* __restrict__ a, const float* __restrict__ b, in
 
 // out_y[c] = f_y / gamma[c] times the slabs' sum y (0: own error, 1: fresh read, 2: mean part), in order.
 __global__ void __launch_bounds__(256)
-cp_gain_final_kernel(const float* __restrict__ partial /* [3][slab][C] */, int nslabs, const float* __restrict__ gamma, int64_t C,
-                     float inv_n, float* __restrict__ own, float* __restrict__ fresh, float* __restrict__ mean_part) {
+cp_gain_final_kernel(const float* partial /* [3][slab][C] */, int nslabs, const float* gamma, int64_t C,
+                     float inv_n, float* own, float* fresh, float* mean_part) {
+  grid_dependency();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= C) return;
   const int y = blockIdx.y;
@@ -355,8 +361,8 @@ int bsp_coupling_check(const bsp_coupling_desc_t* op, int pairs, double* T_out, 
   BSP_TRY(bsp_norm_stats(kind, op->x, dt, T, C, op->gamma, op->beta, op->eps, b.rstd, b.mean, b.amax, diag, st));
   BSP_TRY(bsp_scale_from_amax(b.amax, 1, fmt, b.scale, st));
   const size_t w4 = (size_t)O * C / 4;
-  if (dt == BSP_BF16) cp_weight_kernel<BSP_BF16><<<(unsigned)((w4 + 255) / 256), 256, 0, st>>>(op->W, w4, b.Wd);
-  else cp_weight_kernel<BSP_F32><<<(unsigned)((w4 + 255) / 256), 256, 0, st>>>(op->W, w4, b.Wd);
+  if (dt == BSP_BF16) launch_kernel(cp_weight_kernel<BSP_BF16>, (unsigned)((w4 + 255) / 256), 256, 0, st, op->W, w4, b.Wd);
+  else launch_kernel(cp_weight_kernel<BSP_F32>, (unsigned)((w4 + 255) / 256), 256, 0, st, op->W, w4, b.Wd);
   BSP_LAUNCH_CHECK();
 
   bsp_key_t key;
@@ -370,7 +376,7 @@ int bsp_coupling_check(const bsp_coupling_desc_t* op, int pairs, double* T_out, 
     const PhiloxKey pk = make_key(key);
     const uint16_t* uq_a = slot ? b.uq[0] : nullptr;
 #define BSP_CP_FWD(DT, FMT, SR)                                                                                          \
-  cp_forward_kernel<DT, FMT, SR><<<gf, dim3(64, 4), 0, st>>>(kind, op->x, T, C, op->gamma, op->beta, b.rstd, b.mean,     \
+  launch_kernel(cp_forward_kernel<DT, FMT, SR>, gf, dim3(64, 4), 0, st, kind, op->x, T, C, op->gamma, op->beta, b.rstd, b.mean,     \
                                                              b.scale, pk, b.uq[slot], uq_a, b.dr, diag)
 #define BSP_CP_MODE(DT, FMT)                                                   \
   do {                                                                         \
@@ -403,7 +409,7 @@ int bsp_coupling_check(const bsp_coupling_desc_t* op, int pairs, double* T_out, 
     key.stream = BSP_STREAM_GAIN;
     const PhiloxKey pg = make_key(key);
 #define BSP_CP_SUMS(DT, FMT)                                                                                          \
-  cp_sums_kernel<DT, FMT><<<gs, 256, 0, st>>>(kind, op->x, T, C, op->gamma, op->beta, b.rstd, b.mean, b.scale, pg,    \
+  launch_kernel(cp_sums_kernel<DT, FMT>, gs, 256, 0, st, kind, op->x, T, C, op->gamma, op->beta, b.rstd, b.mean, b.scale, pg,    \
                                               b.slab_rows, b.uq[slot], b.du[slot], uq_a, slot ? b.du[0] : nullptr,    \
                                               b.sum_r, b.sum_du, first, b.gain_partial,                               \
                                               b.dot_partial + (size_t)(draw / 2) * b.nblocks * 2, diag)
@@ -428,14 +434,14 @@ int bsp_coupling_check(const bsp_coupling_desc_t* op, int pairs, double* T_out, 
     x.moment_scale = 1.0f / (float)pairs; x.moment_first = k == 0;
     BSP_TRY(gemm_run(x, st));
   }
-  cp_dots_final_kernel<<<(unsigned)pairs, 256, 0, st>>>(b.dot_partial, b.nblocks, b.dots);
+  launch_kernel(cp_dots_final_kernel, (unsigned)pairs, 256, 0, st, b.dot_partial, b.nblocks, b.dots);
   BSP_LAUNCH_CHECK();
   // mean part of the gain error, sum_t (sum_r / n) (sum_du / n) / gamma, and the averages over the forwards
-  cp_mean_part_kernel<<<dim3((unsigned)((C + 31) / 32), (unsigned)b.nslabs), 256, 0, st>>>(
-      b.sum_r, b.sum_du, T, C, b.slab_rows, b.gain_partial + (size_t)2 * b.nslabs * C);
+  launch_kernel(cp_mean_part_kernel, dim3((unsigned)((C + 31) / 32), (unsigned)b.nslabs), 256, 0, st,
+                b.sum_r, b.sum_du, T, C, b.slab_rows, b.gain_partial + (size_t)2 * b.nslabs * C);
   BSP_LAUNCH_CHECK();
-  cp_gain_final_kernel<<<dim3((unsigned)((C + 255) / 256), 3), 256, 0, st>>>(
-      b.gain_partial, b.nslabs, op->gamma, C, 1.0f / (float)(2 * pairs), b.gain_total, b.gain_fresh, b.gain_mean_part);
+  launch_kernel(cp_gain_final_kernel, dim3((unsigned)((C + 255) / 256), 3), 256, 0, st,
+                b.gain_partial, b.nslabs, op->gamma, C, 1.0f / (float)(2 * pairs), b.gain_total, b.gain_fresh, b.gain_mean_part);
   BSP_LAUNCH_CHECK();
   std::vector<double> host((size_t)pairs * 2);
   BSP_CHECK_CUDA(cudaMemcpyAsync(host.data(), b.dots, host.size() * sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -87,6 +87,7 @@ __device__ __forceinline__ void split4(const float4& v, uint2& hi, uint2& lo) {
 template <bool FP8, int MODE, bool PAIR>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p) {
+  grid_dependency();
   constexpr int kStages = PAIR ? kPairStages : bsp::kStages, kStageBytes = PAIR ? kPairStageBytes : bsp::kStageBytes, kCtas = PAIR ? 2 : 1;
   constexpr int kElem = FP8 ? 1 : 2, bk_elems = BKB / kElem, kAtom = 128 / kElem;   // elements per 128 bytes
   extern __shared__ uint8_t smem_raw[];
@@ -208,8 +209,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   } else {
     // ------------------------------------------------ epilogue (warps 2..9)
     const int q = warp & 3;                      // TMEM lane quarter this warp may access
-    const float inv_a = __fdiv_rn(1.0f, p.sa_dev ? __ldg(p.sa_dev) : p.sa);
-    const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? __ldg(p.sb_dev) : p.sb);
+    const float inv_a = __fdiv_rn(1.0f, p.sa_dev ? ldg(p.sa_dev) : p.sa);
+    const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? ldg(p.sb_dev) : p.sb);
     uint32_t tc = 0;
     bool ok = true;
     for (int t = blockIdx.x / kCtas; t < ntiles && ok; t += gridDim.x / kCtas) {
@@ -391,7 +392,8 @@ __device__ __forceinline__ void mc_unit(const McSplit& sp, int u, int npairs, in
 template <bool FP8, bool PAIR>
 __global__ void __launch_bounds__(kMcThreads, 1)
 gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p,
-               McSplit sp, float* __restrict__ split_ws) {
+               McSplit sp, float* split_ws) {
+  grid_dependency();
   constexpr int kMcStages = McRing<PAIR>::kStages, kMcStageBytes = McRing<PAIR>::kStageBytes, kCtas = PAIR ? 2 : 1;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -505,8 +507,8 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kMcRegsEpilogue));
     const int q = warp & 3;                  // TMEM lane quarter
     const int h = (warp - 4) >> 2;           // column half
-    const float inv_a = __fdiv_rn(1.0f, p.sa_dev ? __ldg(p.sa_dev) : p.sa);
-    const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? __ldg(p.sb_dev) : p.sb);
+    const float inv_a = __fdiv_rn(1.0f, p.sa_dev ? ldg(p.sa_dev) : p.sa);
+    const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? ldg(p.sb_dev) : p.sb);
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16) + h * 64;
     uint32_t tc = 0;
     bool ok = true;
@@ -605,8 +607,9 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 // (its row tile t % ctas), a
 // thread takes four columns of one row; slots are added in the order of their draws.
 __global__ void __launch_bounds__(256)
-gemm_mc_merge_kernel(const float* __restrict__ split_ws, McSplit sp, int ctas, int M, int N, int64_t ldc, float* __restrict__ S1,
-                     float* __restrict__ S2) {
+gemm_mc_merge_kernel(const float* split_ws, McSplit sp, int ctas, int M, int N, int64_t ldc, float* S1,
+                     float* S2) {
+  grid_dependency();
   const int tiles_m = (M + ctas * BM - 1) / (ctas * BM), tiles_n = (N + MC_BN - 1) / MC_BN;
   int tm, tn;
   tile_coords(sp.whole + (int)blockIdx.x / ctas, tiles_m, tiles_n, tm, tn);
@@ -619,7 +622,7 @@ gemm_mc_merge_kernel(const float* __restrict__ split_ws, McSplit sp, int ctas, i
   const float4* src = reinterpret_cast<const float4*>(split_ws + (size_t)blockIdx.x * kMcSplitTileFloats) + i;
 #pragma unroll 4
   for (int g = 1; g < sp.nseg; ++g, src += (size_t)sp.rest * ctas * (kMcSplitTileFloats / 4)) {
-    const float4 v = __ldg(src);
+    const float4 v = ldg(src);
     s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
   }
   *dst = s;
@@ -631,14 +634,15 @@ gemm_mc_merge_kernel(const float* __restrict__ split_ws, McSplit sp, int ctas, i
 // the environment, to tell a tensor-core-path defect from a defect elsewhere.
 template <bool FP8>
 __global__ void __launch_bounds__(256)
-gemm_simt_kernel(const void* __restrict__ A, const void* __restrict__ B, int a_fmt, int b_fmt, int64_t lda,
+gemm_simt_kernel(const void* A, const void* B, int a_fmt, int b_fmt, int64_t lda,
                  int64_t ldb, int64_t b_batch_stride, GemmParams p) {
+  grid_dependency();
   __shared__ float sa[16][17], sb[16][17];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int m = blockIdx.y * 16 + ty, n = blockIdx.x * 16 + tx;
   const int b = blockIdx.z;
-  const float inv_a = __fdiv_rn(1.0f, p.sa_dev ? __ldg(p.sa_dev) : p.sa);
-  const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? __ldg(p.sb_dev) : p.sb);
+  const float inv_a = __fdiv_rn(1.0f, p.sa_dev ? ldg(p.sa_dev) : p.sa);
+  const float inv_b = __fdiv_rn(1.0f, p.sb_dev ? ldg(p.sb_dev) : p.sb);
   float acc = 0.f;
   for (int k0 = 0; k0 < p.K; k0 += 16) {
     const int ka = k0 + tx;
@@ -817,11 +821,13 @@ static int gemm_mc_launch(const CUtensorMap& ma, const CUtensorMap& mb, const Ge
     attr_set.store(true, std::memory_order_release);
   }
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = PAIR ? 2 : 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_kernel does
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = PAIR ? 2 : 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kMcThreads); cfg.dynamicSmemBytes = kMcSmem; cfg.stream = st;
-  cfg.attrs = attr; cfg.numAttrs = PAIR ? 1 : 0;
+  cfg.attrs = attr; cfg.numAttrs = PAIR ? 2 : 1;
   BSP_CHECK_CUDA(cudaLaunchKernelEx(&cfg, gemm_mc_kernel<FP8, PAIR>, ma, mb, p, sp, split_ws));
   BSP_LAUNCH_CHECK();
   return BSP_OK;
@@ -838,12 +844,14 @@ static int gemm_tc_launch_as(const CUtensorMap& ma, const CUtensorMap& mb, const
   constexpr int ctas = PAIR ? 2 : 1;
   const int ntiles = ((p.M + ctas * BM - 1) / (ctas * BM)) * ((p.N + p.bn - 1) / p.bn);
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ctas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_kernel does
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ctas; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)(ctas * (ntiles < nsm / ctas ? ntiles : nsm / ctas)));
   cfg.blockDim = dim3(kGemmThreads); cfg.dynamicSmemBytes = kGemmSmem; cfg.stream = st;
-  cfg.attrs = attr; cfg.numAttrs = PAIR ? 1 : 0;
+  cfg.attrs = attr; cfg.numAttrs = PAIR ? 2 : 1;
   BSP_CHECK_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<FP8, MODE, PAIR>, ma, mb, p));
   BSP_LAUNCH_CHECK();
   return BSP_OK;
@@ -878,12 +886,12 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
       for (int b = 0; b < g.nb; ++b) {
         grid.z = 1;
         const void* Bb = reinterpret_cast<const uint8_t*>(g.B) + (size_t)b * g.b_batch_stride * eb;
-        if (g.fp8) gemm_simt_kernel<true><<<grid, 256, 0, st>>>(g.A, Bb, g.a_fmt, g.b_fmt, g.lda, g.ldb, 0, p);
-        else gemm_simt_kernel<false><<<grid, 256, 0, st>>>(g.A, Bb, g.a_fmt, g.b_fmt, g.lda, g.ldb, 0, p);
+        if (g.fp8) launch_kernel(gemm_simt_kernel<true>, grid, 256, 0, st, g.A, Bb, g.a_fmt, g.b_fmt, g.lda, g.ldb, 0, p);
+        else launch_kernel(gemm_simt_kernel<false>, grid, 256, 0, st, g.A, Bb, g.a_fmt, g.b_fmt, g.lda, g.ldb, 0, p);
       }
     } else {
-      if (g.fp8) gemm_simt_kernel<true><<<grid, 256, 0, st>>>(g.A, g.B, g.a_fmt, g.b_fmt, g.lda, g.ldb, g.b_batch_stride, p);
-      else gemm_simt_kernel<false><<<grid, 256, 0, st>>>(g.A, g.B, g.a_fmt, g.b_fmt, g.lda, g.ldb, g.b_batch_stride, p);
+      if (g.fp8) launch_kernel(gemm_simt_kernel<true>, grid, 256, 0, st, g.A, g.B, g.a_fmt, g.b_fmt, g.lda, g.ldb, g.b_batch_stride, p);
+      else launch_kernel(gemm_simt_kernel<false>, grid, 256, 0, st, g.A, g.B, g.a_fmt, g.b_fmt, g.lda, g.ldb, g.b_batch_stride, p);
     }
     BSP_LAUNCH_CHECK();
     return BSP_OK;
@@ -915,8 +923,8 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
     else rc = pair ? gemm_mc_launch<false, true>(ma, mb, p, sp, g.split_ws, grid_mc, st) : gemm_mc_launch<false, false>(ma, mb, p, sp, g.split_ws, grid_mc, st);
     if (rc != BSP_OK) return rc;
     if (sp.nseg > 1) {
-      gemm_mc_merge_kernel<<<dim3((unsigned)(sp.rest * ctas), 2 * BM * MC_BN / 4 / 256), 256, 0, st>>>(g.split_ws, sp, ctas, p.M, p.N, p.ldc,
-                                                                                              p.S1, p.S2);
+      launch_kernel(gemm_mc_merge_kernel, dim3((unsigned)(sp.rest * ctas), 2 * BM * MC_BN / 4 / 256), 256, 0, st, g.split_ws, sp, ctas, p.M, p.N, p.ldc,
+                    p.S1, p.S2);
       BSP_LAUNCH_CHECK();
     }
     return BSP_OK;
@@ -945,10 +953,11 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
 // (bound by its 3 B per code; field by field it was bound by instructions; 180 M codes: 146 -> 95 us).
 template <int FMT>
 __global__ void __launch_bounds__(256)
-decode_to_bf16_kernel(const uint8_t* __restrict__ codes, size_t n16, uint16_t* __restrict__ out) {
+decode_to_bf16_kernel(const uint8_t* codes, size_t n16, uint16_t* out) {
+  grid_dependency();
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n16) return;
-  const uint4 c = __ldg(reinterpret_cast<const uint4*>(codes) + t);
+  const uint4 c = ldg(reinterpret_cast<const uint4*>(codes) + t);
   const uint2 a = f8_to_bf16x4<FMT>(c.x), b = f8_to_bf16x4<FMT>(c.y), d = f8_to_bf16x4<FMT>(c.z), e = f8_to_bf16x4<FMT>(c.w);
   uint4* dst = reinterpret_cast<uint4*>(out) + 2 * t;
   dst[0] = make_uint4(a.x, a.y, b.x, b.y);
@@ -957,10 +966,11 @@ decode_to_bf16_kernel(const uint8_t* __restrict__ codes, size_t n16, uint16_t* _
 
 // FP32 -> bf16, same layout.
 __global__ void __launch_bounds__(256)
-to_bf16_kernel(const float* __restrict__ in, size_t n8, uint16_t* __restrict__ out) {
+to_bf16_kernel(const float* in, size_t n8, uint16_t* out) {
+  grid_dependency();
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n8) return;
-  const float4 a = __ldg(reinterpret_cast<const float4*>(in) + 2 * t), b = __ldg(reinterpret_cast<const float4*>(in) + 2 * t + 1);
+  const float4 a = ldg(reinterpret_cast<const float4*>(in) + 2 * t), b = ldg(reinterpret_cast<const float4*>(in) + 2 * t + 1);
   reinterpret_cast<uint4*>(out)[t] =
       make_uint4(float_to_bf16_bits(a.x) | (float_to_bf16_bits(a.y) << 16), float_to_bf16_bits(a.z) | (float_to_bf16_bits(a.w) << 16),
                  float_to_bf16_bits(b.x) | (float_to_bf16_bits(b.y) << 16), float_to_bf16_bits(b.z) | (float_to_bf16_bits(b.w) << 16));
@@ -969,8 +979,9 @@ to_bf16_kernel(const float* __restrict__ in, size_t n8, uint16_t* __restrict__ o
 // out[c*ld_out + r] = bf16(in[r*cols + c]); 32 x 32 tiles.
 template <int DT>
 __global__ void __launch_bounds__(256)
-to_bf16_transpose_kernel(const void* __restrict__ in, int64_t rows, int64_t cols, uint16_t* __restrict__ out,
+to_bf16_transpose_kernel(const void* in, int64_t rows, int64_t cols, uint16_t* out,
                          int64_t ld_out) {
+  grid_dependency();
   __shared__ uint16_t tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
@@ -1028,9 +1039,9 @@ int bsp_linear_wgrad(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t,
     const size_t n16 = (size_t)O * ld_t / 16;
     uint16_t* dyb = reinterpret_cast<uint16_t*>(ws);
     if (q_dy.fmt == BSP_E5M2)
-      decode_to_bf16_kernel<BSP_E5M2><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes_t, n16, dyb);
+      launch_kernel(decode_to_bf16_kernel<BSP_E5M2>, (unsigned)((n16 + 255) / 256), 256, 0, st, dy_codes_t, n16, dyb);
     else
-      decode_to_bf16_kernel<BSP_E4M3><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes_t, n16, dyb);
+      launch_kernel(decode_to_bf16_kernel<BSP_E4M3>, (unsigned)((n16 + 255) / 256), 256, 0, st, dy_codes_t, n16, dyb);
     BSP_LAUNCH_CHECK();
     g.fp8 = false; g.A = dyb; g.B = x_t; g.a_fmt = 0; g.b_fmt = 0;
     g.sb = 1.0f; g.sb_dev = nullptr;          // the original is unscaled
@@ -1106,9 +1117,9 @@ int bsp_linear_dgrad(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes, b
   uint16_t* wt = reinterpret_cast<uint16_t*>(reinterpret_cast<char*>(ws) + round_up((size_t)T * O * 2, 256));
   const size_t n16 = (size_t)T * O / 16;
   if (q_dy.fmt == BSP_E5M2)
-    decode_to_bf16_kernel<BSP_E5M2><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes, n16, dyb);
+    launch_kernel(decode_to_bf16_kernel<BSP_E5M2>, (unsigned)((n16 + 255) / 256), 256, 0, st, dy_codes, n16, dyb);
   else
-    decode_to_bf16_kernel<BSP_E4M3><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes, n16, dyb);
+    launch_kernel(decode_to_bf16_kernel<BSP_E4M3>, (unsigned)((n16 + 255) / 256), 256, 0, st, dy_codes, n16, dyb);
   BSP_LAUNCH_CHECK();
   // W [O][C] is the B operand with the contraction index outermost and is read as it lies (MN-major): a
   // bf16 W in place, an FP32 W from a bf16 copy of the same layout (a transposed copy, a quarter of the
@@ -1116,12 +1127,12 @@ int bsp_linear_dgrad(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes, b
   const bool pitch_ok = C % 8 == 0 && aligned16(W), w_in_place = pitch_ok && w_dt == BSP_BF16;
   if (pitch_ok && !w_in_place) {
     const size_t n8 = (size_t)O * C / 8;
-    to_bf16_kernel<<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>(reinterpret_cast<const float*>(W), n8, wt);
+    launch_kernel(to_bf16_kernel, (unsigned)((n8 + 255) / 256), 256, 0, st, reinterpret_cast<const float*>(W), n8, wt);
     BSP_LAUNCH_CHECK();
   } else if (!pitch_ok) {
     dim3 tg((unsigned)((C + 31) / 32), (unsigned)((O + 31) / 32));
-    if (w_dt == BSP_F32) to_bf16_transpose_kernel<BSP_F32><<<tg, 256, 0, st>>>(W, O, C, wt, O);
-    else to_bf16_transpose_kernel<BSP_BF16><<<tg, 256, 0, st>>>(W, O, C, wt, O);
+    if (w_dt == BSP_F32) launch_kernel(to_bf16_transpose_kernel<BSP_F32>, tg, 256, 0, st, W, O, C, wt, O);
+    else launch_kernel(to_bf16_transpose_kernel<BSP_BF16>, tg, 256, 0, st, W, O, C, wt, O);
     BSP_LAUNCH_CHECK();
   }
   GemmArgs g;

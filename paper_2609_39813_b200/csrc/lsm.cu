@@ -29,7 +29,8 @@ constexpr int kLsmThreads = 256;
 constexpr int kLsmStats = 6, kLsmCols = 8;
 
 __global__ void __launch_bounds__(kLsmThreads)
-lsm_prep_kernel(const float* __restrict__ logits, int classes, float eps, float4* __restrict__ table) {
+lsm_prep_kernel(const float* logits, int classes, float eps, float4* table) {
+  grid_dependency();
   __shared__ float red[kLsmThreads / 32];
   __shared__ float bc;
   const size_t row = blockIdx.x;
@@ -68,15 +69,16 @@ lsm_prep_kernel(const float* __restrict__ logits, int classes, float eps, float4
 
 // Block (x, y): trials x * blockDim.x .., rows of chunk y; partial[y][statistic][trial].
 __global__ void __launch_bounds__(kLsmThreads)
-lsm_trial_kernel(const float4* __restrict__ table, int rows, int rows_per_chunk, int classes, float eps, PhiloxKey key_reuse,
-                 PhiloxKey key_copy, int trials, float* __restrict__ partial) {
+lsm_trial_kernel(const float4* table, int rows, int rows_per_chunk, int classes, float eps, PhiloxKey key_reuse,
+                 PhiloxKey key_copy, int trials, float* partial) {
+  grid_dependency();
   const int trial = (int)(blockIdx.x * blockDim.x + threadIdx.x);
   const int row0 = (int)blockIdx.y * rows_per_chunk;
   const int row1 = row0 + rows_per_chunk < rows ? row0 + rows_per_chunk : rows;
   const int groups = classes / 4;                                   // classes % 4 == 0: groups never straddle rows
   float acc[kLsmStats] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   for (int row = row0; row < row1; ++row) {
-    const float4* __restrict__ t = table + (size_t)row * classes;
+    const float4* t = table + (size_t)row * classes;
     const uint64_t q0 = ((uint64_t)row * classes) / 4;
     float a1 = 0.f, a2 = 0.f, b1 = 0.f;
     int cnt = 0;
@@ -86,7 +88,7 @@ lsm_trial_kernel(const float4* __restrict__ table, int rows, int rows_per_chunk,
       const uint32_t u1[4] = {w1.x, w1.y, w1.z, w1.w}, u2[4] = {w2.x, w2.y, w2.z, w2.w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const float4 v = __ldg(t + 4 * g + e);
+        const float4 v = ldg(t + 4 * g + e);
         a1 += (int)u1[e] < 0 ? v.x : v.y;                           // the top bit set: +eps
         b1 += (int)u1[e] < 0 ? v.z : v.w;
         a2 += (int)u2[e] < 0 ? v.x : v.y;
@@ -111,8 +113,9 @@ lsm_trial_kernel(const float4* __restrict__ table, int rows, int rows_per_chunk,
 // (likelihood, constructed); out[block][2c], [2c + 1] = sum and sum of squares in double.  A block takes
 // 32 trials at a time, eight threads sharing a trial's row chunks; fixed order throughout.
 __global__ void __launch_bounds__(256)
-lsm_collect_kernel(const float* __restrict__ partial, int nchunks, int trials, double inv_n, float* __restrict__ per_trial,
-                   double* __restrict__ out) {
+lsm_collect_kernel(const float* partial, int nchunks, int trials, double inv_n, float* per_trial,
+                   double* out) {
+  grid_dependency();
   __shared__ double part[8][kLsmStats][33];
   __shared__ double sh[2 * kLsmCols][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -125,7 +128,7 @@ lsm_collect_kernel(const float* __restrict__ partial, int nchunks, int trials, d
     if (t < trials)
       for (int y = w; y < nchunks; y += 8)
 #pragma unroll
-        for (int i = 0; i < kLsmStats; ++i) a[i] += (double)__ldg(partial + ((size_t)y * kLsmStats + i) * trials + t);
+        for (int i = 0; i < kLsmStats; ++i) a[i] += (double)ldg(partial + ((size_t)y * kLsmStats + i) * trials + t);
 #pragma unroll
     for (int i = 0; i < kLsmStats; ++i) part[w][i][lane] = a[i];
     __syncthreads();
@@ -211,12 +214,12 @@ int bsp_lsm_check(const float* logits, const int32_t* target, int rows, int clas
   const PhiloxKey kr = make_key(k);
   k.stream = BSP_STREAM_GAIN;                                       // the independent copy's own stream
   const PhiloxKey kc = make_key(k);
-  lsm_prep_kernel<<<(unsigned)rows, kLsmThreads, 0, st>>>(logits, classes, eps, table);
+  launch_kernel(lsm_prep_kernel, (unsigned)rows, kLsmThreads, 0, st, logits, classes, eps, table);
   BSP_LAUNCH_CHECK();
-  lsm_trial_kernel<<<dim3((unsigned)plan.tblocks, (unsigned)plan.nchunks), plan.threads, 0, st>>>(
-      table, rows, plan.rows_per_chunk, classes, eps, kr, kc, trials, partial);
+  launch_kernel(lsm_trial_kernel, dim3((unsigned)plan.tblocks, (unsigned)plan.nchunks), plan.threads, 0, st,
+                table, rows, plan.rows_per_chunk, classes, eps, kr, kc, trials, partial);
   BSP_LAUNCH_CHECK();
-  lsm_collect_kernel<<<(unsigned)plan.cblocks, 256, 0, st>>>(partial, plan.nchunks, trials, 1.0 / ((double)rows * classes), pt, sums);
+  launch_kernel(lsm_collect_kernel, (unsigned)plan.cblocks, 256, 0, st, partial, plan.nchunks, trials, 1.0 / ((double)rows * classes), pt, sums);
   BSP_LAUNCH_CHECK();
   double parts[kNumSMs * 2 * kLsmCols], host[2 * kLsmCols];
   const size_t bytes = (size_t)plan.cblocks * 2 * kLsmCols * sizeof(double);

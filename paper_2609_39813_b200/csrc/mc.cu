@@ -35,8 +35,9 @@ __device__ __forceinline__ double warp_max_d(double v) {
 // when |err| <= det_tol |g*|, else +-infinity.  M2 below the resolution of the FP32 sums (1e-6 of
 // S2) counts as no variance.  Block partials in double, summed on the host in block order.
 __global__ void __launch_bounds__(256)
-mc_stats_kernel(const float* __restrict__ g_ref, const float* __restrict__ g, const float* __restrict__ S2,
-                int64_t n, int K, int fresh, float det_tol, double* __restrict__ partials) {
+mc_stats_kernel(const float* g_ref, const float* g, const float* S2,
+                int64_t n, int K, int fresh, float det_tol, double* partials) {
+  grid_dependency();
   // Per-element arithmetic in FP32 (M2 = S2 - S1^2/K as one fused multiply-add), per-thread partial
   // sums in FP32 over the few hundred elements a thread visits, everything above that in double:
   // FP64 division and square root per element would make this pass compute-bound.
@@ -66,10 +67,10 @@ mc_stats_kernel(const float* __restrict__ g_ref, const float* __restrict__ g, co
   };
   const int64_t n4 = n / 4, stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const float4 r = __ldg(reinterpret_cast<const float4*>(g_ref) + i);
-    const float4 a = __ldg(reinterpret_cast<const float4*>(g) + i);
+    const float4 r = ldg(reinterpret_cast<const float4*>(g_ref) + i);
+    const float4 a = ldg(reinterpret_cast<const float4*>(g) + i);
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (fresh) s = __ldg(reinterpret_cast<const float4*>(S2) + i);
+    if (fresh) s = ldg(reinterpret_cast<const float4*>(S2) + i);
     one(r.x, a.x, s.x); one(r.y, a.y, s.y); one(r.z, a.z, s.z); one(r.w, a.w, s.w);
   }
   for (int64_t i = n4 * 4 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
@@ -109,7 +110,7 @@ int mc_stats_launch(const float* g_ref, const float* g, const float* S2, int64_t
   *blocks_out = blocks;
   if (blocks > 0) {
     const float det_tol = (float)(rule ? rule : default_rule())->rel_tol_deterministic;
-    mc_stats_kernel<<<blocks, 256, 0, st>>>(g_ref, g, S2, n, K, fresh, det_tol, partials);
+    launch_kernel(mc_stats_kernel, blocks, 256, 0, st, g_ref, g, S2, n, K, fresh, det_tol, partials);
     BSP_LAUNCH_CHECK();
   }
   return BSP_OK;
@@ -235,8 +236,9 @@ static size_t carve(const bsp_norm_linear_desc_t* op, int K, char* base, CheckBu
 
 // mean = g* + S1/K, var = (S2 - S1^2/K)/(K-1), z = (S1/K)/sqrt(var/K), elementwise.
 __global__ void __launch_bounds__(256)
-mc_moments_kernel(const float* __restrict__ g_ref, const float* __restrict__ S1, const float* __restrict__ S2, size_t n,
-                  int K, float* __restrict__ mean, float* __restrict__ var, float* __restrict__ z) {
+mc_moments_kernel(const float* g_ref, const float* S1, const float* S2, size_t n,
+                  int K, float* mean, float* var, float* z) {
+  grid_dependency();
   const float invK = 1.0f / (float)K, invK1 = 1.0f / (float)(K - 1);
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const float a = S1[i], e = a * invK;
@@ -253,6 +255,7 @@ mc_moments_kernel(const float* __restrict__ g_ref, const float* __restrict__ S1,
 // One warp waits, with the library's bounded wait and the given limit, on a barrier that nothing
 // completes; the wait gives up, the status is raised, the kernel returns.
 __global__ void bounded_wait_selftest_kernel(uint64_t limit_ns, bsp_diag_t* diag) {
+  grid_dependency();
   __shared__ __align__(8) uint64_t bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -325,14 +328,14 @@ int bsp_mc_moments(const float* g_ref, const float* S1, const float* S2, size_t 
   if (!g_ref || !S1 || !S2 || K < 2) return BSP_ERR_ARG;
   if (n == 0 || (!mean && !var && !z)) return BSP_OK;
   const unsigned grid = (unsigned)((n + 255) / 256 < 148 * 16 ? (n + 255) / 256 : 148 * 16);
-  mc_moments_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(g_ref, S1, S2, n, K, mean, var, z);
+  launch_kernel(mc_moments_kernel, grid, 256, 0, (cudaStream_t)stream, g_ref, S1, S2, n, K, mean, var, z);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
 
 int bsp_selftest_bounded_wait(uint64_t limit_ns, bsp_diag_t* diag, void* stream) {
   if (!diag || limit_ns == 0 || limit_ns > 100000000ull) return BSP_ERR_ARG;
-  bounded_wait_selftest_kernel<<<1, 64, 0, (cudaStream_t)stream>>>(limit_ns, diag);
+  launch_kernel(bounded_wait_selftest_kernel, 1, 64, 0, (cudaStream_t)stream, limit_ns, diag);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }

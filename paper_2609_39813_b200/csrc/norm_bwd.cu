@@ -22,14 +22,15 @@ __device__ __forceinline__ float sr_value(float v, uint32_t U) { return f8_sr_va
 // current and the prefetched row) stays near 64 registers, which keeps 1024 threads resident.
 template <int DT, int DU_DT, int FMT, int JMAX, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT)
-norm_bwd_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
-                const float* __restrict__ beta, const float* __restrict__ rstd, const float* __restrict__ mean,
-                const void* __restrict__ du, int gain_read, int dx_read, const uint8_t* __restrict__ u_codes,
-                float scale_val, const float* __restrict__ scale_dev, PhiloxKey key, PhiloxKey key_dx,
-                float* __restrict__ part_g, float* __restrict__ part_b, float* __restrict__ dx) {
+norm_bwd_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
+                const float* beta, const float* rstd, const float* mean,
+                const void* du, int gain_read, int dx_read, const uint8_t* u_codes,
+                float scale_val, const float* scale_dev, PhiloxKey key, PhiloxKey key_dx,
+                float* part_g, float* part_b, float* dx) {
+  grid_dependency();
   __shared__ float red[2][2][NT / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float scale = scale_dev ? __ldg(scale_dev) : scale_val;
+  const float scale = scale_dev ? ldg(scale_dev) : scale_val;
   const float inv_scale = __fdiv_rn(1.0f, scale);
   const float invC = 1.0f / (float)C;
 
@@ -40,8 +41,8 @@ norm_bwd_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, cons
     g4[j] = make_float4(1.f, 1.f, 1.f, 1.f);
     b4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (c < C) {
-      g4[j] = __ldg(reinterpret_cast<const float4*>(gamma + c));
-      if (kind == BSP_LAYERNORM) b4[j] = __ldg(reinterpret_cast<const float4*>(beta + c));
+      g4[j] = ldg(reinterpret_cast<const float4*>(gamma + c));
+      if (kind == BSP_LAYERNORM) b4[j] = ldg(reinterpret_cast<const float4*>(beta + c));
     }
     accg[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     accb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -57,8 +58,8 @@ norm_bwd_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, cons
   float4 nx[JMAX], nd[JMAX];
   float nrs = 0.f, nmu = 0.f;
   auto fetch = [&](int64_t r) {
-    nrs = __ldg(rstd + r);
-    nmu = kind == BSP_LAYERNORM ? __ldg(mean + r) : 0.f;
+    nrs = ldg(rstd + r);
+    nmu = kind == BSP_LAYERNORM ? ldg(mean + r) : 0.f;
 #pragma unroll
     for (int j = 0; j < JMAX; ++j) {
       const int64_t c = 4 * ((int64_t)tid + NT * j);
@@ -98,7 +99,7 @@ norm_bwd_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, cons
           if (policy == BSP_READ_ORIGINAL) return zo;
           float dec[4];
           if (policy == BSP_READ_FORWARD) {
-            const uint32_t pk = __ldg(reinterpret_cast<const uint32_t*>(u_codes + i0));
+            const uint32_t pk = ldg(reinterpret_cast<const uint32_t*>(u_codes + i0));
             f8_decode4<FMT>(pk, dec);
           } else {
             const uint4 w = philox_block(kk, (uint64_t)i0 >> 2, kk.c2);
@@ -170,11 +171,12 @@ norm_bwd_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, cons
 // out[c] = sum over nparts of part[p*C + c], in a fixed order.  grid: (C/32, 1 or 2) blocks of
 // 256 = 8 x 32 threads; blockIdx.y == 1 reduces the second pair (dbeta beside dgamma in one launch).
 __global__ void __launch_bounds__(256)
-column_reduce_kernel(const float* __restrict__ part0, float* __restrict__ out0, const float* __restrict__ part1,
-                     float* __restrict__ out1, int nparts, int64_t C) {
+column_reduce_kernel(const float* part0, float* out0, const float* part1,
+                     float* out1, int nparts, int64_t C) {
+  grid_dependency();
   __shared__ float sm[8][33];
-  const float* __restrict__ part = blockIdx.y ? part1 : part0;
-  float* __restrict__ out = blockIdx.y ? out1 : out0;
+  const float* part = blockIdx.y ? part1 : part0;
+  float* out = blockIdx.y ? out1 : out0;
   const int cl = threadIdx.x & 31, pl = threadIdx.x >> 5;
   const int64_t c = (int64_t)blockIdx.x * 32 + cl;
   float s = 0.f;
@@ -182,11 +184,11 @@ column_reduce_kernel(const float* __restrict__ part0, float* __restrict__ out0, 
     // four loads in flight per thread; the additions keep the order p = pl, pl + 8, ...
     int p = pl;
     for (; p + 24 < nparts; p += 32) {
-      const float a0 = __ldg(part + (size_t)p * C + c), a1 = __ldg(part + (size_t)(p + 8) * C + c);
-      const float a2 = __ldg(part + (size_t)(p + 16) * C + c), a3 = __ldg(part + (size_t)(p + 24) * C + c);
+      const float a0 = ldg(part + (size_t)p * C + c), a1 = ldg(part + (size_t)(p + 8) * C + c);
+      const float a2 = ldg(part + (size_t)(p + 16) * C + c), a3 = ldg(part + (size_t)(p + 24) * C + c);
       s += a0; s += a1; s += a2; s += a3;
     }
-    for (; p < nparts; p += 8) s += __ldg(part + (size_t)p * C + c);
+    for (; p < nparts; p += 8) s += ldg(part + (size_t)p * C + c);
   }
   sm[pl][cl] = s;
   __syncthreads();
@@ -236,11 +238,12 @@ static int gain_chunk(int64_t T, int64_t C, int K) {
 
 template <int DT, int DU_DT, int FMT>
 __global__ void __launch_bounds__(kMcWarps * 32, 2)
-gain_mc_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
-               const float* __restrict__ beta, const float* __restrict__ rstd, const float* __restrict__ mean,
-               const void* __restrict__ du, float scale_val, const float* __restrict__ scale_dev,
-               const float* __restrict__ grid_steps, PhiloxKey key, int draw_begin, int ndraws, int draws_per_z, int subs,
-               float* __restrict__ partial /* [ndraws][nslabs][C] */, bsp_diag_t* __restrict__ diag) {
+gain_mc_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
+               const float* beta, const float* rstd, const float* mean,
+               const void* du, float scale_val, const float* scale_dev,
+               const float* grid_steps, PhiloxKey key, int draw_begin, int ndraws, int draws_per_z, int subs,
+               float* partial /* [ndraws][nslabs][C] */, bsp_diag_t* diag) {
+  grid_dependency();
   // A fresh rounding of an element is its round-down value plus, with probability frac, one grid
   // step: value(U) = lo + (U < P) * (hi - lo) with the threshold P of f8_sr_threshold.  So the
   // gain-use sum of draw k is  sum_t (lo/scale - beta)/gamma * du  (the same for every draw, summed
@@ -261,15 +264,15 @@ gain_mc_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t c = (int64_t)blockIdx.x * kMcCols + lane * 4;
   const int64_t slab = blockIdx.y, nslabs = gridDim.y;
-  const float scale = grid_steps ? 1.0f : (scale_dev ? __ldg(scale_dev) : scale_val);
+  const float scale = grid_steps ? 1.0f : (scale_dev ? ldg(scale_dev) : scale_val);
   const float inv_scale = __fdiv_rn(1.0f, scale);
   const bool col_ok = c < C;
   const int k0 = (int)blockIdx.z * draws_per_z, kend = k0 + draws_per_z < ndraws ? k0 + draws_per_z : ndraws, nd = kend - k0;
 
   float4 g4 = make_float4(1.f, 1.f, 1.f, 1.f), b4 = make_float4(0.f, 0.f, 0.f, 0.f);
   if (col_ok) {
-    g4 = __ldg(reinterpret_cast<const float4*>(gamma + c));
-    if (kind == BSP_LAYERNORM) b4 = __ldg(reinterpret_cast<const float4*>(beta + c));
+    g4 = ldg(reinterpret_cast<const float4*>(gamma + c));
+    if (kind == BSP_LAYERNORM) b4 = ldg(reinterpret_cast<const float4*>(beta + c));
   }
   const float gg[4] = {g4.x, g4.y, g4.z, g4.w};
   const float bb[4] = {b4.x, b4.y, b4.z, b4.w};
@@ -292,8 +295,8 @@ gain_mc_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const
         const size_t i0 = (size_t)r * C + c;
         const float4 xv = load4<DT>(x, i0);
         const float4 dv = load4<DU_DT>(du, i0);
-        const float rs = __ldg(rstd + r);
-        const float mu = kind == BSP_LAYERNORM ? __ldg(mean + r) : 0.f;
+        const float rs = ldg(rstd + r);
+        const float mu = kind == BSP_LAYERNORM ? ldg(mean + r) : 0.f;
         const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
         const float ds[4] = {dv.x, dv.y, dv.z, dv.w};
 #pragma unroll
@@ -304,7 +307,7 @@ gain_mc_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const
           const float w = __fdiv_rn(ds[e], gg[e]);
           if (blockIdx.z == 0 && (!isfinite(xs[e]) || !isfinite(ds[e]))) dc.nonfinite++;
           if (grid_steps) {
-            const float st = __ldg(grid_steps + r);
+            const float st = ldg(grid_steps + r);
             const float t = __fdiv_rn(u, st);
             const float n0 = floorf(t);
             thr[i][e] = __float2uint_rd(__fsub_rn(t, n0) * 4294967296.0f);
@@ -361,7 +364,8 @@ gain_mc_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const
 
 // gk[k*C + c] = sum over slabs of partial[k][slab][c] in a fixed order.
 __global__ void __launch_bounds__(256)
-gain_mc_slab_reduce_kernel(const float* __restrict__ partial, int nslabs, int64_t C, float* __restrict__ gk) {
+gain_mc_slab_reduce_kernel(const float* partial, int nslabs, int64_t C, float* gk) {
+  grid_dependency();
   __shared__ float sm[8][33];
   const int cl = threadIdx.x & 31, pl = threadIdx.x >> 5;
   const int64_t c = (int64_t)blockIdx.x * 32 + cl;
@@ -382,8 +386,9 @@ gain_mc_slab_reduce_kernel(const float* __restrict__ partial, int nslabs, int64_
 // S1[c] += sum_k (gk - ref), S2[c] += sum_k (gk - ref)^2: 32 columns by eight draws per block, the
 // eight partial sums added in order.
 __global__ void __launch_bounds__(256)
-gain_mc_accumulate_kernel(const float* __restrict__ gk, int ndraws, int64_t C, const float* __restrict__ ref,
-                          float* __restrict__ S1, float* __restrict__ S2) {
+gain_mc_accumulate_kernel(const float* gk, int ndraws, int64_t C, const float* ref,
+                          float* S1, float* S2) {
+  grid_dependency();
   __shared__ float sm[2][8][33];
   const int cl = threadIdx.x & 31, pl = threadIdx.x >> 5;
   const int64_t c = (int64_t)blockIdx.x * 32 + cl;
@@ -424,7 +429,7 @@ static int launch_norm_bwd(int jmax, int grid, cudaStream_t st, int kind, const 
   (void)jmax;
   const int64_t groups = C / 4;
 #define BSP_NB(J, NT)                                                                                        \
-  norm_bwd_kernel<DT, DU_DT, FMT, J, NT><<<grid, NT, 0, st>>>(kind, x, T, C, gamma, beta, rstd, mean, du,    \
+  launch_kernel(norm_bwd_kernel<DT, DU_DT, FMT, J, NT>, grid, NT, 0, st, kind, x, T, C, gamma, beta, rstd, mean, du,    \
                                                                gain_read, dx_read, u_codes, q.scale,           \
                                                                q.scale_dev, key, key_dx, part_g, part_b, dx)
   if (groups <= 256) BSP_NB(1, 256);
@@ -512,7 +517,7 @@ int bsp_norm_bwd(int kind, const void* x, int dt, int64_t T, int64_t C, const fl
 #undef BSP_CALL
   if (rc != BSP_OK) return rc;
   const unsigned rb = (unsigned)((C + 31) / 32);
-  column_reduce_kernel<<<dim3(rb, dbeta ? 2 : 1), 256, 0, st>>>(part_g, dgamma, part_b, dbeta, grid, C);
+  launch_kernel(column_reduce_kernel, dim3(rb, dbeta ? 2 : 1), 256, 0, st, part_g, dgamma, part_b, dbeta, grid, C);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -570,7 +575,7 @@ int norm_gain_mc_run(int kind, const void* x, int dt, int64_t T, int64_t C, cons
   do {                                                                                                          \
     BSP_CHECK_CUDA(cudaFuncSetAttribute(gain_mc_kernel<DT, DU, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                         (int)(kMcBlockDraws * kMcCols * sizeof(float))));                       \
-    gain_mc_kernel<DT, DU, FMT><<<grid, kMcWarps * 32, smem, st>>>(kind, x, T, C, gamma, beta, rstd, mean, du,  \
+    launch_kernel(gain_mc_kernel<DT, DU, FMT>, grid, kMcWarps * 32, smem, st, kind, x, T, C, gamma, beta, rstd, mean, du,  \
                                                                  q.scale, q.scale_dev, grid_steps, pk,           \
                                                                  draw0 + kb, nd, per_z, plan.subs, partial,      \
                                                                  kb == 0 ? diag : nullptr);                      \
@@ -591,10 +596,10 @@ int norm_gain_mc_run(int kind, const void* x, int dt, int64_t T, int64_t C, cons
     }
     if (nslabs != 1) {                                   // (a single slab's sums are the draw's)
       dim3 rgrid((unsigned)((C + 31) / 32), (unsigned)nd);
-      gain_mc_slab_reduce_kernel<<<rgrid, 256, 0, st>>>(partial, nslabs, C, gk);
+      launch_kernel(gain_mc_slab_reduce_kernel, rgrid, 256, 0, st, partial, nslabs, C, gk);
       BSP_LAUNCH_CHECK();
     }
-    gain_mc_accumulate_kernel<<<(unsigned)((C + 31) / 32), 256, 0, st>>>(nslabs == 1 ? partial : gk, nd, C, g_ref, S1, S2);
+    launch_kernel(gain_mc_accumulate_kernel, (unsigned)((C + 31) / 32), 256, 0, st, nslabs == 1 ? partial : gk, nd, C, g_ref, S1, S2);
     BSP_LAUNCH_CHECK();
   }
   return BSP_OK;

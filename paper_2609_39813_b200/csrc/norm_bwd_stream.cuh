@@ -62,13 +62,14 @@ __device__ __forceinline__ float warp_sum_packed(const float (&v)[NV], int lane)
 // Requires C == 8 * blockDim.x, T and rows_per_block multiples of kRS (see plan_stream).
 template <int DT, int DU_DT, int FMT, int KIND>
 __global__ void __launch_bounds__(512, 1)
-norm_bwd_stream_kernel(const void* __restrict__ x, int64_t T, int64_t C, int64_t rows_per_block, int nstages_ring,
-                       const float* __restrict__ gamma, const float* __restrict__ beta,
-                       const float* __restrict__ rstd, const float* __restrict__ mean,
-                       const void* __restrict__ du, int gain_read, const uint8_t* __restrict__ u_codes,
-                       float scale_val, const float* __restrict__ scale_dev, PhiloxKey key,
-                       float* __restrict__ part_g, float* __restrict__ part_b, float* __restrict__ dx,
+norm_bwd_stream_kernel(const void* x, int64_t T, int64_t C, int64_t rows_per_block, int nstages_ring,
+                       const float* gamma, const float* beta,
+                       const float* rstd, const float* mean,
+                       const void* du, int gain_read, const uint8_t* u_codes,
+                       float scale_val, const float* scale_dev, PhiloxKey key,
+                       float* part_g, float* part_b, float* dx,
                        bsp_diag_t* diag) {
+  grid_dependency();
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int ESX = DT == BSP_F32 ? 4 : 2, ESD = DU_DT == BSP_F32 ? 4 : 2;
   constexpr bool LN = KIND == BSP_LAYERNORM;
@@ -85,7 +86,7 @@ norm_bwd_stream_kernel(const void* __restrict__ x, int64_t T, int64_t C, int64_t
   float* red = reinterpret_cast<float*>(tail + 8 * 8);                        // [2][4][16]
   volatile int* abort_flag = reinterpret_cast<volatile int*>(red + 2 * 4 * 16);
 
-  const float scale = scale_dev ? __ldg(scale_dev) : scale_val;
+  const float scale = scale_dev ? ldg(scale_dev) : scale_val;
   const float inv_scale = __fdiv_rn(1.0f, scale);
   const float invC = 1.0f / (float)C;
   int col[kNJ];
@@ -120,12 +121,12 @@ norm_bwd_stream_kernel(const void* __restrict__ x, int64_t T, int64_t C, int64_t
   float g[kNJ][4], b[kNJ][4], rg[kNJ][4], accg[kNJ][4], accb[kNJ][4];
 #pragma unroll
   for (int j = 0; j < kNJ; ++j) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(gamma + col[j]));
+    const float4 a = ldg(reinterpret_cast<const float4*>(gamma + col[j]));
     g[j][0] = a.x; g[j][1] = a.y; g[j][2] = a.z; g[j][3] = a.w;
 #pragma unroll
     for (int e = 0; e < 4; ++e) { b[j][e] = 0.f; accg[j][e] = 0.f; accb[j][e] = 0.f; }
     if (LN) {
-      const float4 bb = __ldg(reinterpret_cast<const float4*>(beta + col[j]));
+      const float4 bb = ldg(reinterpret_cast<const float4*>(beta + col[j]));
       b[j][0] = bb.x; b[j][1] = bb.y; b[j][2] = bb.z; b[j][3] = bb.w;
     }
 #pragma unroll
@@ -137,8 +138,8 @@ norm_bwd_stream_kernel(const void* __restrict__ x, int64_t T, int64_t C, int64_t
 #pragma unroll
     for (int rr = 0; rr < kRS; ++rr) {
       const int64_t r = r0 + (int64_t)i * kRS + rr;
-      rs_n[rr] = __ldg(rstd + r);
-      mu_n[rr] = LN ? __ldg(mean + r) : 0.f;
+      rs_n[rr] = ldg(rstd + r);
+      mu_n[rr] = LN ? ldg(mean + r) : 0.f;
     }
   };
   if (nst > 0) fetch_stats(0);
@@ -305,7 +306,7 @@ static int launch_norm_bwd_stream(const StreamPlan& p, cudaStream_t st, int kind
   do {                                                                                                      \
     auto kfn = norm_bwd_stream_kernel<DT, DU_DT, FMT, KIND>;                                                \
     BSP_CHECK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));    \
-    kfn<<<p.grid, p.threads, p.smem, st>>>(x, T, C, p.rows_per_block, p.ring, gamma, beta, rstd, mean, du,  \
+    launch_kernel(kfn, p.grid, p.threads, p.smem, st, x, T, C, p.rows_per_block, p.ring, gamma, beta, rstd, mean, du,  \
                                             gain_read, u_codes, q.scale, q.scale_dev, key, part_g, part_b,  \
                                             dx, diag);                                                      \
   } while (0)

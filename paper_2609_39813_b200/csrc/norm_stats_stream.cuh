@@ -20,10 +20,11 @@ constexpr int kStatNJ = 4;    // column groups per thread
 
 template <int DT, int KIND, int RS, int NJ>
 __global__ void __launch_bounds__(512, 1)
-norm_stats_stream_kernel(const void* __restrict__ x, int64_t T, int64_t C, int64_t rows_per_block, int nstages_ring,
-                         const float* __restrict__ gamma, const float* __restrict__ beta, float eps,
-                         float* __restrict__ rstd, float* __restrict__ mean, uint32_t* __restrict__ amax_bits,
+norm_stats_stream_kernel(const void* x, int64_t T, int64_t C, int64_t rows_per_block, int nstages_ring,
+                         const float* gamma, const float* beta, float eps,
+                         float* rstd, float* mean, uint32_t* amax_bits,
                          bsp_diag_t* diag) {
+  grid_dependency();
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int ESX = DT == BSP_F32 ? 4 : 2;
   constexpr bool LN = KIND == BSP_LAYERNORM;
@@ -68,10 +69,10 @@ norm_stats_stream_kernel(const void* __restrict__ x, int64_t T, int64_t C, int64
 #pragma unroll
     for (int e = 0; e < 4; ++e) { g[j][e] = 1.f; b[j][e] = 0.f; }
     if (amax_bits) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(gamma + col[j]));
+      const float4 a = ldg(reinterpret_cast<const float4*>(gamma + col[j]));
       g[j][0] = a.x; g[j][1] = a.y; g[j][2] = a.z; g[j][3] = a.w;
       if (LN) {
-        const float4 bb = __ldg(reinterpret_cast<const float4*>(beta + col[j]));
+        const float4 bb = ldg(reinterpret_cast<const float4*>(beta + col[j]));
         b[j][0] = bb.x; b[j][1] = bb.y; b[j][2] = bb.z; b[j][3] = bb.w;
       }
     }

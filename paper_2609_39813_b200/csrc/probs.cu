@@ -46,9 +46,10 @@ struct ProbsSmem {
 // generator blocks: each computes the block of one stream and they exchange words by shuffles.
 template <bool SHARE>
 __global__ void __launch_bounds__(kPrMaxN, 1)
-probs_mc_kernel(const float* __restrict__ p_all, const float* __restrict__ V, int n, int d, int law, float param,
-                PhiloxKey kq, PhiloxKey ka, PhiloxKey kb, int draw0, int K, float* __restrict__ ds_sum,
-                float* __restrict__ ds_sq, float* __restrict__ dV_sum, size_t rows) {
+probs_mc_kernel(const float* p_all, const float* V, int n, int d, int law, float param,
+                PhiloxKey kq, PhiloxKey ka, PhiloxKey kb, int draw0, int K, float* ds_sum,
+                float* ds_sq, float* dV_sum, size_t rows) {
+  grid_dependency();
   extern __shared__ __align__(16) float sm[];
   const ProbsSmem lay(n, d, blockDim.x);
   float* Vs = sm;                                  // [npad][d]
@@ -216,9 +217,10 @@ constexpr size_t kPfSmemFloats = (size_t)2 * kPfN * kPfD + kPfDraws * kPfN /*pq*
                                  2 * kPfDraws * kPfN /*eu, ea*/ + (size_t)kPfDraws * kPrOps * kPfN /*err*/;
 
 __global__ void __launch_bounds__(kPfThreads, 2)
-probs_mc_128x64_kernel(const float* __restrict__ p_all, const float* __restrict__ V, int law, float param,
-                       PhiloxKey kq, int draw0, int K, float* __restrict__ ds_sum, float* __restrict__ ds_sq,
-                       float* __restrict__ dV_sum, size_t rows) {
+probs_mc_128x64_kernel(const float* p_all, const float* V, int law, float param,
+                       PhiloxKey kq, int draw0, int K, float* ds_sum, float* ds_sq,
+                       float* dV_sum, size_t rows) {
+  grid_dependency();
   extern __shared__ __align__(16) float sm[];
   float* Vs = sm;                                   // [128][64]
   float* Vt = Vs + kPfN * kPfD;                     // [64][128]: Vt[c][j] = V[j][c]
@@ -425,16 +427,16 @@ int bsp_probs_mc(const float* p, const float* V, int64_t rows, int n, int d, int
     const int64_t ngroups = (rows + kPtSlots / g - 1) / (kPtSlots / g);
     auto kern = law == 1 ? probs_mc_tc_kernel<1> : probs_mc_tc_kernel<0>;
     BSP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPtSmemBytes));
-    kern<<<(unsigned)(ngroups < nsm ? ngroups : nsm), kPtThreads, kPtSmemBytes, (cudaStream_t)stream>>>(
-        p, V, n, d, param, kq, draw0, K, g, ds_sum, ds_sq, dV_sum, (size_t)rows);
+    launch_kernel(kern, (unsigned)(ngroups < nsm ? ngroups : nsm), kPtThreads, kPtSmemBytes, (cudaStream_t)stream,
+                  p, V, n, d, param, kq, draw0, K, g, ds_sum, ds_sq, dV_sum, (size_t)rows);
     BSP_LAUNCH_CHECK();
     return BSP_OK;
   }
   if (n == kPfN && d == kPfD && (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (reinterpret_cast<uintptr_t>(dV_sum) & 15u) == 0) {
     const size_t smem_f = kPfSmemFloats * sizeof(float);
     BSP_CHECK_CUDA(cudaFuncSetAttribute(probs_mc_128x64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f));
-    probs_mc_128x64_kernel<<<(unsigned)rows, kPfThreads, smem_f, (cudaStream_t)stream>>>(p, V, law, param, kq, draw0, K, ds_sum,
-                                                                                      ds_sq, dV_sum, (size_t)rows);
+    launch_kernel(probs_mc_128x64_kernel, (unsigned)rows, kPfThreads, smem_f, (cudaStream_t)stream, p, V, law, param, kq, draw0, K, ds_sum,
+                  ds_sq, dV_sum, (size_t)rows);
     BSP_LAUNCH_CHECK();
     return BSP_OK;
   }
@@ -445,8 +447,8 @@ int bsp_probs_mc(const float* p, const float* V, int64_t rows, int n, int d, int
   auto kern = share ? probs_mc_kernel<true> : probs_mc_kernel<false>;
   if (smem > 48 * 1024)
     BSP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<(unsigned)rows, threads, smem, (cudaStream_t)stream>>>(p, V, n, d, law, param, kq, ka, kb, draw0, K, ds_sum, ds_sq,
-                                                               dV_sum, (size_t)rows);
+  launch_kernel(kern, (unsigned)rows, threads, smem, (cudaStream_t)stream, p, V, n, d, law, param, kq, ka, kb, draw0, K, ds_sum, ds_sq,
+                dV_sum, (size_t)rows);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }

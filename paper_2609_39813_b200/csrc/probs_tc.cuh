@@ -120,9 +120,10 @@ __device__ __forceinline__ void pt_arrive(uint32_t bar, int lane) {
 
 template <int law>
 __global__ void __launch_bounds__(kPtThreads, 1)
-probs_mc_tc_kernel(const float* __restrict__ p_all, const float* __restrict__ V, int n, int d, float param,
-                   PhiloxKey kq, int draw0, int K_all, int g /* slots per row: 64 or 128 */, float* __restrict__ ds_sum,
-                   float* __restrict__ ds_sq, float* __restrict__ dV_sum, size_t rows) {
+probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param,
+                   PhiloxKey kq, int draw0, int K_all, int g /* slots per row: 64 or 128 */, float* ds_sum,
+                   float* ds_sq, float* dV_sum, size_t rows) {
+  grid_dependency();
   extern __shared__ uint8_t pt_raw[];
   const uint32_t raw = smem_u32(pt_raw), base = (raw + 1023u) & ~1023u;
   uint8_t* sm = pt_raw + (base - raw);
@@ -156,14 +157,14 @@ probs_mc_tc_kernel(const float* __restrict__ p_all, const float* __restrict__ V,
   uint32_t* vmax_s = reinterpret_cast<uint32_t*>(hp_s);
   if (tid < kPtD) vmax_s[tid] = 0u;
   __syncthreads();
-  for (int i = tid; i < n * d; i += kPtThreads) atomicMax(&vmax_s[i % d], __float_as_uint(fabsf(__ldg(V + i))));
+  for (int i = tid; i < n * d; i += kPtThreads) atomicMax(&vmax_s[i % d], __float_as_uint(fabsf(ldg(V + i))));
   __syncthreads();
   for (int i = tid; i < kPtN * kPtD; i += kPtThreads) {
     const int j = i >> 6, c = i & 63;
     const float m = __uint_as_float(vmax_s[c]);
     int ex = 0;
     if (m > 0.f && m <= 3.4028234663852886e38f) frexpf(m, &ex);       // m < 2^ex
-    float v = j < n && c < d ? __ldg(V + (size_t)j * d + c) : 0.f;
+    float v = j < n && c < d ? ldg(V + (size_t)j * d + c) : 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const int sh = 8 + 9 * k - ex;                                  // unit 2^-sh
@@ -252,7 +253,7 @@ probs_mc_tc_kernel(const float* __restrict__ p_all, const float* __restrict__ V,
       for (int i = tid; i < R * kPtN; i += kPtWorkers) {
         const size_t row = row0 + (i >> 7);
         const int j = i & (kPtN - 1);
-        const float p = row < rows && j < n ? __ldg(p_all + row * n + j) : 0.f;
+        const float p = row < rows && j < n ? ldg(p_all + row * n + j) : 0.f;
         float lo = 0.f, hi;
         uint32_t thr = law == 1 ? 0xFFFFFFFFu : 0u;                   // never up
         if (j < n && row < rows) probs_cell(p, law, param, lo, hi, thr);

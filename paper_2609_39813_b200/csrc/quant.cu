@@ -13,7 +13,8 @@ namespace bsp {
 // Four generator blocks per thread, a warp's 16-byte stores contiguous: the four chains of dependent
 // multiplies overlap, which is what the draw kernels also rely on.
 __global__ void __launch_bounds__(256)
-philox_fill_kernel(PhiloxKey key, size_t n, uint32_t* __restrict__ out) {
+philox_fill_kernel(PhiloxKey key, size_t n, uint32_t* out) {
+  grid_dependency();
   const size_t nq = (n + 3) / 4;
   const size_t q0 = (size_t)blockIdx.x * (blockDim.x * 4) + threadIdx.x;
   uint4 w[4];
@@ -51,13 +52,14 @@ __device__ __forceinline__ void block_amax(float m, uint32_t* amax_bits) {
 // A load that stays where it is written.
 __device__ __forceinline__ uint4 ldg_now(const uint4* p) {
   uint4 r;
-  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
   return r;
 }
 
 template <int DT>
-__global__ void __launch_bounds__(256) amax_kernel(const void* __restrict__ x, size_t group_size, uint32_t* __restrict__ amax_bits,
+__global__ void __launch_bounds__(256) amax_kernel(const void* x, size_t group_size, uint32_t* amax_bits,
                             bsp_diag_t* diag) {
+  grid_dependency();
   // grid: (blocks_per_group, n_groups); amax_bits pre-cleared to 0.
   const size_t g = blockIdx.y;
   const size_t base = g * group_size;
@@ -111,7 +113,8 @@ __global__ void __launch_bounds__(256) amax_kernel(const void* __restrict__ x, s
   diag_flush_warp(diag, dc);
 }
 
-__global__ void scale_from_amax_kernel(const float* __restrict__ amax, size_t n, int fmt, float* __restrict__ scale) {
+__global__ void scale_from_amax_kernel(const float* amax, size_t n, int fmt, float* scale) {
+  grid_dependency();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float a = amax[i];
@@ -161,15 +164,16 @@ __device__ __forceinline__ uint4 encode16(const float (&v)[16], const PhiloxKey&
 // One thread per 16 elements; group_size % 16 == 0 and elem_offset % 4 == 0 on this path.
 template <int DT, int FMT, int MODE>
 __global__ void __launch_bounds__(256)
-round_vec_kernel(const void* __restrict__ x, size_t n16, size_t group_size, float scale_val,
-                 const float* __restrict__ scales, PhiloxKey key, uint64_t elem_offset,
-                 uint8_t* __restrict__ codes, bsp_diag_t* diag) {
+round_vec_kernel(const void* x, size_t n16, size_t group_size, float scale_val,
+                 const float* scales, PhiloxKey key, uint64_t elem_offset,
+                 uint8_t* codes, bsp_diag_t* diag) {
+  grid_dependency();
   // grid-stride over 16-element chunks, two chunks' loads in flight per thread
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   DiagCounters dc;
   auto finish = [&](size_t t, float (&v)[16]) {
     const size_t i0 = t * 16;
-    const float s = scales ? __ldg(scales + (group_size ? i0 / group_size : 0)) : scale_val;
+    const float s = scales ? ldg(scales + (group_size ? i0 / group_size : 0)) : scale_val;
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = __fmul_rn(v[j], s);
     reinterpret_cast<uint4*>(codes)[t] = encode16<FMT, MODE>(v, key, key.c2, elem_offset + i0, dc);
@@ -192,13 +196,14 @@ round_vec_kernel(const void* __restrict__ x, size_t n16, size_t group_size, floa
 
 // General path: one thread per element (tails, odd group sizes, unaligned offsets).
 template <int DT, int FMT, int MODE>
-__global__ void round_scalar_kernel(const void* __restrict__ x, size_t i_begin, size_t n, size_t group_size,
-                                    float scale_val, const float* __restrict__ scales, PhiloxKey key,
-                                    uint64_t elem_offset, uint8_t* __restrict__ codes, bsp_diag_t* diag) {
+__global__ void round_scalar_kernel(const void* x, size_t i_begin, size_t n, size_t group_size,
+                                    float scale_val, const float* scales, PhiloxKey key,
+                                    uint64_t elem_offset, uint8_t* codes, bsp_diag_t* diag) {
+  grid_dependency();
   const size_t i = i_begin + (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   DiagCounters dc;
   if (i < n) {
-    const float s = scales ? __ldg(scales + (group_size ? i / group_size : 0)) : scale_val;
+    const float s = scales ? ldg(scales + (group_size ? i / group_size : 0)) : scale_val;
     const float v = __fmul_rn(load1<DT>(x, i), s);
     uint32_t U = 0;
     if (MODE == BSP_ROUND_STOCHASTIC) {
@@ -222,19 +227,19 @@ struct PlainProducer {
 struct NormProducer {
   static constexpr bool kCopies = true;
   int kind;
-  const float* __restrict__ gamma;
-  const float* __restrict__ beta;
-  const float* __restrict__ rstd;
-  const float* __restrict__ mean;
+  const float* gamma;
+  const float* beta;
+  const float* rstd;
+  const float* mean;
   float r_, m_;
   __device__ __forceinline__ void row(int64_t r) {
-    r_ = __ldg(rstd + r);
-    m_ = kind == BSP_LAYERNORM ? __ldg(mean + r) : 0.f;
+    r_ = ldg(rstd + r);
+    m_ = kind == BSP_LAYERNORM ? ldg(mean + r) : 0.f;
   }
   // RMS: fl(fl(x*rstd)*gamma).  LN: fl(fl(fl(fl(x-mean)*rstd)*gamma)+beta).
   __device__ __forceinline__ float value(float xin, int64_t c) const {
-    if (kind == BSP_RMSNORM) return __fmul_rn(__fmul_rn(xin, r_), __ldg(gamma + c));
-    return __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(xin, m_), r_), __ldg(gamma + c)), __ldg(beta + c));
+    if (kind == BSP_RMSNORM) return __fmul_rn(__fmul_rn(xin, r_), ldg(gamma + c));
+    return __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(xin, m_), r_), ldg(gamma + c)), ldg(beta + c));
   }
 };
 
@@ -243,16 +248,17 @@ constexpr int kTile = 64;   // 64 x 64 tile, 256 threads, 16 consecutive columns
 // Requires cols % 16 == 0.  Outputs may each be NULL.
 template <class Producer, int DT, int FMT, int MODE>
 __global__ void __launch_bounds__(256)
-quant_tile_kernel(Producer prod, const void* __restrict__ x, int64_t rows, int64_t cols, float scale_val,
-                  const float* __restrict__ scale_dev, PhiloxKey key, uint8_t* __restrict__ codes,
-                  uint8_t* __restrict__ codes_t, int64_t ld_t, float* __restrict__ u_f32,
-                  uint16_t* __restrict__ u_bf16_t, bsp_diag_t* diag) {
+quant_tile_kernel(Producer prod, const void* x, int64_t rows, int64_t cols, float scale_val,
+                  const float* scale_dev, PhiloxKey key, uint8_t* codes,
+                  uint8_t* codes_t, int64_t ld_t, float* u_f32,
+                  uint16_t* u_bf16_t, bsp_diag_t* diag) {
+  grid_dependency();
   __shared__ __align__(16) uint8_t s_codes[kTile][kTile + 4];
   __shared__ __align__(16) uint16_t s_bf16[Producer::kCopies ? kTile : 1][kTile + 2];
   const int64_t r0 = (int64_t)blockIdx.y * kTile, c0 = (int64_t)blockIdx.x * kTile;
   const int tr = threadIdx.x >> 2, tc = (threadIdx.x & 3) * 16;
   const int64_t r = r0 + tr, c = c0 + tc;
-  const float s = scale_dev ? __ldg(scale_dev) : scale_val;
+  const float s = scale_dev ? ldg(scale_dev) : scale_val;
   DiagCounters dc;
   const bool active = (r < rows) && (c < cols);
   if (active) {
@@ -342,14 +348,15 @@ quant_tile_kernel(Producer prod, const void* __restrict__ x, int64_t rows, int64
 // draws of a small tensor (64 x 128, 256 draws: two blocks, 162 us; now 7 us).
 template <int DT, int FMT>
 __global__ void __launch_bounds__(256, 2)
-reround_draws_kernel(NormProducer prod, const void* __restrict__ x, int64_t rows, int64_t cols, float scale_val,
-                     const float* __restrict__ scale_dev, PhiloxKey key, int draw0, int ndraws, int draws_per_z,
-                     uint8_t* __restrict__ codes_t, int64_t ld_t) {
+reround_draws_kernel(NormProducer prod, const void* x, int64_t rows, int64_t cols, float scale_val,
+                     const float* scale_dev, PhiloxKey key, int draw0, int ndraws, int draws_per_z,
+                     uint8_t* codes_t, int64_t ld_t) {
+  grid_dependency();
   const int64_t r = (int64_t)blockIdx.y * kTile + 4 * (threadIdx.x & 15);
   const int64_t c = (int64_t)blockIdx.x * kTile + 4 * (threadIdx.x >> 4);
   // rows up to the next multiple of 16 past `rows` are written as zeros (ld_t covers them)
   if (c >= cols || r >= ((rows + 15) & ~(int64_t)15)) return;
-  const float s = scale_dev ? __ldg(scale_dev) : scale_val;
+  const float s = scale_dev ? ldg(scale_dev) : scale_val;
   // A fresh rounding of an element is its round-down code plus one exactly when the element's
   // generator word falls below the threshold of f8_sr_threshold: both are fixed across draws, so a
   // draw costs one generator block, four comparisons and four conditional adds per four elements.
@@ -411,9 +418,10 @@ reround_draws_kernel(NormProducer prod, const void* __restrict__ x, int64_t rows
 // element, and the norm kind is a template parameter.
 template <int DT, int kind>
 __global__ void __launch_bounds__(256)
-norm_stats_kernel(const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
-                  const float* __restrict__ beta, float eps, float* __restrict__ rstd, float* __restrict__ mean,
-                  uint32_t* __restrict__ amax_bits, bsp_diag_t* diag) {
+norm_stats_kernel(const void* x, int64_t T, int64_t C, const float* gamma,
+                  const float* beta, float eps, float* rstd, float* mean,
+                  uint32_t* amax_bits, bsp_diag_t* diag) {
+  grid_dependency();
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   float amax = 0.f;
@@ -457,13 +465,13 @@ norm_stats_kernel(const void* __restrict__ x, int64_t T, int64_t C, const float*
     if (amax_bits) {
       for (int64_t v = lane; v < nvec; v += 32) {
         const float4 f = load4<DT>(x, base + v * 4);
-        const float4 g = __ldg(reinterpret_cast<const float4*>(gamma) + v);
+        const float4 g = ldg(reinterpret_cast<const float4*>(gamma) + v);
         float u0, u1, u2, u3;
         if (kind == BSP_RMSNORM) {
           u0 = __fmul_rn(__fmul_rn(f.x, rs), g.x); u1 = __fmul_rn(__fmul_rn(f.y, rs), g.y);
           u2 = __fmul_rn(__fmul_rn(f.z, rs), g.z); u3 = __fmul_rn(__fmul_rn(f.w, rs), g.w);
         } else {
-          const float4 b = __ldg(reinterpret_cast<const float4*>(beta) + v);
+          const float4 b = ldg(reinterpret_cast<const float4*>(beta) + v);
           u0 = __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(f.x, mu), rs), g.x), b.x);
           u1 = __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(f.y, mu), rs), g.y), b.y);
           u2 = __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(f.z, mu), rs), g.z), b.z);
@@ -486,11 +494,11 @@ static void launch_tile_mode(int mode, dim3 grid, cudaStream_t st, Producer prod
                              int64_t cols, float scale, const float* scale_dev, PhiloxKey key, uint8_t* codes,
                              uint8_t* codes_t, int64_t ld_t, float* u_f32, uint16_t* u_bf16_t, bsp_diag_t* diag) {
   if (mode == BSP_ROUND_STOCHASTIC)
-    quant_tile_kernel<Producer, DT, FMT, BSP_ROUND_STOCHASTIC><<<grid, 256, 0, st>>>(
-        prod, x, rows, cols, scale, scale_dev, key, codes, codes_t, ld_t, u_f32, u_bf16_t, diag);
+    launch_kernel(quant_tile_kernel<Producer, DT, FMT, BSP_ROUND_STOCHASTIC>, grid, 256, 0, st,
+                  prod, x, rows, cols, scale, scale_dev, key, codes, codes_t, ld_t, u_f32, u_bf16_t, diag);
   else
-    quant_tile_kernel<Producer, DT, FMT, BSP_ROUND_NEAREST><<<grid, 256, 0, st>>>(
-        prod, x, rows, cols, scale, scale_dev, key, codes, codes_t, ld_t, u_f32, u_bf16_t, diag);
+    launch_kernel(quant_tile_kernel<Producer, DT, FMT, BSP_ROUND_NEAREST>, grid, 256, 0, st,
+                  prod, x, rows, cols, scale, scale_dev, key, codes, codes_t, ld_t, u_f32, u_bf16_t, diag);
 }
 
 template <class Producer>
@@ -520,15 +528,15 @@ static int launch_round_flat(const void* x, size_t n, size_t group_size, float s
     const size_t want = (n16 + 511) / 512;                      // two chunks per thread
     const size_t cap = (size_t)kNumSMs * 8;                     // eight 256-thread blocks per SM
     const unsigned blocks = (unsigned)(want < cap ? want : cap);
-    round_vec_kernel<DT, FMT, MODE><<<blocks, 256, 0, st>>>(x, n16, group_size, scale, scales, key, elem_offset,
-                                                           codes, diag);
+    launch_kernel(round_vec_kernel<DT, FMT, MODE>, blocks, 256, 0, st, x, n16, group_size, scale, scales, key, elem_offset,
+                  codes, diag);
     BSP_LAUNCH_CHECK();
   }
   const size_t done = n16 * 16;
   if (done < n) {
     const unsigned blocks = (unsigned)((n - done + 255) / 256);
-    round_scalar_kernel<DT, FMT, MODE><<<blocks, 256, 0, st>>>(x, done, n, group_size, scale, scales, key,
-                                                              elem_offset, codes, diag);
+    launch_kernel(round_scalar_kernel<DT, FMT, MODE>, blocks, 256, 0, st, x, done, n, group_size, scale, scales, key,
+                  elem_offset, codes, diag);
     BSP_LAUNCH_CHECK();
   }
   return BSP_OK;
@@ -569,7 +577,7 @@ int bsp_philox_fill(bsp_key_t key, size_t n, uint32_t* out, void* stream) {
   if (!aligned16(out)) return BSP_ERR_ALIGN;
   if (n == 0) return BSP_OK;
   const size_t nq = (n + 3) / 4;
-  philox_fill_kernel<<<(unsigned)((nq + 1023) / 1024), 256, 0, (cudaStream_t)stream>>>(make_key(key), n, out);
+  launch_kernel(philox_fill_kernel, (unsigned)((nq + 1023) / 1024), 256, 0, (cudaStream_t)stream, make_key(key), n, out);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -588,8 +596,8 @@ int bsp_amax(const void* x, int dt, size_t n_groups, size_t group_size, float* a
   size_t want = (size_t)kNumSMs * 8 / n_groups + 1;
   unsigned bx = (unsigned)(per < want ? (per ? per : 1) : want);
   dim3 grid(bx, (unsigned)n_groups);
-  if (dt == BSP_F32) amax_kernel<BSP_F32><<<grid, 256, 0, st>>>(x, group_size, reinterpret_cast<uint32_t*>(amax), diag);
-  else amax_kernel<BSP_BF16><<<grid, 256, 0, st>>>(x, group_size, reinterpret_cast<uint32_t*>(amax), diag);
+  if (dt == BSP_F32) launch_kernel(amax_kernel<BSP_F32>, grid, 256, 0, st, x, group_size, reinterpret_cast<uint32_t*>(amax), diag);
+  else launch_kernel(amax_kernel<BSP_BF16>, grid, 256, 0, st, x, group_size, reinterpret_cast<uint32_t*>(amax), diag);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -597,7 +605,7 @@ int bsp_amax(const void* x, int dt, size_t n_groups, size_t group_size, float* a
 int bsp_scale_from_amax(const float* amax, size_t n, int fmt, float* scale, void* stream) {
   if (!amax || !scale || !valid_enum(fmt, 1)) return BSP_ERR_ARG;
   if (n == 0) return BSP_OK;
-  scale_from_amax_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(amax, n, fmt, scale);
+  launch_kernel(scale_from_amax_kernel, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, amax, n, fmt, scale);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -657,7 +665,7 @@ int bsp_norm_stats(int kind, const void* x, int dt, int64_t T, int64_t C, const 
   do {                                                                                                       \
     auto kfn = norm_stats_stream_kernel<DT, KIND, kStatRS, kStatNJ>;                                                          \
     BSP_CHECK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp.smem));    \
-    kfn<<<sp.grid, sp.threads, sp.smem, st>>>(x, T, C, sp.rows_per_block, sp.ring, gamma, beta, eps, rstd,   \
+    launch_kernel(kfn, sp.grid, sp.threads, sp.smem, st, x, T, C, sp.rows_per_block, sp.ring, gamma, beta, eps, rstd,   \
                                                mean, ab, diag);                                              \
   } while (0)
     if (dt == BSP_F32) { if (kind == BSP_RMSNORM) BSP_NSS(BSP_F32, BSP_RMSNORM); else BSP_NSS(BSP_F32, BSP_LAYERNORM); }
@@ -667,7 +675,7 @@ int bsp_norm_stats(int kind, const void* x, int dt, int64_t T, int64_t C, const 
     return BSP_OK;
   }
   const unsigned blocks = (unsigned)((T + 7) / 8);
-#define BSP_NS(DT, KIND) norm_stats_kernel<DT, KIND><<<blocks, 256, 0, st>>>(x, T, C, gamma, beta, eps, rstd, mean, ab, diag)
+#define BSP_NS(DT, KIND) launch_kernel(norm_stats_kernel<DT, KIND>, blocks, 256, 0, st, x, T, C, gamma, beta, eps, rstd, mean, ab, diag)
   if (dt == BSP_F32) { if (kind == BSP_RMSNORM) BSP_NS(BSP_F32, BSP_RMSNORM); else BSP_NS(BSP_F32, BSP_LAYERNORM); }
   else { if (kind == BSP_RMSNORM) BSP_NS(BSP_BF16, BSP_RMSNORM); else BSP_NS(BSP_BF16, BSP_LAYERNORM); }
 #undef BSP_NS
@@ -720,7 +728,7 @@ int bsp_norm_fwd_draws(int kind, const void* x, int dt, int64_t T, int64_t C, co
   cudaStream_t st = (cudaStream_t)stream;
   const PhiloxKey pk = make_key(key);
 #define BSP_RR(DT, FMT)                                                                                          \
-  reround_draws_kernel<DT, FMT><<<grid, 256, 0, st>>>(prod, x, T, C, q.scale, q.scale_dev, pk, draw0, n_draws,   \
+  launch_kernel(reround_draws_kernel<DT, FMT>, grid, 256, 0, st, prod, x, T, C, q.scale, q.scale_dev, pk, draw0, n_draws,   \
                                                       per_z, u_codes_t_draws, ld_t)
   if (dt == BSP_F32 && q.fmt == BSP_E4M3) BSP_RR(BSP_F32, BSP_E4M3);
   else if (dt == BSP_F32) BSP_RR(BSP_F32, BSP_E5M2);

@@ -40,13 +40,14 @@ constexpr int kStoreMaxPer = 32;                               // C <= 8192
 
 template <int DT>
 __global__ void __launch_bounds__(kStoreThreads)
-store_fwd_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
-                 const float* __restrict__ beta, const float* __restrict__ rstd, const float* __restrict__ mean,
-                 float levels, PhiloxKey key, int8_t* __restrict__ codes, float* __restrict__ steps) {
+store_fwd_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
+                 const float* beta, const float* rstd, const float* mean,
+                 float levels, PhiloxKey key, int8_t* codes, float* steps) {
+  grid_dependency();
   __shared__ float red[kStoreThreads / 32];
   __shared__ float s_step;
   const int64_t r = blockIdx.x;
-  const float rs = __ldg(rstd + r), mu = kind == BSP_LAYERNORM ? __ldg(mean + r) : 0.f;
+  const float rs = ldg(rstd + r), mu = kind == BSP_LAYERNORM ? ldg(mean + r) : 0.f;
   // thread t holds the groups of four columns 4 (t + 256 j)
   float u[kStoreMaxPer];
   float amax = 0.f;
@@ -55,9 +56,9 @@ store_fwd_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, con
     const int64_t c = 4 * ((int64_t)threadIdx.x + kStoreThreads * j);
     if (c < C) {
       const float4 xv = load4<DT>(x, (size_t)r * C + c);
-      const float4 g4 = __ldg(reinterpret_cast<const float4*>(gamma + c));
+      const float4 g4 = ldg(reinterpret_cast<const float4*>(gamma + c));
       float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (kind == BSP_LAYERNORM) b4 = __ldg(reinterpret_cast<const float4*>(beta + c));
+      if (kind == BSP_LAYERNORM) b4 = ldg(reinterpret_cast<const float4*>(beta + c));
       u[4 * j] = store_chain(kind, xv.x, rs, mu, g4.x, b4.x);
       u[4 * j + 1] = store_chain(kind, xv.y, rs, mu, g4.y, b4.y);
       u[4 * j + 2] = store_chain(kind, xv.z, rs, mu, g4.z, b4.z);
@@ -109,10 +110,11 @@ store_fwd_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, con
 // blocks, no word wasted) and writes 16 consecutive tokens of one column of each half.
 template <int DT>
 __global__ void __launch_bounds__(256)
-store_operand_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
-                     const float* __restrict__ beta, const float* __restrict__ rstd, const float* __restrict__ mean,
-                     const int8_t* __restrict__ codes, const float* __restrict__ steps, int read, PhiloxKey key,
-                     float* __restrict__ out_f32, uint16_t* __restrict__ out_t, int64_t ld_t) {
+store_operand_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
+                     const float* beta, const float* rstd, const float* mean,
+                     const int8_t* codes, const float* steps, int read, PhiloxKey key,
+                     float* out_f32, uint16_t* out_t, int64_t ld_t) {
+  grid_dependency();
   constexpr int TS = 64, PITCH = TS + 2;
   __shared__ __align__(16) uint16_t s_hi[TS][PITCH], s_lo[TS][PITCH];
   const int64_t r0 = (int64_t)blockIdx.y * TS, c0 = (int64_t)blockIdx.x * TS;
@@ -123,13 +125,13 @@ store_operand_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C,
   for (int j = 0; j < 16; ++j) v[j] = 0.f;
   if (r < T && c < C) {
     const size_t i0 = (size_t)r * C + c;
-    const float rs = __ldg(rstd + r), mu = kind == BSP_LAYERNORM ? __ldg(mean + r) : 0.f;
-    const float s = __ldg(steps + r);
+    const float rs = ldg(rstd + r), mu = kind == BSP_LAYERNORM ? ldg(mean + r) : 0.f;
+    const float s = ldg(steps + r);
     float xv[16];
     load16<DT>(x, i0, xv);
     const bool fresh = read == STORE_READ_N || read == STORE_READ_R_EPS;
     const bool fwd = read == STORE_READ_R || read == STORE_READ_R_EPS;
-    const uint4 cq = fwd ? __ldg(reinterpret_cast<const uint4*>(codes + i0)) : make_uint4(0, 0, 0, 0);
+    const uint4 cq = fwd ? ldg(reinterpret_cast<const uint4*>(codes + i0)) : make_uint4(0, 0, 0, 0);
     const uint32_t cw[4] = {cq.x, cq.y, cq.z, cq.w};
 #pragma unroll
     for (int b4 = 0; b4 < 4; ++b4) {
@@ -139,7 +141,7 @@ store_operand_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C,
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int j = 4 * b4 + e;
-        const float u = store_chain(kind, xv[j], rs, mu, __ldg(gamma + c + j), kind == BSP_LAYERNORM ? __ldg(beta + c + j) : 0.f);
+        const float u = store_chain(kind, xv[j], rs, mu, ldg(gamma + c + j), kind == BSP_LAYERNORM ? ldg(beta + c + j) : 0.f);
         float nf = 0.f;
         if (fresh) {
           float n0;
@@ -193,13 +195,14 @@ store_operand_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C,
 // Sixteen codes per thread (ld_t is a multiple of 16; codes need not be aligned); 16.8 M codes: 65 us a code at a time, 18 us here.
 template <int FMT>
 __global__ void __launch_bounds__(256)
-decode_twice_kernel(const uint8_t* __restrict__ codes, int64_t ld_t, size_t n16, uint16_t* __restrict__ out) {
+decode_twice_kernel(const uint8_t* codes, int64_t ld_t, size_t n16, uint16_t* out) {
+  grid_dependency();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n16) return;
   const size_t per = (size_t)ld_t / 16, o = i / per, t = 16 * (i - o * per);
   uint32_t c[4];
   if ((reinterpret_cast<uintptr_t>(codes) & 15u) == 0) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(codes) + i);
+    const uint4 v = ldg(reinterpret_cast<const uint4*>(codes) + i);
     c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
   } else {
 #pragma unroll
@@ -222,13 +225,14 @@ decode_twice_kernel(const uint8_t* __restrict__ codes, int64_t ld_t, size_t n16,
 // the difference, not of the gradient.
 template <int FMT>
 __global__ void __launch_bounds__(256)
-store_dys_kernel(const uint8_t* __restrict__ codes, const float* __restrict__ steps, int64_t T, int64_t ld_t, size_t n8,
-                 uint16_t* __restrict__ out) {
+store_dys_kernel(const uint8_t* codes, const float* steps, int64_t T, int64_t ld_t, size_t n8,
+                 uint16_t* out) {
+  grid_dependency();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n8) return;
   const size_t e0 = i * 8;
   const int64_t t0 = (int64_t)(e0 % (size_t)ld_t);
-  const uint2 c8 = __ldg(reinterpret_cast<const uint2*>(codes + e0));
+  const uint2 c8 = ldg(reinterpret_cast<const uint2*>(codes + e0));
   float d[8];
   f8_decode4<FMT>(c8.x, *reinterpret_cast<float(*)[4]>(&d[0]));
   f8_decode4<FMT>(c8.y, *reinterpret_cast<float(*)[4]>(&d[4]));
@@ -236,8 +240,8 @@ store_dys_kernel(const uint8_t* __restrict__ codes, const float* __restrict__ st
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int64_t ta = t0 + 2 * j, tb = ta + 1;
-    const uint32_t lo = ta < T ? float_to_bf16_bits(d[2 * j] * __ldg(steps + ta)) : 0u;
-    const uint32_t hi = tb < T ? float_to_bf16_bits(d[2 * j + 1] * __ldg(steps + tb)) : 0u;
+    const uint32_t lo = ta < T ? float_to_bf16_bits(d[2 * j] * ldg(steps + ta)) : 0u;
+    const uint32_t hi = tb < T ? float_to_bf16_bits(d[2 * j + 1] * ldg(steps + tb)) : 0u;
     pk[j] = lo | (hi << 16);
   }
   *reinterpret_cast<uint4*>(out + e0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
@@ -253,10 +257,11 @@ store_dys_kernel(const uint8_t* __restrict__ codes, const float* __restrict__ st
 // the loop, 4096 x 1024, 16 draws: 81 us; here 65.
 template <int DT>
 __global__ void __launch_bounds__(256, 3)
-store_diff_draws_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t C, const float* __restrict__ gamma,
-                        const float* __restrict__ beta, const float* __restrict__ rstd, const float* __restrict__ mean,
-                        const int8_t* __restrict__ codes, const float* __restrict__ steps, int read, PhiloxKey key,
-                        int draw0, int ndraws, int draws_per_z, uint16_t* __restrict__ out_t, int64_t ld_t) {
+store_diff_draws_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
+                        const float* beta, const float* rstd, const float* mean,
+                        const int8_t* codes, const float* steps, int read, PhiloxKey key,
+                        int draw0, int ndraws, int draws_per_z, uint16_t* out_t, int64_t ld_t) {
+  grid_dependency();
   const int64_t r = (int64_t)blockIdx.y * 64 + 4 * (threadIdx.x & 15);
   const int64_t c = (int64_t)blockIdx.x * 64 + 4 * (threadIdx.x >> 4);
   if (c >= C || r >= ld_t) return;                              // (ld_t is a multiple of 16: groups of four never straddle it)
@@ -267,13 +272,13 @@ store_diff_draws_kernel(int kind, const void* __restrict__ x, int64_t T, int64_t
     for (int j = 0; j < 4; ++j) thr[i][j] = val[i][j] = 0u;
     if (r + i < T) {
       const size_t i0 = (size_t)(r + i) * C + c;
-      const float rs = __ldg(rstd + r + i), mu = kind == BSP_LAYERNORM ? __ldg(mean + r + i) : 0.f, s = __ldg(steps + r + i);
+      const float rs = ldg(rstd + r + i), mu = kind == BSP_LAYERNORM ? ldg(mean + r + i) : 0.f, s = ldg(steps + r + i);
       const float4 xv = load4<DT>(x, i0);
       const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
-      const uint32_t cw = read == STORE_READ_N ? __ldg(reinterpret_cast<const uint32_t*>(codes + i0)) : 0u;
+      const uint32_t cw = read == STORE_READ_N ? ldg(reinterpret_cast<const uint32_t*>(codes + i0)) : 0u;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float u = store_chain(kind, xs[j], rs, mu, __ldg(gamma + c + j), kind == BSP_LAYERNORM ? __ldg(beta + c + j) : 0.f);
+        const float u = store_chain(kind, xs[j], rs, mu, ldg(gamma + c + j), kind == BSP_LAYERNORM ? ldg(beta + c + j) : 0.f);
         const float t = __fdiv_rn(u, s);
         const float n0 = floorf(t);
         const float f = __fsub_rn(t, n0);
@@ -390,9 +395,9 @@ int bsp_store_fwd(int kind, const void* x, int dt, int64_t T, int64_t C, const f
   const PhiloxKey pk = make_key(key);
   cudaStream_t st = (cudaStream_t)stream;
   if (dt == BSP_F32)
-    store_fwd_kernel<BSP_F32><<<(unsigned)T, kStoreThreads, 0, st>>>(kind, x, T, C, gamma, beta, rstd, mean, (float)store_levels(bits), pk, codes, steps);
+    launch_kernel(store_fwd_kernel<BSP_F32>, (unsigned)T, kStoreThreads, 0, st, kind, x, T, C, gamma, beta, rstd, mean, (float)store_levels(bits), pk, codes, steps);
   else
-    store_fwd_kernel<BSP_BF16><<<(unsigned)T, kStoreThreads, 0, st>>>(kind, x, T, C, gamma, beta, rstd, mean, (float)store_levels(bits), pk, codes, steps);
+    launch_kernel(store_fwd_kernel<BSP_BF16>, (unsigned)T, kStoreThreads, 0, st, kind, x, T, C, gamma, beta, rstd, mean, (float)store_levels(bits), pk, codes, steps);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -413,11 +418,11 @@ int bsp_store_read(int kind, const void* x, int dt, int64_t T, int64_t C, const 
   const int64_t rows = copy_split_t ? ld_t : T;                 // the padding columns are written too
   dim3 grid((unsigned)((C + 63) / 64), (unsigned)((rows + 63) / 64));
   if (dt == BSP_F32)
-    store_operand_kernel<BSP_F32><<<grid, 256, 0, st>>>(kind, x, T, C, gamma, beta, rstd, mean, codes, steps, read, pk, copy_f32,
-                                                        reinterpret_cast<uint16_t*>(copy_split_t), ld_t);
+    launch_kernel(store_operand_kernel<BSP_F32>, grid, 256, 0, st, kind, x, T, C, gamma, beta, rstd, mean, codes, steps, read, pk, copy_f32,
+                  reinterpret_cast<uint16_t*>(copy_split_t), ld_t);
   else
-    store_operand_kernel<BSP_BF16><<<grid, 256, 0, st>>>(kind, x, T, C, gamma, beta, rstd, mean, codes, steps, read, pk, copy_f32,
-                                                         reinterpret_cast<uint16_t*>(copy_split_t), ld_t);
+    launch_kernel(store_operand_kernel<BSP_BF16>, grid, 256, 0, st, kind, x, T, C, gamma, beta, rstd, mean, codes, steps, read, pk, copy_f32,
+                  reinterpret_cast<uint16_t*>(copy_split_t), ld_t);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -434,8 +439,8 @@ namespace bsp {
 // The A operand of bsp_store_wgrad, and the product itself: a check makes the one once for all reads.
 static int store_decode_twice(int64_t O, const uint8_t* dy_codes_t, int fmt, int64_t ld_t, uint16_t* a2, cudaStream_t st) {
   const size_t n16 = (size_t)O * ld_t / 16;
-  if (fmt == BSP_E5M2) decode_twice_kernel<BSP_E5M2><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes_t, ld_t, n16, a2);
-  else decode_twice_kernel<BSP_E4M3><<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(dy_codes_t, ld_t, n16, a2);
+  if (fmt == BSP_E5M2) launch_kernel(decode_twice_kernel<BSP_E5M2>, (unsigned)((n16 + 255) / 256), 256, 0, st, dy_codes_t, ld_t, n16, a2);
+  else launch_kernel(decode_twice_kernel<BSP_E4M3>, (unsigned)((n16 + 255) / 256), 256, 0, st, dy_codes_t, ld_t, n16, a2);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -568,9 +573,9 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
     if (w_mask & 12u) {
       const size_t n8 = (size_t)O * b.ld_t / 8;
       if (op->grad_fmt == BSP_E5M2)
-        store_dys_kernel<BSP_E5M2><<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>(b.dy_codes_t, b.steps, T, b.ld_t, n8, b.dys_t);
+        launch_kernel(store_dys_kernel<BSP_E5M2>, (unsigned)((n8 + 255) / 256), 256, 0, st, b.dy_codes_t, b.steps, T, b.ld_t, n8, b.dys_t);
       else
-        store_dys_kernel<BSP_E4M3><<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>(b.dy_codes_t, b.steps, T, b.ld_t, n8, b.dys_t);
+        launch_kernel(store_dys_kernel<BSP_E4M3>, (unsigned)((n8 + 255) / 256), 256, 0, st, b.dy_codes_t, b.steps, T, b.ld_t, n8, b.dys_t);
       BSP_LAUNCH_CHECK();
     }
     for (int which = 0; which < 2; ++which) {
@@ -596,11 +601,11 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
         const int per_z = (nd + nz - 1) / nz;
         grid.z = (unsigned)((nd + per_z - 1) / per_z);
         if (dt == BSP_F32)
-          store_diff_draws_kernel<BSP_F32><<<grid, 256, 0, st>>>(kind, op->x, T, C, op->gamma, op->beta, b.rstd, b.mean, b.codes,
-                                                                 b.steps, read, pk, k0, nd, per_z, b.diff_t, b.ld_t);
+          launch_kernel(store_diff_draws_kernel<BSP_F32>, grid, 256, 0, st, kind, op->x, T, C, op->gamma, op->beta, b.rstd, b.mean, b.codes,
+                        b.steps, read, pk, k0, nd, per_z, b.diff_t, b.ld_t);
         else
-          store_diff_draws_kernel<BSP_BF16><<<grid, 256, 0, st>>>(kind, op->x, T, C, op->gamma, op->beta, b.rstd, b.mean, b.codes,
-                                                                  b.steps, read, pk, k0, nd, per_z, b.diff_t, b.ld_t);
+          launch_kernel(store_diff_draws_kernel<BSP_BF16>, grid, 256, 0, st, kind, op->x, T, C, op->gamma, op->beta, b.rstd, b.mean, b.codes,
+                        b.steps, read, pk, k0, nd, per_z, b.diff_t, b.ld_t);
         BSP_LAUNCH_CHECK();
         GemmArgs g;
         g.M = O; g.N = C; g.K = T; g.nb = nd; g.fp8 = false;
