@@ -324,7 +324,7 @@ int bsp_gemm(int64_t M, int64_t N, int64_t K, int elem, const void* A, int64_t l
  * bsp_norm_fwd_draws).  For every draw d: dW_d = dY^T X_d, and
  *   S1 += dW_d - g_ref,  S2 += (dW_d - g_ref)^2      (all [O*C] FP32; S1, S2 are read, updated,
  * written back, so draw ranges can be chained).  The per-draw gradients are never written: the
- * running sums of an output tile stay in tensor memory while the kernel walks the draws.
+ * running sums of an output tile stay in registers while the kernel walks the draws.
  * C must be a multiple of 16. */
 int bsp_linear_wgrad_mc(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t, bsp_quant_t q_dy,
                         const uint8_t* x_t_draws, bsp_quant_t q_x, int64_t ld_t, int n_draws,

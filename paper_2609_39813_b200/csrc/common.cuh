@@ -60,12 +60,13 @@ constexpr int kNumSMs = 148;
 
 // The K-draw gain use behind bsp_norm_gain_mc.
 // `grid_steps` (per-token steps [T]) switches the rounding law from the FP8 store to the b-bit
-// per-token grid (q is then ignored apart from its format, which must still be valid).
+// per-token grid (q is then ignored apart from its format, which must still be valid); first: S1 and S2 start
+// with these draws (they need not be cleared).
 size_t norm_gain_mc_workspace(int64_t T, int64_t C, int K);
 int norm_gain_mc_run(int kind, const void* x, int dt, int64_t T, int64_t C, const float* gamma,
                      const float* beta, const float* rstd, const float* mean, const void* du, int du_dt, bsp_quant_t q,
                      bsp_key_t key, int draw0, int K, const float* g_ref, float* S1, float* S2, void* ws, size_t ws_bytes,
-                     bsp_diag_t* diag, void* stream, const float* grid_steps = nullptr);
+                     bsp_diag_t* diag, void* stream, const float* grid_steps = nullptr, bool first = false);
 
 // Index of the current device into a per-device flag array of kMaxDevices entries (a function
 // attribute such as the dynamic shared-memory limit is set once per device, not once per process).

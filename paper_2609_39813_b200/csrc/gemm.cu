@@ -379,6 +379,7 @@ constexpr size_t kMcSplitTileFloats = (size_t)2 * BM * MC_BN;   // S1 and S2 of 
 // Units of the walk: tiles [0, whole) with all draws, then nseg ranges over the other tiles.
 struct McSplit {
   int whole, rest, nseg, pairs_per_seg;
+  int first;                             // the sums start with this launch's draws
 };
 __device__ __forceinline__ void mc_unit(const McSplit& sp, int u, int npairs, int& tile, int& seg, int& p0, int& p1) {
   if (u < sp.whole) { tile = u; seg = 0; p0 = 0; p1 = npairs; return; }
@@ -527,7 +528,7 @@ gemm_mc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           const size_t off = (size_t)row * p.ldc + colbase + c;
           // no reference: the products are differences to the reference already
           if (p.ref) g0 = *reinterpret_cast<const float4*>(p.ref + off);
-          if (seg == 0) {
+          if (seg == 0 && !sp.first) {
             v1 = *reinterpret_cast<const float4*>(p.S1 + off);
             v2 = *reinterpret_cast<const float4*>(p.S2 + off);
           }
@@ -791,6 +792,7 @@ static McSplit mc_split_plan(int64_t M, int64_t N, int64_t k_bytes, int nb, int 
   sp.rest = ntiles - sp.whole;
   sp.nseg = 1;
   sp.pairs_per_seg = npairs;
+  sp.first = 0;
   if (sp.rest == 0) return sp;
   const double pair_us = 1.0 + 0.27 * (double)((k_bytes + BKB - 1) / BKB);
   double best = npairs * pair_us;
@@ -881,6 +883,10 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
 
   if (simt_forced()) {
     dim3 grid((unsigned)((g.N + 15) / 16), (unsigned)((g.M + 15) / 16), (unsigned)g.nb);
+    if (g.mode == EPI_MC && g.mc_first) {
+      BSP_CHECK_CUDA(cudaMemsetAsync(g.S1, 0, (size_t)g.M * g.ldc * sizeof(float), st));
+      BSP_CHECK_CUDA(cudaMemsetAsync(g.S2, 0, (size_t)g.M * g.ldc * sizeof(float), st));
+    }
     // the MC epilogue is a read-modify-write: batches must run one after another
     if (g.mode == EPI_MC && g.nb > 1) {
       for (int b = 0; b < g.nb; ++b) {
@@ -913,6 +919,7 @@ int gemm_run(const GemmArgs& g, cudaStream_t st) {
     p.idesc = make_idesc(fa, fb, ctas * BM, MC_BN);
     p.idesc2 = make_idesc(fa, fb, ctas * BM, 2 * MC_BN);
     McSplit sp = mc_split_plan(g.M, g.N, g.K * eb, g.nb, nsm);
+    sp.first = g.mc_first ? 1 : 0;
     if (!g.split_ws || g.split_ws_bytes < mc_split_bytes(sp, g.M, g.K * eb)) {      // no room: every tile takes all its draws
       sp.whole += sp.rest;
       sp.rest = 0;
@@ -1069,8 +1076,8 @@ int bsp_gemm(int64_t M, int64_t N, int64_t K, int elem, const void* A, int64_t l
 int bsp_linear_wgrad_mc(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t, bsp_quant_t q_dy,
                         const uint8_t* x_t_draws, bsp_quant_t q_x, int64_t ld_t, int n_draws, const float* g_ref,
                         float* S1, float* S2, bsp_diag_t* diag, void* stream) {
-  return bsp::linear_wgrad_mc_run(T, O, C, dy_codes_t, q_dy, x_t_draws, q_x, ld_t, n_draws, g_ref, S1, S2, nullptr, 0,
-                                  diag, stream);
+  return bsp::linear_wgrad_mc_run(T, O, C, dy_codes_t, q_dy, x_t_draws, q_x, ld_t, n_draws, g_ref, S1, S2, false, nullptr,
+                                  0, diag, stream);
 }
 
 }  // extern "C"
@@ -1078,7 +1085,7 @@ int bsp_linear_wgrad_mc(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes
 // The same with room for split ranges of draws (gemm_mc_split_bytes).
 int bsp::linear_wgrad_mc_run(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t, bsp_quant_t q_dy,
                              const uint8_t* x_t_draws, bsp_quant_t q_x, int64_t ld_t, int n_draws, const float* g_ref,
-                             float* S1, float* S2, float* split_ws, size_t split_ws_bytes, bsp_diag_t* diag, void* stream) {
+                             float* S1, float* S2, bool first, float* split_ws, size_t split_ws_bytes, bsp_diag_t* diag, void* stream) {
   if (T < 0 || O < 0 || C < 0 || n_draws < 0 || !valid_enum(q_dy.fmt, 1) || !valid_enum(q_x.fmt, 1)) return BSP_ERR_ARG;
   if (O == 0 || C == 0 || n_draws == 0) return BSP_OK;
   if (!g_ref || !S1 || !S2) return BSP_ERR_ARG;
@@ -1091,7 +1098,7 @@ int bsp::linear_wgrad_mc_run(int64_t T, int64_t O, int64_t C, const uint8_t* dy_
   g.lda = ld_t; g.ldb = ld_t; g.b_batch_stride = (int64_t)C * ld_t;
   g.sa = q_dy.scale; g.sa_dev = q_dy.scale_dev; g.sb = q_x.scale; g.sb_dev = q_x.scale_dev;
   g.mode = EPI_MC; g.C = nullptr; g.ldc = C; g.ref = g_ref; g.S1 = S1; g.S2 = S2; g.diag = diag;
-  g.split_ws = split_ws; g.split_ws_bytes = split_ws_bytes;
+  g.mc_first = first; g.split_ws = split_ws; g.split_ws_bytes = split_ws_bytes;
   return gemm_run(g, (cudaStream_t)stream);
 }
 

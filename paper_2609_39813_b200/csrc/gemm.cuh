@@ -39,6 +39,7 @@ struct GemmArgs {
   uint16_t* diff = nullptr;
   float moment_scale = 1.f;
   bool moment_first = false;
+  bool mc_first = false;               // EPI_MC: the sums start here (S1 and S2 need not be cleared)
   float* split_ws = nullptr;           // EPI_MC: room for split ranges of draws (gemm_mc_split_bytes), or none
   size_t split_ws_bytes = 0;
   bsp_diag_t* diag = nullptr;
@@ -48,9 +49,9 @@ int gemm_run(const GemmArgs& g, cudaStream_t st);
 
 // Workspace with which an EPI_MC contraction of nb draws can split the draws of its last wave of tiles.
 size_t gemm_mc_split_bytes(int64_t M, int64_t N, int64_t K, bool fp8, int nb);
-// bsp_linear_wgrad_mc with such a workspace.
+// bsp_linear_wgrad_mc with such a workspace; first: the sums start with these draws.
 int linear_wgrad_mc_run(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes_t, bsp_quant_t q_dy,
                         const uint8_t* x_t_draws, bsp_quant_t q_x, int64_t ld_t, int n_draws, const float* g_ref, float* S1,
-                        float* S2, float* split_ws, size_t split_ws_bytes, bsp_diag_t* diag, void* stream);
+                        float* S2, bool first, float* split_ws, size_t split_ws_bytes, bsp_diag_t* diag, void* stream);
 
 }  // namespace bsp

@@ -450,14 +450,12 @@ int bsp_mc_check(const bsp_norm_linear_desc_t* op, int K, const bsp_verdict_rule
       emit_dbeta(BSP_READ_FORWARD);
     }
     if (gain_mask & 4u) {
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S1g, 0, C * sizeof(float), st));
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S2g, 0, C * sizeof(float), st));
       gain_n_result = emit(BSP_STREAM_GAIN, BSP_OUT_DGAMMA, BSP_READ_FRESH);
       emit_dbeta(BSP_READ_FRESH);
       gain_key = key;
       if (!overlap_gain) {
-        BSP_TRY(bsp_norm_gain_mc(op->norm_kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt, qu,
-                                 gain_key, 0, K, b.dg_ref, b.S1g, b.S2g, b.ws_gain, b.b_gain, diag, st));
+        BSP_TRY(norm_gain_mc_run(op->norm_kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt, qu,
+                                 gain_key, 0, K, b.dg_ref, b.S1g, b.S2g, b.ws_gain, b.b_gain, diag, st, nullptr, true));
         BSP_TRY(stats(b.dg_ref, b.S1g, b.S2g, C, K, 1, gain_n_result));
       }
     }
@@ -480,13 +478,12 @@ int bsp_mc_check(const bsp_norm_linear_desc_t* op, int K, const bsp_verdict_rule
     }
     if (w_mask & 4u) {
       float* S1w = b.dW_pol;   // the U result has been reduced already
-      BSP_CHECK_CUDA(cudaMemsetAsync(S1w, 0, (size_t)O * C * sizeof(float), st));
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S2w, 0, (size_t)O * C * sizeof(float), st));
       bsp_quant_t qf = qu;
       qf.mode = BSP_ROUND_STOCHASTIC;
       key.stream = BSP_STREAM_WGRAD;
       // draws in chunks: one re-rounding launch writes the chunk's code matrices, one contraction
-      // launch walks them with the running sums resident in tensor memory
+      // launch walks them with the running sums in registers (the first chunk's start there: clearing S1 and
+      // S2 and reading the zeros back was 0.3 of 16.4 ms at 16384 x 4096 x 11008, 5 of 167 us at the smallest)
       const int chunk = draw_chunk(C, b.ld_t, K, op->draw_buffer_bytes);
       key.draw = 0;
       for (int k0 = 0; k0 < K; k0 += chunk) {
@@ -494,21 +491,21 @@ int bsp_mc_check(const bsp_norm_linear_desc_t* op, int K, const bsp_verdict_rule
         BSP_TRY(bsp_norm_fwd_draws(op->norm_kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, qf, key, k0,
                                    nd, b.fresh_t, b.ld_t, st));
         if (overlap_gain && k0 == 0) {
-          // fork: everything the gain kernel reads (du, the statistics, the reference, the cleared
-          // sums) has been queued on the main stream before this point
+          // fork: everything the gain kernel reads (du, the statistics, the reference) has been queued on
+          // the main stream before this point
           sw.side = (cudaStream_t)op->side_stream;
           BSP_CHECK_CUDA(cudaEventCreateWithFlags(&sw.fork, cudaEventDisableTiming));
           BSP_CHECK_CUDA(cudaEventCreateWithFlags(&sw.join, cudaEventDisableTiming));
           BSP_CHECK_CUDA(cudaEventRecord(sw.fork, st));
         }
         BSP_TRY(linear_wgrad_mc_run(T, O, C, b.dy_codes_t, qdy, b.fresh_t, qf, b.ld_t, nd, b.dW_ref, S1w, b.S2w,
-                                    b.ws_split, b.b_split, diag, st));
+                                    k0 == 0, b.ws_split, b.b_split, diag, st));
         if (overlap_gain && k0 == 0) {
           // the contraction is queued first, so its CTAs take the SMs first; the gain blocks fill in
           BSP_CHECK_CUDA(cudaStreamWaitEvent(sw.side, sw.fork, 0));
           sw.launched = true;
           BSP_TRY(norm_gain_mc_run(op->norm_kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt,
-                                   qu, gain_key, 0, K, b.dg_ref, b.S1g, b.S2g, b.ws_gain, b.b_gain, diag, sw.side));
+                                   qu, gain_key, 0, K, b.dg_ref, b.S1g, b.S2g, b.ws_gain, b.b_gain, diag, sw.side, nullptr, true));
           BSP_CHECK_CUDA(cudaEventRecord(sw.join, sw.side));
         }
       }

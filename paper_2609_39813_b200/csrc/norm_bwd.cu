@@ -383,11 +383,11 @@ gain_mc_slab_reduce_kernel(const float* partial, int nslabs, int64_t C, float* g
   }
 }
 
-// S1[c] += sum_k (gk - ref), S2[c] += sum_k (gk - ref)^2: 32 columns by eight draws per block, the
+// S1[c] += sum_k (gk - ref), S2[c] += sum_k (gk - ref)^2 (= if first): 32 columns by eight draws per block, the
 // eight partial sums added in order.
 __global__ void __launch_bounds__(256)
 gain_mc_accumulate_kernel(const float* gk, int ndraws, int64_t C, const float* ref,
-                          float* S1, float* S2) {
+                          float* S1, float* S2, bool first) {
   grid_dependency();
   __shared__ float sm[2][8][33];
   const int cl = threadIdx.x & 31, pl = threadIdx.x >> 5;
@@ -410,7 +410,7 @@ gain_mc_accumulate_kernel(const float* gk, int ndraws, int64_t C, const float* r
     float t = 0.f;
 #pragma unroll
     for (int w = 0; w < 8; ++w) t += sm[pl][w][cl];
-    out[c] += t;
+    out[c] = first ? t : out[c] + t;
   }
 }
 
@@ -547,7 +547,7 @@ size_t norm_gain_mc_workspace(int64_t T, int64_t C, int K) {
 int norm_gain_mc_run(int kind, const void* x, int dt, int64_t T, int64_t C, const float* gamma,
                      const float* beta, const float* rstd, const float* mean, const void* du, int du_dt, bsp_quant_t q,
                      bsp_key_t key, int draw0, int K, const float* g_ref, float* S1, float* S2, void* ws, size_t ws_bytes,
-                     bsp_diag_t* diag, void* stream, const float* grid_steps) {
+                     bsp_diag_t* diag, void* stream, const float* grid_steps, bool first) {
   if (!valid_enum(kind, 1) || !valid_enum(dt, 1) || !valid_enum(du_dt, 1) || !valid_enum(q.fmt, 1)) return BSP_ERR_ARG;
   if (key.tensor_id >= (1u << 24) || key.stream > 255u || key.reserved != 0) return BSP_ERR_ARG;
   if (T < 0 || C <= 0 || K < 0 || draw0 < 0) return BSP_ERR_ARG;
@@ -599,7 +599,8 @@ int norm_gain_mc_run(int kind, const void* x, int dt, int64_t T, int64_t C, cons
       launch_kernel(gain_mc_slab_reduce_kernel, rgrid, 256, 0, st, partial, nslabs, C, gk);
       BSP_LAUNCH_CHECK();
     }
-    launch_kernel(gain_mc_accumulate_kernel, (unsigned)((C + 31) / 32), 256, 0, st, nslabs == 1 ? partial : gk, nd, C, g_ref, S1, S2);
+    launch_kernel(gain_mc_accumulate_kernel, (unsigned)((C + 31) / 32), 256, 0, st, nslabs == 1 ? partial : gk, nd, C, g_ref, S1, S2,
+                  first && kb == 0);
     BSP_LAUNCH_CHECK();
   }
   return BSP_OK;

@@ -535,19 +535,15 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
       // u_q / gamma: the forward's own rounding, regenerated from its key (stream 0, draw 0): one "draw"
       // whose gradient lands in S1 against a zero reference
       BSP_CHECK_CUDA(cudaMemsetAsync(b.zero_c, 0, C * sizeof(float), st));
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.dg_pol, 0, C * sizeof(float), st));
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S2g, 0, C * sizeof(float), st));
       BSP_TRY(norm_gain_mc_run(kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt, qnone, key, 0, 1,
-                               b.zero_c, b.dg_pol, b.S2g, b.ws_gain, b.b_gain, diag, st, b.steps));
+                               b.zero_c, b.dg_pol, b.S2g, b.ws_gain, b.b_gain, diag, st, b.steps, true));
       BSP_TRY(pend.add(b.dg_ref, b.dg_pol, nullptr, C, 1, 0, emit(BSP_STREAM_GAIN, BSP_OUT_DGAMMA, BSP_READ_FORWARD)));
     }
     if (gain_mask & 4u) {
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S1g, 0, C * sizeof(float), st));
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S2g, 0, C * sizeof(float), st));
       bsp_key_t gk = key;
       gk.stream = BSP_STREAM_GAIN;
       BSP_TRY(norm_gain_mc_run(kind, op->x, dt, T, C, op->gamma, op->beta, b.rstd, b.mean, b.du, dt, qnone, gk, 0, K,
-                               b.dg_ref, b.S1g, b.S2g, b.ws_gain, b.b_gain, diag, st, b.steps));
+                               b.dg_ref, b.S1g, b.S2g, b.ws_gain, b.b_gain, diag, st, b.steps, true));
       BSP_TRY(pend.add(b.dg_ref, b.S1g, b.S2g, C, K, 1, emit(BSP_STREAM_GAIN, BSP_OUT_DGAMMA, BSP_READ_FRESH)));
     }
   }
@@ -586,8 +582,6 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
       // sums take them as they come, no per-draw gradient is written, and the bf16 rounding of an
       // operand costs 2^-9 of the difference.
       const int read = which == 0 ? STORE_READ_N : STORE_READ_R_EPS;
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S1w, 0, (size_t)O * C * sizeof(float), st));
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S2w, 0, (size_t)O * C * sizeof(float), st));
       bsp_key_t wk = key;
       wk.stream = BSP_STREAM_WGRAD; wk.draw = 0;
       const PhiloxKey pk = make_key(wk);
@@ -612,13 +606,13 @@ int bsp_mc_check_store(const bsp_store_desc_t* op, int K, const bsp_verdict_rule
         g.A = b.dys_t; g.B = b.diff_t; g.lda = b.ld_t; g.ldb = b.ld_t; g.b_batch_stride = (int64_t)C * b.ld_t;
         g.sa = 1.f; g.sa_dev = b.scale_dy; g.sb = 1.f; g.sb_dev = nullptr;
         g.mode = EPI_MC; g.ldc = C; g.ref = nullptr; g.S1 = b.S1w; g.S2 = b.S2w; g.diag = diag;
-        g.split_ws = b.ws_split; g.split_ws_bytes = b.b_split;
+        g.mc_first = k0 == 0; g.split_ws = b.ws_split; g.split_ws_bytes = b.b_split;
         BSP_TRY(gemm_run(g, st));
       }
       BSP_TRY(pend.add(b.dW_ref, b.S1w, b.S2w, O * C, K, 1,
                        emit(BSP_STREAM_WGRAD, BSP_OUT_DW, which == 0 ? BSP_READ_FRESH : BSP_READ_FORWARD_PLUS_FRESH_ERROR)));
       // the two fresh reads share S1w / S2w: the first one's statistics pass is queued before the
-      // second one clears them (same stream)
+      // second one starts them again (same stream)
     }
   }
   *n_results = nres;

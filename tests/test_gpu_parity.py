@@ -334,6 +334,29 @@ def test_split_draws_equal_one_walk(b, T, C, O, K):
     assert float((S1 - one1).abs().max()) <= tol * float((K * one2).sqrt().max())
 
 
+# a check's running sums start with its first draws, whatever the workspace held
+@pytest.mark.parametrize("T,C,O,K,chunk,simt", [(64, 128, 128, 16, 16, False), (80, 272, 400, 9, 4, False),
+                                                (48, 128, 272, 7, 1, False), (33, 144, 80, 5, 2, True)])
+def test_check_sums_start_by_themselves(b, monkeypatch, T, C, O, K, chunk, simt):
+    if simt:
+        monkeypatch.setenv("BSP_GEMM_SIMT", "1")
+    g = NormLinearGpu(workloads.config1(T=T, C=C, O=O, K=K, seed=8))
+    desc = g.desc(0x24)                                  # fresh reads of both uses
+    desc.draw_buffer_bytes = chunk * C * g.ld_t
+    lay = b.bsp_mc_check_layout(desc, K)
+    sums = []
+    for fill in (0, 255):                                # zeros, and NaN
+        ws = b.workspace(b.bsp_mc_check_workspace_bytes(desc, K))
+        ws.fill_(fill)
+        diag = b.new_diag()
+        b.bsp_mc_check(desc, K, ws, diag)
+        assert b.read_diag(diag)["status"] == 0
+        sums.append([b.ws_view(ws, off, n).clone() for off, n in ((lay.dgamma_S1, C), (lay.dgamma_S2, C),
+                                                                  (lay.dW_S1, O * C), (lay.dW_S2, O * C))])
+    for zeros, nans in zip(*sums):
+        assert torch.equal(zeros, nans) and float(zeros.abs().max()) > 0
+
+
 def test_weight_gradient_fused_monte_carlo_epilogue(b, case):
     inp, g, kind, prep = case
     T, C, O, K = inp.T, inp.C, inp.O, 6
