@@ -1,7 +1,8 @@
 // The rounded-probability averages on the tensor cores, for rows of up to 128 entries and 64 value
 // columns.  A draw of a row needs h = V^T p_q, dp = V h and two outer products with h: per row and draw
 // 4 n d multiply-adds, which on the CUDA cores ran at a quarter of the FP32 rate (V and h from shared
-// memory for every draw: 16384 rows of 128 x 64, 256 draws, 14.7 ms; here 4.2).  Here the draws of a row are the M dimension of small contractions.
+// memory for every draw: 16384 rows of 128 x 64, 256 draws, 14.7 ms; here 4.06).  Here the draws of a row are
+// the M dimension of small contractions.
 //
 // Everything a draw rounds is two-valued: p_q = lo + s q with a bit q per entry (s = param for the grid,
 // 2 param for the +-param law), likewise a and b.  The bits enter the products as exact bf16 0 / 1 and
@@ -25,8 +26,8 @@
 // products.  A tile is 128 slots: one row's 128 draws, or two rows' 64.  Per tile: the generator (three streams)
 // under the H products of the stream before, the slot pass, the dp and outer products, and the entry pass, in
 // which a thread owns an entry and walks 32 slots (the five operators' errors and their squares, in packed
-// FP32 pairs of slots).  Of a tile's 33 thousand cycles at 128 draws and two tiles a row, the generator and
-// the bits take 15, the entry pass 6, the slot pass 3, waits for products 4, and the row's start and end 7:
+// FP32 pairs of slots).  Of a tile's 32 thousand cycles at 128 draws and two tiles a row, the generator and
+// the bits take 14, the entry pass 6, the slot pass 3, waits for products 4, and the row's start and end 7:
 // bound by instruction issue, with the tensor pipe busy a tenth of the time.
 #pragma once
 
@@ -359,9 +360,11 @@ probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param
 #pragma unroll
         for (int s8 = 0; s8 < 8; ++s8) code[s8] = 0u;
         const int nv = K - (chunk * g + ((8 * w) & (g - 1)));           // draws left for this warp's eight slots
-#pragma unroll 1
+        // (unrolled, so that a stream does only its own counting: 4.23 -> 4.06 ms; a second body for whole groups of
+        // eight draws, without their limit, is no faster)
+#pragma unroll
         for (int m = 0; m < 3; ++m) {
-          int ups = 0;                                                // lane s: up-roundings of a in the warp's slot s
+          uint32_t ups[2] = {0u, 0u};                                 // up-roundings of a, a byte per slot (at most 128)
           if (nv <= 0) {                                              // (warp-uniform)
 #pragma unroll
             for (int s8 = 0; s8 < 8; ++s8)
@@ -385,13 +388,17 @@ probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param
             if (m == 0) cnt_q4 += t4 & 0x01010101u;
             if (m == 1) {
               cnt_a4 += t4 & 0x01010101u;
-              const int c = __reduce_add_sync(0xFFFFFFFFu, __popc(t4 & 0x01010101u));
-              if (lane == s8) ups = c;
+              ups[s8 >> 2] += (uint32_t)__popc(t4 & 0x01010101u) << (8 * (s8 & 3));
             }
             *reinterpret_cast<uint2*>(sm + kPtBits + m * kPtMat + (lane >> 4) * kPtTerm + slot * 128 +
                                       ((((uint32_t)(lane & 15) >> 1) ^ s8) << 4) + (lane & 1) * 8) = make_uint2(lo2, hi2);
           }
-          if (m == 1 && lane < 8) suma_s[8 * w + lane] = (float)(sumlo + (double)step * ups);   // 1^T a - 1, in double from the count
+          if (m == 1) {
+            const uint32_t u0 = __reduce_add_sync(0xFFFFFFFFu, ups[0]), u1 = __reduce_add_sync(0xFFFFFFFFu, ups[1]);
+            // 1^T a - 1, in double from the count
+            if (lane < 8)
+              suma_s[8 * w + lane] = (float)(sumlo + (double)step * (double)(((lane & 4 ? u1 : u0) >> (8 * (lane & 3))) & 0xFFu));
+          }
           pt_arrive(bar_go + 8 * m, lane);
         }
 #pragma unroll
