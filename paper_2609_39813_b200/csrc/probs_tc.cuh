@@ -28,7 +28,8 @@
 // which a thread owns an entry and walks 32 slots (the five operators' errors and their squares, in packed
 // FP32 pairs of slots).  Of a tile's 32 thousand cycles at 128 draws and two tiles a row, the generator and
 // the bits take 14, the entry pass 6, the slot pass 3, waits for products 4, and the row's start and end 7:
-// bound by instruction issue, with the tensor pipe busy a tenth of the time.
+// no unit is full (issue slots 48 %, the generator's multiplier 45 %, tensor pipe 15 %), the phases following one
+// another with four warps per scheduler; a second set of bit matrices, to overlap them, does not fit.
 #pragma once
 
 #include "common.cuh"
