@@ -6,16 +6,18 @@
 //
 // Everything a draw rounds is two-valued: p_q = lo + s q with a bit q per entry (s = param for the grid,
 // 2 param for the +-param law), likewise a and b.  The bits enter the products as exact bf16 0 / 1 and
-// the FP32 factors as three bf16 terms, so a product loses nothing an FP32 one would keep:
+// the FP32 factors as three bf16 terms:
 //   H   = bits V            128 slots x 64, for the bits of p_q, a and b        3 x 3 products
 //   delta = s H_q + V^T (lo - p),  h = V^T p + delta  (p_q's; a's and b's likewise), and with them the
 //           dot products x . dp = (V^T x) . h of the operators, one thread per slot
 //   dp^T = V (V^T p) + V delta^T    128 entries x 128 slots, delta in three terms   6 products
 //   sum_k q delta^T, sum_k a delta^T  per row, 128 entries x 64 each, over the row's slots
-// H is exact: V's terms are multiples of 2^-8, 2^-17 and 2^-26 of its column's scale, nine bits each, so
-// the first term's sums (one accumulator) and the other two's (another) are integers below 2^24 of
-// their unit.  That matters because tensor-core accumulation truncates: a truncated H is off to one side
-// in every draw, and such an error, unlike a rounded one, survives the average over the draws.
+// V's terms are multiples of 2^-8, 2^-17 and 2^-26 of its column's scale, nine bits each, so the first term's
+// sums (one accumulator) and the other two's (another) are integers below 2^24 of their unit: H is exact for this V.
+// That matters because tensor-core accumulation truncates: a truncated H is off to one side in every draw, and such
+// an error, unlike a rounded one, survives the average over the draws.  An entry of V is held to 2^-27 of its
+// column's scale, which is FP32's own precision for entries of at least an eighth of it and less below; for a V whose
+// rows differ by more than that bears (probs_wide) the kernel forms the sums in FP32 (probs_fp32_rows).
 // Summing against delta = h - V^T p, whose mean over the draws is zero, rather than against h keeps the
 // sums as small as their results: sum (p - p_q) h^T = -w (V^T p)^T + (p - lo) (sum delta)^T - s sum q delta^T
 // with the scalar w_j = sum_k (p_q - p)_j known from the count of up-roundings.
@@ -95,6 +97,48 @@ __device__ __forceinline__ void bf16_split3(float a, float b, uint32_t (&t)[3]) 
   }
 }
 
+// Whether V's rows differ too widely in size for terms of fixed position: the smallest of the rows' largest
+// magnitudes (rows of zeros aside) below a sixteenth of the power of two above V's largest, or V not finite.  A row of
+// probabilities may lie on the smallest row alone, and then the error of h is 2^-27 of the largest over the
+// smallest.  The line lies where the two forms cross: relative errors of the operators' sums, of their squares and of
+// the gradient-of-V sums against 64 bits, the worst of twelve rows, with one row of V scaled up and unlikely, fixed
+// terms and FP32: x 6 3.4, 3.4, 1.4e-7 and 3.8, 2.6, 2.1e-7; x 100 1.7, 3.9, 0.8e-6 and 1.6, 0.8, 0.2e-6; x 1000 1.1, 2.2,
+// 1.0e-5 and 2.1, 0.2, 0.2e-6.  Scaled down and all but certain: 1/8 0.6, 1.1, 1.2e-6 and 1.3, 1.2, 1.2e-6; 1/32 1.5, 4.0,
+// 0.5e-6 and 1.9, 2.1, 0.9e-6; 1/1000 0.9, 1.0, 0.2e-4 and 1.8, 1.5, 1.5e-6.
+// Also the largest magnitude of each column, to col_max ([64] words).  The kernel's whole block; found is two words.
+__device__ __forceinline__ bool probs_wide(const float* V, int n, int d, uint32_t* found, uint32_t* col_max) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  constexpr int kWarps = kPtThreads / 32, kRows = (kPtN + kWarps - 1) / kWarps;
+  if (threadIdx.x < kPtD) col_max[threadIdx.x] = 0u;
+  if (threadIdx.x == 0) { found[0] = 0u; found[1] = 0xFFFFFFFFu; }
+  uint32_t v[kRows][2];                                               // d <= 64: two columns a lane
+#pragma unroll
+  for (int i = 0; i < kRows; ++i) {
+    const int j = w + kWarps * i;
+    v[i][0] = j < n && lane < d ? __float_as_uint(ldg(V + (size_t)j * d + lane)) & 0x7FFFFFFFu : 0u;
+    v[i][1] = j < n && lane + 32 < d ? __float_as_uint(ldg(V + (size_t)j * d + lane + 32)) & 0x7FFFFFFFu : 0u;
+  }
+  __syncthreads();
+  uint32_t c0 = 0u, c1 = 0u, most = 0u, least = 0xFFFFFFFFu;
+#pragma unroll
+  for (int i = 0; i < kRows; ++i) {
+    c0 = max(c0, v[i][0]);
+    c1 = max(c1, v[i][1]);
+    const uint32_t row = __reduce_max_sync(0xFFFFFFFFu, max(v[i][0], v[i][1]));
+    most = max(most, row);
+    if (row) least = min(least, row);
+  }
+  if (lane < d) atomicMax(&col_max[lane], c0);
+  if (lane + 32 < d) atomicMax(&col_max[lane + 32], c1);
+  if (lane == 0) { atomicMax(&found[0], most); atomicMin(&found[1], least); }
+  __syncthreads();
+  most = found[0]; least = found[1];
+  if (most == 0u) return false;
+  if (most >= 0x7F800000u) return true;
+  int ex;
+  frexpf(__uint_as_float(most), &ex);                                 // most < 2^ex
+  return scalbnf(__uint_as_float(least), 4 - ex) < 1.f;
+}
 // Where an entry sits between its two rounded values (law 0: the uniform grid; law 1: +-param).
 // Up iff the word is below thr (law 0) or above it (law 1: its top bit is set).
 __device__ __forceinline__ void probs_cell(float p, int law, float param, float& lo, float& hi, uint32_t& thr) {
@@ -118,6 +162,171 @@ __device__ __forceinline__ void pt_arrive(uint32_t bar, int lane) {
   tc_fence_before();
   __syncwarp();
   if (lane == 0) mbar_arrive(bar);
+}
+
+// The sums in FP32 on the CUDA cores, for a V that terms of fixed position do not hold (probs_wide).  The whole
+// block; sixteen draws of a row at a time.  Phase 1, a warp per draw: a lane owns four consecutive entries, one
+// generator block per stream; h = V^T p_q with the lane owning two columns, dp = V h from a transposed copy of V;
+// the dot products are warp sums.  Phase 2, a thread per entry and quarter of the columns: adds the draws to its
+// sums.  4096 rows, 32 draws: 128 x 64 662 us (probs_mc_128x64_kernel 663), 64 x 64 523 (probs_mc_kernel 771), 100 x 16
+// 367 (1278), 16 x 16 257 (299).
+constexpr int kPwDraws = 16;
+constexpr size_t kPwFloats = (size_t)2 * kPtN * kPtD + kPwDraws * (3 * kPtN /*pq, eu, ea*/ + kPtD /*h*/ + 5 * kPtN /*err*/);
+static_assert(kPwFloats * sizeof(float) <= kPtEnd, "the FP32 form's shared memory");
+template <int law>
+__device__ __forceinline__ void probs_fp32_rows(float* sm, const float* p_all, const float* V, int n, int d, float param,
+                                                PhiloxKey kq, int draw0, int K, float* ds_sum, float* ds_sq, float* dV_sum,
+                                                size_t rows) {
+  float* Vs = sm;                                                     // [128][64]
+  float* Vt = Vs + kPtN * kPtD;                                       // [64][128]
+  float* pq_s = Vt + kPtN * kPtD;                                     // [16][128]
+  float* eu_s = pq_s + kPwDraws * kPtN;                               // [16][128]: p - p_q
+  float* ea_s = eu_s + kPwDraws * kPtN;                               // [16][128]: a - p_q
+  float* h_s = ea_s + kPwDraws * kPtN;                                // [16][64]
+  float* err_s = h_s + kPwDraws * kPtD;                               // [16][5][128]
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  __syncthreads();
+  for (int i = tid; i < kPtN * kPtD; i += kPtThreads) {
+    const int j = i >> 6, c = i & (kPtD - 1);
+    const float v = j < n && c < d ? ldg(V + (size_t)j * d + c) : 0.f;
+    Vs[i] = v;
+    Vt[c * kPtN + j] = v;
+  }
+  const int j2 = tid & (kPtN - 1), hh = tid >> 7;                     // phase 2: entry, quarter (the fifth is idle)
+  const int op0 = hh == 0 ? 0 : hh + 1, nops = hh == 0 ? 2 : 1;       // its operators: two in the first, one in the others
+  const bool on = 4 * lane < n, on2 = hh < 4 && j2 < n;
+  const uint32_t c3 = kq.c3 & ~0xFFu;
+  __syncthreads();
+  for (size_t row = blockIdx.x; row < rows; row += gridDim.x) {
+    float pv[4], lo[4], hi[4];
+    uint32_t thr[4];
+    double sum_p = 0.0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      pv[e] = lo[e] = hi[e] = 0.f;
+      thr[e] = 0u;                                                    // an entry that is not there stays zero either way
+      if (on) {
+        pv[e] = ldg(p_all + row * n + 4 * lane + e);
+        probs_cell(pv[e], law, param, lo[e], hi[e], thr[e]);
+      }
+      sum_p += (double)pv[e];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum_p += __shfl_xor_sync(0xFFFFFFFFu, sum_p, o);
+    const float sum_p_m1 = (float)(sum_p - 1.0);
+    const uint64_t q = (row * (uint64_t)n) / 4 + (uint64_t)lane;
+    float acc_u[16], acc_a[16], acc_s[2] = {0.f, 0.f}, acc_q[2] = {0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < 16; ++c) acc_u[c] = acc_a[c] = 0.f;
+    for (int k0 = 0; k0 < K; k0 += kPwDraws) {
+      const int nd = K - k0 < kPwDraws ? K - k0 : kPwDraws;
+      if (w < nd) {
+        float pq[4], a[4], b[4];
+        auto draw = [&](uint32_t stream, float (&x)[4]) {
+          const uint4 r = philox4x32_10((uint32_t)q, (uint32_t)(q >> 32), (uint32_t)(draw0 + k0 + w), c3 | stream, kq.k0, kq.k1);
+          const uint32_t u[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[e] = (law == 1 ? u[e] > thr[e] : u[e] < thr[e]) ? hi[e] : lo[e];
+        };
+        draw(0u, pq); draw(1u, a); draw(2u, b);
+        float* pqw = pq_s + w * kPtN;
+        *reinterpret_cast<float4*>(pqw + 4 * lane) = make_float4(pq[0], pq[1], pq[2], pq[3]);
+        __syncwarp();
+        float h0 = 0.f, h1 = 0.f, g0 = 0.f, g1 = 0.f;
+#pragma unroll 2
+        for (int j = 0; j < n; j += 4) {
+          const float4 x = *reinterpret_cast<const float4*>(pqw + j);
+          const float2* v = reinterpret_cast<const float2*>(Vs + j * kPtD) + lane;
+          const float2 v0 = v[0], v1 = v[kPtD / 2], v2 = v[kPtD], v3 = v[3 * kPtD / 2];
+          h0 = fmaf(v0.x, x.x, h0); h1 = fmaf(v0.y, x.x, h1);
+          g0 = fmaf(v1.x, x.y, g0); g1 = fmaf(v1.y, x.y, g1);
+          h0 = fmaf(v2.x, x.z, h0); h1 = fmaf(v2.y, x.z, h1);
+          g0 = fmaf(v3.x, x.w, g0); g1 = fmaf(v3.y, x.w, g1);
+        }
+        float* hw = h_s + w * kPtD;
+        *reinterpret_cast<float2*>(hw + 2 * lane) = make_float2(h0 + g0, h1 + g1);
+        __syncwarp();
+        float dp[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+        for (int c = 0; c < d; ++c) {
+          const float hv = hw[c];
+          const float4 t = *reinterpret_cast<const float4*>(Vt + c * kPtN + 4 * lane);
+          dp[0] = fmaf(t.x, hv, dp[0]); dp[1] = fmaf(t.y, hv, dp[1]); dp[2] = fmaf(t.z, hv, dp[2]); dp[3] = fmaf(t.w, hv, dp[3]);
+        }
+        float dots[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          dots[0] = fmaf(pv[e], dp[e], dots[0]);
+          dots[1] = fmaf(pq[e] - pv[e], dp[e], dots[1]);
+          dots[2] = fmaf(a[e] - pv[e], dp[e], dots[2]);
+          dots[3] = fmaf(b[e] - pv[e], dp[e], dots[3]);
+          dots[4] += a[e] - pv[e];
+        }
+#pragma unroll
+        for (int i = 0; i < 5; ++i) dots[i] = warp_sum(dots[i]);
+        float er[5][4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {                                 // as in the entry pass below
+          const float c = dp[e] - dots[0], dq = pq[e] - pv[e], da = a[e] - pv[e], db = b[e] - pv[e];
+          er[0][e] = dq * c - pq[e] * dots[1];
+          er[1][e] = da * c - a[e] * dots[2];
+          er[2][e] = a[e] * (dots[4] + sum_p_m1) * dp[e] + er[1][e];
+          er[3][e] = 0.5f * ((da + db) * c - (a[e] * dots[3] + b[e] * dots[2]));
+          er[4][e] = 0.5f * ((dq + db) * c - (pq[e] * dots[3] + b[e] * dots[1]));
+        }
+#pragma unroll
+        for (int o = 0; o < 5; ++o)
+          *reinterpret_cast<float4*>(err_s + (w * 5 + o) * kPtN + 4 * lane) = make_float4(er[o][0], er[o][1], er[o][2], er[o][3]);
+        *reinterpret_cast<float4*>(eu_s + w * kPtN + 4 * lane) = make_float4(pv[0] - pq[0], pv[1] - pq[1], pv[2] - pq[2], pv[3] - pq[3]);
+        *reinterpret_cast<float4*>(ea_s + w * kPtN + 4 * lane) = make_float4(a[0] - pq[0], a[1] - pq[1], a[2] - pq[2], a[3] - pq[3]);
+      }
+      __syncthreads();
+      if (on2)
+        for (int k = 0; k < nd; ++k) {
+          const float eu = eu_s[k * kPtN + j2], ea = ea_s[k * kPtN + j2];
+          if (16 * hh < d)
+#pragma unroll
+            for (int c = 0; c < 16; c += 4) {
+              const float4 hv = *reinterpret_cast<const float4*>(h_s + k * kPtD + 16 * hh + c);
+              acc_u[c] = fmaf(eu, hv.x, acc_u[c]); acc_u[c + 1] = fmaf(eu, hv.y, acc_u[c + 1]);
+              acc_u[c + 2] = fmaf(eu, hv.z, acc_u[c + 2]); acc_u[c + 3] = fmaf(eu, hv.w, acc_u[c + 3]);
+              acc_a[c] = fmaf(ea, hv.x, acc_a[c]); acc_a[c + 1] = fmaf(ea, hv.y, acc_a[c + 1]);
+              acc_a[c + 2] = fmaf(ea, hv.z, acc_a[c + 2]); acc_a[c + 3] = fmaf(ea, hv.w, acc_a[c + 3]);
+            }
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            if (i < nops) {
+              const float v = err_s[(k * 5 + op0 + i) * kPtN + j2];
+              acc_s[i] += v;
+              acc_q[i] = fmaf(v, v, acc_q[i]);
+            }
+        }
+      __syncthreads();
+    }
+    if (on2) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (i < nops) {
+          const size_t at = ((size_t)(op0 + i) * rows + row) * n + j2;
+          ds_sum[at] = acc_s[i];
+          if (ds_sq) ds_sq[at] = acc_q[i];
+        }
+      float* o_u = dV_sum + (row * (size_t)n + j2) * d + 16 * hh;
+      float* o_a = o_u + rows * (size_t)n * d;
+#pragma unroll
+      for (int c = 0; c < 16; c += 4) {
+        if (16 * hh + c >= d) break;
+        if ((d & 3) == 0) {
+          *reinterpret_cast<float4*>(o_u + c) = make_float4(acc_u[c], acc_u[c + 1], acc_u[c + 2], acc_u[c + 3]);
+          *reinterpret_cast<float4*>(o_a + c) = make_float4(acc_a[c], acc_a[c + 1], acc_a[c + 2], acc_a[c + 3]);
+        } else {
+#pragma unroll
+          for (int e = c; e < c + 4; ++e)
+            if (16 * hh + e < d) { o_u[e] = acc_u[e]; o_a[e] = acc_a[e]; }
+        }
+      }
+    }
+  }
 }
 
 template <int law>
@@ -153,19 +362,20 @@ probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (w == 16) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+  uint32_t* vmax_s = reinterpret_cast<uint32_t*>(hp_s);
+  if (probs_wide(V, n, d, vmax_s + kPtD, vmax_s)) {
+    if (w == 16) tmem_dealloc(*tmem_slot, 512);
+    probs_fp32_rows<law>(reinterpret_cast<float*>(sm), p_all, V, n, d, param, kq, draw0, K_all, ds_sum, ds_sq, dV_sum, rows);
+    return;
+  }
   // V's three terms, [entry][column] rows of 128 bytes in the 128-byte swizzle: the K-major A operand of
   // dp^T and the MN-major B operand of H.  The scale of a column is the power of two at or above its
   // largest magnitude.
-  uint32_t* vmax_s = reinterpret_cast<uint32_t*>(hp_s);
-  if (tid < kPtD) vmax_s[tid] = 0u;
-  __syncthreads();
-  for (int i = tid; i < n * d; i += kPtThreads) atomicMax(&vmax_s[i % d], __float_as_uint(fabsf(ldg(V + i))));
-  __syncthreads();
   for (int i = tid; i < kPtN * kPtD; i += kPtThreads) {
     const int j = i >> 6, c = i & 63;
     const float m = __uint_as_float(vmax_s[c]);
     int ex = 0;
-    if (m > 0.f && m <= 3.4028234663852886e38f) frexpf(m, &ex);       // m < 2^ex
+    if (m > 0.f) frexpf(m, &ex);                                      // m < 2^ex
     float v = j < n && c < d ? ldg(V + (size_t)j * d + c) : 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {

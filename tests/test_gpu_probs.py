@@ -82,6 +82,37 @@ def test_tensor_core_form_matches_the_oracle(b, R, n, d, law, param, K):
         assert np.max(np.abs(dV[i] - want_dV[i])) <= 2e-5 * f * (np.max(np.abs(want_dV[i])) + 1e-30), i
 
 
+# rows of V that differ widely in size, the large ones unlikely or the likely one small: the errors stay FP32's own.
+# Both sides of the line between the two forms of V (rows within a sixteenth of each other), both tile cuts, the
+# kernel of its own, and more rows than blocks.
+@pytest.mark.parametrize("R,n,d,law,param,K", [(3, 128, 64, 0, 1.0 / 64, 64), (2, 128, 64, 1, 1.0 / 512, 100), (3, 64, 20, 0, 1.0 / 64, 40),
+                                               (700, 32, 8, 0, 1.0 / 64, 32)])
+@pytest.mark.parametrize("scale", [2.0 ** -13, 2.0 ** -10, 0.125, 4.0, 1.0e3, 1.0e4])
+def test_rows_of_values_of_different_sizes(b, R, n, d, law, param, K, scale):
+    p, V = _rows(R, n, d, 19 + n)
+    j = int(np.argmin(p.sum(0)) if scale > 1 else np.argmax(p.sum(0)))
+    p[:, j] *= 1e-4 if scale > 1 else 300.0                  # the large row unlikely, the small one likely
+    p = (p / p.sum(1, keepdims=True, dtype=np.float64)).astype(np.float32)
+    V[j] *= np.float32(scale)
+    ds, sq, dV = _run(b, p, V, law, param, 47, 1, K)
+    want_ds, want_sq, want_dV = probs.mc_sums(p, V, law, param, 47, K, 1)
+    for got, want, tol in ((ds, want_ds, 2e-5), (sq, want_sq, 1e-4), (dV, want_dV, 2e-5)):
+        for r in range(min(R, 4)):                           # row by row: what one row loses another does not hide
+            for i in range(want.shape[0]):
+                assert np.linalg.norm(got[i, r] - want[i, r]) <= tol * np.linalg.norm(want[i, r]) + 1e-30, (r, i)
+
+
+def test_values_that_are_not_finite_stay_with_their_column(b):
+    R, n, d, K = 3, 64, 8, 40
+    p, V = _rows(R, n, d, 3)
+    V[7, 2] = np.inf
+    ds, _, dV = _run(b, p, V, 0, 1.0 / 64, 47, 0, K)
+    assert not np.isfinite(ds).any() and not np.isfinite(dV[:, :, 7, 2]).any()
+    want = probs.mc_sums(p, np.where(np.isfinite(V), V, 0).astype(np.float32), 0, 1.0 / 64, 47, K, 0)[2]
+    keep = [c for c in range(d) if c != 2]                   # h of the other columns does not see it
+    assert np.max(np.abs(dV[..., keep] - want[..., keep])) <= 2e-5 * np.max(np.abs(want))
+
+
 def test_bench_size_on_sampled_rows(b):
     """The size `bench.py` times (16384 rows of 128 probabilities, d = 64, grid 1/64, 256 draws; rows
     drawn by the same recipe): blocks of rows from the start, the middle and the end of the tensor
