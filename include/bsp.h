@@ -652,7 +652,8 @@ int bsp_lsm_check(const float* logits, const int32_t* target, int rows, int clas
  * (g o sigma^2 - tau p - Sigma_r G p)/2, and rows -sigma_j^2 v_j^T for both reads.
  * law 0: stochastic rounding to a uniform grid of spacing `param` (t = fl32(p / param), up iff
  * W < floor(frac(t) 2^32)); law 1: r = +param when the top bit of W is set, else -param.
- * n <= 256, d <= 64, d <= n.  Outputs are overwritten.
+ * n <= 256, d <= 64, d <= n.  Outputs are overwritten; should a bounded wait run out (there is no
+ * diag), the rows it cuts short are NaN in every output.
  * ------------------------------------------------------------------------------------------ */
 int bsp_probs_mc(const float* p, const float* V, int64_t rows, int n, int d, int law, float param,
                  uint64_t seed, uint32_t tensor_id, int draw0, int K, float* ds_sum, float* ds_sq,
@@ -708,6 +709,12 @@ int bsp_coupling_check(const bsp_coupling_desc_t* op, int pairs, double* T, doub
  * after synchronising, diag.status == BSP_ERR_TIMEOUT and the context is intact.
  * ------------------------------------------------------------------------------------------ */
 int bsp_selftest_bounded_wait(uint64_t limit_ns, bsp_diag_t* diag, void* stream);
+/* What bsp_probs_mc leaves when such a wait runs out: the rows a block had not completed are NaN in all
+ * three outputs, the others hold their sums.  As bsp_probs_mc with law 0, tensor 0 and draws from 0, in the
+ * tensor-core form (n <= 128, n % 4 == 0), with every block stopping before its rows from `done` on. */
+int bsp_selftest_probs_unfinished(const float* p, const float* V, int64_t rows, int n, int d, float param,
+                                  uint64_t seed, int K, int64_t done, float* ds_sum, float* ds_sq, float* dV_sum,
+                                  void* stream);
 
 #ifdef __cplusplus
 }

@@ -166,6 +166,7 @@ _SIGNATURES = {
     "bsp_lsm_check_workspace_bytes": (_SZ, [_I, _I, _I]),
     "bsp_lsm_check": (_I, [_P, _P, _I, _I, _F, _I, _U64, C.c_uint32, _P, C.POINTER(LsmStat), _P, _SZ, _P]),
     "bsp_probs_mc": (_I, [_P, _P, _I64, _I, _I, _I, _F, _U64, C.c_uint32, _I, _I, _P, _P, _P, _P]),
+    "bsp_selftest_probs_unfinished": (_I, [_P, _P, _I64, _I, _I, _F, _U64, _I, _I64, _P, _P, _P, _P]),
     "bsp_coupling_check_workspace_bytes": (_SZ, [C.POINTER(CouplingDesc), _I]),
     "bsp_coupling_layout": (_I, [C.POINTER(CouplingDesc), _I, C.POINTER(CouplingLayout)]),
     "bsp_coupling_check": (_I, [C.POINTER(CouplingDesc), _I, C.POINTER(C.c_double), C.POINTER(C.c_double), _P, _SZ, _P, _P]),
@@ -565,6 +566,11 @@ def bsp_lsm_check(logits, target, rows, classes, eps, trials, seed, tensor_id, p
 def bsp_probs_mc(p, V, rows, n, d, law, param, seed, tensor_id, draw0, K, ds_sum, ds_sq, dV_sum, stream=None):
     check(lib().bsp_probs_mc(ptr(p), ptr(V), rows, n, d, law, param, int(seed), tensor_id, draw0, K, ptr(ds_sum),
                              ptr(ds_sq), ptr(dV_sum), _st(stream)), "bsp_probs_mc")
+
+
+def bsp_selftest_probs_unfinished(p, V, rows, n, d, param, seed, K, done, ds_sum, ds_sq, dV_sum, stream=None):
+    check(lib().bsp_selftest_probs_unfinished(ptr(p), ptr(V), rows, n, d, param, int(seed), K, done, ptr(ds_sum), ptr(ds_sq),
+                                              ptr(dV_sum), _st(stream)), "bsp_selftest_probs_unfinished")
 
 
 def bsp_coupling_check_workspace_bytes(desc: CouplingDesc, pairs):

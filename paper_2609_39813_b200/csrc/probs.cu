@@ -398,11 +398,37 @@ probs_mc_128x64_kernel(const float* p_all, const float* V, int law, float param,
   }
 }
 
+// The rows from `stop` on (rounded up to a block's group of rows) are left as after a wait that ran out.
+static int probs_tc_run(const float* p, const float* V, int64_t rows, int n, int d, int law, float param, PhiloxKey kq, int draw0,
+                        int K, float* ds_sum, float* ds_sq, float* dV_sum, int64_t stop, cudaStream_t st) {
+  int dev = 0, nsm = kNumSMs;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int g = K <= 64 ? 64 : 128, R = kPtSlots / g;           // slots per row: two rows' draws share a tile up to 64
+  const int64_t ngroups = (rows + R - 1) / R;
+  auto kern = law == 1 ? probs_mc_tc_kernel<1> : probs_mc_tc_kernel<0>;
+  BSP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPtSmemBytes));
+  launch_kernel(kern, (unsigned)(ngroups < nsm ? ngroups : nsm), kPtThreads, kPtSmemBytes, st, p, V, n, d, param, kq, draw0, K, g,
+                ds_sum, ds_sq, dV_sum, (size_t)rows, (size_t)((stop + R - 1) / R));
+  BSP_LAUNCH_CHECK();
+  return BSP_OK;
+}
+
 }  // namespace bsp
 
 using namespace bsp;
 
 extern "C" {
+
+int bsp_selftest_probs_unfinished(const float* p, const float* V, int64_t rows, int n, int d, float param, uint64_t seed, int K,
+                                  int64_t done, float* ds_sum, float* ds_sq, float* dV_sum, void* stream) {
+  if (!p || !V || !ds_sum || !dV_sum || rows <= 0 || n <= 0 || n > kPtN || n % 4 != 0 || d <= 0 || d > kPtD || d > n || K <= 0 ||
+      !(param > 0.f) || done < 0 || done > rows)
+    return BSP_ERR_ARG;
+  if (!aligned16(dV_sum)) return BSP_ERR_ALIGN;
+  bsp_key_t k;
+  k.seed = seed; k.tensor_id = 0; k.stream = 0; k.draw = 0; k.reserved = 0;
+  return probs_tc_run(p, V, rows, n, d, 0, param, make_key(k), 0, K, ds_sum, ds_sq, dV_sum, done, (cudaStream_t)stream);
+}
 
 int bsp_probs_mc(const float* p, const float* V, int64_t rows, int n, int d, int law, float param, uint64_t seed,
                  uint32_t tensor_id, int draw0, int K, float* ds_sum, float* ds_sq, float* dV_sum, void* stream) {
@@ -420,18 +446,8 @@ int bsp_probs_mc(const float* p, const float* V, int64_t rows, int n, int d, int
   // undercut for few draws: 4096 rows of 128 x 64, 8 draws 348 us here and 350 there, 16 draws 455 and 350; of
   // 64 x 64, 8 draws 336 and 322; of 32 x 32, 24 draws 261 and 298, 32 draws 329 and 299; of 16 x 16 likewise.  It
   // wants whole generator blocks per row and 16-byte stores of the gradient rows.
-  if (n <= kPtN && n % 4 == 0 && K >= (n >= 64 ? 8 : 32) && (d % 4 != 0 || aligned16(dV_sum))) {
-    int dev = 0, nsm = kNumSMs;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int g = K <= 64 ? 64 : 128;                           // slots per row: two rows' draws share a tile up to 64
-    const int64_t ngroups = (rows + kPtSlots / g - 1) / (kPtSlots / g);
-    auto kern = law == 1 ? probs_mc_tc_kernel<1> : probs_mc_tc_kernel<0>;
-    BSP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPtSmemBytes));
-    launch_kernel(kern, (unsigned)(ngroups < nsm ? ngroups : nsm), kPtThreads, kPtSmemBytes, (cudaStream_t)stream,
-                  p, V, n, d, param, kq, draw0, K, g, ds_sum, ds_sq, dV_sum, (size_t)rows);
-    BSP_LAUNCH_CHECK();
-    return BSP_OK;
-  }
+  if (n <= kPtN && n % 4 == 0 && K >= (n >= 64 ? 8 : 32) && (d % 4 != 0 || aligned16(dV_sum)))
+    return probs_tc_run(p, V, rows, n, d, law, param, kq, draw0, K, ds_sum, ds_sq, dV_sum, rows, (cudaStream_t)stream);
   if (n == kPfN && d == kPfD && (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (reinterpret_cast<uintptr_t>(dV_sum) & 15u) == 0) {
     const size_t smem_f = kPfSmemFloats * sizeof(float);
     BSP_CHECK_CUDA(cudaFuncSetAttribute(probs_mc_128x64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f));

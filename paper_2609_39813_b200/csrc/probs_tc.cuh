@@ -333,7 +333,7 @@ template <int law>
 __global__ void __launch_bounds__(kPtThreads, 1)
 probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param,
                    PhiloxKey kq, int draw0, int K_all, int g /* slots per row: 64 or 128 */, float* ds_sum,
-                   float* ds_sq, float* dV_sum, size_t rows) {
+                   float* ds_sq, float* dV_sum, size_t rows, size_t stop /* groups from here on are left undone (self-test) */) {
   grid_dependency();
   extern __shared__ uint8_t pt_raw[];
   const uint32_t raw = smem_u32(pt_raw), base = (raw + 1023u) & ~1023u;
@@ -410,7 +410,7 @@ probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param
                      v_k = make_smem_desc(base + kPtV), v_mn = make_smem_desc_mn(base + kPtV, kPtTerm),
                      dl_k = make_smem_desc(base + kPtDelta), dl_mn = make_smem_desc_mn(base + kPtDelta, kPtTerm);
       constexpr uint32_t mat = kPtMat >> 4, term = kPtTerm >> 4;      // descriptor addresses count 16 bytes
-      for (size_t grp = blockIdx.x; grp < ngroups && ok; grp += gridDim.x)
+      for (size_t grp = blockIdx.x; grp < stop && ok; grp += gridDim.x)
         for (int unit = 0; unit < K_all && ok; unit += g, ++tile) {   // (a segment is a whole number of tiles)
           const uint32_t ph = tile & 1u;
           const bool fresh = unit % kPtSegment == 0;
@@ -448,6 +448,8 @@ probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param
                 }
           tc_commit(bar_v);
         }
+      if (!ok)                                                        // let the products in flight end
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);
     }
   } else {
     // ------------------------------------------------ sixteen worker warps
@@ -455,7 +457,8 @@ probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param
     const float step = law == 1 ? 2.f * param : param;
     const uint32_t c3 = kq.c3 & ~0xFFu;
     const float inv_param = 1.f / param;
-    for (size_t it = (size_t)blockIdx.x * nsegs; it < ngroups * nsegs && ok;
+    size_t it = (size_t)blockIdx.x * nsegs;
+    for (; it < stop * nsegs && ok;
          it += (it + 1) % nsegs ? 1 : ((size_t)gridDim.x - 1) * nsegs + 1) {      // group by group, its segments in order
       const size_t row0 = it / nsegs * R;
       const int seg = (int)(it % nsegs), k_seg = seg * kPtSegment, K = K_all - k_seg < kPtSegment ? K_all - k_seg : kPtSegment,
@@ -872,8 +875,17 @@ probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param
       pt_sync();                                                      // the scratch is reused
       tc_fence_after();
     }
-    if (!ok)                                                          // a bounded wait ran out: no sums that look valid
-      for (size_t i = (size_t)blockIdx.x * kPtWorkers + tid; i < 5 * rows * n; i += (size_t)gridDim.x * kPtWorkers) ds_sum[i] = NAN;
+    // a bounded wait ran out: the sums of this block's rows that are not complete do not look valid
+    for (size_t grp = it / nsegs; grp < ngroups; grp += gridDim.x) {
+      const size_t r0 = grp * R, nr = rows - r0 < (size_t)R ? rows - r0 : (size_t)R;
+      for (int o = 0; o < 5; ++o)
+        for (size_t i = tid; i < nr * n; i += kPtWorkers) {
+          ds_sum[(o * rows + r0) * n + i] = NAN;
+          if (ds_sq) ds_sq[(o * rows + r0) * n + i] = NAN;
+        }
+      for (int o = 0; o < 2; ++o)
+        for (size_t i = tid; i < nr * n * d; i += kPtWorkers) dV_sum[(o * rows + r0) * (size_t)n * d + i] = NAN;
+    }
   }
   tc_fence_before();
   __syncthreads();

@@ -113,6 +113,23 @@ def test_values_that_are_not_finite_stay_with_their_column(b):
     assert np.max(np.abs(dV[..., keep] - want[..., keep])) <= 2e-5 * np.max(np.abs(want))
 
 
+# a bounded wait that runs out cuts a block short: its incomplete rows are NaN in every output, all others are whole
+# (two rows a group and one; more groups than blocks; draws in segments)
+@pytest.mark.parametrize("R,n,d,K,done", [(301, 32, 8, 40, 100), (301, 32, 8, 40, 0), (7, 64, 20, 300, 3), (4, 16, 3, 70, 4)])
+@pytest.mark.parametrize("squares", [True, False])
+def test_rows_cut_short_are_not_numbers(b, R, n, d, K, done, squares):
+    p, V = (torch.from_numpy(x).cuda() for x in _rows(R, n, d, 23))
+    shapes = [(5, R, n), (5, R, n) if squares else None, (2, R, n, d)]
+    want, got = ([None if s is None else torch.zeros(s, device="cuda") for s in shapes] for _ in range(2))
+    b.bsp_probs_mc(p, V, R, n, d, 0, 1.0 / 64, 9, 0, 0, K, *want)
+    b.bsp_selftest_probs_unfinished(p, V, R, n, d, 1.0 / 64, 9, K, done, *got)
+    whole = (done + 1) // 2 * 2 if K <= 64 else done         # a group is two rows up to 64 draws
+    for w, x in zip(want, got):
+        if w is not None:
+            assert torch.equal(x[:, :whole], w[:, :whole]) and torch.isfinite(w).all()
+            assert torch.isnan(x[:, whole:]).all()
+
+
 def test_bench_size_on_sampled_rows(b):
     """The size `bench.py` times (16384 rows of 128 probabilities, d = 64, grid 1/64, 256 draws; rows
     drawn by the same recipe): blocks of rows from the start, the middle and the end of the tensor
