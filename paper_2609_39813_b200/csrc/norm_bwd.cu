@@ -227,12 +227,15 @@ struct GainPlan {
     draws_per_z = (int)((K + nz - 1) / nz);
   }
 };
-// Draws per launch: the partial sums of a launch stay within 64 MiB, at least kMcBlockDraws draws.
+// Draws per launch: the partial sums of a launch stay within 64 MiB, at least kMcBlockDraws draws, and no more
+// than a grid's second dimension holds (gain_mc_slab_reduce_kernel has a row of blocks per draw).
+constexpr int64_t kMcMostDraws = 65535;
 static int gain_chunk(int64_t T, int64_t C, int K) {
   const GainPlan plan(T, C, K);
   const int64_t per = (int64_t)(plan.nslabs > 0 ? plan.nslabs : 1) * C * (int64_t)sizeof(float);
   int64_t fit = ((int64_t)64 << 20) / (per > 0 ? per : 1);
   if (fit < kMcBlockDraws) fit = kMcBlockDraws;
+  if (fit > kMcMostDraws) fit = kMcMostDraws;
   return (int)(fit < K ? fit : K);
 }
 

@@ -309,6 +309,32 @@ def test_weight_gradient_three_reads(b, case, policy):
     assert rel_l2(down(dW).reshape(O, C), want) <= TOL_TC
 
 
+# more draws than a grid's second dimension holds: two calls over the halves of the draws add up to one
+def test_gain_draws_beyond_a_grid_dimension(b):
+    T, C, K = 64, 64, 70000
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(12)
+    x, du = (torch.randn(T, C, generator=gen, device="cuda") for _ in range(2))
+    gamma, ref = torch.ones(C, device="cuda"), torch.zeros(C, device="cuda")
+    rstd, mean, amax, scale = (torch.zeros(n, device="cuda") for n in (T, T, 1, 1))
+    b.bsp_norm_stats(b.RMSNORM, x, T, C, gamma, None, 1e-6, rstd, mean, amax)
+    b.bsp_scale_from_amax(amax, 1, b.E4M3, scale)
+    q = b.quant(b.E4M3, b.ROUND_STOCHASTIC, 1.0, scale)
+    ws = b.workspace(b.bsp_norm_gain_mc_workspace_bytes(T, C, K))
+    sums = []
+    for cuts in ((0, K), (0, K // 2, K)):
+        S1, S2 = torch.zeros(C, device="cuda"), torch.zeros(C, device="cuda")
+        for k0, k1 in zip(cuts, cuts[1:]):
+            b.bsp_norm_gain_mc(b.RMSNORM, x, T, C, gamma, None, rstd, mean, du, q, b.key(9, 1, b.STREAM_GAIN, 0), k0, k1 - k0,
+                               ref, S1, S2, ws)
+        sums.append((S1, S2))
+    # the same terms in FP32, summed in another order: an eighth of K roundings of the sums of magnitudes at most
+    (a1, a2), (b1, b2) = sums
+    tol = K / 8 * 2.0 ** -24
+    assert float((a2 - b2).abs().max()) <= tol * float(b2.max()) and float(b2.min()) > 0
+    assert float((a1 - b1).abs().max()) <= tol * float((K * b2).sqrt().max())
+
+
 # the check may cut a contraction's draws into ranges (few tiles, or a last partial wave of them) and
 # merge the ranges' sums; bsp_linear_wgrad_mc, which has no workspace, walks them in one go
 @pytest.mark.parametrize("T,C,O,K", [(64, 128, 128, 41), (80, 272, 400, 32), (48, 128, 272, 9), (33, 2064, 1168, 20)])
