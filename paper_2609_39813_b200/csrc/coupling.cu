@@ -53,7 +53,7 @@ __device__ __forceinline__ void bf16x4_to_float(const uint2& b, float (&v)[4]) {
 // One forward's rounding: code = round(u scale), uq = decode(code) as bf16 (exact).  uq_a given: also
 // dr[t] = dr[T + t] = uq_a - uq, the first operand of X (twice, to meet both terms of the second; zero or
 // one grid step, exact in bf16).
-// Block (64, 4): 64 groups of four columns by 16 rows.
+// Block (64, 4): 64 groups of four columns by 16 rows; the rows along grid.x, which holds any T.
 constexpr int kCpRows = 16;
 template <int DT, int FMT, bool SR>
 __global__ void __launch_bounds__(256)
@@ -62,7 +62,7 @@ cp_forward_kernel(int kind, const void* x, int64_t T, int64_t C, const float* ga
                   const float* scale_dev, PhiloxKey key, uint16_t* uq,
                   const uint16_t* uq_a, uint16_t* dr, bsp_diag_t* diag) {
   grid_dependency();
-  const int64_t c = 4 * ((int64_t)blockIdx.x * 64 + threadIdx.x);
+  const int64_t c = 4 * ((int64_t)blockIdx.y * 64 + threadIdx.x);
   const float scale = ldg(scale_dev);
   DiagCounters dc;
   if (c < C) {
@@ -71,7 +71,7 @@ cp_forward_kernel(int kind, const void* x, int64_t T, int64_t C, const float* ga
     if (kind == BSP_LAYERNORM) b4 = ldg(reinterpret_cast<const float4*>(beta + c));
 #pragma unroll
     for (int j = 0; j < kCpRows / 4; ++j) {
-      const int64_t t = (int64_t)blockIdx.y * kCpRows + threadIdx.y + 4 * j;
+      const int64_t t = (int64_t)blockIdx.x * kCpRows + threadIdx.y + 4 * j;
       if (t >= T) break;
       const size_t i = (size_t)t * C + c;
       float u[4];
@@ -367,7 +367,7 @@ int bsp_coupling_check(const bsp_coupling_desc_t* op, int pairs, double* T_out, 
 
   bsp_key_t key;
   key.seed = op->seed; key.tensor_id = op->tensor_id; key.reserved = 0;
-  const dim3 gf((unsigned)((C / 4 + 63) / 64), (unsigned)((T + kCpRows - 1) / kCpRows));
+  const dim3 gf((unsigned)((T + kCpRows - 1) / kCpRows), (unsigned)((C / 4 + 63) / 64));
   const dim3 gs((unsigned)((C + 127) / 128), (unsigned)b.nslabs);
 
   auto forward = [&](int draw, int slot) -> int {

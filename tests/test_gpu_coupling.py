@@ -93,6 +93,19 @@ def test_at_the_390m_shape(b):
     assert rel_l2(got["X"], want["X"]) <= 2e-3
 
 
+def test_more_tokens_than_a_grid_dimension_of_row_blocks(b):
+    """T above 65535 blocks of 16 rows, against the oracle on the same draws."""
+    inp = workloads.config4(T=65537 * 16 + 3, C=16, O=16, K=4, seed=26)
+    inp.W = workloads.to_bf16_grid(inp.W)
+    got, rstd, mean = _run(b, inp, 1)
+    prep = coupling.prepare(inp.x, inp.gamma, inp.beta, inp.W, norm.LAYER, inp.eps, rstd32=rstd, mean32=mean)
+    want = coupling.run(prep, inp.seed, 1)
+    assert np.allclose(got["T"], want["T"], rtol=5e-4)
+    assert rel_l2(got["gain_total"], want["gain_total"]) <= 5e-4 and rel_l2(got["gain_fresh"], want["gain_fresh"]) <= 5e-4
+    # X sums 2 T products, sixteen to a tensor-core step that may drop 2^-23 of the sum so far
+    assert rel_l2(got["X"], want["X"]) <= 2 * inp.T / 16 * 2.0 ** -23
+
+
 def test_closed_forms_and_round_to_nearest(b):
     inp = workloads.config2(T=256, C=128, O=128, K=4, seed=23)
     pairs = 200
