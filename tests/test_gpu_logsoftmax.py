@@ -118,3 +118,18 @@ def test_cuts_by_trials_and_row_chunks(b, rows, classes, trials):
     for c in range(8):
         assert abs(stats[c].mean - mean[c]) <= 2e-4 * max(abs(mean[c]), eps * eps)
         assert abs(stats[c].se - se[c]) <= 1e-3 * se[c] + 1e-9
+
+
+# long rows lose nothing to the length of their sums.  A table entry, the difference of two rounded terms some ten times
+# its size, is good to 2e-6 of itself; the statistics, sums of 8192 entries of either sign per row, to a few times that
+@pytest.mark.parametrize("rows,classes,trials", [(16, 8192, 24), (4, 8192, 300)])
+def test_long_rows_keep_their_precision(b, rows, classes, trials):
+    eps = 0.1
+    logits, target = _inputs(rows, classes, 5)
+    pt = torch.zeros(trials * 6, device="cuda")
+    ws = b.workspace(b.bsp_lsm_check_workspace_bytes(rows, classes, trials))
+    b.bsp_lsm_check(torch.from_numpy(logits).cuda(), torch.from_numpy(target).cuda(), rows, classes, eps, trials, 7, ls.TENSOR_S, pt, ws)
+    want, _ = ls.run(logits, target, eps, 7, trials)
+    got = pt.cpu().numpy().reshape(trials, 6).astype(np.float64)
+    for i in range(4):
+        assert np.linalg.norm(got[:, i] - want[:, i]) <= 2e-5 * np.linalg.norm(want[:, i]), i
