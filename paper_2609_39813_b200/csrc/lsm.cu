@@ -125,6 +125,58 @@ lsm_trial_kernel(const float4* table, int rows, int rows_per_chunk, int classes,
     for (int i = 0; i < kLsmStats; ++i) partial[((size_t)blockIdx.y * kLsmStats + i) * trials + trial] = acc[i];
 }
 
+// The same for few trials of few rows, with the classes of a row cut as well: block (x, y) takes range y % nranges of row
+// y / nranges, its threadIdx.y parts of `per` groups each; ranges[y][4][trial] the sums of A, A', B and the count.
+__global__ void __launch_bounds__(kLsmThreads)
+lsm_range_kernel(const float4* table, int nranges, int per, int classes, PhiloxKey key_reuse, PhiloxKey key_copy, int trials,
+                 float* ranges) {
+  grid_dependency();
+  __shared__ float sm[4][kLsmThreads];
+  const int trial = (int)(blockIdx.x * blockDim.x + threadIdx.x), row = (int)blockIdx.y / nranges;
+  const int groups = classes / 4, g0 = ((int)(blockIdx.y % nranges) * (int)blockDim.y + (int)threadIdx.y) * per;
+  float a1, a2, b1;
+  int cnt;
+  lsm_walk(table + (size_t)row * classes + 4 * g0, (uint64_t)row * groups + g0, groups - g0 < per ? groups - g0 : per, key_reuse, key_copy,
+           (uint32_t)trial, a1, a2, b1, cnt);
+  const int at = (int)(threadIdx.y * blockDim.x + threadIdx.x);
+  sm[0][at] = a1; sm[1][at] = a2; sm[2][at] = b1; sm[3][at] = (float)cnt;
+  __syncthreads();
+  if (threadIdx.y == 0 && trial < trials)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float v = 0.f;
+      for (int y = 0; y < (int)blockDim.y; ++y) v += sm[i][y * blockDim.x + threadIdx.x];
+      ranges[((size_t)blockIdx.y * 4 + i) * trials + trial] = v;
+    }
+}
+
+// The ranges of a row together, and its six terms, as lsm_trial_kernel leaves them for a chunk of one row.  Block (x, y):
+// 32 trials of row y, eight threads sharing a trial's ranges.
+__global__ void __launch_bounds__(256)
+lsm_join_kernel(const float* ranges, int nranges, int classes, float eps, int trials, float* partial) {
+  grid_dependency();
+  __shared__ float sm[8][4][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = (int)blockIdx.x * 32 + lane;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  if (t < trials)
+#pragma unroll 4
+    for (int r = w; r < nranges; r += 8)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s[i] += ldg(ranges + (((size_t)blockIdx.y * nranges + r) * 4 + i) * trials + t);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) sm[w][i][lane] = s[i];
+  __syncthreads();
+  if (w != 0 || t >= trials) return;
+#pragma unroll
+  for (int k = 1; k < 8; ++k)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] += sm[k][i][lane];
+  const float sum_r = eps * (2.f * s[3] - (float)classes);            // (the count is below 2^24: exact)
+  const float v[kLsmStats] = {s[0], s[1], -s[0] * sum_r, -s[1] * sum_r, s[2], -s[2] * sum_r};
+#pragma unroll
+  for (int i = 0; i < kLsmStats; ++i) partial[((size_t)blockIdx.y * kLsmStats + i) * trials + t] = v[i];
+}
+
 // Per trial the statistics as means over rows and classes (FP32 out), and per block the sums over its
 // trials: column c < 6 the statistic itself, 6 and 7 the paired contrasts reuse - independent
 // (likelihood, constructed); out[block][2c], [2c + 1] = sum and sum of squares in double.  A block takes
@@ -178,10 +230,15 @@ lsm_collect_kernel(const float* partial, int nchunks, int trials, double inv_n, 
 }
 
 // How a call is cut: blocks of up to 256 trials by chunks of rows, about seven blocks per SM (one wave
-// of the eight that fit) where the rows allow it.
+// of the eight that fit) where the rows allow it.  Where a chunk is one row and that leaves an eighth of the threads or
+// fewer, each row's groups of classes are cut too, into parts of at least 16 groups; a block takes as many parts of a
+// row as make it 256 threads, the rest go over nranges blocks.  Thread per trial and so: 16 x 8192, 64 trials 637 and
+// 70 us; 16 x 512, 256 trials 71 and 47; 16 x 4096, 1024 trials (an eighth and less) 380 and 182; 64 x 512, 1024 (a quarter)
+// 106 and 112.
 struct LsmPlan {
   int threads, tblocks, rows_per_chunk, nchunks, cblocks;
-  LsmPlan(int rows, int trials) {
+  int parts, per, nranges;                                          // nranges 0: classes are not cut
+  LsmPlan(int rows, int classes, int trials) {
     threads = trials >= kLsmThreads ? kLsmThreads : (trials + 31) / 32 * 32;
     tblocks = (trials + threads - 1) / threads;
     int want = (kNumSMs * 7 + tblocks - 1) / tblocks;
@@ -190,7 +247,18 @@ struct LsmPlan {
     nchunks = (rows + rows_per_chunk - 1) / rows_per_chunk;
     cblocks = (trials + 31) / 32;
     if (cblocks > kNumSMs) cblocks = kNumSMs;
+    const int groups = classes / 4;
+    int64_t cuts = (int64_t)kNumSMs * 7 * kLsmThreads / ((int64_t)tblocks * threads * rows);   // of the threads wanted over those there
+    parts = 1; per = groups; nranges = 0;
+    if (rows_per_chunk > 1 || cuts < 8 || groups < 32) return;
+    if (cuts > groups / 16) cuts = groups / 16;
+    parts = kLsmThreads / threads < cuts ? kLsmThreads / threads : (int)cuts;
+    nranges = (int)((cuts + parts - 1) / parts);
+    per = (groups + nranges * parts - 1) / (nranges * parts);
   }
+  // floats: the chunks' terms, and before them the ranges' sums
+  size_t partials(int trials) const { return (size_t)nchunks * kLsmStats * trials; }
+  size_t ranges(int trials) const { return (size_t)nchunks * nranges * 4 * trials; }
 };
 
 }  // namespace bsp
@@ -201,9 +269,9 @@ extern "C" {
 
 size_t bsp_lsm_check_workspace_bytes(int rows, int classes, int trials) {
   if (rows <= 0 || classes <= 0 || trials <= 0) return 0;
-  const LsmPlan plan(rows, trials);
+  const LsmPlan plan(rows, classes, trials);
   return round_up((size_t)rows * classes * sizeof(float4), 256) +
-         round_up((size_t)plan.nchunks * trials * kLsmStats * sizeof(float), 256) +
+         round_up(plan.ranges(trials) * sizeof(float), 256) + round_up(plan.partials(trials) * sizeof(float), 256) +
          round_up((size_t)trials * kLsmStats * sizeof(float), 256) + (size_t)kNumSMs * 2 * kLsmCols * sizeof(double);
 }
 
@@ -217,12 +285,14 @@ int bsp_lsm_check(const float* logits, const int32_t* target, int rows, int clas
     return BSP_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t n = (size_t)rows * classes;
-  const LsmPlan plan(rows, trials);
+  const LsmPlan plan(rows, classes, trials);
   char* base = reinterpret_cast<char*>(ws);
   float4* table = reinterpret_cast<float4*>(base);
   base += round_up(n * sizeof(float4), 256);
+  float* ranges = reinterpret_cast<float*>(base);
+  base += round_up(plan.ranges(trials) * sizeof(float), 256);
   float* partial = reinterpret_cast<float*>(base);
-  base += round_up((size_t)plan.nchunks * trials * kLsmStats * sizeof(float), 256);
+  base += round_up(plan.partials(trials) * sizeof(float), 256);
   float* pt = per_trial ? per_trial : reinterpret_cast<float*>(base);
   base += round_up((size_t)trials * kLsmStats * sizeof(float), 256);
   double* sums = reinterpret_cast<double*>(base);
@@ -233,8 +303,15 @@ int bsp_lsm_check(const float* logits, const int32_t* target, int rows, int clas
   const PhiloxKey kc = make_key(k);
   launch_kernel(lsm_prep_kernel, (unsigned)rows, kLsmThreads, 0, st, logits, classes, eps, table);
   BSP_LAUNCH_CHECK();
-  launch_kernel(lsm_trial_kernel, dim3((unsigned)plan.tblocks, (unsigned)plan.nchunks), plan.threads, 0, st,
-                table, rows, plan.rows_per_chunk, classes, eps, kr, kc, trials, partial);
+  if (plan.nranges) {
+    launch_kernel(lsm_range_kernel, dim3((unsigned)plan.tblocks, (unsigned)(rows * plan.nranges)), dim3(plan.threads, plan.parts), 0, st,
+                  table, plan.nranges, plan.per, classes, kr, kc, trials, ranges);
+    launch_kernel(lsm_join_kernel, dim3((unsigned)((trials + 31) / 32), (unsigned)rows), 256, 0, st, ranges, plan.nranges, classes, eps,
+                  trials, partial);
+  } else {
+    launch_kernel(lsm_trial_kernel, dim3((unsigned)plan.tblocks, (unsigned)plan.nchunks), plan.threads, 0, st,
+                  table, rows, plan.rows_per_chunk, classes, eps, kr, kc, trials, partial);
+  }
   BSP_LAUNCH_CHECK();
   launch_kernel(lsm_collect_kernel, (unsigned)plan.cblocks, 256, 0, st, partial, plan.nchunks, trials, 1.0 / ((double)rows * classes), pt, sums);
   BSP_LAUNCH_CHECK();

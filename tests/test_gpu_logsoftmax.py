@@ -103,8 +103,10 @@ def test_argument_errors(b):
         b.bsp_lsm_check(x, y, 6, 8, 0.1, 1 << 20, 0, 3, None, ws)         # workspace too small
 
 
-# one thread per trial: trials that do not fill a warp, a block, two blocks; rows cut into chunks or not
-@pytest.mark.parametrize("rows,classes,trials", [(1, 4, 2), (40, 8, 33), (9, 36, 257), (300, 32, 513)])
+# one thread per trial: trials that do not fill a warp, a block, two blocks; rows cut into chunks or not; classes cut
+# into parts of one block and into ranges over several, the last one short or empty
+@pytest.mark.parametrize("rows,classes,trials", [(1, 4, 2), (40, 8, 33), (9, 36, 257), (300, 32, 513), (16, 8192, 64), (1, 8192, 3),
+                                                (5, 68, 40), (2, 1796, 300), (33, 2052, 130)])
 def test_cuts_by_trials_and_row_chunks(b, rows, classes, trials):
     eps = 0.25
     logits, target = _inputs(rows, classes, 5)
