@@ -232,6 +232,32 @@ __device__ __forceinline__ uint32_t f8_sr_threshold(float v) {
   return __float2uint_rd(f * 4294967296.0f);
 }
 
+// Both halves of a stochastic rounding at once: returns f8_sr_threshold(v); lo = f8_sr_value(v, ~0), the value rounded
+// toward zero, and step = f8_sr_value(v, 0) - lo, what rounding up adds (0 where the threshold is 0).
+template <int FMT>
+__device__ __forceinline__ uint32_t f8_sr_cell(float v, float& lo, float& step) {
+  using F = F8<FMT>;
+  const uint32_t b = __float_as_uint(v), a = b & 0x7FFFFFFFu, s = b & 0x80000000u;
+  if (a >= F::FMAX_BITS) {
+    lo = __uint_as_float(a > 0x7F800000u ? 0x7FC00000u : s | F::FMAX_BITS);
+    step = 0.f;
+    return 0u;
+  }
+  if (a >= F::MINNORM_BITS) {
+    constexpr int d = 23 - F::MB;
+    const uint32_t rem = a & ((1u << d) - 1u);
+    lo = __uint_as_float(b - rem);
+    step = rem ? __uint_as_float(b - rem + (1u << d)) - lo : 0.f;
+    return rem << (32 - d);
+  }
+  const float t = __uint_as_float(a) * __uint_as_float((uint32_t)(F::MB - F::EMIN + 127) << 23);
+  const float n = (float)(uint32_t)t, unit = __uint_as_float((uint32_t)(F::EMIN - F::MB + 127) << 23);
+  const uint32_t thr = __float2uint_rd((t - n) * 4294967296.0f);
+  lo = __uint_as_float(s | __float_as_uint(n * unit));
+  step = thr ? __uint_as_float(s | __float_as_uint(unit)) : 0.f;
+  return thr;
+}
+
 // Nearest-even rounding of two in-range FP32 values (|v| below the format's maximum) to two codes
 // with the hardware conversion: `lo` in bits 0..7, `hi` in bits 8..15.  NaN, infinities and
 // magnitudes at or above the maximum never come here (the callers route those to f8_encode).

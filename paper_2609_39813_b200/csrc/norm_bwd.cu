@@ -239,6 +239,17 @@ static int gain_chunk(int64_t T, int64_t C, int K) {
   return (int)(fit < K ? fit : K);
 }
 
+// Shared memory of a block: the sums of its draws, [draw][kMcCols]; the inputs of a sub-slab, each thread's own four
+// rows of four elements, [row][thread]; and rstd, mean and step of a warp's rows, [warp][3][kMcRows].
+constexpr size_t gain_smem_bytes(int draws, int x_size, int du_size) {
+  return (size_t)draws * kMcCols * sizeof(float) + (size_t)kMcSub * kMcCols * (x_size + du_size) + (size_t)kMcSub * 3 * sizeof(float);
+}
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* smem, const void* global) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(global), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <int DT, int DU_DT, int FMT>
 __global__ void __launch_bounds__(kMcWarps * 32, 2)
 gain_mc_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
@@ -248,9 +259,9 @@ gain_mc_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
                float* partial /* [ndraws][nslabs][C] */, bsp_diag_t* diag) {
   grid_dependency();
   // A fresh rounding of an element is its round-down value plus, with probability frac, one grid
-  // step: value(U) = lo + (U < P) * (hi - lo) with the threshold P of f8_sr_threshold.  So the
-  // gain-use sum of draw k is  sum_t (lo/scale - beta)/gamma * du  (the same for every draw, summed
-  // once) plus  sum_t [U_k,t < P_t] * (hi - lo)/scale/gamma * du : per element and draw one generator
+  // step: value(U) = lo + (U < P) * step with the threshold P of f8_sr_cell.  So the
+  // gain-use sum of draw k is  sum_t (lo/scale - beta) * du  (the same for every draw, summed
+  // once) plus  sum_t [U_k,t < P_t] * step/scale * du,  over gamma: per element and draw one generator
   // word, one comparison and one conditional add.
   // grid_steps != NULL selects the b-bit per-token store instead of the FP8 store: the element sits at
   // t = u / s on the uniform grid of its token's step s, lo = s floor(t), the step weight is s and the
@@ -258,11 +269,17 @@ gain_mc_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
   //
   // Bound by the generator's integer multiplies (the heavy half of the FMA pipe), behind chains of
   // dependent multiplies: two draws of four rows give a thread eight independent chains, with the
-  // thresholds and step weights in registers.  4096 x 1024, 64 draws: 214 us = 1.25 T draws/s (one draw at
-  // a time with both in shared memory, three blocks per SM: 255 us); 64 x 128, 256 draws, which were one
-  // block: 290 -> 9 us.
+  // thresholds and step weights in registers.  What a sub-slab costs besides its draws matters when they are few: its
+  // inputs are copied to shared memory under the draws of the sub-slab before, and gamma divides the
+  // sums, not the elements.  16384 x 4096 bf16: 16 draws 925 us (read where they are needed and divided
+  // each: 1024), 4 draws 352 (464); 4096 x 1024, 64 draws 214 = 1.25 T draws/s (one draw at a time with thresholds and
+  // weights in shared memory, three blocks per SM: 262; 988, 403 at the larger shape); 64 x 128, 256 draws, which were
+  // one block: 290 -> 9.
+  constexpr int NT = kMcWarps * 32, ESX = DT == BSP_F32 ? 4 : 2, ESD = DU_DT == BSP_F32 ? 4 : 2;
   extern __shared__ __align__(16) float mc_sum[];        // [draws of this block][kMcCols]
-  constexpr int NT = kMcWarps * 32;
+  char* x_s = reinterpret_cast<char*>(mc_sum + draws_per_z * kMcCols);
+  char* du_s = x_s + (size_t)kMcSub * kMcCols * ESX;
+  float* row_s = reinterpret_cast<float*>(du_s + (size_t)kMcSub * kMcCols * ESD);
   __shared__ __align__(16) float red[2][2][kMcWarps][kMcCols];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t c = (int64_t)blockIdx.x * kMcCols + lane * 4;
@@ -271,7 +288,26 @@ gain_mc_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
   const float inv_scale = __fdiv_rn(1.0f, scale);
   const bool col_ok = c < C;
   const int k0 = (int)blockIdx.z * draws_per_z, kend = k0 + draws_per_z < ndraws ? k0 + draws_per_z : ndraws, nd = kend - k0;
+  row_s += warp * 3 * kMcRows;
 
+  // the inputs of sub-slab `sub`: a thread copies what it will read, a warp's first lanes the values of its rows
+  auto fetch = [&](int sub) {
+    const int64_t row0 = (slab * subs + sub) * kMcSub + warp;
+#pragma unroll
+    for (int i = 0; i < kMcRows; ++i) {
+      const int64_t r = row0 + kMcWarps * i;
+      if (r < T && col_ok) {
+        const size_t i0 = (size_t)r * C + c;
+        copy_async<4 * ESX>(x_s + (i * NT + tid) * 4 * ESX, reinterpret_cast<const char*>(x) + i0 * ESX);
+        copy_async<4 * ESD>(du_s + (i * NT + tid) * 4 * ESD, reinterpret_cast<const char*>(du) + i0 * ESD);
+      }
+    }
+    const int which = lane / kMcRows;
+    const int64_t r = row0 + kMcWarps * (lane % kMcRows);
+    const float* src = which == 0 ? rstd : which == 1 && kind == BSP_LAYERNORM ? mean : which == 2 ? grid_steps : nullptr;
+    if (src && r < T) copy_async<4>(row_s + lane, src + r);
+  };
+  fetch(0);
   float4 g4 = make_float4(1.f, 1.f, 1.f, 1.f), b4 = make_float4(0.f, 0.f, 0.f, 0.f);
   if (col_ok) {
     g4 = ldg(reinterpret_cast<const float4*>(gamma + c));
@@ -289,17 +325,18 @@ gain_mc_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
     const uint64_t q0 = (uint64_t)(row0 * C + (col_ok ? c : 0)) >> 2, qstep = (uint64_t)(kMcWarps * C) / 4;
     uint32_t thr[kMcRows][4];
     float wgt[kMcRows][4], base[4] = {0.f, 0.f, 0.f, 0.f};   // base: the draw-independent part of this thread's sums
+    copy_async_wait();
+    __syncwarp();
 #pragma unroll
     for (int i = 0; i < kMcRows; ++i) {
       const int64_t r = row0 + kMcWarps * i;
 #pragma unroll
       for (int e = 0; e < 4; ++e) { thr[i][e] = 0u; wgt[i][e] = 0.f; }
       if (r < T && col_ok) {
-        const size_t i0 = (size_t)r * C + c;
-        const float4 xv = load4<DT>(x, i0);
-        const float4 dv = load4<DU_DT>(du, i0);
-        const float rs = ldg(rstd + r);
-        const float mu = kind == BSP_LAYERNORM ? ldg(mean + r) : 0.f;
+        const float4 xv = load4<DT>(x_s, 4 * (i * NT + tid));
+        const float4 dv = load4<DU_DT>(du_s, 4 * (i * NT + tid));
+        const float rs = row_s[i];
+        const float mu = kind == BSP_LAYERNORM ? row_s[kMcRows + i] : 0.f;
         const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
         const float ds[4] = {dv.x, dv.y, dv.z, dv.w};
 #pragma unroll
@@ -307,25 +344,25 @@ gain_mc_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
           float u;
           if (kind == BSP_RMSNORM) u = __fmul_rn(__fmul_rn(xs[e], rs), gg[e]);
           else u = __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(xs[e], mu), rs), gg[e]), bb[e]);
-          const float w = __fdiv_rn(ds[e], gg[e]);
           if (blockIdx.z == 0 && (!isfinite(xs[e]) || !isfinite(ds[e]))) dc.nonfinite++;
+          float lo, step;                                // (NaN has threshold 0: it stays in base)
           if (grid_steps) {
-            const float st = ldg(grid_steps + r);
+            const float st = row_s[2 * kMcRows + i];
             const float t = __fdiv_rn(u, st);
             const float n0 = floorf(t);
             thr[i][e] = __float2uint_rd(__fsub_rn(t, n0) * 4294967296.0f);
-            base[e] = fmaf(fmaf(st, n0, -bb[e]), w, base[e]);
-            wgt[i][e] = thr[i][e] ? st * w : 0.f;
+            base[e] = fmaf(fmaf(st, n0, -bb[e]), ds[e], base[e]);
+            wgt[i][e] = thr[i][e] ? st * ds[e] : 0.f;
             continue;
           }
-          const float v = __fmul_rn(u, scale);
-          const float lo = sr_value<FMT>(v, 0xFFFFFFFFu), hi = sr_value<FMT>(v, 0u);   // never up / up whenever possible
-          thr[i][e] = f8_sr_threshold<FMT>(v);
-          base[e] = fmaf(fmaf(lo, inv_scale, -bb[e]), w, base[e]);
-          wgt[i][e] = thr[i][e] ? (hi - lo) * inv_scale * w : 0.f;    // (NaN has threshold 0: it stays in base)
+          thr[i][e] = f8_sr_cell<FMT>(__fmul_rn(u, scale), lo, step);
+          base[e] = fmaf(fmaf(lo, inv_scale, -bb[e]), ds[e], base[e]);
+          wgt[i][e] = thr[i][e] ? step * inv_scale * ds[e] : 0.f;
         }
       }
     }
+    __syncwarp();                                        // every lane has read the rows' values
+    if (sub + 1 < subs) fetch(sub + 1);
     for (int k = 0; k < nd; k += 2) {                    // an odd count ends with a draw nobody stores
       float acc[2][4];
 #pragma unroll
@@ -361,7 +398,7 @@ gain_mc_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
   diag_flush_warp(diag, dc);                             // (the host hands diag to the first chunk of draws only)
   for (int k = tid / kMcCols; k < nd; k += 2) {
     const int64_t cc = (int64_t)blockIdx.x * kMcCols + tid % kMcCols;
-    if (cc < C) partial[((size_t)(k0 + k) * nslabs + slab) * C + cc] = mc_sum[k * kMcCols + tid % kMcCols];
+    if (cc < C) partial[((size_t)(k0 + k) * nslabs + slab) * C + cc] = __fdiv_rn(mc_sum[k * kMcCols + tid % kMcCols], ldg(gamma + cc));
   }
 }
 
@@ -573,12 +610,12 @@ int norm_gain_mc_run(int kind, const void* x, int dt, int64_t T, int64_t C, cons
     const int per_z = plan.draws_per_z < nd ? plan.draws_per_z : nd;
     if (nslabs > 0) {
       dim3 grid((unsigned)((C + kMcCols - 1) / kMcCols), (unsigned)nslabs, (unsigned)((nd + per_z - 1) / per_z));
-      const size_t smem = (size_t)per_z * kMcCols * sizeof(float);
 #define BSP_GM(DT, DU, FMT)                                                                                     \
   do {                                                                                                          \
+    constexpr int esx = DT == BSP_F32 ? 4 : 2, esd = DU == BSP_F32 ? 4 : 2;                                     \
     BSP_CHECK_CUDA(cudaFuncSetAttribute(gain_mc_kernel<DT, DU, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                        (int)(kMcBlockDraws * kMcCols * sizeof(float))));                       \
-    launch_kernel(gain_mc_kernel<DT, DU, FMT>, grid, kMcWarps * 32, smem, st, kind, x, T, C, gamma, beta, rstd, mean, du,  \
+                                        (int)gain_smem_bytes(kMcBlockDraws, esx, esd)));                        \
+    launch_kernel(gain_mc_kernel<DT, DU, FMT>, grid, kMcWarps * 32, gain_smem_bytes(per_z, esx, esd), st, kind, x, T, C, gamma, beta, rstd, mean, du,  \
                                                                  q.scale, q.scale_dev, grid_steps, pk,           \
                                                                  draw0 + kb, nd, per_z, plan.subs, partial,      \
                                                                  kb == 0 ? diag : nullptr);                      \

@@ -309,6 +309,37 @@ def test_weight_gradient_three_reads(b, case, policy):
     assert rel_l2(down(dW).reshape(O, C), want) <= TOL_TC
 
 
+# slabs of two sub-slabs (the second one's inputs copied under the first one's draws), a ragged last one, every pair of
+# types of x and du, LayerNorm: the values of a row (rstd, mean) and of a column (gamma, beta) both enter
+@pytest.mark.parametrize("x_type", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("du_type", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("fmt", ["E4M3", "E5M2"])
+def test_gain_draws_of_a_layernorm_over_sub_slabs(b, x_type, du_type, fmt):
+    T, C, K = 3610, 4096, 3
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(31)
+    x = (torch.randn(T, C, generator=gen, device="cuda") * torch.exp2(torch.randint(-3, 4, (T, 1), generator=gen, device="cuda"))).to(x_type)
+    du = torch.randn(T, C, generator=gen, device="cuda").to(du_type)
+    gamma = 1.0 + 0.3 * torch.randn(C, generator=gen, device="cuda")
+    beta = 0.1 * torch.randn(C, generator=gen, device="cuda")
+    rstd, mean, amax, scale = (torch.zeros(n, device="cuda") for n in (T, T, 1, 1))
+    f = getattr(b, fmt)
+    b.bsp_norm_stats(b.LAYERNORM, x, T, C, gamma, beta, 1e-5, rstd, mean, amax)
+    b.bsp_scale_from_amax(amax, 1, f, scale)
+    q = b.quant(f, b.ROUND_STOCHASTIC, 1.0, scale)
+    one, db, ref = (torch.zeros(C, device="cuda") for _ in range(3))
+    ws = b.workspace(b.bsp_norm_bwd_workspace_bytes(T, C))
+    want = torch.zeros(C, dtype=torch.float64)
+    for k in range(K):
+        b.bsp_norm_bwd(b.LAYERNORM, x, T, C, gamma, beta, rstd, mean, du, 2, None, q, b.key(9, 1, b.STREAM_GAIN, 5 + k), one, db, None, ws)
+        want += one.double().cpu()
+    S1, S2 = torch.zeros(C, device="cuda"), torch.zeros(C, device="cuda")
+    ws = b.workspace(b.bsp_norm_gain_mc_workspace_bytes(T, C, K))
+    b.bsp_norm_gain_mc(b.LAYERNORM, x, T, C, gamma, beta, rstd, mean, du, q, b.key(9, 1, b.STREAM_GAIN, 0), 5, K, ref, S1, S2, ws)
+    # both are FP32 sums over the tokens of terms (value - beta) du / gamma
+    assert rel_l2(down(S1), want.numpy()) <= TOL_FP32 * 4
+
+
 # more draws than a grid's second dimension holds: two calls over the halves of the draws add up to one
 def test_gain_draws_beyond_a_grid_dimension(b):
     T, C, K = 64, 64, 70000

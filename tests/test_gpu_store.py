@@ -184,3 +184,24 @@ def test_mc_check_store_at_the_390m_shape(b):
     b.bsp_store_wgrad(T, O, C, g.dy_codes_t, g.q_dy, split, g.ld_t, dW, wsw)
     want = prep["dy"]["value"].T @ store.copy_for(prep, 3, inp.seed, philox.STREAM_WGRAD, 5, cols)
     assert rel_l2(down(dW).reshape(O, C)[:, cols], want) <= 1e-4
+
+
+def test_gain_use_over_sub_slabs(b):
+    """Slabs of two sub-slabs of rows, each with its own steps, the last one ragged: the fresh read's statistics against
+    the oracle on the same draws."""
+    inp = workloads.config4(T=3610, C=4096, O=16, K=4)
+    g = NormLinearGpu(inp)
+    K, bits = 4, 6
+    d = _desc(b, g, inp, bits, mask=0x04)
+    ws = b.workspace(b.bsp_mc_check_store_workspace_bytes(d, K))
+    diag = b.new_diag()
+    res = b.bsp_mc_check_store(d, K, ws, diag)
+    assert len(res) == 1 and b.read_diag(diag)["status"] == 0
+    du = torch.zeros(inp.T * inp.C, device="cuda")
+    wsd = b.workspace(b.bsp_linear_dgrad_workspace_bytes(inp.T, inp.O, inp.C))
+    b.bsp_linear_dgrad(inp.T, inp.O, inp.C, g.dy_codes, g.q_dy, g.W, du, wsd)
+    prep = store.prepare(inp.x, inp.gamma, inp.beta, inp.W, inp.dY, norm.LAYER, inp.eps, inp.seed, bits, inp.dtype,
+                         rstd32=down(g.rstd), mean32=down(g.mean), du=down(du).reshape(inp.T, inp.C).astype(np.float64))
+    want = store.gain_use(inp.x, inp.gamma, inp.beta, norm.LAYER, inp.eps, prep, 2, K, inp.seed)["stats"]
+    for f in ("rel_l2_mean_err", "R"):
+        assert np.isclose(getattr(res[0], f), getattr(want, f), rtol=5e-3), (res[0].as_dict(), want, f)
