@@ -1120,7 +1120,7 @@ int bsp_linear_dgrad(int64_t T, int64_t O, int64_t C, const uint8_t* dy_codes, b
   if (!ws || ws_bytes < bsp_linear_dgrad_workspace_bytes(T, O, C) || (reinterpret_cast<uintptr_t>(ws) & 255u))
     return BSP_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
-  uint16_t* dyb = reinterpret_cast<uint16_t*>(ws);
+  uint16_t* dyb = reinterpret_cast<uint16_t*>(ws);             // (bsp_mc_check reads it here afterwards)
   uint16_t* wt = reinterpret_cast<uint16_t*>(reinterpret_cast<char*>(ws) + round_up((size_t)T * O * 2, 256));
   const size_t n16 = (size_t)T * O / 16;
   if (q_dy.fmt == BSP_E5M2)

@@ -309,6 +309,30 @@ def test_weight_gradient_three_reads(b, case, policy):
     assert rel_l2(down(dW).reshape(O, C), want) <= TOL_TC
 
 
+# the check's weight gradient under the original is the single operator's, though it takes dY's decoded codes from the
+# product before: ragged token counts, one and several tiles a side
+@pytest.mark.parametrize("T,C,O", [(64, 128, 128), (77, 144, 272), (301, 528, 1040), (1, 16, 16)])
+@pytest.mark.parametrize("make", [workloads.config2, workloads.config4])
+def test_check_original_read_of_the_weight_use(b, make, T, C, O):
+    inp = make(T=T, C=C, O=O, K=4, seed=13)
+    g = NormLinearGpu(inp)
+    desc = g.desc(0x08)
+    ws = b.workspace(b.bsp_mc_check_workspace_bytes(desc, 4))
+    diag = b.new_diag()
+    b.bsp_mc_check(desc, 4, ws, diag)
+    assert b.read_diag(diag)["status"] == 0
+    got = b.ws_view(ws, b.bsp_mc_check_layout(desc, 4).dW_S1, O * C).clone()
+    u_t = torch.zeros(C * g.ld_t, dtype=torch.bfloat16, device="cuda")
+    q = g.q
+    b.bsp_norm_fwd(g.kind, g.x, T, C, g.gamma, g.beta, g.rstd, g.mean, q, b.key(inp.seed, g.tensor_id, b.STREAM_FORWARD, 0),
+                   None, None, g.ld_t, None, u_t)
+    want = torch.zeros(O * C, device="cuda")
+    wsw = b.workspace(b.bsp_linear_wgrad_workspace_bytes(T, O, C, b.READ_ORIGINAL))
+    b.bsp_linear_wgrad(T, O, C, g.dy_codes_t, g.q_dy, b.READ_ORIGINAL, u_t, q, g.ld_t, want, ws=wsw, diag=diag)
+    # the same products of the same values, summed in FP32 over the tokens
+    assert rel_l2(down(got), down(want)) <= 1e-6 and float(want.abs().max()) > 0
+
+
 # slabs of two sub-slabs (the second one's inputs copied under the first one's draws), a ragged last one, every pair of
 # types of x and du, LayerNorm: the values of a row (rstd, mean) and of a column (gamma, beta) both enter
 @pytest.mark.parametrize("x_type", [torch.float32, torch.bfloat16])
