@@ -398,17 +398,18 @@ probs_mc_128x64_kernel(const float* p_all, const float* V, int law, float param,
   }
 }
 
-// The rows from `stop` on (rounded up to a block's group of rows) are left as after a wait that ran out.
+// few: in the FP32 form, a block per row.  The rows from `stop` on (rounded up to a block's group of rows) are left as
+// after a wait that ran out.
 static int probs_tc_run(const float* p, const float* V, int64_t rows, int n, int d, int law, float param, PhiloxKey kq, int draw0,
-                        int K, float* ds_sum, float* ds_sq, float* dV_sum, int64_t stop, cudaStream_t st) {
+                        int K, float* ds_sum, float* ds_sq, float* dV_sum, bool few, int64_t stop, cudaStream_t st) {
   int dev = 0, nsm = kNumSMs;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int g = K <= 64 ? 64 : 128, R = kPtSlots / g;           // slots per row: two rows' draws share a tile up to 64
-  const int64_t ngroups = (rows + R - 1) / R;
+  const int64_t ngroups = few ? rows : (rows + R - 1) / R;
   auto kern = law == 1 ? probs_mc_tc_kernel<1> : probs_mc_tc_kernel<0>;
   BSP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPtSmemBytes));
   launch_kernel(kern, (unsigned)(ngroups < nsm ? ngroups : nsm), kPtThreads, kPtSmemBytes, st, p, V, n, d, param, kq, draw0, K, g,
-                ds_sum, ds_sq, dV_sum, (size_t)rows, (size_t)((stop + R - 1) / R));
+                ds_sum, ds_sq, dV_sum, (size_t)rows, few, (size_t)((stop + R - 1) / R));
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
@@ -427,7 +428,7 @@ int bsp_selftest_probs_unfinished(const float* p, const float* V, int64_t rows, 
   if (!aligned16(dV_sum)) return BSP_ERR_ALIGN;
   bsp_key_t k;
   k.seed = seed; k.tensor_id = 0; k.stream = 0; k.draw = 0; k.reserved = 0;
-  return probs_tc_run(p, V, rows, n, d, 0, param, make_key(k), 0, K, ds_sum, ds_sq, dV_sum, done, (cudaStream_t)stream);
+  return probs_tc_run(p, V, rows, n, d, 0, param, make_key(k), 0, K, ds_sum, ds_sq, dV_sum, false, done, (cudaStream_t)stream);
 }
 
 int bsp_probs_mc(const float* p, const float* V, int64_t rows, int n, int d, int law, float param, uint64_t seed,
@@ -442,12 +443,18 @@ int bsp_probs_mc(const float* p, const float* V, int64_t rows, int n, int d, int
   k.stream = 0; const PhiloxKey kq = make_key(k);
   k.stream = 1; const PhiloxKey ka = make_key(k);
   k.stream = 2; const PhiloxKey kb = make_key(k);
-  // The tensor-core kernel's tile costs the same whatever part of its 128 slots is drawn, which the kernels below
-  // undercut for few draws: 4096 rows of 128 x 64, 8 draws 348 us here and 350 there, 16 draws 455 and 350; of
-  // 64 x 64, 8 draws 336 and 322; of 32 x 32, 24 draws 261 and 298, 32 draws 329 and 299; of 16 x 16 likewise.  It
-  // wants whole generator blocks per row and 16-byte stores of the gradient rows.
+  // Which kernel, by what was measured over 64 to 4096 rows, in us: probs_mc_kernel (128 x 64: probs_mc_128x64_kernel), the
+  // tensor-core form and the same kernel's FP32 form.  The tensor-core form's tile costs the same whatever part
+  // of its 128 slots is drawn and whatever d, the FP32 form costs a pass of all its warps for sixteen draws.  4096 rows:
+  //   64 x 8,   8 draws 144, 266, 122;  16 draws 266, 268, 166;  24 draws 387, 270, 254;  32 draws 508, 272, 298
+  //   128 x 64, 8 draws 334, 336, 316;  12 draws 399, 337, 353;  100 x 64, 12 draws 919, 326, 312;  16 draws 1140, 327, 359
+  //   16 x 8,   4 draws 44, 260, 85;    24 draws 206, 264, 203;  32 draws 270, 266, 240;  48 draws 399, 306, 343
+  //   32 x 32,  24 draws 250, 273, 285; 32 draws 319, 275, 336
+  // (1024 rows of 16 x 8, 32 draws: 70, 83, 65.)  Both want whole generator blocks per row and 16-byte stores of the
+  // gradient rows.
+  const bool few = n >= 64 ? K <= 16 && (int64_t)K * n * d <= 80000 : K <= 32 && n * d <= 512;
   if (n <= kPtN && n % 4 == 0 && K >= (n >= 64 ? 8 : 32) && (d % 4 != 0 || aligned16(dV_sum)))
-    return probs_tc_run(p, V, rows, n, d, law, param, kq, draw0, K, ds_sum, ds_sq, dV_sum, rows, (cudaStream_t)stream);
+    return probs_tc_run(p, V, rows, n, d, law, param, kq, draw0, K, ds_sum, ds_sq, dV_sum, few, rows, (cudaStream_t)stream);
   if (n == kPfN && d == kPfD && (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (reinterpret_cast<uintptr_t>(dV_sum) & 15u) == 0) {
     const size_t smem_f = kPfSmemFloats * sizeof(float);
     BSP_CHECK_CUDA(cudaFuncSetAttribute(probs_mc_128x64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f));

@@ -164,8 +164,8 @@ __device__ __forceinline__ void pt_arrive(uint32_t bar, int lane) {
   if (lane == 0) mbar_arrive(bar);
 }
 
-// The sums in FP32 on the CUDA cores, for a V that terms of fixed position do not hold (probs_wide).  The whole
-// block; sixteen draws of a row at a time.  Phase 1, a warp per draw: a lane owns four consecutive entries, one
+// The sums in FP32 on the CUDA cores, for few draws (probs.cu) and for a V that terms of fixed position do not hold
+// (probs_wide).  The whole block; sixteen draws of a row at a time.  Phase 1, a warp per draw: a lane owns four consecutive entries, one
 // generator block per stream; h = V^T p_q with the lane owning two columns, dp = V h from a transposed copy of V;
 // the dot products are warp sums.  Phase 2, a thread per entry and quarter of the columns: adds the draws to its
 // sums.  4096 rows, 32 draws: 128 x 64 662 us (probs_mc_128x64_kernel 663), 64 x 64 523 (probs_mc_kernel 771), 100 x 16
@@ -333,7 +333,8 @@ template <int law>
 __global__ void __launch_bounds__(kPtThreads, 1)
 probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param,
                    PhiloxKey kq, int draw0, int K_all, int g /* slots per row: 64 or 128 */, float* ds_sum,
-                   float* ds_sq, float* dV_sum, size_t rows, size_t stop /* groups from here on are left undone (self-test) */) {
+                   float* ds_sq, float* dV_sum, size_t rows, bool few /* draws: the FP32 form */,
+                   size_t stop /* groups from here on are left undone (self-test) */) {
   grid_dependency();
   extern __shared__ uint8_t pt_raw[];
   const uint32_t raw = smem_u32(pt_raw), base = (raw + 1023u) & ~1023u;
@@ -355,6 +356,10 @@ probs_mc_tc_kernel(const float* p_all, const float* V, int n, int d, float param
   double* sumlo_s = reinterpret_cast<double*>(sm + kPtBar + 64);      // [2]: sum of lo - 1
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, wq = w & 3, wg = w >> 2;
 
+  if (few) {
+    probs_fp32_rows<law>(reinterpret_cast<float*>(sm), p_all, V, n, d, param, kq, draw0, K_all, ds_sum, ds_sq, dV_sum, rows);
+    return;
+  }
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) mbar_init(bar_go + 8 * i, kPtWorkers / 32);
     mbar_init(bar_h, 1); mbar_init(bar_d, 1); mbar_init(bar_v, 1);

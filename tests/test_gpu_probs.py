@@ -82,6 +82,23 @@ def test_tensor_core_form_matches_the_oracle(b, R, n, d, law, param, K):
         assert np.max(np.abs(dV[i] - want_dV[i])) <= 2e-5 * f * (np.max(np.abs(want_dV[i])) + 1e-30), i
 
 
+# the FP32 form of the same kernel, which takes few draws: a pass of sixteen draws partly filled and full, two passes,
+# entries and columns that fill a warp's or a thread's share partly, more rows than blocks
+@pytest.mark.parametrize("R,n,d,law,param,K", [
+    (3, 128, 64, 0, 1.0 / 64, 8), (2, 128, 64, 1, 1.0 / 512, 9), (301, 68, 9, 0, 1.0 / 64, 15), (5, 64, 63, 1, 1.0 / 256, 16),
+    (160, 20, 16, 0, 1.0 / 32, 32), (3, 4, 4, 1, 1.0 / 64, 32), (7, 36, 1, 0, 0.125, 32)])
+def test_few_draws_match_the_oracle(b, R, n, d, law, param, K):
+    p, V = _rows(R, n, d, 9 + n)
+    ds, sq, dV = _run(b, p, V, law, param, 45, 1, K)
+    want_ds, want_sq, want_dV = probs.mc_sums(p, V, law, param, 45, K, 1)
+    f = max(1.0, np.sqrt(K / 9))                             # as above
+    for i in range(5):
+        assert np.max(np.abs(ds[i] - want_ds[i])) <= 2e-5 * f * (np.max(np.abs(want_ds[i])) + 1e-30), i
+        assert np.max(np.abs(sq[i] - want_sq[i])) <= 1e-4 * (np.max(np.abs(want_sq[i])) + 1e-30), i
+    for i in range(2):
+        assert np.max(np.abs(dV[i] - want_dV[i])) <= 2e-5 * f * (np.max(np.abs(want_dV[i])) + 1e-30), i
+
+
 # rows of V that differ widely in size, the large ones unlikely or the likely one small: the errors stay FP32's own.
 # Both sides of the line between the two forms of V (rows within a sixteenth of each other), both tile cuts, the
 # kernel of its own, and more rows than blocks.
