@@ -391,15 +391,23 @@ def test_gain_draws_beyond_a_grid_dimension(b):
 
 
 # the check may cut a contraction's draws into ranges (few tiles, or a last partial wave of them) and
-# merge the ranges' sums; bsp_linear_wgrad_mc, which has no workspace, walks them in one go
-@pytest.mark.parametrize("T,C,O,K", [(64, 128, 128, 41), (80, 272, 400, 32), (48, 128, 272, 9), (33, 2064, 1168, 20)])
+# merge the ranges' sums; bsp_linear_wgrad_mc, which has no workspace, walks them in one go.  An odd count of draws, an even
+# count of tile rows (pairs of CTAs), an odd one below nine (single CTAs) and of nine (pairs, the last one's second CTA
+# beyond the output)
+@pytest.mark.parametrize("T,C,O,K", [(64, 128, 128, 41), (80, 272, 400, 32), (48, 128, 272, 17), (33, 2064, 1168, 20), (80, 144, 1152, 33),
+                                     (80, 144, 1104, 32)])
 def test_split_draws_equal_one_walk(b, T, C, O, K):
     inp = workloads.config1(T=T, C=C, O=O, K=K, seed=6)
     g = NormLinearGpu(inp)
     desc = g.desc(0x30)                                  # weight use: the forward's read and fresh reads
-    ws = b.workspace(b.bsp_mc_check_workspace_bytes(desc, K))
     diag = b.new_diag()
-    b.bsp_mc_check(desc, K, ws, diag)
+    launches = []
+    for draws in (4, K):                                 # four draws, two pairs, are never split
+        ws = b.workspace(b.bsp_mc_check_workspace_bytes(desc, draws))
+        before = b.bsp_launch_count()
+        b.bsp_mc_check(desc, draws, ws, diag)
+        launches.append(b.bsp_launch_count() - before)
+    assert launches[1] == launches[0] + 1                # the merge
     assert b.read_diag(diag)["status"] == 0
     lay = b.bsp_mc_check_layout(desc, K)
     ref, S1, S2 = (b.ws_view(ws, off, O * C).clone() for off in (lay.dW_ref, lay.dW_S1, lay.dW_S2))

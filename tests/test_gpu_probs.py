@@ -44,9 +44,9 @@ def _run(b, p, V, law, param, seed, draw0, K):
 
 @pytest.mark.parametrize("R,n,d,law,param", [(7, 4, 3, 0, 0.125), (5, 3, 2, 1, 0.125), (33, 48, 16, 0, 1.0 / 64),
                                             (9, 200, 64, 1, 1.0 / 512), (3, 256, 64, 0, 1.0 / 256),
-                                            # 128 x 64 takes the kernel of its own (eight draws at a time: K = 9 leaves one over)
+                                            # nine draws of 128 x 64 take the FP32 form of the tensor-core kernel
                                             (11, 128, 64, 0, 1.0 / 64), (6, 128, 64, 1, 1.0 / 512),
-                                            (600, 128, 64, 0, 1.0 / 64)])       # more blocks than the GPU holds at once
+                                            (600, 128, 64, 0, 1.0 / 64)])       # four rows a block and more
 def test_sums_match_the_oracle_draw_for_draw(b, R, n, d, law, param):
     p, V = _rows(R, n, d, 5 + n)
     K, draw0 = 9, 3
@@ -62,13 +62,27 @@ def test_sums_match_the_oracle_draw_for_draw(b, R, n, d, law, param):
         assert np.max(np.abs(dV[i] - want_dV[i])) <= 2e-5 * scale
 
 
-# the tensor-core form (16 draws up, whole generator blocks per row): both cuts of a tile (up to 64 draws two
+# fewer than eight draws of 128 x 64 have a kernel of their own, a warp per draw: one warp, some, all but one; more blocks than
+# the GPU holds at once
+@pytest.mark.parametrize("R,law,param,K", [(11, 0, 1.0 / 64, 1), (6, 1, 1.0 / 512, 5), (600, 0, 1.0 / 64, 7)])
+def test_128x64_kernel_matches_the_oracle(b, R, law, param, K):
+    p, V = _rows(R, 128, 64, 6 + K)
+    ds, sq, dV = _run(b, p, V, law, param, 49, 2, K)
+    want_ds, want_sq, want_dV = probs.mc_sums(p, V, law, param, 49, K, 2)
+    for i in range(5):
+        assert np.max(np.abs(ds[i] - want_ds[i])) <= 2e-5 * (np.max(np.abs(want_ds[i])) + 1e-30), i
+        assert np.max(np.abs(sq[i] - want_sq[i])) <= 1e-4 * (np.max(np.abs(want_sq[i])) + 1e-30), i
+    for i in range(2):
+        assert np.max(np.abs(dV[i] - want_dV[i])) <= 2e-5 * (np.max(np.abs(want_dV[i])) + 1e-30), i
+
+
+# the tensor-core form (more draws than the FP32 form takes, whole generator blocks per row): both cuts of a tile (up to 64 draws two
 # rows share one), partly filled tiles and slot groups, draws beyond a segment of 256, entries and columns
 # that are not whole products, an odd row count, more groups than SMs
 @pytest.mark.parametrize("R,n,d,law,param,K", [
     (3, 128, 64, 0, 1.0 / 64, 16), (3, 128, 64, 1, 1.0 / 512, 64), (2, 128, 64, 0, 1.0 / 64, 65),
-    (1, 128, 64, 0, 1.0 / 128, 257), (5, 4, 1, 0, 0.125, 31), (4, 16, 3, 1, 1.0 / 64, 33), (3, 36, 33, 0, 1.0 / 64, 129),
-    (2, 124, 62, 0, 1.0 / 128, 100), (301, 20, 16, 0, 1.0 / 32, 17), (2, 100, 64, 1, 1.0 / 256, 128)])
+    (1, 128, 64, 0, 1.0 / 128, 257), (5, 4, 1, 0, 0.125, 40), (4, 16, 3, 1, 1.0 / 64, 33), (3, 36, 33, 0, 1.0 / 64, 129),
+    (2, 124, 62, 0, 1.0 / 128, 100), (301, 20, 16, 0, 1.0 / 32, 33), (2, 100, 64, 1, 1.0 / 256, 128)])
 def test_tensor_core_form_matches_the_oracle(b, R, n, d, law, param, K):
     p, V = _rows(R, n, d, 7 + n)
     ds, sq, dV = _run(b, p, V, law, param, 43, 2, K)
