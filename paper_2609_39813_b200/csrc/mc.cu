@@ -488,7 +488,7 @@ int bsp_mc_check(const bsp_norm_linear_desc_t* op, int K, const bsp_verdict_rule
       key.stream = BSP_STREAM_WGRAD;
       // draws in chunks: one re-rounding launch writes the chunk's code matrices, one contraction
       // launch walks them with the running sums in registers (the first chunk's start there: clearing S1 and
-      // S2 and reading the zeros back was 0.3 of 16.4 ms at 16384 x 4096 x 11008, 5 of 167 us at the smallest)
+      // S2 and reading the zeros back was 65 us of memsets at 16384 x 4096 x 11008, 5 of 167 us at the smallest)
       const int chunk = draw_chunk(C, b.ld_t, K, op->draw_buffer_bytes);
       key.draw = 0;
       for (int k0 = 0; k0 < K; k0 += chunk) {
