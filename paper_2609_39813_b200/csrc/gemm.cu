@@ -357,7 +357,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 // PAIR: two CTAs of a cluster take two tile rows of the same columns as one product over 256 rows
 // (cta_group::2): each loads its own A rows and one of the two draws' B tiles, 32 KB per 128 bytes of K
 // instead of 48, which is what L2 has to deliver to every SM (96 bytes per cycle at the tensor rate
-// without pairs, of about 80 it gives with all SMs loading): see mc_pairs for what it measured.  The leader's (rank 0) warp 1
+// without pairs, of about 80 that the times of unpaired products allow; no counter was read): see mc_pairs for what it measured.  The leader's (rank 0) warp 1
 // issues for both; its full barriers count both CTAs' bytes, its commits arrive in both.
 //
 // The walk is over units (tile, range of draws).  Whole waves of tiles take all their draws; the tiles
@@ -744,7 +744,7 @@ static int device_sms() {
 // How a plain contraction is tiled: columns of a tile, 64 .. 256 in steps of 16 (of 32 for a pair of CTAs),
 // and whether pairs take two tile rows together.  The time goes with the number of rounds the tiles take
 // over the SMs times what a tile costs: per 32 bytes of K the product's bn / 2 cycles or, with every SM
-// loading, the 32 bytes of each operand row at the 80 bytes per cycle and SM that L2 was seen to give
+// loading, the 32 bytes of each operand row at the 80 bytes per cycle and SM that fit the times
 // (alone, 256 columns reach 0.83 of the tensor rate, 128 columns 0.6), and the epilogue of the last tile
 // (about 12 cycles a column).  Fewer columns only where they save a twentieth (3001 x 1552 x 4112 bf16, 144 columns: 66 -> 54 us); pairs wherever they
 // cost no more (16384 x 4096 x 11008 bf16: 1070 -> 954 us; 4096 x 1024 x 8192: 63 -> 55).
