@@ -782,9 +782,12 @@ def run_ours(args):
     flops = 2.0 * T * O * C * K               # one launch contracts all K draws
     achieved = flops / (gemm_ms * 1e-3) / 1e12
     peak = 2.0 * peaks["bf16_tflops"]        # FP8 dense = 2 x the measured BF16 burst figure
+    # DRAM bytes of one launch of this kernel at this shape: dram__bytes_read.sum + dram__bytes_write.sum
+    # of one ncu capture of this command (profiles/gemm_mc_kernel_cfg5.md); null for any other shape
+    traffic = GEMM_MC_TRAFFIC.get((T, C, O, K))
     roofline = dict(bound="tensor", kernel="gemm_mc_kernel (FP8 weight gradient over K draws, sums in registers)",
-                    achieved=achieved, peak=peak, unit="TFLOP/s", frac=achieved / peak, traffic=None,
-                    traffic_unit="bytes per launch",
+                    achieved=achieved, peak=peak, unit="TFLOP/s", frac=achieved / peak, traffic=traffic,
+                    traffic_unit="bytes per launch (ncu dram read + write, one capture)",
                     algorithmic_bytes=float(K * C * g.ld_t + O * g.ld_t + 5 * 4 * O * C),
                     us_per_launch=gemm_ms * 1e3, draws_per_launch=K,
                     share_of_step=gemm_ms / (ms_total / args.steps),
@@ -838,6 +841,12 @@ def run_ours(args):
     print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()
+
+
+# DRAM traffic of one gemm_mc_kernel launch by (T, C, O, K), bytes: dram__bytes_read.sum +
+# dram__bytes_write.sum of one ncu capture of `python bench.py --steps 1 --warmup 3 --no-extras
+# --no-cpu-baseline` (profiles/gemm_mc_kernel_cfg5.md)
+GEMM_MC_TRAFFIC = {(16384, 4096, 11008, 16): 8519097600.0 + 367267072.0}
 
 
 def main():
