@@ -18,18 +18,17 @@
 //
 // Per inner step: S = Q K^T and dP = dO V^T (128x128x64 each; the dK/dV mode forms the transposes) land
 // in TMEM columns [0,128) and [128,256); eight softmax warps (two per TMEM lane quarter, 64 columns
-// each) turn them into P and dS and write those back into tensor memory as packed bf16 pairs (FP8-
-// operand mode: as codes), where the accumulating products read them as their A operand, row per
-// lane; the TMA-loaded 128 x 64 tiles are the MN-major B operands.  320 threads: warp 0 TMA, warp 1
-// MMA (the whole warp walks the loop, one elected lane issues), warps 2..9 softmax + epilogue.
-// Head dimension 64, bf16 inputs, FP32 outputs.  Every wait is bounded.
+// each) turn them into P and dS and write those back into tensor memory as packed bf16 pairs, where the
+// accumulating products read them as their A operand, row per lane; the TMA-loaded 128 x 64 tiles are the
+// MN-major B operands.  320 threads: warp 0 TMA, warp 1 MMA (the whole warp walks the loop, one elected
+// lane issues), warps 2..9 softmax + epilogue.
+// Head dimension 64, bf16 inputs, FP32 outputs.  Every wait is bounded.  The backward of the FP8-operand mode
+// is in attn_f8.cu.
 #include <string.h>
 
 #include <atomic>
 
-
 #include "attn_common.cuh"
-#include "mc_stats.cuh"
 
 namespace bsp {
 
@@ -52,59 +51,34 @@ struct AttnParams {
   float* out1;                   // DKV: dK                         [BH*S*64]
   float* out2;                   // DKV with the fused dQ: dQ (zero at launch), else NULL
   float* lse_out;                // FWD
-  // Monte-Carlo epilogue (DQ, and DKV without dV): instead of storing the gradient g, the kernel adds
-  // g - mc_ref to out0 and (g - mc_ref)^2 to out1 (the running sums S1, S2 of that gradient)
-  const float* mc_ref;           // [BH*S*64] or NULL
-  int nd;                        // draws per launch (1; 2 in the Monte-Carlo dQ kernel: dterm holds [2][BH*S])
   bsp_diag_t* diag;
-  // FP8-operand mode: q, k, v, dO hold decoded FP8 codes (exact in bf16); their per-(b,h) scales
-  // are folded into the softmax argument, dP and the outputs; P and dS are rounded onto the E4M3 /
-  // E5M2 grids (at p_scale / ds_scale) before their products.  All NULL / 0 in BF16-operand mode.
+  // FWD in FP8-operand mode: q, k, v hold decoded FP8 codes (exact in bf16); their per-(b,h) scales are folded
+  // into the softmax argument and the output.  All NULL / 0 in BF16-operand mode.
   int fp8;
   const float* sc_q;             // [BH]
   const float* sc_k;
   const float* sc_v;
-  const float* sc_do;
-  float p_scale, ds_scale;
-  const uint8_t *cq, *ck, *cv, *cdo;   // the operands' codes: what the backward modes load in FP8-operand mode
 };
 
-// Two floats rounded to the nearest FP8 grid value (ties to even, saturating: what f8_rn_value
-// gives) and packed as a bf16 pair, through the hardware conversions: f32 pair -> FP8 pair -> f16 pair
-// (every FP8 value is an f16 value) -> f32 -> bf16 pair (every FP8 value is a bf16 value too).
-template <int FMT>
-__device__ __forceinline__ uint32_t f8_grid_bf16x2(float lo, float hi) {
-  const uint16_t c = (uint16_t)f8_encode_rn_pair_inrange<FMT>(lo, hi);
-  uint32_t h2;
-  if (FMT == BSP_E4M3) asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"(c));
-  else asm("cvt.rn.f16x2.e5m2x2 %0, %1;" : "=r"(h2) : "h"(c));
-  const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h2));
-  return pack_bf16x2(f.x, f.y);
-}
-
-// FP8: the FP8-operand mode (per-head operand scales, P and dS rounded onto the FP8 grids); a
-// template parameter because its tests and extra multiplications sit in the innermost loop.
+// FP8 (forward only): the FP8-operand mode, per-head operand scales; a template parameter because its
+// multiplications sit in the innermost loop.
 // DV (dK/dV mode only): false leaves dV out (its product, the P operand and its store): dV does
-// not read the correction term, so the draws of a fresh read need it once, not K times.
-// MC: the Monte-Carlo epilogue (see AttnParams::mc_ref); a template parameter so that the plain
-// kernels carry none of its registers.
-// ND (Monte-Carlo dQ and dK kernels only): draws per launch.  S, dP and P do not depend on the correction
-// term, so with ND = 2 a step forms them once and builds two dS operands, one per draw's D (at
-// p.dterm and p.dterm + BH*S), into two accumulators; the epilogue adds both draws to the sums.
-// DQF (dK/dV mode, BF16 operands only): the same CTA also forms the step's share of dQ, dS_ij K_j, and
+// not read the correction term.
+// DQF (dK/dV mode only): the same CTA also forms the step's share of dQ, dS_ij K_j, and
 // adds it to dQ in global memory (one tiled bulk reduce-add per step and column half), so S, dP and
 // the exponentials are formed once per score tile for all three gradients.  dS^T then goes to
 // shared memory instead of tensor memory (K-major A operand of dK, MN-major A operand of dQ) and
 // the tile ring has two stages.  dQ must hold zeros at launch; the order of its FP32 additions is
 // not fixed, so dQ is not bit-reproducible in this form.
-template <int MODE, bool FP8, bool DV, bool MC, int ND, bool DQF = false>
+template <int MODE, bool FP8, bool DV, bool DQF = false>
 __global__ void __launch_bounds__(kAtThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
             const __grid_constant__ CUtensorMap tm_o0, const __grid_constant__ CUtensorMap tm_o1,
             const __grid_constant__ CUtensorMap tm_o2, AttnParams p) {
   grid_dependency();
-  static_assert(!DQF || (MODE == AT_DKV && !FP8 && DV && !MC && ND == 1), "fused dQ: plain BF16 dK/dV kernel only");
+  static_assert(!DQF || (MODE == AT_DKV && DV), "fused dQ: dK/dV kernel only");
+  static_assert(!FP8 || MODE == AT_FWD, "the backward of the FP8-operand mode is attn_f8_kernel");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -138,17 +112,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const uint32_t b_bias = bars + 2240;                       // three barriers, one per buffer
   const uint32_t bias0 = bars + 4096;                        // ones tile; buffer b: X_lse at 1 + 2b, X_d at 2 + 2b
 
-  // dK kernel with two draws: the extra product step carries the first draw's -D; the second draw
-  // needs, per query (a column of S^T), delta = D_first - D_second, kept as FP32 in three buffers of
-  // 128 values that the threads writing the X tiles fill alongside them
-  const uint32_t delta0 = bars + 2304;
   // DQF: the step's dQ share is complete / has been read out of tensor memory
   const uint32_t b_dq_full = bars + 3848, b_dq_free = bars + 3856;
   // Plain dQ kernel: the two halves of 64 keys of a step are two pipelines (their own S and dP
   // products, 128 x 64 each, their own hand-over barriers with the four softmax warps that own those
   // columns, their own share of the dQ product), issued in turn by the one MMA warp, so that one half's
   // hand-overs run under the other half's work.
-  constexpr bool PP = (MODE == AT_DQ || MODE == AT_FWD) && !FP8 && !MC && ND == 1;
+  constexpr bool PP = MODE == AT_DQ || (MODE == AT_FWD && !FP8);
   const uint32_t b_sdp_full1 = bars + 3864, b_sdp_free1 = bars + 3872, b_pds_ready1 = bars + 3880, b_pds_free1 = bars + 3888;
   const uint32_t id_sdp64 = make_idesc(1u, 1u, 128, 64);
 
@@ -206,9 +176,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   // bf16 operands P and dS as the softmax warps write them back (64 columns each: two elements per
   // column) at [256,320) and [320,384), and one accumulator buffer of two 64-column halves at 384.
   const uint32_t t_s = tmem, t_dp = tmem + 128, t_p = tmem + 256, t_ds = tmem + 320;
-  // two draws (dQ kernel): the second draw's dS operand takes the P columns (no product reads P
-  // there) and its accumulator the second half of the accumulator buffer
-  const uint32_t t_ds2 = tmem + 256;
   const uint32_t t_dq = tmem + 320;                           // DQF: the step's dQ share (dS^T is in shared memory)
   const uint32_t t_accbase = MODE == AT_FWD ? tmem + 256 : tmem + 384;
   constexpr bool kAccDouble = MODE == AT_FWD;   // accumulators double-buffered across items
@@ -217,17 +184,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const uint32_t id_sdp = make_idesc(1u, 1u, 128, 128);                                   // A, B K-major
   const uint32_t id_kmn = make_idesc(1u, 1u, 128, 64) | (1u << 16);                       // A K-major, B MN-major
   const uint32_t id_mn = make_idesc(1u, 1u, 128, 64) | (1u << 15) | (1u << 16);           // A, B MN-major
-  // FP8-operand mode of the backward: every product is an FP8 tensor-core product (kind::f8f6f4) on the
-  // codes themselves.  The streamed and resident tiles are 128 rows of 64 bytes (64-byte swizzle), a
-  // K step is 32 elements, and P (E4M3) and dS (E5M2) go back into tensor memory four codes per column.
-  constexpr bool F8K = FP8 && MODE != AT_FWD;
-  constexpr uint32_t kTileB = F8K ? (uint32_t)(AT_BLK * AT_D) : (uint32_t)kAtTile;        // bytes a tile load brings
-  // operand formats (E4M3 = 0, E5M2 = 1): S from Q and K; dP from dO (E5M2) and V
-  const uint32_t id8_s = make_idesc(0u, 0u, 128, 128);
-  const uint32_t id8_dp = MODE == AT_DKV ? make_idesc(0u, 1u, 128, 128) : make_idesc(1u, 0u, 128, 128);
-  const uint32_t id8_pdo = make_idesc(0u, 1u, 128, 64) | (1u << 16);                      // P^T (E4M3) x dO (E5M2, MN-major)
-  const uint32_t id8_ds = make_idesc(1u, 0u, 128, 64) | (1u << 16);                       // dS (E5M2) x Q or K (E4M3, MN-major)
-
   if (warp == 0) {
     // ------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -242,7 +198,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         const uint32_t rb = item & 1u, rph = (item >> 1) & 1u;
         if (!mbar_wait(b_res_empty + 8 * rb, rph ^ 1u, abort_flag)) { ok = false; break; }
         const uint32_t r0 = res_base + rb * 2 * kAtTile, r1 = r0 + kAtTile;
-        mbar_expect_tx(b_res + 8 * rb, (MODE == AT_FWD ? 1 : 2) * kTileB);
+        mbar_expect_tx(b_res + 8 * rb, (MODE == AT_FWD ? 1 : 2) * kAtTile);
         if (MODE == AT_DKV) {
           tma_load_3d(r0, &tm_k, b_res + 8 * rb, 0, blk * AT_BLK, bh);
           tma_load_3d(r1, &tm_v, b_res + 8 * rb, 0, blk * AT_BLK, bh);
@@ -256,7 +212,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           const uint32_t s = itg % kStg, ph = (itg / kStg) & 1u;
           if (!mbar_wait(b_sempty + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t d0 = stage_at(s), d1 = d0 + kAtTile;
-          mbar_expect_tx(b_sfull + 8 * s, 2 * kTileB);
+          mbar_expect_tx(b_sfull + 8 * s, 2 * kAtTile);
           if (MODE == AT_DKV) {
             tma_load_3d(d0, &tm_q, b_sfull + 8 * s, 0, step * AT_BLK, bh);
             tma_load_3d(d1, &tm_do, b_sfull + 8 * s, 0, step * AT_BLK, bh);
@@ -308,25 +264,15 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         const uint32_t do_t = MODE == AT_DKV ? st1 : res1, v_t = MODE == AT_DKV ? res1 : st1;
         // DKV forms the transposes, S^T = K Q^T and dP^T = V dO^T (rows = keys), so that P^T and dS^T
         // come out of the softmax warps as the row-per-lane A operands of dV = P^T dO, dK = dS^T Q
-        if (F8K) {
-          // 64 bytes of K per row: two steps of 32 elements
-          const uint64_t a = make_smem_desc_sw64(MODE == AT_DKV ? k_t : q_t), b = make_smem_desc_sw64(MODE == AT_DKV ? q_t : k_t);
+        {
+          const uint64_t a = make_smem_desc(MODE == AT_DKV ? k_t : q_t), b = make_smem_desc(MODE == AT_DKV ? q_t : k_t);
 #pragma unroll
-          for (int k = 0; k < 2; ++k) tc_mma_l<true>(leader, t_s, a + 2u * k, b + 2u * k, id8_s, k != 0);
-          const uint64_t a2 = make_smem_desc_sw64(MODE == AT_DKV ? v_t : do_t), b2 = make_smem_desc_sw64(MODE == AT_DKV ? do_t : v_t);
+          for (int k = 0; k < 4; ++k) tc_mma_l<false>(leader, t_s, a + 2u * k, b + 2u * k, id_sdp, k != 0);
+        }
+        if (MODE != AT_FWD) {
+          const uint64_t a = make_smem_desc(MODE == AT_DKV ? v_t : do_t), b = make_smem_desc(MODE == AT_DKV ? do_t : v_t);
 #pragma unroll
-          for (int k = 0; k < 2; ++k) tc_mma_l<true>(leader, t_dp, a2 + 2u * k, b2 + 2u * k, id8_dp, k != 0);
-        } else {
-          {
-            const uint64_t a = make_smem_desc(MODE == AT_DKV ? k_t : q_t), b = make_smem_desc(MODE == AT_DKV ? q_t : k_t);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) tc_mma_l<false>(leader, t_s, a + 2u * k, b + 2u * k, id_sdp, k != 0);
-          }
-          if (MODE != AT_FWD) {
-            const uint64_t a = make_smem_desc(MODE == AT_DKV ? v_t : do_t), b = make_smem_desc(MODE == AT_DKV ? do_t : v_t);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) tc_mma_l<false>(leader, t_dp, a + 2u * k, b + 2u * k, id_sdp, k != 0);
-          }
+          for (int k = 0; k < 4; ++k) tc_mma_l<false>(leader, t_dp, a + 2u * k, b + 2u * k, id_sdp, k != 0);
         }
         if (MODE == AT_DKV) {
           // the extra K = 16 step: minus LSE/c into S^T, minus D into dP^T (see the X tiles)
@@ -400,28 +346,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         tc_fence_after();
         const uint32_t first = it == 0 ? 0u : 1u;             // overwrite on the first product
         if (!kAccDouble && it == 0 && !wait_all(b_acc_free + 8 * ab, aph ^ 1u)) { ok = false; break; }
-        if (F8K && MODE == AT_DKV) {
-          // the same products on the codes: eight columns per 32 queries, 128 queries = 4 x 32 along K
-          const uint64_t bdo = make_smem_desc_mn_sw64(st1), bq = make_smem_desc_mn_sw64(st0);
-          if (DV) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) tc_mma_ts_l<true>(leader, t_acc0, t_p + 8u * k, bdo + 128u * k, id8_pdo, first | (k != 0));
-          }
-#pragma unroll
-          for (int k = 0; k < 4; ++k) tc_mma_ts_l<true>(leader, t_acc1, t_ds + 8u * k, bq + 128u * k, id8_ds, first | (k != 0));
-          if (ND == 2 && !DV) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) tc_mma_ts_l<true>(leader, t_acc0, t_ds2 + 8u * k, bq + 128u * k, id8_ds, first | (k != 0));
-          }
-        } else if (F8K && MODE == AT_DQ) {
-          const uint64_t bk = make_smem_desc_mn_sw64(st0);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) tc_mma_ts_l<true>(leader, t_acc0, t_ds + 8u * k, bk + 128u * k, id8_ds, first | (k != 0));
-          if (ND == 2) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) tc_mma_ts_l<true>(leader, t_acc1, t_ds2 + 8u * k, bk + 128u * k, id8_ds, first | (k != 0));
-          }
-        } else if (DQF) {
+        if (DQF) {
           // dV += P^T dO with P^T from tensor memory; dK += dS^T Q with dS^T K-major from shared memory
           // (two halves of 64 queries, four K = 16 steps each); then the step's dQ share = dS K_j: the same
           // buffer read MN-major (128 queries wide, 16 keys per step), K_j = the resident tile, MN-major
@@ -450,20 +375,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           }
 #pragma unroll
           for (int k = 0; k < 8; ++k) tc_mma_ts_l<false>(leader, t_acc1, t_ds + 8u * k, bq + 128u * k, id_kmn, first | (k != 0));
-          if (ND == 2 && !DV) {
-            // second draw: its dS^T operand sits in the P columns, its dK in the dV accumulator
-#pragma unroll
-            for (int k = 0; k < 8; ++k) tc_mma_ts_l<false>(leader, t_acc0, t_ds2 + 8u * k, bq + 128u * k, id_kmn, first | (k != 0));
-          }
-        } else if (MODE == AT_DQ) {
-          // dQ += dS K : A from tensor memory (row = query, eight columns per 16 keys), B MN-major = streamed K
-          const uint64_t bk = make_smem_desc_mn(st0, 16384u);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) tc_mma_ts_l<false>(leader, t_acc0, t_ds + 8u * k, bk + 128u * k, id_kmn, first | (k != 0));
-          if (ND == 2) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) tc_mma_ts_l<false>(leader, t_acc1, t_ds2 + 8u * k, bk + 128u * k, id_kmn, first | (k != 0));
-          }
         } else {
           // O_h += P_h V_h for the two halves of 64 keys, each into its own accumulator (its own running
           // maximum): A = P from tensor memory (eight columns per 16 keys), B MN-major = streamed V
@@ -516,38 +427,26 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     const uint32_t ab = kAccDouble ? (item & 1u) : 0u;
     const uint32_t iph = kAccDouble ? ((item >> 1) & 1u) : ((uint32_t)item & 1u);
     const uint32_t t_acc0 = t_accbase + ab * 128, t_acc1 = t_acc0 + 64;
-    float inv_q = 1.f, inv_k = 1.f, inv_v = 1.f, inv_do = 1.f;
+    float inv_q = 1.f, inv_k = 1.f, inv_v = 1.f;
     if (FP8) {
       inv_q = __fdiv_rn(1.0f, ldg(p.sc_q + bh)); inv_k = __fdiv_rn(1.0f, ldg(p.sc_k + bh));
-      inv_v = __fdiv_rn(1.0f, ldg(p.sc_v + bh)); inv_do = __fdiv_rn(1.0f, ldg(p.sc_do + bh));
+      inv_v = __fdiv_rn(1.0f, ldg(p.sc_v + bh));
     }
     const float c2 = FP8 ? p.c * kLog2e * inv_q * inv_k : p.c * kLog2e;   // scores arrive as products of decoded codes
-    const float dp_mul = FP8 ? inv_do * inv_v : 1.0f;                     // likewise dP
     // DKV: softmax thread ts owns row (ts & 127) of the X tiles: the LSE tile for ts < 128, the D tile
     // above.  bias_fetch reads the raw value of a step's query (nothing may depend on that load
     // before the step's arithmetic is done, or the in-order warp sits out its latency); bias_put
     // writes the three-term row into buffer (global step) % 3 and signals the MMA issuer.
     const int ts = (int)threadIdx.x - kAtSoftThread0;
     const float* bias_src = ts < 128 ? p.lse : p.dterm;
-    const float bias_mul = ts < 128 ? -kLog2e / c2 : -1.0f / dp_mul;
-    float nx_mul = bias_mul;                                  // the same factor for the next item's head
+    const float bias_mul = ts < 128 ? -kLog2e / c2 : -1.0f;
     auto bias_fetch = [&](int tbh, int step) -> float {
       const int q = step * AT_BLK + (ts & 127);
       return ldg(bias_src + (size_t)tbh * p.S + (q < p.S ? q : 0));
     };
-    // the second draw's correction term of the same query (threads of the D tile only)
-    auto bias_fetch2 = [&](int tbh, int step) -> float {
-      if (ND != 2 || ts < 128) return 0.f;
-      const int q = step * AT_BLK + (ts & 127);
-      return ldg(p.dterm + (size_t)p.BH * p.S + (size_t)tbh * p.S + (q < p.S ? q : 0));
-    };
-    auto bias_put = [&](int step, uint32_t jt, float raw, float mul, float raw2) {
+    auto bias_put = [&](int step, uint32_t jt, float raw) {
       const int q = ts & 127;
-      if (ND == 2 && ts >= 128) {
-        const float dl = step * AT_BLK + q < p.S ? raw - raw2 : 0.f;
-        asm volatile("st.shared.f32 [%0], %1;" ::"r"(delta0 + ((jt % 3u) * 128u + (uint32_t)q) * 4u), "f"(dl) : "memory");
-      }
-      const float x = step * AT_BLK + q < p.S ? raw * mul : 0.f;
+      const float x = step * AT_BLK + q < p.S ? raw * bias_mul : 0.f;
       const __nv_bfloat16 h1 = __float2bfloat16_rn(x);
       const float r1 = x - __bfloat162float(h1);
       const __nv_bfloat16 h2 = __float2bfloat16_rn(r1);
@@ -572,15 +471,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         int nb, ns;
         decode_item(wn, nb, nx_bh, nx_begin, ns);
         nx_total = ns;
-        if (FP8) {                                            // per-head operand scales
-          const float nq = __fdiv_rn(1.0f, ldg(p.sc_q + nx_bh)), nk = __fdiv_rn(1.0f, ldg(p.sc_k + nx_bh));
-          const float nv = __fdiv_rn(1.0f, ldg(p.sc_v + nx_bh)), ndo = __fdiv_rn(1.0f, ldg(p.sc_do + nx_bh));
-          nx_mul = ts < 128 ? -kLog2e / (p.c * kLog2e * nq * nk) : -1.0f / (ndo * nv);
-        }
       }
       while (bias_written < itg + (uint32_t)(total < 2 ? total : 2)) {
         const int l = (int)(bias_written - itg);
-        bias_put(it_begin + l, bias_written, bias_fetch(bh, it_begin + l), bias_mul, bias_fetch2(bh, it_begin + l));
+        bias_put(it_begin + l, bias_written, bias_fetch(bh, it_begin + l));
         ++bias_written;
       }
     }
@@ -591,14 +485,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       if (t - total < nx_total) { tbh = nx_bh; tstep = nx_begin + (t - total); return true; }
       return false;
     };
-    float lse2 = 0.f, dq = 0.f, dq2 = 0.f;                    // this row's LSE*log2e and D (dq2: the second draw's D)
+    float lse2 = 0.f, dq = 0.f;                               // this row's LSE*log2e and D
     int qrow = 0;                                             // global query index of this thread's row
     if (MODE != AT_DKV) {
       qrow = blk * AT_BLK + r;
       if (MODE == AT_DQ && qrow < p.S) {
         lse2 = ldg(p.lse + (size_t)bh * p.S + qrow) * kLog2e;
         dq = ldg(p.dterm + (size_t)bh * p.S + qrow);
-        if (ND == 2) dq2 = ldg(p.dterm + (size_t)p.BH * p.S + (size_t)bh * p.S + qrow);
       }
       if (lse_known && qrow < p.S) lse2 = ldg(p.lse + (size_t)bh * p.S + qrow) * kLog2e;
     }
@@ -639,7 +532,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       const int step = it_begin + (it % nsteps);
       const uint32_t ip = (itg + (uint32_t)it) & 1u;
       int kblk;                                               // key block of this step
-      float bias_next = 0.f, bias_next2 = 0.f;                // DKV: this thread's raw value(s) for the row two steps ahead
+      float bias_next = 0.f;                                  // DKV: this thread's raw value for the row two steps ahead
       int bias_bh = 0, bias_step = 0;
       const bool bias_due = MODE == AT_DKV && bias_written == itg + (uint32_t)it + 2u && bias_target(it, bias_bh, bias_step);
       if (MODE == AT_DKV) {
@@ -664,10 +557,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive((PP && h) ? b_sdp_free1 : b_sdp_free);
-      if (bias_due) {                                         // lands under this step's arithmetic
-        bias_next = bias_fetch(bias_bh, bias_step);
-        bias_next2 = bias_fetch2(bias_bh, bias_step);
-      }
+      if (bias_due) bias_next = bias_fetch(bias_bh, bias_step);   // lands under this step's arithmetic
 
       const int key0 = kblk * AT_BLK + h * 64;
       // masking is needed only on the diagonal block and where the sequence ends inside the block
@@ -713,48 +603,22 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       }
       {
         uint32_t pk[32], dk[32];
-        // two neighbouring keys: P and dS = P (dP - D) as packed bf16 operands.  FP8-operand mode
-        // first rounds P onto the E4M3 grid at p_scale and dS onto the E5M2 grid at ds_scale (the
-        // grid values are exact in bf16; the scales come back in the epilogue).
-        // a pair of dS values as a packed bf16 operand (FP8-operand mode: on the E5M2 grid at ds_scale)
-        auto pack_ds = [&](float s0, float s1) -> uint32_t {
-          if (F8K) return f8_encode_rn_pair_inrange<BSP_E5M2>(s0 * p.ds_scale, s1 * p.ds_scale);   // two codes, 16 bits
-          if (FP8) return f8_grid_bf16x2<BSP_E5M2>(s0 * p.ds_scale, s1 * p.ds_scale);
-          return pack_bf16x2(s0, s1);
-        };
-        // 32 of this thread's 64 columns of an operand (16 packed pairs) back into tensor memory: two
-        // 16-bit elements per column, or (codes) four per column
+        // 32 of this thread's 64 columns of an operand (16 packed pairs) back into tensor memory
         auto st_half = [&](uint32_t t_base, int half, const uint32_t (&wv)[16]) {
-          if (F8K) {
-            uint32_t c8[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) c8[i] = (wv[2 * i] & 0xFFFFu) | (wv[2 * i + 1] << 16);
-            tmem_st8(t_base + lane_off + h * 16 + half * 8, c8);
-          } else {
-            tmem_st16(t_base + lane_off + h * 32 + half * 16, wv);
-          }
+          tmem_st16(t_base + lane_off + h * 32 + half * 16, wv);
         };
+        // two neighbouring keys: P and dS = P (dP - D) as packed bf16 operands
         auto pack_pair = [&](float p0, float p1, uint32_t dp0, uint32_t dp1, float d0, float d1, uint32_t& po,
                              uint32_t& dso) {
           float s0 = 0.f, s1 = 0.f;
           if (MODE == AT_FWD) run_l += p0 + p1;             // the row's normaliser, from the unrounded values
-          if (MODE == AT_DKV && !FP8) {
+          if (MODE == AT_DKV) {
             // (the accumulators already hold dP - D): both products in one packed instruction
             mul_f32x2(s0, s1, p0, p1, __uint_as_float(dp0), __uint_as_float(dp1));
           } else if (MODE != AT_FWD) {
             float t0, t1;
-            fma_f32x2(t0, t1, __uint_as_float(dp0), __uint_as_float(dp1), dp_mul, dp_mul, -d0, -d1);
+            fma_f32x2(t0, t1, __uint_as_float(dp0), __uint_as_float(dp1), 1.0f, 1.0f, -d0, -d1);
             mul_f32x2(s0, s1, p0, p1, t0, t1);
-          }
-          if (FP8 && MODE != AT_FWD) {                      // the forward keeps P unrounded
-            if (F8K) {                                      // the codes themselves (two per word for now)
-              po = f8_encode_rn_pair_inrange<BSP_E4M3>(p0 * p.p_scale, p1 * p.p_scale);
-              dso = f8_encode_rn_pair_inrange<BSP_E5M2>(s0 * p.ds_scale, s1 * p.ds_scale);
-              return;
-            }
-            po = f8_grid_bf16x2<BSP_E4M3>(p0 * p.p_scale, p1 * p.p_scale);
-            dso = f8_grid_bf16x2<BSP_E5M2>(s0 * p.ds_scale, s1 * p.ds_scale);
-            return;
           }
           po = pack_bf16x2(p0, p1);
           if (MODE != AT_FWD) dso = pack_bf16x2(s0, s1);
@@ -820,48 +684,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           st_half(t_dp, 1, *reinterpret_cast<const uint32_t(*)[16]>(&pk[16]));
           tmem_wait_st();
           tc_fence_before();
-        } else if (MODE == AT_DQ && ND == 2) {
-          // two draws: one exponential per element, two dS values; 32 columns at a time so that the
-          // packed operands of both draws stay within the register budget
-          uint32_t da[16], db[16];
-          auto pair2_at = [&](int j, bool masked) {
-            float a0, a1;
-            fma_f32x2(a0, a1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), c2, c2, -lse2, -lse2);
-            if (masked) {
-              if (!valid_at(j)) a0 = -INFINITY;
-              if (!valid_at(j + 1)) a1 = -INFINITY;
-            }
-            const float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
-            float t0, t1, u0, u1, s0, s1, r0, r1;
-            fma_f32x2(t0, t1, __uint_as_float(dv[j]), __uint_as_float(dv[j + 1]), dp_mul, dp_mul, -dq, -dq);
-            fma_f32x2(u0, u1, __uint_as_float(dv[j]), __uint_as_float(dv[j + 1]), dp_mul, dp_mul, -dq2, -dq2);
-            mul_f32x2(s0, s1, p0, p1, t0, t1);
-            mul_f32x2(r0, r1, p0, p1, u0, u1);
-            da[(j & 31) >> 1] = pack_ds(s0, s1);
-            db[(j & 31) >> 1] = pack_ds(r0, r1);
-          };
-          if (!edge) {
-#pragma unroll
-            for (int j = 0; j < 32; j += 2) pair2_at(j, false);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 32; j += 2) pair2_at(j, true);
-          }
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_pds_free, ip ^ 1u, abort_flag));
-          if (!ok) break;
-          st_half(t_ds, 0, da);
-          st_half(t_ds2, 0, db);
-          if (!edge) {
-#pragma unroll
-            for (int j = 32; j < 64; j += 2) pair2_at(j, false);
-          } else {
-#pragma unroll
-            for (int j = 32; j < 64; j += 2) pair2_at(j, true);
-          }
-          st_half(t_ds, 1, da);
-          st_half(t_ds2, 1, db);
-          tmem_wait_st();
-          tc_fence_before();
         } else if (MODE == AT_DQ) {
           if (!edge) {
 #pragma unroll
@@ -876,47 +698,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           if (!ok) break;
           st_half(t_ds, 0, *reinterpret_cast<const uint32_t(*)[16]>(&dk[0]));
           st_half(t_ds, 1, *reinterpret_cast<const uint32_t(*)[16]>(&dk[16]));
-          tmem_wait_st();
-          tc_fence_before();
-        } else if (MODE == AT_DKV && ND == 2) {
-          // dK kernel, two draws: the accumulators hold s - LSE/c and dP - D of the first draw; the
-          // second draw's dP - D is that plus delta of the column's query.  32 columns at a time.
-          uint32_t da[16], db[16];
-          const uint32_t dbase = delta0 + (((itg + (uint32_t)it) % 3u) * 128u + (uint32_t)h * 64u) * 4u;
-          auto pair2_at = [&](int j, bool masked) {
-            // (scalar arithmetic here: the packed forms cost this variant registers it does not have)
-            float a0 = __uint_as_float(sv[j]) * c2, a1 = __uint_as_float(sv[j + 1]) * c2;
-            if (masked) {
-              if (!valid_at(j)) a0 = -INFINITY;
-              if (!valid_at(j + 1)) a1 = -INFINITY;
-            }
-            const float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
-            float e0, e1;
-            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(e0), "=f"(e1) : "r"(dbase + (uint32_t)j * 4u));
-            const float x0 = __uint_as_float(dv[j]) * dp_mul, x1 = __uint_as_float(dv[j + 1]) * dp_mul;
-            da[(j & 31) >> 1] = pack_ds(p0 * x0, p1 * x1);
-            db[(j & 31) >> 1] = pack_ds(p0 * (x0 + e0), p1 * (x1 + e1));
-          };
-          if (!edge) {
-#pragma unroll
-            for (int j = 0; j < 32; j += 2) pair2_at(j, false);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 32; j += 2) pair2_at(j, true);
-          }
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_pds_free, ip ^ 1u, abort_flag));
-          if (!ok) break;
-          st_half(t_ds, 0, da);
-          st_half(t_ds2, 0, db);
-          if (!edge) {
-#pragma unroll
-            for (int j = 32; j < 64; j += 2) pair2_at(j, false);
-          } else {
-#pragma unroll
-            for (int j = 32; j < 64; j += 2) pair2_at(j, true);
-          }
-          st_half(t_ds, 1, da);
-          st_half(t_ds2, 1, db);
           tmem_wait_st();
           tc_fence_before();
         } else {
@@ -979,8 +760,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       }
       if (bias_due) {
         // (the empty asm pins the first use of the fetched value here, after the step's arithmetic)
-        asm volatile("" : "+f"(bias_next), "+f"(bias_next2));
-        bias_put(bias_step, bias_written, bias_next, bias_bh == bh && it + 2 < total ? bias_mul : nx_mul, bias_next2);
+        asm volatile("" : "+f"(bias_next));
+        bias_put(bias_step, bias_written, bias_next);
         ++bias_written;
       }
     }
@@ -1008,19 +789,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     // time through the item's resident-tile buffer (no product reads it any more): every thread puts
     // its row's 32 FP32 values of column half h into the 128-byte-swizzle box that a tiled bulk store
     // then writes (whole 128-byte lines; rows beyond the sequence are clipped by the store).
-    constexpr bool mc = MC;
-    // Monte-Carlo epilogue: the reference values of the warp's 32 rows x 32 columns, fetched by the
-    // warp together (load t: four rows of 128 contiguous bytes, lane -> row 4t + lane / 8, 16-byte
-    // chunk lane % 8) and handed to the row-owning threads through the staging buffer further down
-    float4 rc[8];
-    if (mc) {
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const int orow = blk * AT_BLK + q4 * 32 + 4 * t + (lane >> 3);
-        rc[t] = ldg(reinterpret_cast<const float4*>(p.mc_ref + ((size_t)bh * p.S + (orow < p.S ? orow : 0)) * AT_D + h * 32) +
-                      (lane & 7));
-      }
-    }
     if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_acc + 8 * ab, iph, abort_flag));
     if (ok) {
       tc_fence_after();
@@ -1036,37 +804,16 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         tma_store_wait_read();                                // the last share's reduce-adds have read the staging buffer
         red_pending = false;
       }
-      if (MODE == AT_DKV || mc) named_bar_sync(3, 256);       // ... before anyone writes the second staging buffer again
-      float rv[32];                                           // this thread's 32 reference values
-      if (mc) {
-        // through the warp's own 4 KB of the (now free) second staging buffer: chunk (row, c) sits
-        // where the output boxes keep it, so every thread finds its row at its own output slots
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const uint32_t row = (uint32_t)(q4 * 32 + 4 * t + (lane >> 3));
-          const uint32_t off = (uint32_t)h * 16384u + row * 128u + ((((uint32_t)lane & 7u) ^ (row & 7u)) << 4);
-          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage2 + off), "f"(rc[t].x), "f"(rc[t].y), "f"(rc[t].z),
-                       "f"(rc[t].w) : "memory");
-        }
-        __syncwarp();
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const uint32_t off = (uint32_t)h * 16384u + (uint32_t)r * 128u + ((uint32_t)(t ^ (r & 7)) << 4);
-          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                       : "=f"(rv[4 * t]), "=f"(rv[4 * t + 1]), "=f"(rv[4 * t + 2]), "=f"(rv[4 * t + 3]) : "r"(stage2 + off));
-        }
-        __syncwarp();
-      }
+      if (MODE == AT_DKV) named_bar_sync(3, 256);            // ... before anyone writes the second staging buffer again
 #pragma unroll
       for (int o = (MODE == AT_DKV && !DV) ? 1 : 0; o < nout; ++o) {
         const uint32_t stg = o == 0 ? res_base + rbi * 2 * kAtTile : stage2;
         float mul;
-        if (MODE == AT_DKV) mul = o == 0 ? (FP8 ? inv_do / p.p_scale : 1.f) : p.c * (FP8 ? inv_q / p.ds_scale : 1.f);
-        else if (MODE == AT_DQ) mul = p.c * (FP8 ? inv_k / p.ds_scale : 1.f);
+        if (MODE == AT_DKV) mul = o == 0 ? 1.f : p.c;
+        else if (MODE == AT_DQ) mul = p.c;
         else mul = inv_v * fwd_w0;
-        uint32_t a[32], a2[ND == 2 ? 32 : 1];
+        uint32_t a[32];
         tmem_ld32((o == 0 ? t_acc0 : t_acc1) + lane_off + h * 32, a);
-        if (ND == 2) tmem_ld32((o == 0 ? t_acc1 : t_acc0) + lane_off + h * 32, *reinterpret_cast<uint32_t(*)[32]>(&a2[0]));
         if (MODE == AT_FWD) {
           // O = w0 O_0 + w1 O_1: fold the second half's accumulator in here
           uint32_t a1[32];
@@ -1082,34 +829,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           __syncwarp();
           if (lane == 0) mbar_arrive(b_acc_free + 8 * ab);
         }
-        if (mc) {
-          // g - ref into this output's staging buffer, its square into the other one
-          const uint32_t stg2 = o == 0 ? stage2 : res_base + rbi * 2 * kAtTile;
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            const uint32_t off = (uint32_t)h * 16384u + (uint32_t)r * 128u + ((uint32_t)(t ^ (r & 7)) << 4);
-            float d[4], q[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              d[e] = __uint_as_float(a[4 * t + e]) * mul - rv[4 * t + e];
-              q[e] = d[e] * d[e];
-              if (ND == 2) {                                  // the second draw of this launch joins the first
-                const float e2 = __uint_as_float(a2[ND == 2 ? 4 * t + e : 0]) * mul - rv[4 * t + e];
-                d[e] += e2;
-                q[e] = fmaf(e2, e2, q[e]);
-              }
-            }
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg + off), "f"(d[0]), "f"(d[1]), "f"(d[2]), "f"(d[3]) : "memory");
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg2 + off), "f"(q[0]), "f"(q[1]), "f"(q[2]), "f"(q[3]) : "memory");
-          }
-        } else {
-#pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            const uint32_t off = (uint32_t)h * 16384u + (uint32_t)r * 128u + ((uint32_t)(t ^ (r & 7)) << 4);
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg + off), "f"(__uint_as_float(a[4 * t]) * mul),
-                         "f"(__uint_as_float(a[4 * t + 1]) * mul), "f"(__uint_as_float(a[4 * t + 2]) * mul),
-                         "f"(__uint_as_float(a[4 * t + 3]) * mul) : "memory");
-          }
+        for (int t = 0; t < 8; ++t) {
+          const uint32_t off = (uint32_t)h * 16384u + (uint32_t)r * 128u + ((uint32_t)(t ^ (r & 7)) << 4);
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stg + off), "f"(__uint_as_float(a[4 * t]) * mul),
+                       "f"(__uint_as_float(a[4 * t + 1]) * mul), "f"(__uint_as_float(a[4 * t + 2]) * mul),
+                       "f"(__uint_as_float(a[4 * t + 3]) * mul) : "memory");
         }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1117,23 +842,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       if (warp == kAtSoftWarp0 && lane == 0) {
         // issue the stores and go on: their completion is only needed before the staging buffers are
         // written again (next epilogue) or handed back (after the next item's first step)
-        if (mc) {
-          // S1 += g - ref, S2 += (g - ref)^2: each element of the sums is added to once per launch
-          const uint32_t sx = MODE == AT_DKV ? stage2 : res_base + rbi * 2 * kAtTile;
-          const uint32_t sy = MODE == AT_DKV ? res_base + rbi * 2 * kAtTile : stage2;
-          tma_reduce_add_3d(&tm_o0, sx, 0, blk * AT_BLK, bh);
-          tma_reduce_add_3d(&tm_o0, sx + 16384u, 32, blk * AT_BLK, bh);
-          tma_reduce_add_3d(&tm_o1, sy, 0, blk * AT_BLK, bh);
-          tma_reduce_add_3d(&tm_o1, sy + 16384u, 32, blk * AT_BLK, bh);
-        } else {
-          if (MODE != AT_DKV || DV) {
-            tma_store_3d(&tm_o0, res_base + rbi * 2 * kAtTile, 0, blk * AT_BLK, bh);
-            tma_store_3d(&tm_o0, res_base + rbi * 2 * kAtTile + 16384u, 32, blk * AT_BLK, bh);
-          }
-          if (MODE == AT_DKV) {
-            tma_store_3d(&tm_o1, stage2, 0, blk * AT_BLK, bh);
-            tma_store_3d(&tm_o1, stage2 + 16384u, 32, blk * AT_BLK, bh);
-          }
+        if (MODE != AT_DKV || DV) {
+          tma_store_3d(&tm_o0, res_base + rbi * 2 * kAtTile, 0, blk * AT_BLK, bh);
+          tma_store_3d(&tm_o0, res_base + rbi * 2 * kAtTile + 16384u, 32, blk * AT_BLK, bh);
+        }
+        if (MODE == AT_DKV) {
+          tma_store_3d(&tm_o1, stage2, 0, blk * AT_BLK, bh);
+          tma_store_3d(&tm_o1, stage2 + 16384u, 32, blk * AT_BLK, bh);
         }
         tma_store_commit();
         store_pending = true;
@@ -1259,7 +974,7 @@ attn_dterm_kernel(const void* dO, const float* o_orig, const uint8_t* o_codes,
 
 // ------------------------------------------------------------------------------- host side
 
-template <int MODE, bool FP8, bool DV, bool MC = false, int ND = 1, bool DQF = false>
+template <int MODE, bool FP8, bool DV, bool DQF = false>
 static int launch_attn_mode(const void* q, const void* k, const void* v, const void* dO, AttnParams p, cudaStream_t st) {
   CUtensorMap mq, mk, mv, mdo, mo0, mo1, mo2;
   int rc;
@@ -1267,24 +982,14 @@ static int launch_attn_mode(const void* q, const void* k, const void* v, const v
   if ((rc = make_out_map(&mo0, p.out0 ? p.out0 : p.out1, p.BH, p.S)) != BSP_OK) return rc;
   if ((rc = make_out_map(&mo1, p.out1 ? p.out1 : p.out0, p.BH, p.S)) != BSP_OK) return rc;
   if ((rc = make_out_map(&mo2, DQF ? p.out2 : (p.out0 ? p.out0 : p.out1), p.BH, p.S)) != BSP_OK) return rc;
-  if (FP8 && MODE != AT_FWD) {
-    // the backward of the FP8-operand mode loads the codes
-    if (!p.cq || !p.ck || !p.cv || !p.cdo) return BSP_ERR_ARG;
-    if (!aligned16(p.cq) || !aligned16(p.ck) || !aligned16(p.cv) || !aligned16(p.cdo)) return BSP_ERR_ALIGN;
-    if ((rc = make_head_map_u8(&mq, p.cq, p.BH, p.S)) != BSP_OK) return rc;
-    if ((rc = make_head_map_u8(&mk, p.ck, p.BH, p.S)) != BSP_OK) return rc;
-    if ((rc = make_head_map_u8(&mv, p.cv, p.BH, p.S)) != BSP_OK) return rc;
-    if ((rc = make_head_map_u8(&mdo, p.cdo, p.BH, p.S)) != BSP_OK) return rc;
-  } else {
-    if ((rc = make_head_map(&mq, q, p.BH, p.S)) != BSP_OK) return rc;
-    if ((rc = make_head_map(&mk, k, p.BH, p.S)) != BSP_OK) return rc;
-    if ((rc = make_head_map(&mv, v, p.BH, p.S)) != BSP_OK) return rc;
-    if ((rc = make_head_map(&mdo, dO ? dO : q, p.BH, p.S)) != BSP_OK) return rc;
-  }
+  if ((rc = make_head_map(&mq, q, p.BH, p.S)) != BSP_OK) return rc;
+  if ((rc = make_head_map(&mk, k, p.BH, p.S)) != BSP_OK) return rc;
+  if ((rc = make_head_map(&mv, v, p.BH, p.S)) != BSP_OK) return rc;
+  if ((rc = make_head_map(&mdo, dO ? dO : q, p.BH, p.S)) != BSP_OK) return rc;
   static std::atomic<bool> attr_set_dev[kMaxDevices];       // per kernel instantiation and device
   std::atomic<bool>& attr_set = attr_set_dev[device_slot()];
   if (!attr_set.load(std::memory_order_acquire)) {
-    BSP_CHECK_CUDA(cudaFuncSetAttribute(attn_kernel<MODE, FP8, DV, MC, ND, DQF>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAtSmem));
+    BSP_CHECK_CUDA(cudaFuncSetAttribute(attn_kernel<MODE, FP8, DV, DQF>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAtSmem));
     attr_set.store(true, std::memory_order_release);
   }
   // persistent: one CTA per SM walks the (block, head) items, heaviest first
@@ -1294,24 +999,16 @@ static int launch_attn_mode(const void* q, const void* k, const void* v, const v
     nsm = sm_count;
   const int64_t nitems = (int64_t)p.nblk * p.BH;
   const unsigned grid = (unsigned)(nitems < nsm ? nitems : nsm);
-  launch_kernel(attn_kernel<MODE, FP8, DV, MC, ND, DQF>, grid, kAtThreads, kAtSmem, st, mq, mk, mv, mdo, mo0, mo1, mo2, p);
+  launch_kernel(attn_kernel<MODE, FP8, DV, DQF>, grid, kAtThreads, kAtSmem, st, mq, mk, mv, mdo, mo0, mo1, mo2, p);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
 
 template <int MODE>
 static int launch_attn(const void* q, const void* k, const void* v, const void* dO, AttnParams p, cudaStream_t st) {
-  if (MODE != AT_FWD && p.mc_ref != nullptr) {               // Monte-Carlo epilogue: BF16 operands, no dV
-    if (p.fp8) {
-      if (p.nd == 2) return launch_attn_mode<MODE, true, MODE != AT_DKV, MODE != AT_FWD, MODE != AT_FWD ? 2 : 1>(q, k, v, dO, p, st);
-      return launch_attn_mode<MODE, true, MODE != AT_DKV, MODE != AT_FWD>(q, k, v, dO, p, st);
-    }
-    if (p.nd == 2) return launch_attn_mode<MODE, false, MODE != AT_DKV, MODE != AT_FWD, MODE != AT_FWD ? 2 : 1>(q, k, v, dO, p, st);
-    return launch_attn_mode<MODE, false, MODE != AT_DKV, MODE != AT_FWD>(q, k, v, dO, p, st);
-  }
-  if (MODE == AT_DKV && p.out0 == nullptr)                   // dK only
-    return p.fp8 ? launch_attn_mode<MODE, true, false>(q, k, v, dO, p, st) : launch_attn_mode<MODE, false, false>(q, k, v, dO, p, st);
-  return p.fp8 ? launch_attn_mode<MODE, true, true>(q, k, v, dO, p, st) : launch_attn_mode<MODE, false, true>(q, k, v, dO, p, st);
+  if (MODE == AT_DKV && p.out0 == nullptr) return launch_attn_mode<MODE, false, MODE != AT_DKV>(q, k, v, dO, p, st);   // dK only
+  if (MODE == AT_FWD && p.fp8) return launch_attn_mode<MODE, MODE == AT_FWD, true>(q, k, v, dO, p, st);
+  return launch_attn_mode<MODE, false, true>(q, k, v, dO, p, st);
 }
 
 static bool valid_enum(int v, int hi) { return v >= 0 && v <= hi; }
@@ -1319,9 +1016,7 @@ static bool valid_enum(int v, int hi) { return v >= 0 && v <= hi; }
 static int set_fp8(AttnParams& p, const bsp_attn_fp8_t* f) {
   p.fp8 = f ? 1 : 0;
   p.sc_q = f ? f->q_scale : nullptr; p.sc_k = f ? f->k_scale : nullptr;
-  p.sc_v = f ? f->v_scale : nullptr; p.sc_do = f ? f->do_scale : nullptr;
-  p.p_scale = f ? f->p_scale : 1.f; p.ds_scale = f ? f->ds_scale : 1.f;
-  p.cq = f ? f->q_codes : nullptr; p.ck = f ? f->k_codes : nullptr; p.cv = f ? f->v_codes : nullptr; p.cdo = f ? f->do_codes : nullptr;
+  p.sc_v = f ? f->v_scale : nullptr;
   if (f && (!f->q_scale || !f->k_scale || !f->v_scale || !f->do_scale || !(f->p_scale > 0.f) || !(f->ds_scale > 0.f)))
     return BSP_ERR_ARG;
   return BSP_OK;
@@ -1336,7 +1031,7 @@ int attn_fwd_impl(int B, int H, int S, int Dh, int causal, float softmax_scale, 
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o)) return BSP_ERR_ALIGN;
   AttnParams p{};
   p.BH = B * H; p.S = S; p.nblk = (S + AT_BLK - 1) / AT_BLK; p.causal = causal ? 1 : 0; p.c = softmax_scale;
-  p.lse = lse_known; p.dterm = nullptr; p.out0 = o; p.out1 = nullptr; p.lse_out = lse; p.diag = diag; p.mc_ref = nullptr; p.nd = 1;
+  p.lse = lse_known; p.dterm = nullptr; p.out0 = o; p.out1 = nullptr; p.lse_out = lse; p.diag = diag;
   if ((rc = set_fp8(p, f)) != BSP_OK) return rc;
   return launch_attn<AT_FWD>(q, k, v, nullptr, p, (cudaStream_t)stream);
 }
@@ -1415,9 +1110,10 @@ int attn_bwd_dterm_impl(int B, int H, int S, int Dh, int causal, float softmax_s
     return BSP_ERR_ALIGN;
   AttnParams p{};
   p.BH = B * H; p.S = S; p.nblk = (S + AT_BLK - 1) / AT_BLK; p.causal = causal ? 1 : 0; p.c = softmax_scale;
-  p.lse = lse; p.dterm = dterm; p.lse_out = nullptr; p.diag = diag; p.mc_ref = nullptr; p.nd = 1;
+  p.lse = lse; p.dterm = dterm; p.lse_out = nullptr; p.diag = diag;
   if ((rc = set_fp8(p, f)) != BSP_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
+  if (f) return attn_f8_bwd(B * H, S, causal, softmax_scale, f, lse, dterm, dq, dk, dv, diag, st);
   if (dk) {
     p.out0 = dv; p.out1 = dk;
     if ((rc = launch_attn<AT_DKV>(q, k, v, dO, p, st)) != BSP_OK) return rc;
@@ -1442,39 +1138,12 @@ int attn_bwd_fused_impl(int B, int H, int S, int Dh, int causal, float softmax_s
     return BSP_ERR_ALIGN;
   AttnParams p{};
   p.BH = B * H; p.S = S; p.nblk = (S + AT_BLK - 1) / AT_BLK; p.causal = causal ? 1 : 0; p.c = softmax_scale;
-  p.lse = lse; p.dterm = dterm; p.lse_out = nullptr; p.diag = diag; p.mc_ref = nullptr; p.nd = 1;
+  p.lse = lse; p.dterm = dterm; p.lse_out = nullptr; p.diag = diag;
   if ((rc = set_fp8(p, nullptr)) != BSP_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   BSP_CHECK_CUDA(cudaMemsetAsync(dq, 0, (size_t)B * H * S * AT_D * sizeof(float), st));
   p.out0 = dv; p.out1 = dk; p.out2 = dq;
-  return launch_attn_mode<AT_DKV, false, true, false, 1, true>(q, k, v, dO, p, st);
-}
-
-// nd (1 or 2) draws of the D use for dQ and dK with the Monte-Carlo epilogue: the kernels add g - ref
-// and its square to the running sums of their gradient and write no gradient (dV is not computed).
-// dterm holds the draws' correction terms back to back, [nd][B*H*S]; with nd = 2 (BF16-operand mode
-// only) both kernels take the two draws in one launch (S, dP and P are formed once per step).  The
-// sums must not be touched by anything else while this runs.
-int attn_bwd_dterm_mc(int B, int H, int S, int Dh, int causal, float softmax_scale, const void* q, const void* k,
-                      const void* v, const void* dO, int dt, const bsp_attn_fp8_t* f, const float* lse,
-                      const float* dterm, int nd, const float* ref_dq, float* S1q, float* S2q, const float* ref_dk,
-                      float* S1k, float* S2k, bsp_diag_t* diag, void* stream) {
-  int rc = check_attn_shape(B, H, S, Dh, dt);
-  if (rc != BSP_OK) return rc;
-  if (!q || !k || !v || !dO || !lse || !dterm || !ref_dq || !S1q || !S2q || !ref_dk || !S1k || !S2k) return BSP_ERR_ARG;
-  if (nd < 1 || nd > 2) return BSP_ERR_ARG;
-  if (!aligned16(ref_dq) || !aligned16(ref_dk) || !aligned16(S1q) || !aligned16(S2q) || !aligned16(S1k) || !aligned16(S2k))
-    return BSP_ERR_ALIGN;
-  AttnParams p{};
-  p.BH = B * H; p.S = S; p.nblk = (S + AT_BLK - 1) / AT_BLK; p.causal = causal ? 1 : 0; p.c = softmax_scale;
-  p.lse = lse; p.lse_out = nullptr; p.diag = diag;
-  if ((rc = set_fp8(p, f)) != BSP_OK) return rc;
-  cudaStream_t st = (cudaStream_t)stream;
-  p.dterm = dterm; p.nd = nd;
-  p.mc_ref = ref_dk; p.out0 = S1k; p.out1 = S2k;
-  if ((rc = launch_attn<AT_DKV>(q, k, v, dO, p, st)) != BSP_OK) return rc;
-  p.mc_ref = ref_dq; p.out0 = S1q; p.out1 = S2q;
-  return launch_attn<AT_DQ>(q, k, v, dO, p, st);
+  return launch_attn_mode<AT_DKV, false, true, true>(q, k, v, dO, p, st);
 }
 
 // x (bf16 [groups][group_size]) -> nearest FP8 codes at each group's own amax scale -> the decoded

@@ -127,9 +127,20 @@ int attn_dterm_impl(int B, int H, int S, int Dh, const void* dO, int dt, const f
 int attn_bwd_dterm_impl(int B, int H, int S, int Dh, int causal, float softmax_scale, const void* q, const void* k,
                         const void* v, const void* dO, int dt, const bsp_attn_fp8_t* f, const float* lse,
                         const float* dterm, float* dq, float* dk, float* dv, bsp_diag_t* diag, void* stream);
-int attn_bwd_dterm_mc(int B, int H, int S, int Dh, int causal, float softmax_scale, const void* q, const void* k,
-                      const void* v, const void* dO, int dt, const bsp_attn_fp8_t* f, const float* lse,
-                      const float* dterm, int nd, const float* ref_dq, float* S1q, float* S2q, const float* ref_dk,
-                      float* S1k, float* S2k, bsp_diag_t* diag, void* stream);
+// The draws of a fresh read go through the scores kDrawsPerPass at a time, and where (block, head) items are fewer than
+// the SMs they are spread over attn_draw_sets(BH, S, K) sets with sums of their own, [sets][BH * S * 64] per array,
+// which attn_sum_sets adds in order into S1 and S2 (n floats each).
+constexpr int kDrawsPerPass = 4;
+int attn_draw_sets(int64_t BH, int S, int K);
+int attn_sum_sets(const float* p1, const float* p2, int sets, float* S1, float* S2, size_t n, cudaStream_t st);
+
+// FP8-operand mode (attn_f8.cu): the backward of one evaluation (dv with dk only; dk or dq may be left out), and K
+// draws of the correction term (dterm [K][B*H*S]) with S1 = sum (g_k - ref), S2 = sum (g_k - ref)^2 of dQ and dK
+// written.  `partials`: 4 x attn_draw_sets(BH, S, K) x BH x S x 64 floats, unused where the sets are one.
+int attn_f8_bwd(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, const float* lse, const float* dterm, float* dq,
+                float* dk, float* dv, bsp_diag_t* diag, cudaStream_t st);
+int attn_f8_draws(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, const float* lse, const float* dterm, int K,
+                  const float* ref_dq, float* S1q, float* S2q, const float* ref_dk, float* S1k, float* S2k, float* partials,
+                  bsp_diag_t* diag, cudaStream_t st);
 
 }  // namespace bsp

@@ -526,6 +526,7 @@ struct AttnCheckBuffers {
   void* op8[4];
   uint8_t* opc[4];                                // the operands' codes (FP8-operand mode)
   float *op_amax[4], *op_scale[4];
+  float* partials;                                // sums of the sets of draws (FP8-operand mode, few (block, head) items)
   void* ws_stats;
   size_t b_stats;
 };
@@ -552,6 +553,8 @@ static size_t attn_carve(const bsp_attn_desc_t* op, int K, char* base, AttnCheck
     for (int t = 0; t < 4; ++t) {
       c.op8[t] = take(n * 2); c.opc[t] = (uint8_t*)take(n); c.op_amax[t] = (float*)take(BH * 4); c.op_scale[t] = (float*)take(BH * 4);
     }
+    const size_t sets = (size_t)attn_draw_sets((int64_t)BH, op->S, K > 0 ? K : 1);
+    if (sets > 1) c.partials = (float*)take(4 * sets * n * 4);
   }
   c.b_stats = kMaxPendingStats * kStatSlotBytes;
   c.ws_stats = take(c.b_stats);
@@ -677,10 +680,6 @@ int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t
     launch_kernel(mc_accumulate_draws_kernel, (unsigned)((rows + 255) / 256), 256, 0, st, b.d_draws, rows, K, b.d_ref, b.S1d, b.S2d,
                   rows);
     BSP_LAUNCH_CHECK();
-    for (int t = 0; t < 2; ++t) {
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S1[t], 0, n * 4, st));
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S2[t], 0, n * 4, st));
-    }
     if (!fp8) {
       // dQ: P K once (the forward kernel with K in place of V and the rows' LSE given, so it takes one
       // pass over the keys; g_pol[0] is free by now), then the K draws collapse to one elementwise pass
@@ -689,17 +688,17 @@ int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t
                     n / 4);
       BSP_LAUNCH_CHECK();
       // dK: four draws per launch
+      BSP_CHECK_CUDA(cudaMemsetAsync(b.S1[1], 0, n * 4, st));
+      BSP_CHECK_CUDA(cudaMemsetAsync(b.S2[1], 0, n * 4, st));
       for (int k0 = 0; k0 < K; k0 += kDkND) {
         const int nd = K - k0 < kDkND ? K - k0 : kDkND;
         BSP_TRY(attn_dk_diff((int)BH, S, op->causal, c, q, k, b.lse, b.d_ref, b.d_draws + (size_t)k0 * rows, nd, b.S1[1],
                              b.S2[1], diag, st));
       }
     } else {
-      // the rounded backward once per draw; dQ and dK go from the accumulators straight into their sums
-      // (two draws per launch: the scores, dP and the exponentials are formed once for both)
-      for (int k0 = 0; k0 < K; k0 += 2)
-        BSP_TRY(attn_bwd_dterm_mc(B, H, S, Dh, op->causal, c, q, k, v, dO, dt, f, b.lse, b.d_draws + (size_t)k0 * rows,
-                                  K - k0 >= 2 ? 2 : 1, b.g_ref[0], b.S1[0], b.S2[0], b.g_ref[1], b.S1[1], b.S2[1], diag, st));
+      // the rounded backward of every draw; dQ and dK go from the accumulators straight into their sums
+      BSP_TRY(attn_f8_draws((int)BH, S, op->causal, c, f, b.lse, b.d_draws, K, b.g_ref[0], b.S1[0], b.S2[0], b.g_ref[1], b.S1[1],
+                            b.S2[1], b.partials, diag, st));
     }
     BSP_TRY(pend.add(b.d_ref, b.S1d, b.S2d, (int64_t)rows, K, 1, emit(out_ids[0], BSP_READ_FRESH)));
     for (int t = 0; t < 2; ++t)
