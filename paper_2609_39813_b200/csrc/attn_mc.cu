@@ -19,11 +19,15 @@
 // Rounding an operand to bf16 now costs 2^-9 of the *difference*, not of the whole dS, so the
 // statistics see the read and not the operand format, and no per-draw gradient is ever written.
 //
-// attn_dk_diff_kernel: persistent, one CTA per SM walking (key block, head) items, heaviest first.
-// 320 threads: warp 0 TMA producer, warp 1 MMA issuer, warps 2..9 probabilities, operand scaling and
-// epilogue.  Tensor memory: S^T 128 columns, P^T operand 64, four accumulators of 64.  -LSE enters
-// S^T through one extra K = 16 product step (a tile of ones against rows holding -LSE/c as three
-// bf16 terms), as in the dK/dV kernel of the plain backward.  Every wait is bounded.
+// attn_dk_diff_kernel: persistent, one CTA per SM walking (key block, head, set of draws) items, heaviest
+// first; a CTA takes the draws of its set four at a time and adds to the sums in that order (sets as in
+// attn_f8.cu, whose sum_sets_kernel joins them).  640 threads: warps 0..15 probabilities, operand scaling and
+// epilogue (32 columns of S^T each), warp 16 TMA, warp 17 MMA issue.  Tensor memory: two S^T buffers of 128
+// columns, four accumulators of 64.  P^T goes back into the columns its thread read S^T from (two K = 16
+// steps per 32 columns, the first 16 of them), so the scores are double-buffered in the room that one buffer
+// and a separate operand would take, and S^T of a step is formed under the exponentials and stores of the
+// step before.  -LSE enters S^T through one extra K = 16 product step (a tile of ones against rows holding
+// -LSE/c as three bf16 terms), written two steps ahead, so P^T = exp2(c2 acc) needs no per-column operand.
 #include <string.h>
 
 #include <atomic>
@@ -33,12 +37,13 @@
 
 namespace bsp {
 
-constexpr int kDkThreads = 320;
-constexpr int kDkND = 4;                           // draws per launch
+constexpr int kDkThreads = 640;
+constexpr int kDkWarps = 16;
+constexpr int kDkND = kDrawsPerPass;               // draws per pass over the steps
 constexpr uint32_t kDkStages = 3;                  // ring of streamed Q tiles
+constexpr uint32_t kDkBuf = kDkND * kAtTile;       // one buffer of scaled Q tiles (also the epilogue's 64 KB of staging)
 constexpr int kDkBiasTile = AT_BLK * 16 * 2;       // 4 KB: one 128 x 16 bf16 tile of the extra K = 16 step
-// shared memory: K tiles [2], Q ring [3], two buffers of the scaled Q tiles [2][4] (the first one is
-// also the epilogue's 64 KB of staging), barriers, then the ones tile and three buffers of the -LSE tile
+// shared memory: K tiles [2], Q ring [3], scaled Q tiles [2][4], barriers, the ones tile and three -LSE tiles
 constexpr int kDkSmem = 1024 + (2 + (int)kDkStages + 2 * kDkND) * kAtTile + 1024 + 4 * kDkBiasTile;
 static_assert(kDkSmem <= 232448, "dynamic shared memory of attn_dk_diff_kernel exceeds the SM's");
 
@@ -47,8 +52,8 @@ struct DkDiffParams {
   float c;                       // softmax scale
   const float* lse;              // [BH*S]
   const float* d_ref;            // [BH*S]      the reference's correction term
-  const float* d_draws;          // [nd][BH*S]  the draws' correction terms
-  int nd;                        // draws in this launch, 1 .. kDkND (the rest contribute zeros)
+  const float* d_draws;          // [K][BH*S]   the draws' correction terms
+  int K, sets, passes;           // draws; sets per (block, head); passes of up to four draws per set
   bsp_diag_t* diag;
 };
 
@@ -66,374 +71,386 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
-  const uint32_t res_base = base;                                   // K tile of the item, two buffers
+  const uint32_t res_base = base;                                   // K tile of the pass, two buffers
   const uint32_t q0 = base + 2 * kAtTile;                           // stage s: q0 + s * kAtTile
-  const uint32_t bs0 = q0 + kDkStages * kAtTile;                    // buffer pb, draw d: bs0 + (4 pb + d) * kAtTile
-  const uint32_t bars = bs0 + 2 * kDkND * kAtTile;
-  // P^T and the scaled tiles are double-buffered (buffer = step & 1), so the probabilities of step
-  // j + 1 are formed while the accumulating product of step j runs
+  const uint32_t bs0 = q0 + kDkStages * kAtTile;                    // buffer pb, draw d: bs0 + pb * kDkBuf + d * kAtTile
+  const uint32_t bars = bs0 + 2 * kDkBuf;
   const uint32_t b_res = bars, b_res_empty = bars + 16, b_sfull = bars + 32, b_sempty = bars + 56,
-                 b_sdp_full = bars + 80, b_sdp_free = bars + 88, b_pds_ready = bars + 96 /* [2] */,
-                 b_pds_free = bars + 112 /* [2] */, b_acc = bars + 128, b_acc_free = bars + 136, b_bias = bars + 144;
+                 b_s_full = bars + 80 /* [2] */, b_op_ready = bars + 96 /* [2] */, b_op_free = bars + 112 /* [2] */,
+                 b_acc = bars + 128, b_acc_free = bars + 136, b_bias = bars + 144 /* [3] */, b_staged = bars + 184,
+                 b_stg_free = bars + 192;
   const uint32_t bias0 = bars + 1024;                               // ones tile; buffer b: the -LSE tile at 1 + b
   uint8_t* bars_gen = smem_raw + (bars - raw);
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars_gen + 176);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 180);
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars_gen + 208);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 212);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nitems = p.nblk * p.BH;
+  const int nwork = p.nblk * p.BH * p.sets;
   // the CTA's n-th item: rounds of gridDim.x items, walked forwards and backwards in turn
   auto item_at = [&](int n) -> int {
     const int b = (int)blockIdx.x, G = (int)gridDim.x;
     return n * G + ((n & 1) ? G - 1 - b : b);
   };
-  auto decode_item = [&](int w, int& blk, int& bh, int& it_begin, int& nsteps) {
-    blk = w / p.BH;                                                 // key block j: steps i = j .. nblk-1 (causal)
-    bh = w % p.BH;
+  // draws [d_begin, d_end) of the item, in passes of up to kDkND
+  auto decode = [&](int w, int& blk, int& bh, int& set, int& it_begin, int& nsteps, int& d_begin, int& d_end) {
+    set = w % p.sets;
+    const int i = w / p.sets;
+    blk = i / p.BH;                                                 // key block j: steps i = j .. nblk-1 (causal)
+    bh = i % p.BH;
     it_begin = p.causal ? blk : 0;
     nsteps = p.nblk - it_begin;
+    d_begin = set * p.passes * kDkND;
+    d_end = d_begin + p.passes * kDkND < p.K ? d_begin + p.passes * kDkND : p.K;
   };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 2; ++s) { mbar_init(b_res + 8 * s, 1); mbar_init(b_res_empty + 8 * s, 1); }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(b_res + 8 * s, 1); mbar_init(b_res_empty + 8 * s, 1); mbar_init(b_s_full + 8 * s, 1);
+      mbar_init(b_op_ready + 8 * s, kDkWarps); mbar_init(b_op_free + 8 * s, 1);
+    }
     for (uint32_t s = 0; s < kDkStages; ++s) { mbar_init(b_sfull + 8 * s, 1); mbar_init(b_sempty + 8 * s, 1); }
-    for (uint32_t s = 0; s < 3; ++s) mbar_init(b_bias + 8 * s, 8);
-    mbar_init(b_sdp_full, 1); mbar_init(b_sdp_free, 8);
-    for (int s = 0; s < 2; ++s) { mbar_init(b_pds_ready + 8 * s, 8); mbar_init(b_pds_free + 8 * s, 1); }
-    mbar_init(b_acc, 1); mbar_init(b_acc_free, 8);
+    for (uint32_t s = 0; s < 3; ++s) mbar_init(b_bias + 8 * s, 4);
+    mbar_init(b_acc, 1); mbar_init(b_acc_free, kDkWarps);
+    mbar_init(b_staged, kDkWarps); mbar_init(b_stg_free, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+  if (threadIdx.x < 256) {
+    // constant parts of the four extra tiles: thread t clears 16 bytes of each (row t & 127, half t >> 7); the
+    // first three columns of the ones tile are 1
+    const int t0 = (int)threadIdx.x;
+    const uint32_t off = (uint32_t)((t0 & 127) >> 3) * 256u + (uint32_t)(t0 >> 7) * 128u + (uint32_t)(t0 & 7) * 16u;
+#pragma unroll
+    for (uint32_t t = 0; t < 4; ++t) {
+      const bool one = t == 0 && t0 < 128;
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %3};" ::"r"(bias0 + t * kDkBiasTile + off),
+                   "r"(one ? 0x3F803F80u : 0u), "r"(one ? 0x00003F80u : 0u), "r"(0u) : "memory");
+    }
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (warp == 17) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  // S^T 128 columns, two P^T operands of 64, the accumulator of draw d at t_acc + 64 d
-  const uint32_t t_s = tmem, t_p = tmem + 128, t_acc = tmem + 256;
+  // two S^T buffers of 128 columns (P^T in place), the accumulator of draw d at t_acc + 64 d
+  const uint32_t t_s = tmem, t_acc = tmem + 256;
 
   const uint32_t id_s = make_idesc(1u, 1u, 128, 128);                          // A, B K-major
   const uint32_t id_acc = make_idesc(1u, 1u, 128, 64 * kDkND) | (1u << 16);    // A from tensor memory, B MN-major
 
-  if (warp == 0) {
-    // ------------------------------------------------ TMA producer
-    if (lane == 0) {
-      tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k);
-      bool ok = true;
-      uint32_t itg = 0;
-      int item = 0;
-      for (int w = item_at(0); w < nitems && ok; w = item_at(++item)) {
-        int blk, bh, it_begin, nsteps;
-        decode_item(w, blk, bh, it_begin, nsteps);
-        const uint32_t rb = item & 1u, rph = (item >> 1) & 1u;
-        if (!mbar_wait(b_res_empty + 8 * rb, rph ^ 1u, abort_flag)) { ok = false; break; }
-        mbar_expect_tx(b_res + 8 * rb, kAtTile);
-        tma_load_3d(res_base + rb * kAtTile, &tm_k, b_res + 8 * rb, 0, blk * AT_BLK, bh);
-        for (int it = 0; it < nsteps; ++it, ++itg) {
-          const uint32_t s = itg % kDkStages, ph = (itg / kDkStages) & 1u;
-          if (!mbar_wait(b_sempty + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
-          mbar_expect_tx(b_sfull + 8 * s, kAtTile);
-          tma_load_3d(q0 + s * kAtTile, &tm_q, b_sfull + 8 * s, 0, (it_begin + it) * AT_BLK, bh);
+  // the block starts with 640 x 96 registers: the control warpgroup keeps 32 a thread, the others take 112
+  if (warp >= kDkWarps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+    if (warp == 16) {
+      // ------------------------------------------------ TMA producer
+      if (lane == 0) {
+        tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k);
+        bool ok = true;
+        uint32_t itg = 0, vi = 0;                                   // global step, pass
+        int n = 0;
+        for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+          int blk, bh, set, it_begin, nsteps, d0, d_end;
+          decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
+          for (; d0 < d_end && ok; d0 += kDkND, ++vi) {
+            const uint32_t rb = vi & 1u;
+            if (!mbar_wait(b_res_empty + 8 * rb, ((vi >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+            mbar_expect_tx(b_res + 8 * rb, kAtTile);
+            tma_load_3d(res_base + rb * kAtTile, &tm_k, b_res + 8 * rb, 0, blk * AT_BLK, bh);
+            for (int it = 0; it < nsteps; ++it, ++itg) {
+              const uint32_t s = itg % kDkStages, ph = (itg / kDkStages) & 1u;
+              if (!mbar_wait(b_sempty + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
+              mbar_expect_tx(b_sfull + 8 * s, kAtTile);
+              tma_load_3d(q0 + s * kAtTile, &tm_q, b_sfull + 8 * s, 0, (it_begin + it) * AT_BLK, bh);
+            }
+          }
         }
+        if (!ok) for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let copies in flight land
       }
-      if (!ok) for (int i = 0; i < 200; ++i) __nanosleep(1000);     // let copies in flight land
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    } else if (warp == 17) {
+      // ------------------------------------------------ MMA issuer (the whole warp walks, one lane issues)
+      const uint32_t leader = elect_one() ? 1u : 0u;
+      auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
+        return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag));
+      };
       bool ok = true;
-      uint32_t itg = 0;
-      int item = 0;
-      for (int w = item_at(0); w < nitems && ok; w = item_at(++item)) {
-        int blk, bh, it_begin, nsteps;
-        decode_item(w, blk, bh, it_begin, nsteps);
-        const uint32_t rb = item & 1u, iph = (item >> 1) & 1u, aph = (uint32_t)item & 1u;
-        const uint32_t k_t = res_base + rb * kAtTile;
-        if (!mbar_wait(b_res + 8 * rb, iph, abort_flag)) { ok = false; break; }
-        // S^T = K Q^T of global step jt (rows = keys), plus the K = 16 step that subtracts LSE / c.
-        // Issued one step ahead: the other warps hand the S^T columns back as soon as they hold them
-        // in registers.
-        auto issue_s = [&](uint32_t jt) -> bool {
-          const uint32_t s = jt % kDkStages, ph = (jt / kDkStages) & 1u;
-          if (!mbar_wait(b_sfull + 8 * s, ph, abort_flag)) return false;
-          if (!mbar_wait(b_sdp_free, (jt & 1u) ^ 1u, abort_flag)) return false;
-          tc_fence_after();
-          const uint64_t a = make_smem_desc(k_t), b = make_smem_desc(q0 + s * kAtTile);
+      uint32_t itg = 0, vi = 0;
+      int n = 0;
+      for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+        int blk, bh, set, it_begin, nsteps, d0, d_end;
+        decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
+        for (; d0 < d_end && ok; d0 += kDkND, ++vi) {
+          const uint32_t rb = vi & 1u;
+          const uint32_t k_t = res_base + rb * kAtTile;
+          if (!wait_all(b_res + 8 * rb, (vi >> 1) & 1u)) { ok = false; break; }
+          // S^T = K Q^T of global step jt (rows = keys), plus the K = 16 step that subtracts LSE / c, one step
+          // ahead; its buffer is free once the product of two steps ago has read P^T there
+          auto issue_s = [&](uint32_t jt) -> bool {
+            const uint32_t s = jt % kDkStages, sb = jt & 1u, bb = jt % 3u;
+            if (!wait_all(b_sfull + 8 * s, (jt / kDkStages) & 1u)) return false;
+            if (!wait_all(b_op_free + 8 * sb, ((jt >> 1) & 1u) ^ 1u)) return false;
+            if (!wait_all(b_bias + 8 * bb, (jt / 3u) & 1u)) return false;
+            tc_fence_after();
+            const uint64_t a = make_smem_desc(k_t), b = make_smem_desc(q0 + s * kAtTile);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) tc_mma<false>(t_s, a + 2u * k, b + 2u * k, id_s, k != 0);
-          const uint32_t bb = jt % 3u;
-          if (!mbar_wait(b_bias + 8 * bb, (jt / 3u) & 1u, abort_flag)) return false;
-          tc_mma<false>(t_s, make_smem_desc_k16(bias0), make_smem_desc_k16(bias0 + (1u + bb) * kDkBiasTile), id_s, 1u);
-          tc_commit(b_sdp_full);
-          return true;
-        };
-        if (nsteps > 0) ok = issue_s(itg);
-        for (int it = 0; it < nsteps && ok; ++it) {
-          const uint32_t jg = itg + (uint32_t)it;
-          const uint32_t s = jg % kDkStages, pb = jg & 1u, pph = (jg >> 1) & 1u;
-          if (it + 1 < nsteps && !issue_s(jg + 1)) { ok = false; break; }
-          if (!mbar_wait(b_pds_ready + 8 * pb, pph, abort_flag)) { ok = false; break; }
-          tc_fence_after();
-          // the accumulators are free once the epilogue of the item before has read them
-          if (it == 0 && !mbar_wait(b_acc_free, aph ^ 1u, abort_flag)) { ok = false; break; }
-          // all four draws at once: P^T (tensor memory, eight columns per 16 queries) against the four
-          // scaled Q tiles side by side (MN-major, one 128-byte atom of 64 columns per draw)
-          const uint64_t bq = make_smem_desc_mn(bs0 + pb * kDkND * kAtTile, (uint32_t)kAtTile);
+            for (int k = 0; k < 4; ++k) tc_mma_l<false>(leader, t_s + 128u * sb, a + 2u * k, b + 2u * k, id_s, k != 0);
+            tc_mma_l<false>(leader, t_s + 128u * sb, make_smem_desc_k16(bias0), make_smem_desc_k16(bias0 + (1u + bb) * kDkBiasTile), id_s, 1u);
+            tc_commit_l(leader, b_s_full + 8 * sb);
+            return true;
+          };
+          ok = issue_s(itg);
+          for (int it = 0; it < nsteps && ok; ++it) {
+            const uint32_t jg = itg + (uint32_t)it, s = jg % kDkStages, pb = jg & 1u;
+            if (it + 1 < nsteps && !issue_s(jg + 1)) { ok = false; break; }
+            if (!wait_all(b_op_ready + 8 * pb, (jg >> 1) & 1u)) { ok = false; break; }
+            // the accumulators are free once the epilogue of the pass before has read them
+            if (it == 0 && !wait_all(b_acc_free, (vi & 1u) ^ 1u)) { ok = false; break; }
+            tc_fence_after();
+            // all four draws at once: P^T (tensor memory, eight columns per 16 queries, 16 of every 32 columns)
+            // against the four scaled Q tiles side by side (MN-major, one 128-byte atom of 64 columns per draw)
+            const uint64_t bq = make_smem_desc_mn(bs0 + pb * kDkBuf, (uint32_t)kAtTile);
 #pragma unroll
-          for (int k = 0; k < 8; ++k) tc_mma_ts(t_acc, t_p + 64u * pb + 8u * k, bq + 128u * k, id_acc, (it != 0) | (k != 0));
-          tc_commit(b_pds_free + 8 * pb);
-          tc_commit(b_sempty + 8 * s);
+            for (uint32_t k = 0; k < 8; ++k)
+              tc_mma_ts_l<false>(leader, t_acc, t_s + 128u * pb + 32u * (k >> 1) + 8u * (k & 1u), bq + 128u * k, id_acc,
+                                 (it != 0 || k != 0) ? 1u : 0u);
+            tc_commit_l(leader, b_op_free + 8 * pb);
+            tc_commit_l(leader, b_sempty + 8 * s);
+          }
+          itg += (uint32_t)nsteps;
+          if (ok) {
+            tc_commit_l(leader, b_res_empty + 8 * rb);
+            tc_commit_l(leader, b_acc);
+          }
         }
-        itg += (uint32_t)nsteps;
-        if (ok) tc_commit(b_acc);
       }
     }
   } else {
     // ------------------------------------------------ probabilities, operand scaling, epilogue
-    const int q4 = warp & 3, h = (warp - 2) >> 2;
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+    const int q4 = warp & 3, h = warp >> 2;                         // lane quarter; 32 of the 128 columns
     const int r = q4 * 32 + lane;                                   // row of the 128-row block: a key (S^T), a query (Q tile)
     const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
-    const int ts = (int)threadIdx.x - 64;                           // 0 .. 255
-    {
-      // constant parts of the four extra tiles: thread ts clears 16 bytes of each (row ts & 127, half
-      // ts >> 7); the first three columns of the ones tile are 1
-      const uint32_t off = (uint32_t)((ts & 127) >> 3) * 256u + (uint32_t)(ts >> 7) * 128u + (uint32_t)(ts & 7) * 16u;
-#pragma unroll
-      for (uint32_t t = 0; t < 4; ++t) {
-        const bool one = t == 0 && ts < 128;
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %3};" ::"r"(bias0 + t * kDkBiasTile + off),
-                     "r"(one ? 0x3F803F80u : 0u), "r"(one ? 0x00003F80u : 0u), "r"(0u) : "memory");
-      }
-      named_bar_sync(1, 256);
-    }
+    const uint32_t row_off = (uint32_t)r * 128u;
     const float c2 = p.c * kLog2e;
     const float bias_mul = -kLog2e / c2;                            // the accumulator holds s - LSE / c
-    const size_t rows_total = (size_t)p.BH * p.S;
-    bool ok = true;
-    bool store_pending = false;                                     // the epilogue's bulk adds may still read the staging
-    uint32_t bias_written = 0, itg = 0;
-    int item = 0;
-    // the -LSE row of one step: threads ts < 128 own query ts of the tile
+    const size_t rows = (size_t)p.BH * p.S;
+    bool ok = true, store_pending = false;
+    uint32_t bias_written = 0, jt = 0, vi = 0, stg_ph = 0;          // -LSE rows written; global step, pass; last epilogue's phase
+    // the pass whose accumulators have not been read yet
+    bool due = false, e_first = true;
+    int e_blk = 0, e_bh = 0, e_set = 0;
+    // the -LSE row of one step (the warps of column quarter 0: thread r writes query r of the tile)
     auto bias_fetch = [&](int tbh, int step) -> float {
-      if (ts >= 128) return 0.f;
-      const int q = step * AT_BLK + ts;
+      const int q = step * AT_BLK + r;
       return q < p.S ? ldg(p.lse + (size_t)tbh * p.S + q) : 0.f;
     };
-    // (fenced = false: the caller issues the proxy fence itself, after other stores that need one too)
-    auto bias_put = [&](uint32_t jt, float rawv, bool fenced = true) {
-      if (ts < 128) {
-        const float x = rawv * bias_mul;
-        const __nv_bfloat16 h1 = __float2bfloat16_rn(x);
-        const float r1 = x - __bfloat162float(h1);
-        const __nv_bfloat16 h2 = __float2bfloat16_rn(r1);
-        const __nv_bfloat16 h3 = __float2bfloat16_rn(r1 - __bfloat162float(h2));
-        const uint32_t w0 = (uint32_t)__bfloat16_as_ushort(h1) | ((uint32_t)__bfloat16_as_ushort(h2) << 16);
-        const uint32_t w1 = (uint32_t)__bfloat16_as_ushort(h3);
-        const uint32_t tile = bias0 + (1u + jt % 3u) * kDkBiasTile;
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %3};" ::"r"(tile + (uint32_t)(ts >> 3) * 256u + (uint32_t)(ts & 7) * 16u),
-                     "r"(w0), "r"(w1), "r"(0u) : "memory");
-        if (fenced) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      }
-      if (!fenced) return;
-      __syncwarp();
-      if (lane == 0) mbar_arrive(b_bias + 8 * (jt % 3u));
+    auto bias_put = [&](uint32_t j, float rawv) {
+      const float x = rawv * bias_mul;
+      const __nv_bfloat16 h1 = __float2bfloat16_rn(x);
+      const float r1 = x - __bfloat162float(h1);
+      const __nv_bfloat16 h2 = __float2bfloat16_rn(r1);
+      const __nv_bfloat16 h3 = __float2bfloat16_rn(r1 - __bfloat162float(h2));
+      const uint32_t w0 = (uint32_t)__bfloat16_as_ushort(h1) | ((uint32_t)__bfloat16_as_ushort(h2) << 16);
+      const uint32_t w1 = (uint32_t)__bfloat16_as_ushort(h3);
+      const uint32_t tile = bias0 + (1u + j % 3u) * kDkBiasTile;
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %3};" ::"r"(tile + (uint32_t)(r >> 3) * 256u + (uint32_t)(r & 7) * 16u),
+                   "r"(w0), "r"(w1), "r"(0u) : "memory");
     };
-    for (int w = item_at(0); w < nitems && ok; w = item_at(++item)) {
-      int blk, bh, it_begin, nsteps;
-      decode_item(w, blk, bh, it_begin, nsteps);
-      const uint32_t rb = (uint32_t)item & 1u, aph = (uint32_t)item & 1u;
-      // the next item's head and first step: its first two -LSE rows are written under this item's tail
-      int nx_bh = 0, nx_begin = 0, nx_total = 0;
-      {
-        const int wn = item_at(item + 1);
-        if (wn < nitems) { int nb; decode_item(wn, nb, nx_bh, nx_begin, nx_total); }
-      }
-      while (bias_written < itg + (uint32_t)(nsteps < 2 ? nsteps : 2)) {
-        const int l = (int)(bias_written - itg);
-        bias_put(bias_written, bias_fetch(bh, it_begin + l));
-        ++bias_written;
-      }
-      auto bias_target = [&](int it, int& tbh, int& tstep) -> bool {
-        const int t = it + 2;
-        if (t < nsteps) { tbh = bh; tstep = it_begin + t; return true; }
-        if (t - nsteps < nx_total) { tbh = nx_bh; tstep = nx_begin + (t - nsteps); return true; }
-        return false;
-      };
-      const int key = blk * AT_BLK + r;                             // this thread's row of S^T
-      for (int it = 0; it < nsteps && ok; ++it) {
-        const int step = it_begin + it;
-        const uint32_t jt = itg + (uint32_t)it, ip = jt & 1u, pb = jt & 1u, pph = (jt >> 1) & 1u;
-        const uint32_t t_pb = t_p + 64u * pb, bsb = bs0 + pb * kDkND * kAtTile;
-        // this step's correction terms of query step*128 + r: requested here, first used after the
-        // exponentials (nothing may depend on these loads before then, or the in-order warp sits out
-        // their latency)
-        float draw_raw[kDkND], dref_raw;
-        const bool q_in = step * AT_BLK + r < p.S;
-        {
-          const size_t qi = (size_t)bh * p.S + (q_in ? step * AT_BLK + r : 0);
-          dref_raw = ldg(p.d_ref + qi);
+    // Reads the accumulators of pass `v` (its last global step: last) and adds the draws' sum and sum of squares to
+    // S1 and S2 (the first pass of an item sets them), staged in that step's operand buffer, which no product reads
+    // any more.
+    auto epilogue = [&](uint32_t v, uint32_t last) -> bool {
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait(b_acc, v & 1u, abort_flag))) return false;
+      tc_fence_after();
+      const uint32_t stg = bs0 + (last & 1u) * kDkBuf;
+      float s1[16], s2[16];
 #pragma unroll
-          for (int d = 0; d < kDkND; ++d) draw_raw[d] = d < p.nd ? ldg(p.d_draws + (size_t)d * rows_total + qi) : 0.f;
-        }
-        int bias_bh = 0, bias_step = 0;
-        const bool bias_due = bias_written == jt + 2u && bias_target(it, bias_bh, bias_step);
-        float bias_next = 0.f;
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_sdp_full, ip, abort_flag));
-        if (!ok) break;
-        tc_fence_after();
-        uint32_t sv[64];
-        tmem_ld32_nowait(t_s + lane_off + h * 64, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
-        tmem_ld32_nowait(t_s + lane_off + h * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
-        // the step's Q tile has landed long ago (S^T read it); this thread still has to see its barrier
-        // before it reads the tile further down: the test goes out here, under the tensor-memory load
-        const uint32_t q_seen = mbar_try_wait(b_sfull + 8 * (jt % kDkStages), (jt / kDkStages) & 1u);
+      for (int e = 0; e < 16; ++e) s1[e] = s2[e] = 0.f;
+#pragma unroll
+      for (int d = 0; d < kDkND; ++d) {                             // (draws that a pass does not have add zeros)
+        uint32_t a[16];
+        tmem_ld16(t_acc + 64u * d + lane_off + h * 16, a);
         tmem_wait_ld();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(b_sdp_free);
-        if (bias_due) bias_next = bias_fetch(bias_bh, bias_step);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          const float g = __uint_as_float(a[e]);
+          s1[e] += g;
+          s2[e] = fmaf(g, g, s2[e]);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_acc_free);
+      // box h >> 1 of 32 columns, four 16-byte chunks of this thread's half of it
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const uint32_t at = stg + (uint32_t)(h >> 1) * 16384u + row_off + ((uint32_t)(((h & 1) * 4 + t) ^ (r & 7)) << 4);
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(s1[4 * t]), "f"(s1[4 * t + 1]), "f"(s1[4 * t + 2]),
+                     "f"(s1[4 * t + 3]) : "memory");
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + 32768u), "f"(s2[4 * t]), "f"(s2[4 * t + 1]),
+                     "f"(s2[4 * t + 2]), "f"(s2[4 * t + 3]) : "memory");
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_staged);
+      if (warp == 0 && !__all_sync(0xFFFFFFFFu, mbar_wait(b_staged, v & 1u, abort_flag))) return false;
+      if (warp == 0 && lane == 0) {
+        const int y = e_blk * AT_BLK, z = e_set * p.BH + e_bh;
+        if (e_first) {
+          tma_store_3d(&tm_s1, stg, 0, y, z);
+          tma_store_3d(&tm_s1, stg + 16384u, 32, y, z);
+          tma_store_3d(&tm_s2, stg + 32768u, 0, y, z);
+          tma_store_3d(&tm_s2, stg + 49152u, 32, y, z);
+        } else {
+          tma_store_wait_all();                                     // this thread's stores of the passes before have landed
+          tma_reduce_add_3d(&tm_s1, stg, 0, y, z);
+          tma_reduce_add_3d(&tm_s1, stg + 16384u, 32, y, z);
+          tma_reduce_add_3d(&tm_s2, stg + 32768u, 0, y, z);
+          tma_reduce_add_3d(&tm_s2, stg + 49152u, 32, y, z);
+        }
+        tma_store_commit();
+      }
+      store_pending = true;
+      stg_ph = v & 1u;
+      return true;
+    };
 
-        const int col0 = step * AT_BLK + h * 64;                    // first query of this thread's 64 columns
-        const bool edge = (p.causal && blk == step) || (blk + 1) * AT_BLK > p.S || (step + 1) * AT_BLK > p.S;
-        auto valid_at = [&](int j) {
-          const int qy = col0 + j;
-          return key < p.S && qy < p.S && (!p.causal || key <= qy);
-        };
-        uint32_t pk[32];
-        auto pair_at = [&](int j, bool masked) {
-          float a0, a1;
-          mul_f32x2(a0, a1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), c2, c2);
-          if (masked) {
-            if (!valid_at(j)) a0 = -INFINITY;
-            if (!valid_at(j + 1)) a1 = -INFINITY;
+    int n = 0;
+    for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+      int blk, bh, set, it_begin, nsteps, d0, d_end;
+      decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
+      const int d_first = d0;
+      for (; d0 < d_end && ok; d0 += kDkND, ++vi) {
+        const int nd = d_end - d0 < kDkND ? d_end - d0 : kDkND;
+        // the next pass's head and steps: its first two -LSE rows are written under this pass's tail
+        int nx_bh = bh, nx_begin = it_begin, nx_total = nsteps;
+        if (d0 + kDkND >= d_end) {
+          const int wn = item_at(n + 1);
+          nx_total = 0;
+          if (wn < nwork) { int b0, s0, x0, x1; decode(wn, b0, nx_bh, s0, nx_begin, nx_total, x0, x1); }
+        }
+        if (h == 0) {
+          while (bias_written < jt + (uint32_t)(nsteps < 2 ? nsteps : 2)) {
+            bias_put(bias_written, bias_fetch(bh, it_begin + (int)(bias_written - jt)));
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b_bias + 8 * (bias_written % 3u));
+            ++bias_written;
           }
-          pk[j >> 1] = pack_bf16x2(ex2_approx(a0), ex2_approx(a1));
-        };
-        if (!edge) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 2) pair_at(j, false);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; j += 2) pair_at(j, true);
         }
-        // this buffer of the P^T operand and of the scaled tiles is free once the product of two steps
-        // ago has read it
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_pds_free + 8 * pb, pph ^ 1u, abort_flag));
-        if (!ok) break;
-        tmem_st16(t_pb + lane_off + h * 32, *reinterpret_cast<const uint32_t(*)[16]>(&pk[0]));
-        if (!edge) {
+        const int key = blk * AT_BLK + r;                           // this thread's row of S^T
+        for (int it = 0; it < nsteps && ok; ++it, ++jt) {
+          const int step = it_begin + it;
+          const uint32_t pb = jt & 1u, t_pb = t_s + 128u * pb + lane_off + 32u * (uint32_t)h, bsb = bs0 + pb * kDkBuf + row_off;
+          // this step's correction terms of query step*128 + r: requested here, first used after the exponentials
+          float draw_raw[kDkND], dref_raw;
+          const bool q_in = step * AT_BLK + r < p.S;
+          {
+            const size_t qi = (size_t)bh * p.S + (q_in ? step * AT_BLK + r : 0);
+            dref_raw = ldg(p.d_ref + qi);
 #pragma unroll
-          for (int j = 32; j < 64; j += 2) pair_at(j, false);
-        } else {
+            for (int d = 0; d < kDkND; ++d) draw_raw[d] = d < nd ? ldg(p.d_draws + (size_t)(d0 + d) * rows + qi) : 0.f;
+          }
+          // the -LSE row two steps ahead
+          const int bt = it + 2;
+          const bool bias_due = h == 0 && bias_written == jt + 2u && (bt < nsteps || bt - nsteps < nx_total);
+          float bias_next = 0.f;
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_s_full + 8 * pb, (jt >> 1) & 1u, abort_flag));
+          if (!ok) break;
+          tc_fence_after();
+          uint32_t sv[32];
+          tmem_ld32_nowait(t_pb, sv);
+          if (bias_due) bias_next = bt < nsteps ? bias_fetch(bh, it_begin + bt) : bias_fetch(nx_bh, nx_begin + (bt - nsteps));
+          // the step's Q tile has landed (S^T read it); this thread still has to see its barrier before it reads it
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_sfull + 8 * (jt % kDkStages), (jt / kDkStages) & 1u, abort_flag));
+          tmem_wait_ld();
+          if (!ok) break;
+          const int col0 = step * AT_BLK + h * 32;                  // first query of this thread's 32 columns
+          const bool edge = (p.causal && blk == step) || (blk + 1) * AT_BLK > p.S || (step + 1) * AT_BLK > p.S;
+          uint32_t pk[16];
+          if (!edge) {
 #pragma unroll
-          for (int j = 32; j < 64; j += 2) pair_at(j, true);
-        }
-        tmem_st16(t_pb + lane_off + h * 32 + 16, *reinterpret_cast<const uint32_t(*)[16]>(&pk[16]));
-        // ---- the B operand: row r of the streamed Q tile times this row's factor of each draw, written
-        // at the same (swizzled) place of the draw's tile.  Thread (r, h) takes the four 16-byte chunks
-        // whose logical index is 4h .. 4h+3; chunk c of row r sits at position c ^ (r & 7), so the lanes
-        // of a warp (consecutive rows) spread over all banks.
-        if (store_pending) {
-          if (warp == 2 && lane == 0) tma_store_wait_read();
-          named_bar_sync(2, 256);
-          store_pending = false;
-        }
-        {
-          const uint32_t s = jt % kDkStages, ph = (jt / kDkStages) & 1u;
-          if (!__all_sync(0xFFFFFFFFu, q_seen)) {
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_sfull + 8 * s, ph, abort_flag));
+            for (int j = 0; j < 32; j += 2) {
+              float a0, a1;
+              mul_f32x2(a0, a1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), c2, c2);
+              pk[j >> 1] = pack_bf16x2(ex2_approx(a0), ex2_approx(a1));
+            }
+          } else {
+            // valid queries of this key: first <= column < end
+            const int first = (p.causal ? key : 0) - col0, end = (key < p.S ? p.S : 0) - col0;
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+              float a0, a1;
+              mul_f32x2(a0, a1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), c2, c2);
+              if (j < first || j >= end) a0 = -INFINITY;
+              if (j + 1 < first || j + 1 >= end) a1 = -INFINITY;
+              pk[j >> 1] = pack_bf16x2(ex2_approx(a0), ex2_approx(a1));
+            }
+          }
+          tmem_st16(t_pb, pk);                                      // in place: the first 16 of the thread's own 32 columns
+          if (store_pending) {                                      // an epilogue's staging has left this buffer
+            if (warp == 0 && lane == 0) { tma_store_wait_read(); mbar_arrive(b_stg_free); }
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_stg_free, stg_ph, abort_flag));
+            if (!ok) break;
+            store_pending = false;
+          }
+          // ---- the B operand: row r of the streamed Q tile times this row's factor of each draw, written at the same
+          // (swizzled) place of the draw's tile.  Thread (r, h) takes the 16-byte chunks 2h and 2h + 1; chunk c of row r
+          // sits at position c ^ (r & 7), so the lanes of a warp (consecutive rows) spread over all banks.  (The
+          // buffer is free: S^T of this step was only formed after the product of two steps ago.)
+          {
+            uint32_t f2[kDkND];
+            asm volatile("" : "+f"(dref_raw));                      // keeps the first use of the loads here
+#pragma unroll
+            for (int d = 0; d < kDkND; ++d) {
+              asm volatile("" : "+f"(draw_raw[d]));
+              const float fk = (q_in && d < nd) ? -p.c * (draw_raw[d] - dref_raw) : 0.f;
+              f2[d] = pack_bf16x2(fk, fk);
+            }
+            const uint32_t qt = q0 + (jt % kDkStages) * kAtTile + row_off;
+#pragma unroll
+            for (int cch = 0; cch < 2; ++cch) {
+              uint32_t a0, a1, a2, a3;
+              const uint32_t off = (uint32_t)((2 * h + cch) ^ (r & 7)) << 4;
+              asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(a0), "=r"(a1), "=r"(a2), "=r"(a3) : "r"(qt + off));
+#pragma unroll
+              for (int d = 0; d < kDkND; ++d)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(bsb + (uint32_t)d * kAtTile + off),
+                             "r"(mul_bf16x2(a0, f2[d])), "r"(mul_bf16x2(a1, f2[d])), "r"(mul_bf16x2(a2, f2[d])),
+                             "r"(mul_bf16x2(a3, f2[d])) : "memory");
+            }
+          }
+          if (bias_due) {
+            asm volatile("" : "+f"(bias_next));
+            bias_put(bias_written, bias_next);
+          }
+          tmem_wait_st();
+          tc_fence_before();
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(b_op_ready + 8 * pb);
+            if (bias_due) mbar_arrive(b_bias + 8 * (bias_written % 3u));
+          }
+          if (bias_due) ++bias_written;
+          if (it == 0 && due) {
+            ok = epilogue(vi - 1u, jt - 1u);
+            due = false;
             if (!ok) break;
           }
-          // the row factors -c (D_k - D*) of the draws (zero for a draw this launch does not have)
-          uint32_t f2[kDkND];
-          asm volatile("" : "+f"(dref_raw));
-#pragma unroll
-          for (int d = 0; d < kDkND; ++d) {
-            asm volatile("" : "+f"(draw_raw[d]));
-            const float fk = (q_in && d < p.nd) ? -p.c * (draw_raw[d] - dref_raw) : 0.f;
-            f2[d] = pack_bf16x2(fk, fk);
-          }
-          const uint32_t row_off = (uint32_t)r * 128u;
-#pragma unroll
-          for (int cch = 0; cch < 4; ++cch) {
-            uint32_t a0, a1, a2, a3;
-            const uint32_t off = row_off + ((uint32_t)((4 * h + cch) ^ (r & 7)) << 4);
-            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(a0), "=r"(a1), "=r"(a2), "=r"(a3) : "r"(q0 + s * kAtTile + off));
-#pragma unroll
-            for (int d = 0; d < kDkND; ++d)
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(bsb + (uint32_t)d * kAtTile + off),
-                           "r"(mul_bf16x2(a0, f2[d])), "r"(mul_bf16x2(a1, f2[d])), "r"(mul_bf16x2(a2, f2[d])),
-                           "r"(mul_bf16x2(a3, f2[d])) : "memory");
-          }
         }
-        tmem_wait_st();
-        tc_fence_before();
-        if (bias_due) {
-          // the -LSE row two steps ahead goes out under the same proxy fence as the scaled tiles (a
-          // fence waits for the thread's shared-memory stores to drain: one per step, not two)
-          asm volatile("" : "+f"(bias_next));                       // keeps the first use of the load here
-          bias_put(bias_written, bias_next, false);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(b_pds_ready + 8 * pb);
-          if (bias_due) mbar_arrive(b_bias + 8 * (bias_written % 3u));
-        }
-        if (bias_due) ++bias_written;
-      }
-      itg += (uint32_t)nsteps;
-      // ---- epilogue: the four accumulators hold the draws' differences; their sum and sum of squares
-      // leave through the (now idle) scaled-tile buffers as bulk adds into S1 and S2
-      if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_acc, aph, abort_flag));
-      if (ok) {
-        tc_fence_after();
-        float s1[32], s2[32];
-#pragma unroll
-        for (int e = 0; e < 32; ++e) s1[e] = s2[e] = 0.f;
-#pragma unroll
-        for (int d = 0; d < kDkND; ++d) {
-          uint32_t a[32];
-          tmem_ld32(t_acc + 64u * d + lane_off + h * 32, a);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const float v = __uint_as_float(a[e]);
-            s1[e] += v;
-            s2[e] = fmaf(v, v, s2[e]);
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(b_acc_free);
-        if (warp == 2 && lane == 0) mbar_arrive(b_res_empty + 8 * rb);   // the item's K tile is no longer read
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const uint32_t off = (uint32_t)h * 16384u + (uint32_t)r * 128u + ((uint32_t)(t ^ (r & 7)) << 4);
-          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(bs0 + off), "f"(s1[4 * t]), "f"(s1[4 * t + 1]),
-                       "f"(s1[4 * t + 2]), "f"(s1[4 * t + 3]) : "memory");
-          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(bs0 + 32768u + off), "f"(s2[4 * t]),
-                       "f"(s2[4 * t + 1]), "f"(s2[4 * t + 2]), "f"(s2[4 * t + 3]) : "memory");
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        named_bar_sync(3, 256);
-        if (warp == 2 && lane == 0) {
-          tma_reduce_add_3d(&tm_s1, bs0, 0, blk * AT_BLK, bh);
-          tma_reduce_add_3d(&tm_s1, bs0 + 16384u, 32, blk * AT_BLK, bh);
-          tma_reduce_add_3d(&tm_s2, bs0 + 32768u, 0, blk * AT_BLK, bh);
-          tma_reduce_add_3d(&tm_s2, bs0 + 49152u, 32, blk * AT_BLK, bh);
-          tma_store_commit();
-        }
-        store_pending = true;
+        e_blk = blk; e_bh = bh; e_set = set; e_first = d0 == d_first;
+        due = true;
       }
     }
-    if (warp == 2 && lane == 0) tma_store_wait_all();
+    if (ok && due) ok = epilogue(vi - 1u, jt - 1u);
+    if (warp == 0 && lane == 0) tma_store_wait_all();
   }
 
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag && p.diag) atomicMax(&p.diag->status, (int)BSP_ERR_TIMEOUT);
-  if (warp == 1) {
+  if (warp == 17) {
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, 512);
@@ -490,32 +507,35 @@ __global__ void mc_accumulate_draws_kernel(const float* g, size_t stride, int nd
   S2[i] = s2;
 }
 
-// nd (1 .. 4) draws of the dK difference, added to the running sums.
+// The sums over the K draws of the dK difference; `partials` as in attn_f8_draws (two arrays of it).
 static int attn_dk_diff(int BH, int S, int causal, float c, const void* q, const void* k, const float* lse,
-                        const float* d_ref, const float* d_draws, int nd, float* S1k, float* S2k, bsp_diag_t* diag,
-                        cudaStream_t st) {
-  if (nd < 1 || nd > kDkND) return BSP_ERR_ARG;
+                        const float* d_ref, const float* d_draws, int K, float* S1k, float* S2k, float* partials,
+                        bsp_diag_t* diag, cudaStream_t st) {
+  DkDiffParams p;
+  p.BH = BH; p.S = S; p.nblk = (S + AT_BLK - 1) / AT_BLK; p.causal = causal ? 1 : 0; p.c = c;
+  p.lse = lse; p.d_ref = d_ref; p.d_draws = d_draws; p.K = K; p.diag = diag;
+  p.sets = attn_draw_sets(BH, S, K);
+  p.passes = ((K + kDkND - 1) / kDkND + p.sets - 1) / p.sets;
+  const size_t n = (size_t)BH * S * AT_D;
+  float* o1 = p.sets > 1 ? partials : S1k;
+  float* o2 = p.sets > 1 ? partials + (size_t)p.sets * n : S2k;
   CUtensorMap mq, mk, m1, m2;
   int rc;
   if ((rc = make_head_map(&mq, q, BH, S)) != BSP_OK) return rc;
   if ((rc = make_head_map(&mk, k, BH, S)) != BSP_OK) return rc;
-  if ((rc = make_out_map(&m1, S1k, BH, S)) != BSP_OK) return rc;
-  if ((rc = make_out_map(&m2, S2k, BH, S)) != BSP_OK) return rc;
+  if ((rc = make_out_map(&m1, o1, BH * p.sets, S)) != BSP_OK) return rc;
+  if ((rc = make_out_map(&m2, o2, BH * p.sets, S)) != BSP_OK) return rc;
   static std::atomic<bool> attr_set_dev[kMaxDevices];
   std::atomic<bool>& attr_set = attr_set_dev[device_slot()];
   if (!attr_set.load(std::memory_order_acquire)) {
     BSP_CHECK_CUDA(cudaFuncSetAttribute(attn_dk_diff_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDkSmem));
     attr_set.store(true, std::memory_order_release);
   }
-  DkDiffParams p;
-  p.BH = BH; p.S = S; p.nblk = (S + AT_BLK - 1) / AT_BLK; p.causal = causal ? 1 : 0; p.c = c;
-  p.lse = lse; p.d_ref = d_ref; p.d_draws = d_draws; p.nd = nd; p.diag = diag;
   const int nsm = sm_count_or_default();
-  const int64_t nitems = (int64_t)p.nblk * BH;
-  const unsigned grid = (unsigned)(nitems < nsm ? nitems : nsm);
-  launch_kernel(attn_dk_diff_kernel, grid, kDkThreads, kDkSmem, st, mq, mk, m1, m2, p);
+  const int64_t nwork = (int64_t)p.nblk * BH * p.sets;
+  launch_kernel(attn_dk_diff_kernel, (unsigned)(nwork < nsm ? nwork : nsm), kDkThreads, kDkSmem, st, mq, mk, m1, m2, p);
   BSP_LAUNCH_CHECK();
-  return BSP_OK;
+  return p.sets > 1 ? attn_sum_sets(o1, o2, p.sets, S1k, S2k, n, st) : BSP_OK;
 }
 
 struct AttnCheckBuffers {
@@ -526,7 +546,7 @@ struct AttnCheckBuffers {
   void* op8[4];
   uint8_t* opc[4];                                // the operands' codes (FP8-operand mode)
   float *op_amax[4], *op_scale[4];
-  float* partials;                                // sums of the sets of draws (FP8-operand mode, few (block, head) items)
+  float* partials;                                // sums of the sets of draws (where (block, head) items are few)
   void* ws_stats;
   size_t b_stats;
 };
@@ -553,9 +573,9 @@ static size_t attn_carve(const bsp_attn_desc_t* op, int K, char* base, AttnCheck
     for (int t = 0; t < 4; ++t) {
       c.op8[t] = take(n * 2); c.opc[t] = (uint8_t*)take(n); c.op_amax[t] = (float*)take(BH * 4); c.op_scale[t] = (float*)take(BH * 4);
     }
-    const size_t sets = (size_t)attn_draw_sets((int64_t)BH, op->S, K > 0 ? K : 1);
-    if (sets > 1) c.partials = (float*)take(4 * sets * n * 4);
   }
+  const size_t sets = (size_t)attn_draw_sets((int64_t)BH, op->S, K > 0 ? K : 1);
+  if (sets > 1) c.partials = (float*)take((op->fp8_operands ? 4 : 2) * sets * n * 4);
   c.b_stats = kMaxPendingStats * kStatSlotBytes;
   c.ws_stats = take(c.b_stats);
   if (out) *out = c;
@@ -687,14 +707,8 @@ int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t
       launch_kernel(attn_dq_sums_kernel, (unsigned)((n / 4 + 255) / 256), 256, 0, st, b.g_pol[0], b.S1d, b.S2d, c, b.S1[0], b.S2[0],
                     n / 4);
       BSP_LAUNCH_CHECK();
-      // dK: four draws per launch
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S1[1], 0, n * 4, st));
-      BSP_CHECK_CUDA(cudaMemsetAsync(b.S2[1], 0, n * 4, st));
-      for (int k0 = 0; k0 < K; k0 += kDkND) {
-        const int nd = K - k0 < kDkND ? K - k0 : kDkND;
-        BSP_TRY(attn_dk_diff((int)BH, S, op->causal, c, q, k, b.lse, b.d_ref, b.d_draws + (size_t)k0 * rows, nd, b.S1[1],
-                             b.S2[1], diag, st));
-      }
+      // dK: all draws in one launch
+      BSP_TRY(attn_dk_diff((int)BH, S, op->causal, c, q, k, b.lse, b.d_ref, b.d_draws, K, b.S1[1], b.S2[1], b.partials, diag, st));
     } else {
       // the rounded backward of every draw; dQ and dK go from the accumulators straight into their sums
       BSP_TRY(attn_f8_draws((int)BH, S, op->causal, c, f, b.lse, b.d_draws, K, b.g_ref[0], b.S1[0], b.S2[0], b.g_ref[1], b.S1[1],
