@@ -7,16 +7,22 @@
 // The scores, dP and the exponentials do not depend on the draw, so a step forms them once for up to
 // four draws.  What limits the number of draws is tensor memory: S and dP take 128 columns each, an
 // accumulator 64; the operands dS_k therefore go through shared memory (16 KB of codes per draw and
-// step, double-buffered) and the four accumulators fill the other 256 columns.  A thread owns a query row
+// step) and the four accumulators fill the other 256 columns.  A thread owns a query row
 // in both kernels, so LSE and the D_k are scalars of the thread: the dQ kernel reads the codes K-major
 // (rows = queries), the dK / dV kernel reads the same layout MN-major (rows = the contraction).
 //
-// Nothing the softmax warps wait for is on their own path: S and dP of the next step are issued as soon as
-// they hold this step's in registers, operand buffers alternate, and an item's epilogue is taken after the
-// next item's first step, when its last products have long finished.
+// Little that the softmax warps wait for is on their own path: S and dP of the next step are issued as soon as
+// they hold this step's in registers; a step's products run under the exponentials of the next, so one buffer
+// of operands is enough; an item's accumulators are read after the next item's first step.  The running sums of
+// an item stay in shared memory, in the place of a second buffer, from its first pass to its last, and leave
+// in one store.  (Bulk reduce-adds per pass instead: 64 KB each, 3000 cycles of every pass spent waiting for
+// their staging to be read.)
 //
-// Measured at B H = 128, S = 2048, causal, 32 draws: both kernels 4.5 ms; a launch per pair of draws, with the
-// operands in tensor memory and eight softmax warps, 8.2 ms (the whole check 9.54 -> 6.32 ms).
+// Measured at B H = 128, S = 2048, causal, 32 draws: both kernels 4.35 ms (a launch per pair of draws, with the
+// operands in tensor memory and eight softmax warps, 8.2; two operand buffers and reduce-adds 4.5), the whole
+// check 9.54 -> 6.15 ms.  Of a step's 4600 cycles the conversions take 1700 and the exponentials 1200, one after the
+// other in all warps (a start half a step apart does not last: a step's products need every warp's codes); 450
+// are a pass's end, the rest waits for barriers and tensor memory.
 //
 // Persistent CTA, one per SM, walking (block, head, set of draws) items, heaviest first.  A CTA takes the
 // draws of its set four at a time and adds to the sums in that order; where there are fewer (block, head)
@@ -37,11 +43,27 @@ constexpr int kF8ND = kDrawsPerPass;               // draws per pass over the st
 constexpr uint32_t kF8Stages = 3;                  // ring of streamed tile pairs
 constexpr uint32_t kF8Tile = AT_BLK * AT_D;        // 8 KB: 128 rows of 64 codes
 constexpr uint32_t kF8Op = AT_BLK * AT_BLK;        // 16 KB: one operand, 128 x 128 codes
-constexpr uint32_t kF8Buf = kF8ND * kF8Op;         // one buffer of operands (the epilogue's staging: two FP32 tiles)
-// resident tiles [2][2], ring [3][2], operand buffers [2][4], barriers
-constexpr int kF8Smem = 1024 + 4 * kF8Tile + kF8Stages * 2 * kF8Tile + 2 * kF8Buf + 512;
+constexpr uint32_t kF8Buf = kF8ND * kF8Op;         // the step's operands
+constexpr uint32_t kF8Out = AT_BLK * AT_D * 4;     // 32 KB: an FP32 output tile, as two boxes of 32 columns
+// operands [4], two output tiles (the running sums), resident tiles [2][2], ring [3][2], barriers
+constexpr int kF8Smem = 1024 + kF8Buf + 2 * kF8Out + 4 * kF8Tile + kF8Stages * 2 * kF8Tile + 512;
 static_assert(kF8Smem <= 232448, "dynamic shared memory of attn_f8_kernel exceeds the SM's");
-static_assert(kF8Buf == 2 * AT_BLK * AT_D * 4, "an operand buffer holds the two staged outputs");
+
+// Two pairs of floats to four FP8 codes in one word (nearest, saturating).
+template <int FMT>
+__device__ __forceinline__ uint32_t f8_encode4(uint64_t ab, uint64_t cd) {
+  uint32_t r;
+  float a, b, c, d;
+  f2_unpack(ab, a, b);
+  f2_unpack(cd, c, d);
+  if (FMT == BSP_E4M3)
+    asm("{\n\t.reg .b16 lo, hi;\n\tcvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\tcvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
+        "mov.b32 %0, {lo, hi};\n\t}" : "=r"(r) : "f"(a), "f"(b), "f"(c), "f"(d));
+  else
+    asm("{\n\t.reg .b16 lo, hi;\n\tcvt.rn.satfinite.e5m2x2.f32 lo, %2, %1;\n\tcvt.rn.satfinite.e5m2x2.f32 hi, %4, %3;\n\t"
+        "mov.b32 %0, {lo, hi};\n\t}" : "=r"(r) : "f"(a), "f"(b), "f"(c), "f"(d));
+  return r;
+}
 
 struct AttnF8Params {
   int BH, S, nblk, causal;
@@ -68,12 +90,12 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
-  const uint32_t op0 = base;                                        // operand buffer pb: op0 + pb * kF8Buf
-  const uint32_t res_base = op0 + 2 * kF8Buf;                       // resident pair rb: res_base + rb * 2 * kF8Tile
+  const uint32_t op0 = base, out0 = op0 + kF8Buf;                   // operand o: op0 + o * kF8Op
+  const uint32_t res_base = out0 + 2 * kF8Out;                      // resident pair rb: res_base + rb * 2 * kF8Tile
   const uint32_t str0 = res_base + 4 * kF8Tile;                     // stage s: str0 + s * 2 * kF8Tile
   const uint32_t bars = str0 + kF8Stages * 2 * kF8Tile;
   const uint32_t b_res = bars, b_res_empty = bars + 16, b_sfull = bars + 32, b_sempty = bars + 56, b_sdp_full = bars + 80,
-                 b_sdp_free = bars + 88, b_op_ready = bars + 96 /* [2] */, b_op_free = bars + 112 /* [2] */, b_acc = bars + 128,
+                 b_sdp_free = bars + 88, b_op_ready = bars + 96, b_op_free = bars + 112, b_acc = bars + 128,
                  b_acc_free = bars + 136, b_staged = bars + 144, b_stg_free = bars + 152;
   uint8_t* bars_gen = smem_raw + (bars - raw);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars_gen + 176);
@@ -108,8 +130,8 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
       mbar_init(b_res + 8 * s, 1); mbar_init(b_res_empty + 8 * s, 1);
-      mbar_init(b_op_ready + 8 * s, kF8Warps); mbar_init(b_op_free + 8 * s, 1);
     }
+    mbar_init(b_op_ready, kF8Warps); mbar_init(b_op_free, 1);
     for (uint32_t s = 0; s < kF8Stages; ++s) { mbar_init(b_sfull + 8 * s, 1); mbar_init(b_sempty + 8 * s, 1); }
     mbar_init(b_sdp_full, 1); mbar_init(b_sdp_free, kF8Warps);
     mbar_init(b_acc, 1); mbar_init(b_acc_free, kF8Warps);
@@ -198,9 +220,9 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           };
           ok = issue_sdp(itg);
           for (int it = 0; it < nsteps && ok; ++it) {
-            const uint32_t jg = itg + (uint32_t)it, s = jg % kF8Stages, pb = jg & 1u;
+            const uint32_t jg = itg + (uint32_t)it, s = jg % kF8Stages;
             if (it + 1 < nsteps && !issue_sdp(jg + 1)) { ok = false; break; }
-            if (!wait_all(b_op_ready + 8 * pb, (jg >> 1) & 1u)) { ok = false; break; }
+            if (!wait_all(b_op_ready, jg & 1u)) { ok = false; break; }
             // the accumulators are free once the epilogue of the pass before has read them
             if (it == 0 && !wait_all(b_acc_free, (vi & 1u) ^ 1u)) { ok = false; break; }
             tc_fence_after();
@@ -209,7 +231,7 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             const uint32_t acc = it == 0 ? 0u : 1u;
             // 128 = 4 x 32 along the contraction: 32 bytes of a row (K-major A) or 32 rows (MN-major A) per step
             auto products = [&](uint32_t o, uint64_t b, uint32_t id) {
-              const uint32_t op = op0 + pb * kF8Buf + o * kF8Op;
+              const uint32_t op = op0 + o * kF8Op;
               const uint64_t a = MODE == AT_DKV ? make_smem_desc_mn(op, 16384u) : make_smem_desc(op);
 #pragma unroll
               for (uint32_t i = 0; i < 4; ++i)
@@ -221,7 +243,7 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               products(0u, bs, id_ds);
               if (DV) products(1u, bdo, id_p);
             }
-            tc_commit_l(leader, b_op_free + 8 * pb);
+            tc_commit_l(leader, b_op_free);
             tc_commit_l(leader, b_sempty + 8 * s);
           }
           itg += (uint32_t)nsteps;
@@ -241,41 +263,57 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const size_t rows = (size_t)p.BH * p.S;
     const uint32_t row_off = (uint32_t)r * 128u;
     const uint32_t ch0 = (uint32_t)((2 * h) ^ (r & 7)) << 4, ch1 = (uint32_t)((2 * h + 1) ^ (r & 7)) << 4;
-    bool ok = true, store_pending = false;
-    uint32_t jt = 0, vi = 0, stg_ph = 0;                            // global step, pass; phase of the last epilogue
+    bool ok = true;
+    uint32_t jt = 0, vi = 0, stored = 0;                            // global step, pass; items whose outputs have been sent off
     // the pass whose accumulators have not been read yet
     bool due = false;
     int e_blk = 0, e_bh = 0, e_set = 0, e_nd = 0;
-    bool e_first = true;
-    // Reads the accumulators of pass `v` (its last global step: last) and sends off its outputs, staged in that
-    // step's operand buffer, which no product reads any more.
-    auto epilogue = [&](uint32_t v, uint32_t last) -> bool {
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(b_acc, v & 1u, abort_flag))) return false;
-      tc_fence_after();
-      const float inv_q = __fdiv_rn(1.0f, ldg(p.sc_q + e_bh)), inv_k = __fdiv_rn(1.0f, ldg(p.sc_k + e_bh));
-      const float mul = p.c * ((MODE == AT_DKV ? inv_q : inv_k) / p.ds_scale);
-      const uint32_t stg = op0 + (last & 1u) * kF8Buf;
+    bool e_first = true, e_last = true;
+    // Reads the accumulators of pass `v` into the item's output tiles; after its last pass the tiles leave.
+    auto epilogue = [&](uint32_t v) -> bool {
       const int orow = e_blk * AT_BLK + r;                          // a key (dK / dV) or a query
-      // box h >> 1 of 32 columns, four 16-byte chunks of this thread's half of it
-      const uint32_t box = stg + (uint32_t)(h >> 1) * 16384u + row_off;
-      auto chunk = [&](int t) -> uint32_t { return box + ((uint32_t)(((h & 1) * 4 + t) ^ (r & 7)) << 4); };
+      float ref[MC ? 16 : 1];
       if (MC) {
-        float s1[16], s2[16], ref[16];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
           if (orow < p.S) f = ldg(reinterpret_cast<const float4*>(p.mc_ref + ((size_t)e_bh * p.S + orow) * AT_D + h * 16) + t);
-          ref[4 * t] = f.x; ref[4 * t + 1] = f.y; ref[4 * t + 2] = f.z; ref[4 * t + 3] = f.w;
+          ref[MC ? 4 * t : 0] = f.x; ref[MC ? 4 * t + 1 : 0] = f.y; ref[MC ? 4 * t + 2 : 0] = f.z; ref[MC ? 4 * t + 3 : 0] = f.w;
         }
+      }
+      const float inv_q = __fdiv_rn(1.0f, ldg(p.sc_q + e_bh)), inv_k = __fdiv_rn(1.0f, ldg(p.sc_k + e_bh));
+      const float mul = p.c * ((MODE == AT_DKV ? inv_q : inv_k) / p.ds_scale);
+      if (e_first && stored) {                                      // the stores of the item before have read the tiles
+        if (warp == 0 && lane == 0) { tma_store_wait_read(); mbar_arrive(b_stg_free); }
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(b_stg_free, (stored - 1u) & 1u, abort_flag))) return false;
+      }
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait(b_acc, v & 1u, abort_flag))) return false;
+      tc_fence_after();
+      // box h >> 1 of 32 columns, four 16-byte chunks of this thread's half of it
+      const uint32_t box = out0 + (uint32_t)(h >> 1) * 16384u + row_off;
+      auto chunk = [&](int t) -> uint32_t { return box + ((uint32_t)(((h & 1) * 4 + t) ^ (r & 7)) << 4); };
+      auto put4 = [&](uint32_t at, float a, float b, float c, float d) {
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+      };
+      if (MC) {
+        float s1[16], s2[16];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) s1[e] = s2[e] = 0.f;
+        for (int t = 0; t < 4; ++t) {
+          if (e_first) {
+#pragma unroll
+            for (int e = 4 * t; e < 4 * t + 4; ++e) s1[e] = s2[e] = 0.f;
+          } else {
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(s1[4 * t]), "=f"(s1[4 * t + 1]), "=f"(s1[4 * t + 2]), "=f"(s1[4 * t + 3]) : "r"(chunk(t)));
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(s2[4 * t]), "=f"(s2[4 * t + 1]), "=f"(s2[4 * t + 2]), "=f"(s2[4 * t + 3]) : "r"(chunk(t) + kF8Out));
+          }
+        }
         for (int d = 0; d < e_nd; ++d) {
           uint32_t a[16];
           tmem_ld16(t_acc + 64u * (uint32_t)d + lane_off + h * 16, a);
           tmem_wait_ld();
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
-            const float g = __fmul_rn(__uint_as_float(a[e]), mul) - ref[e];   // zero where the draw is the reference
+            const float g = __fmul_rn(__uint_as_float(a[e]), mul) - ref[MC ? e : 0];   // zero where the draw is the reference
             s1[e] += g;
             s2[e] = fmaf(g, g, s2[e]);
           }
@@ -285,11 +323,10 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (lane == 0) mbar_arrive(b_acc_free);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(chunk(t)), "f"(s1[4 * t]), "f"(s1[4 * t + 1]),
-                       "f"(s1[4 * t + 2]), "f"(s1[4 * t + 3]) : "memory");
-          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(chunk(t) + 32768u), "f"(s2[4 * t]), "f"(s2[4 * t + 1]),
-                       "f"(s2[4 * t + 2]), "f"(s2[4 * t + 3]) : "memory");
+          put4(chunk(t), s1[4 * t], s1[4 * t + 1], s1[4 * t + 2], s1[4 * t + 3]);
+          put4(chunk(t) + kF8Out, s2[4 * t], s2[4 * t + 1], s2[4 * t + 2], s2[4 * t + 3]);
         }
+        if (!e_last) return true;
       } else {
         const float mul_v = DV ? __fdiv_rn(1.0f, ldg(p.sc_do + e_bh)) / p.p_scale : 0.f;
 #pragma unroll
@@ -300,9 +337,8 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const float m = o == 0 ? mul : mul_v;
 #pragma unroll
           for (int t = 0; t < 4; ++t)
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(chunk(t) + 32768u * o), "f"(__uint_as_float(a[4 * t]) * m),
-                         "f"(__uint_as_float(a[4 * t + 1]) * m), "f"(__uint_as_float(a[4 * t + 2]) * m),
-                         "f"(__uint_as_float(a[4 * t + 3]) * m) : "memory");
+            put4(chunk(t) + kF8Out * o, __uint_as_float(a[4 * t]) * m, __uint_as_float(a[4 * t + 1]) * m,
+                 __uint_as_float(a[4 * t + 2]) * m, __uint_as_float(a[4 * t + 3]) * m);
         }
         tc_fence_before();
         __syncwarp();
@@ -311,36 +347,23 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(b_staged);
-      if (warp == 0 && !__all_sync(0xFFFFFFFFu, mbar_wait(b_staged, v & 1u, abort_flag))) return false;
-      if (warp == 0 && lane == 0) {
-        const int y = e_blk * AT_BLK;
-        if (MC) {
-          const int z = e_set * p.BH + e_bh;
-          if (e_first) {
-            tma_store_3d(&tm_o0, stg, 0, y, z);
-            tma_store_3d(&tm_o0, stg + 16384u, 32, y, z);
-            tma_store_3d(&tm_o1, stg + 32768u, 0, y, z);
-            tma_store_3d(&tm_o1, stg + 49152u, 32, y, z);
-          } else {
-            tma_store_wait_all();                                   // this thread's stores of the passes before have landed
-            tma_reduce_add_3d(&tm_o0, stg, 0, y, z);
-            tma_reduce_add_3d(&tm_o0, stg + 16384u, 32, y, z);
-            tma_reduce_add_3d(&tm_o1, stg + 32768u, 0, y, z);
-            tma_reduce_add_3d(&tm_o1, stg + 49152u, 32, y, z);
+      if (warp == 0) {
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(b_staged, stored & 1u, abort_flag))) return false;
+        if (lane == 0) {
+          // MC: S1, S2; else dQ, or dK and dV
+          const CUtensorMap* m0 = !MC && MODE == AT_DKV ? &tm_o1 : &tm_o0;
+          const CUtensorMap* m1 = !MC && MODE == AT_DKV ? &tm_o0 : &tm_o1;
+          const int y = e_blk * AT_BLK, z = e_set * p.BH + e_bh;
+          tma_store_3d(m0, out0, 0, y, z);
+          tma_store_3d(m0, out0 + 16384u, 32, y, z);
+          if (MC || DV) {
+            tma_store_3d(m1, out0 + kF8Out, 0, y, z);
+            tma_store_3d(m1, out0 + kF8Out + 16384u, 32, y, z);
           }
-        } else {
-          const CUtensorMap* mo = MODE == AT_DKV ? &tm_o1 : &tm_o0;
-          tma_store_3d(mo, stg, 0, y, e_bh);
-          tma_store_3d(mo, stg + 16384u, 32, y, e_bh);
-          if (DV) {
-            tma_store_3d(&tm_o0, stg + 32768u, 0, y, e_bh);
-            tma_store_3d(&tm_o0, stg + 49152u, 32, y, e_bh);
-          }
+          tma_store_commit();
         }
-        tma_store_commit();
       }
-      store_pending = true;
-      stg_ph = v & 1u;
+      ++stored;
       return true;
     };
 
@@ -352,6 +375,8 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const float inv_q = __fdiv_rn(1.0f, ldg(p.sc_q + bh)), inv_k = __fdiv_rn(1.0f, ldg(p.sc_k + bh));
       const float inv_v = __fdiv_rn(1.0f, ldg(p.sc_v + bh)), inv_do = __fdiv_rn(1.0f, ldg(p.sc_do + bh));
       const float c2 = p.c * kLog2e * inv_q * inv_k, dp_mul = inv_do * inv_v;   // scores and dP arrive as products of codes
+      const uint64_t c2_2 = f2_pack(c2, c2), dp_mul_2 = f2_pack(dp_mul, dp_mul);
+      const uint64_t ds_2 = f2_pack(p.ds_scale, p.ds_scale), ps_2 = f2_pack(p.p_scale, p.p_scale);
       for (; d0 < d_end && ok; d0 += kF8ND, ++vi) {
         const int nd = MC ? (d_end - d0 < kF8ND ? d_end - d0 : kF8ND) : 1;
         // LSE and the draws' correction terms of the thread's query: of the item (dQ), or of the step (dK / dV,
@@ -367,12 +392,11 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         fetch(MODE == AT_DKV ? it_begin : blk);
         for (int it = 0; it < nsteps && ok; ++it, ++jt) {
           const int step = it_begin + it;
-          const uint32_t pb = jt & 1u;
           const int qblk = MODE == AT_DKV ? step : blk, kblk = MODE == AT_DKV ? blk : step;
-          const float lse2 = lse_q * kLog2e;
-          float dk[kF8ND];
+          const uint64_t nlse_2 = f2_pack(-lse_q * kLog2e, -lse_q * kLog2e);
+          uint64_t ndk_2[kF8ND];
 #pragma unroll
-          for (int d = 0; d < kF8ND; ++d) dk[d] = dd[d];
+          for (int d = 0; d < kF8ND; ++d) ndk_2[d] = f2_pack(-dd[d], -dd[d]);
           ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_sdp_full, jt & 1u, abort_flag));
           if (!ok) break;
           tc_fence_after();
@@ -384,38 +408,37 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           __syncwarp();
           if (lane == 0) mbar_arrive(b_sdp_free);
           if (MODE == AT_DKV && it + 1 < nsteps) fetch(step + 1);
-          // the probabilities, in place; masking only on the diagonal block and where the sequence ends
+          // the probabilities, in place (masking only on the diagonal block and where the sequence ends)
           const int key0 = kblk * AT_BLK + h * 32, qy = qblk * AT_BLK + r;
           const bool edge = (p.causal && kblk >= qblk) || (kblk + 1) * AT_BLK > p.S || (qblk + 1) * AT_BLK > p.S;
-          if (!edge) {
+          uint64_t pr[16], dp[16];                                  // pairs of columns
 #pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-              float a0, a1;
-              fma_f32x2(a0, a1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), c2, c2, -lse2, -lse2);
-              sv[j] = __float_as_uint(ex2_approx(a0)); sv[j + 1] = __float_as_uint(ex2_approx(a1));
-            }
-          } else {
+          for (int j = 0; j < 16; ++j) {
+            pr[j] = f2_fma(f2_pack(__uint_as_float(sv[2 * j]), __uint_as_float(sv[2 * j + 1])), c2_2, nlse_2);
+            dp[j] = f2_pack(__uint_as_float(dv[2 * j]), __uint_as_float(dv[2 * j + 1]));
+          }
+          if (edge) {
             // the last valid key of this row, relative to the thread's first column
             const int last = (qy < p.S ? (p.causal && qy < p.S - 1 ? qy : p.S - 1) : -1) - key0;
 #pragma unroll
-            for (int j = 0; j < 32; j += 2) {
+            for (int j = 0; j < 16; ++j) {
               float a0, a1;
-              fma_f32x2(a0, a1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), c2, c2, -lse2, -lse2);
-              if (j > last) a0 = -INFINITY;
-              if (j + 1 > last) a1 = -INFINITY;
-              sv[j] = __float_as_uint(ex2_approx(a0)); sv[j + 1] = __float_as_uint(ex2_approx(a1));
+              f2_unpack(pr[j], a0, a1);
+              if (2 * j > last) a0 = -INFINITY;
+              if (2 * j + 1 > last) a1 = -INFINITY;
+              pr[j] = f2_pack(a0, a1);
             }
           }
-          // the staging of an epilogue has left this buffer / the products of two steps ago have read it
-          if (store_pending) {
-            if (warp == 0 && lane == 0) { tma_store_wait_read(); mbar_arrive(b_stg_free); }
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_stg_free, stg_ph, abort_flag));
-            if (!ok) break;
-            store_pending = false;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            float a0, a1;
+            f2_unpack(pr[j], a0, a1);
+            pr[j] = f2_pack(ex2_approx(a0), ex2_approx(a1));
           }
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_op_free + 8 * pb, ((jt >> 1) & 1u) ^ 1u, abort_flag));
+          // the products of the step before have read the operands
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(b_op_free, (jt & 1u) ^ 1u, abort_flag));
           if (!ok) break;
-          const uint32_t op = op0 + pb * kF8Buf + row_off;
+          const uint32_t op = op0 + row_off;
           auto put = [&](uint32_t o, const uint32_t (&w8)[8]) {
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(op + o * kF8Op + ch0), "r"(w8[0]), "r"(w8[1]), "r"(w8[2]), "r"(w8[3]) : "memory");
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(op + o * kF8Op + ch1), "r"(w8[4]), "r"(w8[5]), "r"(w8[6]), "r"(w8[7]) : "memory");
@@ -423,49 +446,35 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           if (DV) {
             uint32_t w8[8];
 #pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-              float f0, f1, f2, f3;
-              mul_f32x2(f0, f1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), p.p_scale, p.p_scale);
-              mul_f32x2(f2, f3, __uint_as_float(sv[j + 2]), __uint_as_float(sv[j + 3]), p.p_scale, p.p_scale);
-              w8[j >> 2] = f8_encode_rn_pair_inrange<BSP_E4M3>(f0, f1) | (f8_encode_rn_pair_inrange<BSP_E4M3>(f2, f3) << 16);
-            }
+            for (int j = 0; j < 8; ++j) w8[j] = f8_encode4<BSP_E4M3>(f2_mul(pr[2 * j], ps_2), f2_mul(pr[2 * j + 1], ps_2));
             put(1u, w8);
           }
 #pragma unroll
-          for (int j = 0; j < 32; j += 2) {                         // P ds_scale: once for all draws
-            float f0, f1;
-            mul_f32x2(f0, f1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), p.ds_scale, p.ds_scale);
-            sv[j] = __float_as_uint(f0); sv[j + 1] = __float_as_uint(f1);
-          }
+          for (int j = 0; j < 16; ++j) pr[j] = f2_mul(pr[j], ds_2);  // P ds_scale: once for all draws
 #pragma unroll
           for (int d = 0; d < (MC ? kF8ND : 1); ++d) {
             if (MC && d >= nd) break;
             uint32_t w8[8];
 #pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-              float t0, t1, t2, t3;
-              fma_f32x2(t0, t1, __uint_as_float(dv[j]), __uint_as_float(dv[j + 1]), dp_mul, dp_mul, -dk[d], -dk[d]);
-              fma_f32x2(t2, t3, __uint_as_float(dv[j + 2]), __uint_as_float(dv[j + 3]), dp_mul, dp_mul, -dk[d], -dk[d]);
-              mul_f32x2(t0, t1, __uint_as_float(sv[j]), __uint_as_float(sv[j + 1]), t0, t1);
-              mul_f32x2(t2, t3, __uint_as_float(sv[j + 2]), __uint_as_float(sv[j + 3]), t2, t3);
-              w8[j >> 2] = f8_encode_rn_pair_inrange<BSP_E5M2>(t0, t1) | (f8_encode_rn_pair_inrange<BSP_E5M2>(t2, t3) << 16);
-            }
+            for (int j = 0; j < 8; ++j)
+              w8[j] = f8_encode4<BSP_E5M2>(f2_mul(pr[2 * j], f2_fma(dp[2 * j], dp_mul_2, ndk_2[d])),
+                                           f2_mul(pr[2 * j + 1], f2_fma(dp[2 * j + 1], dp_mul_2, ndk_2[d])));
             put((uint32_t)d, w8);
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
-          if (lane == 0) mbar_arrive(b_op_ready + 8 * pb);
+          if (lane == 0) mbar_arrive(b_op_ready);
           if (it == 0 && due) {
-            ok = epilogue(vi - 1u, jt - 1u);
+            ok = epilogue(vi - 1u);
             due = false;
             if (!ok) break;
           }
         }
-        e_blk = blk; e_bh = bh; e_set = set; e_nd = nd; e_first = d0 == d_first;
+        e_blk = blk; e_bh = bh; e_set = set; e_nd = nd; e_first = d0 == d_first; e_last = d0 + kF8ND >= d_end;
         due = true;
       }
     }
-    if (ok && due) ok = epilogue(vi - 1u, jt - 1u);
+    if (ok && due) ok = epilogue(vi - 1u);
     if (warp == 0 && lane == 0) tma_store_wait_all();
   }
 
