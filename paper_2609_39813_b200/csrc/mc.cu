@@ -101,6 +101,26 @@ bool rule_valid(const bsp_verdict_rule_t* r) {
          r->qprime_fail >= r->qprime_hold && r->r_fail >= r->r_hold;
 }
 
+// A block per slot, a warp per field: lane l sums the blocks l, l + 32, ... in order, then the lanes in pairs.
+__global__ void __launch_bounds__(32 * kStatFields)
+mc_stats_sum_kernel(const double* slots, StatBlocks blocks, double* out) {
+  grid_dependency();
+  const int f = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* p = slots + (size_t)blockIdx.x * kStatSlotDoubles + f;
+  double a = 0.0;
+  for (int b = lane; b < blocks.n[blockIdx.x]; b += 32) {
+    const double v = ldg(p + (size_t)b * kStatFields);
+    a = f == 5 ? fmax(a, v) : a + v;
+  }
+  a = f == 5 ? warp_max_d(a) : warp_sum_d(a);
+  if (lane == 0) out[(size_t)blockIdx.x * kStatFields + f] = a;
+}
+int mc_stats_sum_slots(const double* slots, const StatBlocks& blocks, int count, double* out, cudaStream_t st) {
+  launch_kernel(mc_stats_sum_kernel, count, 32 * kStatFields, 0, st, slots, blocks, out);
+  BSP_LAUNCH_CHECK();
+  return BSP_OK;
+}
+
 // Launches the statistics pass over n elements into one slot of block partials; returns the number
 // of blocks whose partials the slot then holds.
 int mc_stats_launch(const float* g_ref, const float* g, const float* S2, int64_t n, int K, int fresh,
