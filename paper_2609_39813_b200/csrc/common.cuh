@@ -187,6 +187,39 @@ __device__ __forceinline__ uint32_t f8_encode(float v, uint32_t U, DiagCounters&
   return sign | (base + up);
 }
 
+// Four stochastic roundings at once, the codes packed in the order of the values: what f8_encode gives for each.  In the
+// format's normal range the up-rounding is a carry: with d dropped bits, U < rem 2^(32 - d) exactly when
+// rem > U >> (32 - d), i.e. when adding 2^d - 1 - (U >> (32 - d)) to the FP32 pattern carries into the kept bits; so a
+// thread whose four values all lie there takes no branch per value (3001 x 1552 FP32, LayerNorm chain, generator and
+// both code layouts: 18.2 -> 16.6 us; 8.4 M attention outputs: 11.6 -> 9 us).
+template <int FMT>
+__device__ __forceinline__ uint32_t f8_encode4_sr(const float (&v)[4], const uint4& w, DiagCounters& dc) {
+  using F = F8<FMT>;
+  constexpr int d = 23 - F::MB;
+  const uint32_t U[4] = {w.x, w.y, w.z, w.w};
+  uint32_t b[4], a[4], far = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    b[i] = __float_as_uint(v[i]);
+    a[i] = b[i] & 0x7FFFFFFFu;
+    far = max(far, a[i] - F::MINNORM_BITS);                         // (below the smallest normal value: wraps)
+  }
+  if (far < F::FMAX_BITS - F::MINNORM_BITS) {
+    uint32_t c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      // the smallest normal value has the code 1 << MB; the code's seven bits go to bits 24 .. 30
+      const uint32_t t = a[i] + ((1u << 23) - F::MINNORM_BITS + ((1u << d) - 1u)) - (U[i] >> (32 - d));
+      c[i] = ((t << (24 - d)) & 0x7F000000u) | (b[i] & 0x80000000u);
+    }
+    return __byte_perm(__byte_perm(c[0], c[1], 0x0073), __byte_perm(c[2], c[3], 0x0073), 0x5410);
+  }
+  uint32_t packed = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) packed |= f8_encode<FMT, true>(v[i], U[i], dc) << (8 * i);
+  return packed;
+}
+
 // Value of the stochastic rounding of v as FP32, i.e. decode(encode_SR(v)) without the detour
 // through the code: in the normal range the FP32 pattern is truncated and bumped in place.
 template <int FMT>

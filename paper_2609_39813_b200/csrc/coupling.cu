@@ -76,12 +76,14 @@ cp_forward_kernel(int kind, const void* x, int64_t T, int64_t C, const float* ga
       const size_t i = (size_t)t * C + c;
       float u[4];
       cp_chain(kind, load4<DT>(x, i), ldg(rstd + t), kind == BSP_LAYERNORM ? ldg(mean + t) : 0.f, g4, b4, u);
-      uint4 w = make_uint4(0, 0, 0, 0);
-      if (SR) w = philox_block(key, (uint64_t)i >> 2, key.c2);
-      const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+      const float v[4] = {__fmul_rn(u[0], scale), __fmul_rn(u[1], scale), __fmul_rn(u[2], scale), __fmul_rn(u[3], scale)};
       uint32_t packed = 0;
+      if (SR) {
+        packed = f8_encode4_sr<FMT>(v, philox_block(key, (uint64_t)i >> 2, key.c2), dc);
+      } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) packed |= f8_encode<FMT, SR>(__fmul_rn(u[e], scale), ww[e], dc) << (8 * e);
+        for (int e = 0; e < 4; ++e) packed |= f8_encode<FMT, false>(v[e], 0u, dc) << (8 * e);
+      }
       const uint2 q = f8_to_bf16x4<FMT>(packed);
       *reinterpret_cast<uint2*>(uq + i) = q;
       if (uq_a) {
@@ -161,11 +163,8 @@ cp_sums_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
       }
       float u[4], q4[4], dec[4];
       cp_chain(kind, xv, ldg(rstd + t), kind == BSP_LAYERNORM ? ldg(mean + t) : 0.f, g4, b4, u);
-      const uint4 wd = philox_block(key, (uint64_t)i >> 2, key.c2);
-      const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
-      uint32_t packed = 0;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) packed |= f8_encode<FMT, true>(__fmul_rn(u[e], scale), ww[e], dc) << (8 * e);
+      const float v[4] = {__fmul_rn(u[0], scale), __fmul_rn(u[1], scale), __fmul_rn(u[2], scale), __fmul_rn(u[3], scale)};
+      const uint32_t packed = f8_encode4_sr<FMT>(v, philox_block(key, (uint64_t)i >> 2, key.c2), dc);
       f8_decode4<FMT>(packed, dec);
       bf16x4_to_float(qv, q4);
       const float d4[4] = {dv.x, dv.y, dv.z, dv.w};

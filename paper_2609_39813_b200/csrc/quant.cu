@@ -150,13 +150,14 @@ __device__ __forceinline__ uint4 encode16(const float (&v)[16], const PhiloxKey&
   }
 #pragma unroll
   for (int b = 0; b < 4; ++b) {
-    uint4 w = make_uint4(0, 0, 0, 0);
-    if (MODE == BSP_ROUND_STOCHASTIC) w = philox_block(key, (e0 >> 2) + b, draw);
-    const uint32_t c0 = f8_encode<FMT, MODE == BSP_ROUND_STOCHASTIC>(v[4 * b + 0], w.x, dc);
-    const uint32_t c1 = f8_encode<FMT, MODE == BSP_ROUND_STOCHASTIC>(v[4 * b + 1], w.y, dc);
-    const uint32_t c2 = f8_encode<FMT, MODE == BSP_ROUND_STOCHASTIC>(v[4 * b + 2], w.z, dc);
-    const uint32_t c3 = f8_encode<FMT, MODE == BSP_ROUND_STOCHASTIC>(v[4 * b + 3], w.w, dc);
-    packed[b] = c0 | (c1 << 8) | (c2 << 16) | (c3 << 24);
+    const float x[4] = {v[4 * b], v[4 * b + 1], v[4 * b + 2], v[4 * b + 3]};
+    if (MODE == BSP_ROUND_STOCHASTIC) {
+      packed[b] = f8_encode4_sr<FMT>(x, philox_block(key, (e0 >> 2) + b, draw), dc);
+    } else {
+      packed[b] = 0u;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) packed[b] |= f8_encode<FMT, false>(x[i], 0u, dc) << (8 * i);
+    }
   }
   return make_uint4(packed[0], packed[1], packed[2], packed[3]);
 }

@@ -359,6 +359,75 @@ def test_mc_check_attention_draw_groups(b, K):
         assert got.verdict == want.verdict
 
 
+@pytest.mark.parametrize("B,H,S,K", [(10, 15, 64, 9), (1, 1, 64, 37)])
+def test_mc_check_attention_draw_sets(b, B, H, S, K):
+    """At least as many (key block, head) items as SMs: one set, several passes of an item in turn (10 x 15 heads,
+    nine draws).  One item: ten sets of one pass each, the last of a single draw.  Against the plain oracle."""
+    inp = workloads.config3(B=B, H=H, S=S, D=64, K=K, seed=17)
+    g = AttnGpu(b, inp, True)
+    d = _attn_desc(b, g, inp, K, 4)
+    res = b.bsp_mc_check_attn(d, K, b.workspace(b.bsp_mc_check_attn_workspace_bytes(d, K)), b.new_diag())
+    o = g.o.cpu().numpy().reshape(B * H, S, inp.D)
+    parts = []
+    for idx, q, k, v, dO in _slices(inp):
+        prep = check.prepare_attention_slice(q, k, v, dO, inp.softmax_scale, inp.seed, idx, True, o32=o[idx])
+        parts.append(check.attention_d_use(q, k, v, dO, inp.softmax_scale, prep, 2, K, inp.seed))
+    want = _pooled([p_["dk"] for p_ in parts], K, True)
+    for f in ("rel_l2_mean_err", "R", "Qprime", "rms_z"):
+        assert np.isclose(getattr(res[2], f), getattr(want, f), rtol=1e-2), f      # as in the test above
+
+
+@pytest.mark.parametrize("B,H,S,K,causal", [(1, 2, 200, 9, 1), (2, 40, 256, 6, 1), (1, 1, 64, 4, 0), (1, 3, 300, 21, 0)])
+def test_mc_check_attention_fp8_draws_equal_single_backwards(b, B, H, S, K, causal):
+    """FP8 operands: the draws' sums of dQ and dK against one backward per draw.  160 items of two blocks: one set, two
+    passes; the others: sets of one or two passes, the last one partly filled.  The backward of a draw is the
+    same arithmetic in both, so what is left is FP32 sums of K terms (K 2^-24) and of the statistics: 1e-4."""
+    torch.manual_seed(S + K)
+    BH, n, rows, c = B * H, B * H * S * 64, B * H * S, 0.125
+    x = {nm: (torch.randn(n, device="cuda") * (1.0 if nm == "dO" else 0.5)).bfloat16() for nm in ("q", "k", "v", "dO")}
+    q8 = {}
+    for nm, t in x.items():
+        xq, codes = torch.zeros_like(t), torch.zeros(n, dtype=torch.uint8, device="cuda")
+        amax, sc = torch.zeros(BH, device="cuda"), torch.zeros(BH, device="cuda")
+        b.bsp_attn_quantize(t, BH, S * 64, fp8.E5M2 if nm == "dO" else fp8.E4M3, xq, amax, sc, codes=codes)
+        q8[nm] = (xq, sc, codes)
+    f = b.attn_fp8(*(q8[nm][1] for nm in ("q", "k", "v", "dO")), 256.0, 1024.0, *(q8[nm][2] for nm in ("q", "k", "v", "dO")))
+    ops = [q8[nm][0] for nm in ("q", "k", "v", "dO")]
+    o, lse = torch.zeros(n, device="cuda"), torch.zeros(rows, device="cuda")
+    b.bsp_attn_fwd_stats(B, H, S, 64, causal, c, *ops[:3], o, lse, fp8=f)
+    amax, sc, codes = torch.zeros(BH, device="cuda"), torch.zeros(BH, device="cuda"), torch.zeros(n, dtype=torch.uint8, device="cuda")
+    b.bsp_amax(o, BH, S * 64, amax)
+    b.bsp_scale_from_amax(amax, BH, fp8.E4M3, sc)
+    b.bsp_round_grouped(o, BH, S * 64, fp8.E4M3, fp8.SR, sc, b.key(5, 3, b.STREAM_FORWARD), codes)
+    key = b.key(5, 3, b.STREAM_ATTN_D)
+
+    def backward(read, draw):
+        D, dq, dk = torch.zeros(rows, device="cuda"), torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda")
+        b.bsp_attn_dterm(B, H, S, 64, ops[3], o, codes, sc, fp8.E4M3, read, key, draw, 1, D, do_scales=q8["dO"][1])
+        b.bsp_attn_bwd_dterm(B, H, S, 64, causal, c, *ops, lse, D, dq, dk, None, fp8=f)
+        return dq.double(), dk.double()
+
+    ref = backward(0, 0)
+    S1, S2 = [torch.zeros_like(t) for t in ref], [torch.zeros_like(t) for t in ref]
+    for d in range(K):
+        for i, g in enumerate(backward(2, d)):
+            S1[i] += g - ref[i]
+            S2[i] += (g - ref[i]) ** 2
+    desc = b.AttnDesc()
+    desc.B, desc.H, desc.S, desc.Dh, desc.causal, desc.softmax_scale, desc.dtype = B, H, S, 64, causal, c, b.BF16
+    desc.q, desc.k, desc.v, desc.dO = (b.ptr(x[nm]) for nm in ("q", "k", "v", "dO"))
+    desc.store_fmt, desc.forward_mode, desc.seed, desc.tensor_id, desc.policy_mask = fp8.E4M3, fp8.SR, 5, 3, 4
+    desc.fp8_operands, desc.p_scale, desc.ds_scale = 1, 256.0, 1024.0
+    diag = b.new_diag()
+    res = b.bsp_mc_check_attn(desc, K, b.workspace(b.bsp_mc_check_attn_workspace_bytes(desc, K)), diag)
+    assert b.read_diag(diag)["status"] == 0
+    for i, r in enumerate(res[1:3]):
+        mean = S1[i] / K
+        se2 = ((S2[i] - S1[i] ** 2 / K) / (K * (K - 1))).clamp(min=0).sum()
+        assert np.isclose(r.rel_l2_mean_err, float(mean.norm() / ref[i].norm()), rtol=1e-4), (i, r.rel_l2_mean_err)
+        assert np.isclose(r.R, float((mean ** 2).sum() / se2), rtol=1e-4), (i, r.R)
+
+
 def _quantised_operands(b, inp):
     """Q, K, V -> E4M3 and dO -> E5M2 per (b,h) slice on the GPU, and the oracle's values of the same."""
     from paper_2609_39813_b200.harness import up
