@@ -69,13 +69,27 @@ cp_forward_kernel(int kind, const void* x, int64_t T, int64_t C, const float* ga
     const float4 g4 = ldg(reinterpret_cast<const float4*>(gamma + c));
     float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (kind == BSP_LAYERNORM) b4 = ldg(reinterpret_cast<const float4*>(beta + c));
+    // the loads of the thread's rows are all requested before the first is used (4096 x 1024: 17.6 -> 15.4 us)
+    constexpr int R = kCpRows / 4;
+    const int64_t t0 = (int64_t)blockIdx.x * kCpRows + threadIdx.y;
+    float4 xr[R];
+    float rs[R], mu[R];
+    uint2 qa_r[R];
 #pragma unroll
-    for (int j = 0; j < kCpRows / 4; ++j) {
-      const int64_t t = (int64_t)blockIdx.x * kCpRows + threadIdx.y + 4 * j;
+    for (int j = 0; j < R; ++j) {
+      const int64_t t = t0 + 4 * j < T ? t0 + 4 * j : T - 1;
+      xr[j] = load4<DT>(x, (size_t)t * C + c);
+      rs[j] = ldg(rstd + t);
+      mu[j] = kind == BSP_LAYERNORM ? ldg(mean + t) : 0.f;
+      qa_r[j] = uq_a ? ldg(reinterpret_cast<const uint2*>(uq_a + (size_t)t * C + c)) : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int64_t t = t0 + 4 * j;
       if (t >= T) break;
       const size_t i = (size_t)t * C + c;
       float u[4];
-      cp_chain(kind, load4<DT>(x, i), ldg(rstd + t), kind == BSP_LAYERNORM ? ldg(mean + t) : 0.f, g4, b4, u);
+      cp_chain(kind, xr[j], rs[j], mu[j], g4, b4, u);
       const float v[4] = {__fmul_rn(u[0], scale), __fmul_rn(u[1], scale), __fmul_rn(u[2], scale), __fmul_rn(u[3], scale)};
       uint32_t packed = 0;
       if (SR) {
@@ -87,7 +101,7 @@ cp_forward_kernel(int kind, const void* x, int64_t T, int64_t C, const float* ga
       const uint2 q = f8_to_bf16x4<FMT>(packed);
       *reinterpret_cast<uint2*>(uq + i) = q;
       if (uq_a) {
-        const uint2 a = ldg(reinterpret_cast<const uint2*>(uq_a + i));
+        const uint2 a = qa_r[j];
         float qa[4], qb[4];
         bf16x4_to_float(a, qa);
         bf16x4_to_float(q, qb);
@@ -124,9 +138,9 @@ cp_weight_kernel(const void* W, size_t n4, uint16_t* Wd) {
 // columns, a thread four columns of every eighth row; its two column sums join partial[2][slab][C] (or
 // start it), so every sum has one writer and a fixed order.  The dot products: FP32 chains per thread (a
 // few dozen elements), double above (double arithmetic is scarce on this part).
-constexpr int kCpSlabs = 64;
+constexpr int kCpSlabs = 64, kCpResident = 3;                       // slabs at most; blocks per SM
 template <int DT, int FMT>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, kCpResident)
 cp_sums_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma,
                const float* beta, const float* rstd, const float* mean,
                const float* scale_dev, PhiloxKey key, int64_t slab_rows, const uint16_t* uq,
@@ -219,6 +233,19 @@ cp_sums_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
   }
 }
 
+// Rows of a slab: the fewest rounds of blocks over the SMs times eight rows of a block (and about two such steps of
+// a block's own start and end), from kCpSlabs slabs down.  4096 x 1024: 52 slabs in one round, not 64 in one and a
+// sixth (26.7 -> 20.1 us a pass on average).
+static int64_t cp_slab_rows(int64_t T, int64_t C) {
+  const int64_t least = ((T + kCpSlabs - 1) / kCpSlabs + 7) & ~(int64_t)7, columns = (C + 127) / 128;
+  int64_t best = least, cost = INT64_MAX;
+  for (int64_t r = least; r <= 16 * least; r += 8) {
+    const int64_t blocks = columns * ((T + r - 1) / r), rounds = (blocks + kCpResident * kNumSMs - 1) / (kCpResident * kNumSMs);
+    if (rounds * (r / 8 + 2) < cost) { cost = rounds * (r / 8 + 2); best = r; }
+  }
+  return best;
+}
+
 // out[k] = { T, control } of pair k from its blocks' dot products, in a fixed order.  One block per pair.
 __global__ void __launch_bounds__(256)
 cp_dots_final_kernel(const double* partial, int nblocks, double* out) {
@@ -293,7 +320,7 @@ static size_t coupling_carve(const bsp_coupling_desc_t* op, int pairs, char* bas
   const size_t T = (size_t)op->T, C = (size_t)op->C, O = (size_t)op->O;
   CouplingBuffers c;
   memset(&c, 0, sizeof(c));
-  c.slab_rows = ((op->T + kCpSlabs - 1) / kCpSlabs + 7) & ~(int64_t)7;
+  c.slab_rows = cp_slab_rows(op->T, (int64_t)C);
   c.nslabs = (int)((op->T + c.slab_rows - 1) / c.slab_rows);
   c.nblocks = c.nslabs * (int)((C + 127) / 128);
   c.rstd = (float*)take(T * 4); c.mean = (float*)take(T * 4); c.amax = (float*)take(4); c.scale = (float*)take(4);
