@@ -154,7 +154,8 @@ int attn_sum_sets(const float* p1, const float* p2, int sets, float* S1, float* 
 
 // FP8-operand mode (attn_f8.cu): the backward of one evaluation (dv with dk only; dk or dq may be left out), and K
 // draws of the correction term (dterm [K][B*H*S]) with S1 = sum (g_k - ref), S2 = sum (g_k - ref)^2 of dQ and dK
-// written.  `partials`: 4 x attn_draw_sets(BH, S, K) x BH x S x 64 floats, unused where the sets are one.
+// written.  `partials`: 4 x attn_draw_sets(BH, S, K) x BH x S x 64 floats, unused where the sets are one;
+// NULL: one set.
 int attn_f8_bwd(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, const float* lse, const float* dterm, float* dq,
                 float* dk, float* dv, bsp_diag_t* diag, cudaStream_t st);
 int attn_f8_draws(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, const float* lse, const float* dterm, int K,

@@ -577,7 +577,7 @@ int attn_f8_draws(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, c
   int rc = f8_params(p, BH, S, causal, c, f, lse, dterm, diag);
   if (rc != BSP_OK) return rc;
   p.K = K;
-  p.sets = attn_draw_sets(BH, S, K);
+  p.sets = partials ? attn_draw_sets(BH, S, K) : 1;
   p.passes = ((K + kF8ND - 1) / kF8ND + p.sets - 1) / p.sets;
   const size_t n = (size_t)BH * S * AT_D;
   float* part[4] = {S1k, S2k, S1q, S2q};

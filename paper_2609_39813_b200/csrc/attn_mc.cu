@@ -26,7 +26,8 @@
 // columns, four accumulators of 64.  P^T goes back into the columns its thread read S^T from (two K = 16
 // steps per 32 columns, the first 16 of them), so the scores are double-buffered in the room that one buffer
 // and a separate operand would take, and S^T of a step is formed under the exponentials and stores of the
-// step before.  -LSE enters S^T through one extra K = 16 product step (a tile of ones against rows holding
+// step before (B H = 128, S = 2048, causal, 32 draws: 1.68 ms; with one buffer, eight warps and a launch per four
+// draws 1.89).  -LSE enters S^T through one extra K = 16 product step (a tile of ones against rows holding
 // -LSE/c as three bf16 terms), written two steps ahead, so P^T = exp2(c2 acc) needs no per-column operand.
 #include <string.h>
 
@@ -514,7 +515,7 @@ static int attn_dk_diff(int BH, int S, int causal, float c, const void* q, const
   DkDiffParams p;
   p.BH = BH; p.S = S; p.nblk = (S + AT_BLK - 1) / AT_BLK; p.causal = causal ? 1 : 0; p.c = c;
   p.lse = lse; p.d_ref = d_ref; p.d_draws = d_draws; p.K = K; p.diag = diag;
-  p.sets = attn_draw_sets(BH, S, K);
+  p.sets = partials ? attn_draw_sets(BH, S, K) : 1;
   p.passes = ((K + kDkND - 1) / kDkND + p.sets - 1) / p.sets;
   const size_t n = (size_t)BH * S * AT_D;
   float* o1 = p.sets > 1 ? partials : S1k;
@@ -551,7 +552,7 @@ struct AttnCheckBuffers {
   size_t b_stats;
 };
 
-static size_t attn_carve(const bsp_attn_desc_t* op, int K, char* base, AttnCheckBuffers* out) {
+static size_t attn_carve(const bsp_attn_desc_t* op, int K, char* base, AttnCheckBuffers* out, bool room_for_sets = true) {
   size_t off = 0;
   auto take = [&](size_t bytes) -> void* {
     void* p = base ? base + off : nullptr;
@@ -574,10 +575,11 @@ static size_t attn_carve(const bsp_attn_desc_t* op, int K, char* base, AttnCheck
       c.op8[t] = take(n * 2); c.opc[t] = (uint8_t*)take(n); c.op_amax[t] = (float*)take(BH * 4); c.op_scale[t] = (float*)take(BH * 4);
     }
   }
-  const size_t sets = (size_t)attn_draw_sets((int64_t)BH, op->S, K > 0 ? K : 1);
-  if (sets > 1) c.partials = (float*)take((op->fp8_operands ? 4 : 2) * sets * n * 4);
   c.b_stats = kMaxPendingStats * kStatSlotBytes;
   c.ws_stats = take(c.b_stats);
+  // last: a workspace without room for them is taken too, and then every item's draws stay in one set
+  const size_t sets = room_for_sets ? (size_t)attn_draw_sets((int64_t)BH, op->S, K > 0 ? K : 1) : 1;
+  if (sets > 1) c.partials = (float*)take((op->fp8_operands ? 4 : 2) * sets * n * 4);
   if (out) *out = c;
   return off;
 }
@@ -618,11 +620,12 @@ int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t
   if (rc != BSP_OK) return rc;
   const bool fp8 = op->fp8_operands != 0;
   if (fp8 && (!(op->p_scale > 0.f) || !(op->ds_scale > 0.f))) return BSP_ERR_ARG;
-  if (!ws || ws_bytes < bsp_mc_check_attn_workspace_bytes(op, K) || (reinterpret_cast<uintptr_t>(ws) & 255u))
+  const bool room_for_sets = ws_bytes >= bsp_mc_check_attn_workspace_bytes(op, K);
+  if (!ws || ws_bytes < attn_carve(op, K, nullptr, nullptr, false) || (reinterpret_cast<uintptr_t>(ws) & 255u))
     return BSP_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   AttnCheckBuffers b;
-  attn_carve(op, K, reinterpret_cast<char*>(ws), &b);
+  attn_carve(op, K, reinterpret_cast<char*>(ws), &b, room_for_sets);
   const int B = op->B, H = op->H, S = op->S, Dh = op->Dh, dt = op->dtype;
   const size_t BH = (size_t)B * H, rows = BH * S, n = rows * Dh;
   const float c = op->softmax_scale;

@@ -55,7 +55,7 @@ struct PendingStats {
     return mc_stats_launch(g_ref, g, S2, n_, K_, fresh_, rule, slots + (size_t)slot * kStatSlotDoubles, st, &blocks[slot]);
   }
   // One small copy, one synchronisation.  The stream is idle when this returns.  (The slots themselves are 38 KB
-  // each: copying and summing them here took 24 us of the smallest check.)
+  // each: copying and summing them here took 21 us of the smallest check.)
   int flush() {
     double host[kMaxPendingStats * kStatFields];
     if (count > 0) {
