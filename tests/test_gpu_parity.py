@@ -73,6 +73,43 @@ def test_round_special_values_bit_exact(b, fmt, mode):
     assert d["n_saturated"] == n_sat and d["n_nonfinite"] == n_nf and d["status"] == b.ERR_NONFINITE
 
 
+@pytest.mark.parametrize("fmt", [fp8.E4M3, fp8.E5M2])
+@pytest.mark.parametrize("two_d", [False, True])
+def test_round_decided_by_the_last_bits_of_the_word(b, fmt, two_d):
+    """Stochastic rounding of values whose fraction of a step is the generator word itself, cut to the FP32 value below it
+    or raised to the one above, in the subnormal range and in the normal one, mixed within every four with ordinary,
+    saturating, non-finite and zero values."""
+    F = fp8.FORMATS[fmt]
+    rng = np.random.default_rng(6)
+    rows, cols = 64, 256
+    n = rows * cols
+    key = (42, 3, 1, 2)
+    words = philox.tensor_words(*key, n)
+    frac = words.astype(np.float64) * 2.0 ** -32
+    step = 2.0 ** (F.emin - F.mbits)
+    level = rng.integers(0, 2 ** F.mbits, n) * rng.integers(0, 2, n)                 # steps below the fraction, 0 in half of them
+    octave = np.where(rng.random(n) < 0.3, 2.0 ** rng.integers(0, 5, n), 1.0)
+    exact = np.where(octave > 1, (2 ** F.mbits + level) * octave, level) * step + frac * step * octave
+    v = exact.astype(np.float32)
+    below = np.where(v > exact, np.nextafter(v, np.float32(0)), v)
+    v = np.where(rng.random(n) < 0.5, below, np.nextafter(below, np.float32(np.inf))).astype(np.float32)
+    other = rng.random(n)
+    v = np.where(other < 0.1, rng.standard_normal(n) * F.fmax / 3, v)
+    v = np.where((other > 0.9) & (other < 0.92), rng.choice([0.0, 1e-40, F.fmax, F.fmax * 1.01, np.inf, np.nan], n), v)
+    v = (v * rng.choice([-1.0, 1.0], n)).astype(np.float32)
+    x, codes, codes_t, diag = up(v), torch.zeros(n, dtype=torch.uint8, device="cuda"), torch.zeros(n, dtype=torch.uint8, device="cuda"), b.new_diag()
+    q = b.quant(fmt, fp8.SR, 1.0)
+    if two_d:
+        b.bsp_round_2d(x, rows, cols, q, b.key(*key), codes, codes_t, rows, diag)
+        assert torch.equal(codes_t.view(cols, rows).T, codes.view(rows, cols))
+    else:
+        b.bsp_round(x, n, q, b.key(*key), 0, codes, diag)
+    want, n_sat, n_nf = fp8.encode(v, fmt, fp8.SR, words)
+    assert np.array_equal(codes.cpu().numpy(), want)
+    d = b.read_diag(diag)
+    assert d["n_saturated"] == n_sat and d["n_nonfinite"] == n_nf
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("n,offset", [(100003, 0), (4096, 64), (777, 5)])
 def test_round_scaled_ragged_bit_exact(b, dtype, n, offset):
