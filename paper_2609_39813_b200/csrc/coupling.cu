@@ -136,8 +136,10 @@ cp_weight_kernel(const void* W, size_t n4, uint16_t* Wd) {
 // and sum dua r, and both forwards join sum_r and sum_du (or start them, first).  u is formed from x
 // again, which costs less traffic than an FP32 r would.  Block (x, y) walks slab y of rows for 128
 // columns, a thread four columns of every eighth row; its two column sums join partial[2][slab][C] (or
-// start it), so every sum has one writer and a fixed order.  The dot products: FP32 chains per thread (a
-// few dozen elements), double above (double arithmetic is scarce on this part).
+// start it), so every sum has one writer and a fixed order.  A column's sum is an FP32
+// chain of a thread's rows (cp_slab_rows bounds them); the dot products are summed in double from the products on
+// (eight FP32 chains per thread instead took more registers than there are: 16 forwards of 4096 x 1024 -> 64
+// 1277 -> 1202 us, and an error of T of 5e-8 of the terms' norm, not 1e-8).
 constexpr int kCpSlabs = 64, kCpResident = 3;                       // slabs at most; blocks per SM
 template <int DT, int FMT>
 __global__ void __launch_bounds__(256, kCpResident)
@@ -154,14 +156,17 @@ cp_sums_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
   const int64_t c = (int64_t)blockIdx.x * 128 + 4 * lane;
   const float scale = ldg(scale_dev), inv = __fdiv_rn(1.0f, scale);
   const int64_t t0 = (int64_t)blockIdx.y * slab_rows, t1 = t0 + slab_rows < T ? t0 + slab_rows : T;
-  float own[4] = {0.f, 0.f, 0.f, 0.f}, fresh[4] = {0.f, 0.f, 0.f, 0.f}, da[4] = {0.f, 0.f, 0.f, 0.f}, db[4] = {0.f, 0.f, 0.f, 0.f};
+  float own[4] = {0.f, 0.f, 0.f, 0.f}, fresh[4] = {0.f, 0.f, 0.f, 0.f};
+  double da = 0.0, db = 0.0;
   DiagCounters dc;
   if (c < C) {
     const float4 g4 = ldg(reinterpret_cast<const float4*>(gamma + c));
     float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (kind == BSP_LAYERNORM) b4 = ldg(reinterpret_cast<const float4*>(beta + c));
+    const int rows = (int)(t1 - t0);
 #pragma unroll 1
-    for (int64_t t = t0 + w; t < t1; t += 8) {
+    for (int n = w; n < rows; n += 8) {
+      const int64_t t = t0 + n;
       const size_t i = (size_t)t * C + c;
       const float4 xv = load4<DT>(x, i), dv = ldg(reinterpret_cast<const float4*>(du + i));
       const uint2 qv = ldg(reinterpret_cast<const uint2*>(uq + i));
@@ -196,8 +201,8 @@ cp_sums_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           ra[e] = qa[e] * inv - u[e];
-          da[e] = fmaf(ra[e] - r4[e], y4[e] - d4[e], da[e]);
-          db[e] = fmaf(y4[e], r4[e], db[e]);
+          da += (double)((ra[e] - r4[e]) * (y4[e] - d4[e]));
+          db += (double)(y4[e] * r4[e]);
         }
         *reinterpret_cast<float4*>(sum_r + i) =
             make_float4((sr.x + ra[0]) + r4[0], (sr.y + ra[1]) + r4[1], (sr.z + ra[2]) + r4[2], (sr.w + ra[3]) + r4[3]);
@@ -210,11 +215,9 @@ cp_sums_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
   *reinterpret_cast<float4*>(&sm[0][w][4 * lane]) = make_float4(own[0], own[1], own[2], own[3]);
   *reinterpret_cast<float4*>(&sm[1][w][4 * lane]) = make_float4(fresh[0], fresh[1], fresh[2], fresh[3]);
   if (uq_a) {
-    double a = ((double)da[0] + (double)da[1]) + ((double)da[2] + (double)da[3]);
-    double b = ((double)db[0] + (double)db[1]) + ((double)db[2] + (double)db[3]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) { a += __shfl_xor_sync(0xFFFFFFFFu, a, o); b += __shfl_xor_sync(0xFFFFFFFFu, b, o); }
-    if (lane == 0) { sd[0][w] = a; sd[1][w] = b; }
+    for (int o = 16; o > 0; o >>= 1) { da += __shfl_xor_sync(0xFFFFFFFFu, da, o); db += __shfl_xor_sync(0xFFFFFFFFu, db, o); }
+    if (lane == 0) { sd[0][w] = da; sd[1][w] = db; }
   }
   __syncthreads();
   const int which = threadIdx.x >> 7, cl = threadIdx.x & 127;
@@ -234,13 +237,18 @@ cp_sums_kernel(int kind, const void* x, int64_t T, int64_t C, const float* gamma
 }
 
 // Rows of a slab: the fewest rounds of blocks over the SMs times eight rows of a block (and about two such steps of
-// a block's own start and end), from kCpSlabs slabs down.  4096 x 1024: 52 slabs in one round, not 64 in one and a
-// sixth (26.7 -> 20.1 us a pass on average).
+// a block's own start and end), from kCpSlabs slabs down.  4096 x 1024: 52 slabs, 416 blocks in one round of 444
+// places, where 64 slabs are 512 blocks in two (26.7 -> 20.1 us a pass on average).  Up to kCpMostRows rows, 64 of a
+// thread: with terms of random signs the rounding of a column's sum has the variance T r / 16 in the threads' chains
+// and T^2 / 2 r over the slabs, and at r = 512 that is what 64 slabs give for any T; more tokens take 64 slabs.
+constexpr int64_t kCpMostRows = 512;
 static int64_t cp_slab_rows(int64_t T, int64_t C) {
-  const int64_t least = ((T + kCpSlabs - 1) / kCpSlabs + 7) & ~(int64_t)7, columns = (C + 127) / 128;
-  int64_t best = least, cost = INT64_MAX;
-  for (int64_t r = least; r <= 16 * least; r += 8) {
-    const int64_t blocks = columns * ((T + r - 1) / r), rounds = (blocks + kCpResident * kNumSMs - 1) / (kCpResident * kNumSMs);
+  const int64_t columns = (C + 127) / 128, places = kCpResident * kNumSMs;
+  int64_t best = 0, cost = INT64_MAX;
+  for (int64_t n = kCpSlabs; n > 0; --n) {
+    const int64_t r = ((T + n - 1) / n + 7) & ~(int64_t)7;
+    if (best && r > kCpMostRows) break;
+    const int64_t rounds = (columns * ((T + r - 1) / r) + places - 1) / places;
     if (rounds * (r / 8 + 2) < cost) { cost = rounds * (r / 8 + 2); best = r; }
   }
   return best;

@@ -60,6 +60,19 @@ def test_struct_layouts_match_header(built):
     assert b.bsp_mc_check_workspace_bytes(d, 16) < full
 
 
+@pytest.mark.parametrize("T,C", [(1, 16), (77, 144), (1003, 4112), (4096, 1024), (16384, 3600), (16352, 7936), (65537 * 16 + 3, 16)])
+def test_coupling_slabs_bound_the_sums_chains(built, T, C):
+    """A slab of the coupling check holds at most 512 rows (a thread's FP32 chain then has 64), or what 64 slabs need.
+    The slabs show in the workspace: two doubles per block and pair."""
+    from paper_2609_39813_b200 import binding as b
+    d = b.CouplingDesc()
+    d.T, d.C, d.O = T, C, 16
+    blocks = (b.bsp_coupling_check_workspace_bytes(d, 32) - b.bsp_coupling_check_workspace_bytes(d, 16) - 256) // 256
+    columns = -(-C // 128)
+    assert blocks % columns == 0 and 1 <= blocks // columns <= 64
+    assert -(-T // (blocks // columns)) <= max(512, -(-T // 64) + 7)
+
+
 def test_check_argument_errors_need_no_gpu(built):
     from paper_2609_39813_b200 import binding as b
     import ctypes as C

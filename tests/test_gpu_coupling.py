@@ -55,6 +55,7 @@ CASES = {
     "rms_bf16_ragged": lambda: workloads.config2(T=200, C=128, O=96, K=4, seed=21),
     "layernorm_f32": lambda: workloads.config4(T=160, C=96, O=64, K=4, seed=22),
     "odd_tokens": lambda: workloads.config2(T=77, C=144, O=272, K=4, seed=24),          # ragged tiles, K = 2 T odd halves
+    "wide_long_slabs": lambda: workloads.config2(T=1003, C=4112, O=64, K=4, seed=27),   # slabs five times the shortest, ragged
     "one_token": lambda: workloads.config4(T=1, C=16, O=16, K=4, seed=25),
 }
 
