@@ -715,6 +715,11 @@ int bsp_selftest_bounded_wait(uint64_t limit_ns, bsp_diag_t* diag, void* stream)
 int bsp_selftest_probs_unfinished(const float* p, const float* V, int64_t rows, int n, int d, float param,
                                   uint64_t seed, int K, int64_t done, float* ds_sum, float* ds_sq, float* dV_sum,
                                   void* stream);
+/* The same for the sums over the draws in bsp_mc_check_attn: blocks of a head that were not completed are NaN
+ * in the sums of dK (FP8 operands: and of dQ), so the statistics of a fresh read say so even without a diag.  As
+ * bsp_mc_check_attn with the default rule, the kernels over the draws stopping before work item `done`. */
+int bsp_selftest_attn_unfinished(const bsp_attn_desc_t* op, int K, int done, bsp_use_result_t* results,
+                                 int* n_results, void* ws, size_t ws_bytes, bsp_diag_t* diag, void* stream);
 
 #ifdef __cplusplus
 }

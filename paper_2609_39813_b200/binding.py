@@ -156,6 +156,7 @@ _SIGNATURES = {
     "bsp_mc_check_attn_workspace_bytes": (_SZ, [C.POINTER(AttnDesc), _I]),
     "bsp_mc_check_attn": (_I, [C.POINTER(AttnDesc), _I, C.POINTER(VerdictRule), C.POINTER(UseResult), C.POINTER(_I),
                                _P, _SZ, _P, _P]),
+    "bsp_selftest_attn_unfinished": (_I, [C.POINTER(AttnDesc), _I, _I, C.POINTER(UseResult), C.POINTER(_I), _P, _SZ, _P, _P]),
     "bsp_mc_stats_workspace_bytes": (_SZ, [_I64]),
     "bsp_mc_stats": (_I, [_P, _P, _P, _I64, _I, _I, C.POINTER(VerdictRule), C.POINTER(UseResult), _P, _SZ, _P]),
     "bsp_mc_check_workspace_bytes": (_SZ, [C.POINTER(NormLinearDesc), _I]),
@@ -484,6 +485,14 @@ def bsp_mc_check_attn(desc: AttnDesc, K, ws, diag=None, stream=None, rule=None):
     n = C.c_int(0)
     check(lib().bsp_mc_check_attn(C.byref(desc), K, _ruleref(rule), res, C.byref(n), ptr(ws), ws.numel(), ptr(diag),
                                   _st(stream)), "bsp_mc_check_attn")
+    return [res[i] for i in range(n.value)]
+
+
+def bsp_selftest_attn_unfinished(desc: AttnDesc, K, done, ws, diag=None, stream=None):
+    res = (UseResult * 12)()
+    n = C.c_int(0)
+    check(lib().bsp_selftest_attn_unfinished(C.byref(desc), K, done, res, C.byref(n), ptr(ws), ws.numel(), ptr(diag), _st(stream)),
+          "bsp_selftest_attn_unfinished")
     return [res[i] for i in range(n.value)]
 
 

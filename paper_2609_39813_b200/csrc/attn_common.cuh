@@ -118,6 +118,18 @@ static inline int make_head_map_u8(CUtensorMap* map, const void* base, int BH, i
   return r == CUDA_SUCCESS ? BSP_OK : BSP_ERR_CUDA;
 }
 
+// Block `blk` of head z in both sums, NaN: what a block of `threads` threads leaves of an item that a wait which ran out
+// cut short, instead of what the memory held before.
+__device__ __forceinline__ void attn_fill_nan(float* o0, float* o1, int z, int blk, int S, int threads) {
+  const int rows = min(AT_BLK, S - blk * AT_BLK);
+  const size_t at = ((size_t)z * S + (size_t)blk * AT_BLK) * (AT_D / 4);
+  const float4 bad = make_float4(NAN, NAN, NAN, NAN);
+  for (int i = threadIdx.x; i < rows * (AT_D / 4); i += threads) {
+    reinterpret_cast<float4*>(o0)[at + i] = bad;
+    reinterpret_cast<float4*>(o1)[at + i] = bad;
+  }
+}
+
 inline int check_attn_shape(int B, int H, int S, int Dh, int dt) {
   if (B <= 0 || H <= 0 || S <= 0) return BSP_ERR_ARG;
   if (Dh != AT_D || dt != BSP_BF16) return BSP_ERR_UNSUPPORTED;
@@ -155,11 +167,11 @@ int attn_sum_sets(const float* p1, const float* p2, int sets, float* S1, float* 
 // FP8-operand mode (attn_f8.cu): the backward of one evaluation (dv with dk only; dk or dq may be left out), and K
 // draws of the correction term (dterm [K][B*H*S]) with S1 = sum (g_k - ref), S2 = sum (g_k - ref)^2 of dQ and dK
 // written.  `partials`: 4 x attn_draw_sets(BH, S, K) x BH x S x 64 floats, unused where the sets are one;
-// NULL: one set.
+// NULL: one set.  walk: items from here on are left as after a wait that ran out (INT_MAX: none).
 int attn_f8_bwd(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, const float* lse, const float* dterm, float* dq,
                 float* dk, float* dv, bsp_diag_t* diag, cudaStream_t st);
 int attn_f8_draws(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, const float* lse, const float* dterm, int K,
                   const float* ref_dq, float* S1q, float* S2q, const float* ref_dk, float* S1k, float* S2k, float* partials,
-                  bsp_diag_t* diag, cudaStream_t st);
+                  int walk, bsp_diag_t* diag, cudaStream_t st);
 
 }  // namespace bsp

@@ -76,6 +76,12 @@ struct AttnF8Params {
   float p_scale, ds_scale;
   bsp_diag_t* diag;
 };
+struct AttnF8Draws : AttnF8Params {
+  float *s1, *s2;                // what tm_o0 and tm_o1 map
+  int walk;                      // items from here on are left as after a wait that ran out (self-test; else all)
+};
+template <bool MC> struct AttnF8Arg { using type = AttnF8Params; };
+template <> struct AttnF8Arg<true> { using type = AttnF8Draws; };
 
 // MODE: AT_DQ (the CTA owns a query block, streams K_j, V_j) or AT_DKV (owns a key block, streams Q_i, dO_i).
 // MC: the draws with their sums S1 (tm_o0), S2 (tm_o1); else one evaluation: dQ (tm_o0), or dK (tm_o1) and,
@@ -84,7 +90,8 @@ template <int MODE, bool MC, bool DV>
 __global__ void __launch_bounds__(kF8Threads, 1)
 attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
-               const __grid_constant__ CUtensorMap tm_o0, const __grid_constant__ CUtensorMap tm_o1, AttnF8Params p) {
+               const __grid_constant__ CUtensorMap tm_o0, const __grid_constant__ CUtensorMap tm_o1,
+               typename AttnF8Arg<MC>::type p) {
   static_assert(!DV || (MODE == AT_DKV && !MC), "dV: one evaluation of the dK / dV kernel");
   grid_dependency();
   extern __shared__ uint8_t smem_raw[];
@@ -100,9 +107,12 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   uint8_t* bars_gen = smem_raw + (bars - raw);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars_gen + 176);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 180);
+  volatile int* items_out = abort_flag + 1;                         // items whose outputs have been sent off
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwork = p.nblk * p.BH * p.sets;
+  int nwalk = nwork;
+  if constexpr (MC) nwalk = p.walk;
   // the CTA's n-th item: rounds of gridDim.x items, walked forwards and backwards in turn
   auto item_at = [&](int n) -> int {
     const int b = (int)blockIdx.x, G = (int)gridDim.x;
@@ -137,6 +147,7 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     mbar_init(b_acc, 1); mbar_init(b_acc_free, kF8Warps);
     mbar_init(b_staged, kF8Warps); mbar_init(b_stg_free, 1);
     *abort_flag = 0;
+    if (MC) *items_out = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -163,7 +174,7 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         bool ok = true;
         uint32_t itg = 0, vi = 0;                                   // global step, pass
         int n = 0;
-        for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+        for (int w = item_at(0); w < nwalk && ok; w = item_at(++n)) {
           int blk, bh, set, it_begin, nsteps, d0, d_end;
           decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
           for (; d0 < d_end && ok; d0 += kF8ND, ++vi) {
@@ -194,7 +205,7 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       bool ok = true;
       uint32_t itg = 0, vi = 0;
       int n = 0;
-      for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+      for (int w = item_at(0); w < nwalk && ok; w = item_at(++n)) {
         int blk, bh, set, it_begin, nsteps, d0, d_end;
         decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
         for (; d0 < d_end && ok; d0 += kF8ND, ++vi) {
@@ -361,6 +372,7 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             tma_store_3d(m1, out0 + kF8Out + 16384u, 32, y, z);
           }
           tma_store_commit();
+          if (MC) *items_out = (int)stored + 1;
         }
       }
       ++stored;
@@ -368,7 +380,7 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     };
 
     int n = 0;
-    for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+    for (int w = item_at(0); w < nwalk && ok; w = item_at(++n)) {
       int blk, bh, set, it_begin, nsteps, d0, d_end;
       decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
       const int d_first = d0;
@@ -481,6 +493,13 @@ attn_f8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag && p.diag) atomicMax(&p.diag->status, (int)BSP_ERR_TIMEOUT);
+  if constexpr (MC) {
+    for (int n = *items_out, w; (w = item_at(n)) < nwork; ++n) {    // none, unless a wait ran out
+      int blk, bh, set, a, b, c, d;
+      decode(w, blk, bh, set, a, b, c, d);
+      attn_fill_nan(p.s1, p.s2, set * p.BH + bh, blk, p.S, kF8Threads);
+    }
+  }
   if (warp == 17) {
     __syncwarp();
     tc_fence_after();
@@ -517,7 +536,7 @@ static int f8_params(AttnF8Params& p, int BH, int S, int causal, float c, const 
 }
 
 template <int MODE, bool MC, bool DV>
-static int launch_f8(const bsp_attn_fp8_t* f, float* out0, float* out1, const AttnF8Params& p, cudaStream_t st) {
+static int launch_f8(const bsp_attn_fp8_t* f, float* out0, float* out1, typename AttnF8Arg<MC>::type p, cudaStream_t st) {
   CUtensorMap mq, mk, mv, mdo, mo0, mo1;
   int rc;
   if ((rc = make_head_map_u8(&mq, f->q_codes, p.BH, p.S)) != BSP_OK) return rc;
@@ -534,6 +553,10 @@ static int launch_f8(const bsp_attn_fp8_t* f, float* out0, float* out1, const At
   }
   const int nsm = sm_count_or_default();
   const int64_t nwork = (int64_t)p.nblk * p.BH * p.sets;
+  if constexpr (MC) {
+    p.s1 = out0; p.s2 = out1;
+    if (p.walk > nwork) p.walk = (int)nwork;
+  }
   launch_kernel(attn_f8_kernel<MODE, MC, DV>, (unsigned)(nwork < nsm ? nwork : nsm), kF8Threads, kF8Smem, st, mq, mk, mv, mdo, mo0,
                 mo1, p);
   BSP_LAUNCH_CHECK();
@@ -572,11 +595,12 @@ int attn_sum_sets(const float* p1, const float* p2, int sets, float* S1, float* 
 
 int attn_f8_draws(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, const float* lse, const float* dterm, int K,
                   const float* ref_dq, float* S1q, float* S2q, const float* ref_dk, float* S1k, float* S2k, float* partials,
-                  bsp_diag_t* diag, cudaStream_t st) {
-  AttnF8Params p{};
+                  int walk, bsp_diag_t* diag, cudaStream_t st) {
+  AttnF8Draws p{};
   int rc = f8_params(p, BH, S, causal, c, f, lse, dterm, diag);
   if (rc != BSP_OK) return rc;
   p.K = K;
+  p.walk = walk;
   p.sets = partials ? attn_draw_sets(BH, S, K) : 1;
   p.passes = ((K + kF8ND - 1) / kF8ND + p.sets - 1) / p.sets;
   const size_t n = (size_t)BH * S * AT_D;

@@ -29,6 +29,7 @@
 // step before (B H = 128, S = 2048, causal, 32 draws: 1.68 ms; with one buffer, eight warps and a launch per four
 // draws 1.89).  -LSE enters S^T through one extra K = 16 product step (a tile of ones against rows holding
 // -LSE/c as three bf16 terms), written two steps ahead, so P^T = exp2(c2 acc) needs no per-column operand.
+#include <limits.h>
 #include <string.h>
 
 #include <atomic>
@@ -55,6 +56,8 @@ struct DkDiffParams {
   const float* d_ref;            // [BH*S]      the reference's correction term
   const float* d_draws;          // [K][BH*S]   the draws' correction terms
   int K, sets, passes;           // draws; sets per (block, head); passes of up to four draws per set
+  float *s1, *s2;                // what tm_s1 and tm_s2 map
+  int walk;                      // items from here on are left as after a wait that ran out (self-test; else all)
   bsp_diag_t* diag;
 };
 
@@ -84,6 +87,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   uint8_t* bars_gen = smem_raw + (bars - raw);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars_gen + 208);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 212);
+  volatile int* items_out = abort_flag + 1;                         // items whose sums have been sent off whole
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwork = p.nblk * p.BH * p.sets;
@@ -114,6 +118,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     mbar_init(b_acc, 1); mbar_init(b_acc_free, kDkWarps);
     mbar_init(b_staged, kDkWarps); mbar_init(b_stg_free, 1);
     *abort_flag = 0;
+    *items_out = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x < 256) {
@@ -150,7 +155,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         bool ok = true;
         uint32_t itg = 0, vi = 0;                                   // global step, pass
         int n = 0;
-        for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+        for (int w = item_at(0); w < p.walk && ok; w = item_at(++n)) {
           int blk, bh, set, it_begin, nsteps, d0, d_end;
           decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
           for (; d0 < d_end && ok; d0 += kDkND, ++vi) {
@@ -177,7 +182,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       bool ok = true;
       uint32_t itg = 0, vi = 0;
       int n = 0;
-      for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+      for (int w = item_at(0); w < p.walk && ok; w = item_at(++n)) {
         int blk, bh, set, it_begin, nsteps, d0, d_end;
         decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
         for (; d0 < d_end && ok; d0 += kDkND, ++vi) {
@@ -238,7 +243,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     bool ok = true, store_pending = false;
     uint32_t bias_written = 0, jt = 0, vi = 0, stg_ph = 0;          // -LSE rows written; global step, pass; last epilogue's phase
     // the pass whose accumulators have not been read yet
-    bool due = false, e_first = true;
+    bool due = false, e_first = true, e_last = true;
     int e_blk = 0, e_bh = 0, e_set = 0;
     // the -LSE row of one step (the warps of column quarter 0: thread r writes query r of the tile)
     auto bias_fetch = [&](int tbh, int step) -> float {
@@ -310,6 +315,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           tma_reduce_add_3d(&tm_s2, stg + 49152u, 32, y, z);
         }
         tma_store_commit();
+        if (e_last) *items_out = *items_out + 1;
       }
       store_pending = true;
       stg_ph = v & 1u;
@@ -317,7 +323,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     };
 
     int n = 0;
-    for (int w = item_at(0); w < nwork && ok; w = item_at(++n)) {
+    for (int w = item_at(0); w < p.walk && ok; w = item_at(++n)) {
       int blk, bh, set, it_begin, nsteps, d0, d_end;
       decode(w, blk, bh, set, it_begin, nsteps, d0, d_end);
       const int d_first = d0;
@@ -328,7 +334,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (d0 + kDkND >= d_end) {
           const int wn = item_at(n + 1);
           nx_total = 0;
-          if (wn < nwork) { int b0, s0, x0, x1; decode(wn, b0, nx_bh, s0, nx_begin, nx_total, x0, x1); }
+          if (wn < p.walk) { int b0, s0, x0, x1; decode(wn, b0, nx_bh, s0, nx_begin, nx_total, x0, x1); }
         }
         if (h == 0) {
           while (bias_written < jt + (uint32_t)(nsteps < 2 ? nsteps : 2)) {
@@ -440,7 +446,7 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             if (!ok) break;
           }
         }
-        e_blk = blk; e_bh = bh; e_set = set; e_first = d0 == d_first;
+        e_blk = blk; e_bh = bh; e_set = set; e_first = d0 == d_first; e_last = d0 + kDkND >= d_end;
         due = true;
       }
     }
@@ -451,6 +457,11 @@ attn_dk_diff_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag && p.diag) atomicMax(&p.diag->status, (int)BSP_ERR_TIMEOUT);
+  for (int n = *items_out, w; (w = item_at(n)) < nwork; ++n) {      // none, unless a wait ran out
+    int blk, bh, set, a, b, c, d;
+    decode(w, blk, bh, set, a, b, c, d);
+    attn_fill_nan(p.s1, p.s2, set * p.BH + bh, blk, p.S, kDkThreads);
+  }
   if (warp == 17) {
     __syncwarp();
     tc_fence_after();
@@ -510,7 +521,7 @@ __global__ void mc_accumulate_draws_kernel(const float* g, size_t stride, int nd
 
 // The sums over the K draws of the dK difference; `partials` as in attn_f8_draws (two arrays of it).
 static int attn_dk_diff(int BH, int S, int causal, float c, const void* q, const void* k, const float* lse,
-                        const float* d_ref, const float* d_draws, int K, float* S1k, float* S2k, float* partials,
+                        const float* d_ref, const float* d_draws, int K, float* S1k, float* S2k, float* partials, int walk,
                         bsp_diag_t* diag, cudaStream_t st) {
   DkDiffParams p;
   p.BH = BH; p.S = S; p.nblk = (S + AT_BLK - 1) / AT_BLK; p.causal = causal ? 1 : 0; p.c = c;
@@ -534,6 +545,8 @@ static int attn_dk_diff(int BH, int S, int causal, float c, const void* q, const
   }
   const int nsm = sm_count_or_default();
   const int64_t nwork = (int64_t)p.nblk * BH * p.sets;
+  p.s1 = o1; p.s2 = o2;
+  p.walk = walk < nwork ? walk : (int)nwork;
   launch_kernel(attn_dk_diff_kernel, (unsigned)(nwork < nsm ? nwork : nsm), kDkThreads, kDkSmem, st, mq, mk, m1, m2, p);
   BSP_LAUNCH_CHECK();
   return p.sets > 1 ? attn_sum_sets(o1, o2, p.sets, S1k, S2k, n, st) : BSP_OK;
@@ -612,8 +625,8 @@ size_t bsp_mc_check_attn_workspace_bytes(const bsp_attn_desc_t* op, int K) {
     if (_rc != BSP_OK) return _rc; \
   } while (0)
 
-int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t* rule, bsp_use_result_t* results,
-                      int* n_results, void* ws, size_t ws_bytes, bsp_diag_t* diag, void* stream) {
+static int attn_check(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t* rule, bsp_use_result_t* results,
+                      int* n_results, void* ws, size_t ws_bytes, int walk, bsp_diag_t* diag, void* stream) {
   if (!op || !results || !n_results || K < 4 || !rule_valid(rule)) return BSP_ERR_ARG;
   if (!op->q || !op->k || !op->v || !op->dO) return BSP_ERR_ARG;
   int rc = check_attn_shape(op->B, op->H, op->S, op->Dh, op->dtype);
@@ -711,11 +724,11 @@ int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t
                     n / 4);
       BSP_LAUNCH_CHECK();
       // dK: all draws in one launch
-      BSP_TRY(attn_dk_diff((int)BH, S, op->causal, c, q, k, b.lse, b.d_ref, b.d_draws, K, b.S1[1], b.S2[1], b.partials, diag, st));
+      BSP_TRY(attn_dk_diff((int)BH, S, op->causal, c, q, k, b.lse, b.d_ref, b.d_draws, K, b.S1[1], b.S2[1], b.partials, walk, diag, st));
     } else {
       // the rounded backward of every draw; dQ and dK go from the accumulators straight into their sums
       BSP_TRY(attn_f8_draws((int)BH, S, op->causal, c, f, b.lse, b.d_draws, K, b.g_ref[0], b.S1[0], b.S2[0], b.g_ref[1], b.S1[1],
-                            b.S2[1], b.partials, diag, st));
+                            b.S2[1], b.partials, walk, diag, st));
     }
     BSP_TRY(pend.add(b.d_ref, b.S1d, b.S2d, (int64_t)rows, K, 1, emit(out_ids[0], BSP_READ_FRESH)));
     for (int t = 0; t < 2; ++t)
@@ -725,6 +738,17 @@ int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t
   }
   *n_results = nres;
   return pend.flush();
+}
+
+int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t* rule, bsp_use_result_t* results,
+                      int* n_results, void* ws, size_t ws_bytes, bsp_diag_t* diag, void* stream) {
+  return attn_check(op, K, rule, results, n_results, ws, ws_bytes, INT_MAX, diag, stream);
+}
+
+int bsp_selftest_attn_unfinished(const bsp_attn_desc_t* op, int K, int done, bsp_use_result_t* results, int* n_results,
+                                 void* ws, size_t ws_bytes, bsp_diag_t* diag, void* stream) {
+  if (done < 0) return BSP_ERR_ARG;
+  return attn_check(op, K, nullptr, results, n_results, ws, ws_bytes, done, diag, stream);
 }
 
 }  // extern "C"

@@ -359,6 +359,29 @@ def test_mc_check_attention_draw_groups(b, K):
         assert got.verdict == want.verdict
 
 
+@pytest.mark.parametrize("fp8_operands", [0, 1])
+@pytest.mark.parametrize("B,H,S,K,done", [(10, 15, 200, 9, 0), (10, 15, 200, 9, 299), (1, 3, 200, 37, 20), (1, 1, 64, 4, 0)])
+def test_mc_check_attention_cut_short_says_so(b, B, H, S, K, done, fp8_operands):
+    """What a wait that runs out leaves of the sums over the draws: NaN where a block was not completed, not what a check
+    before left in the workspace.  More items than blocks and fewer, one set of draws and several, one item missing or all."""
+    inp = workloads.config3(B=B, H=H, S=S, D=64, K=K, seed=18)
+    g = AttnGpu(b, inp, True)
+    d = _attn_desc(b, g, inp, K, 4)
+    d.fp8_operands, d.p_scale, d.ds_scale = fp8_operands, 256.0, 1024.0
+    ws, diag = b.workspace(b.bsp_mc_check_attn_workspace_bytes(d, K)), b.new_diag()
+    whole = b.bsp_mc_check_attn(d, K, ws, diag)
+    assert all(np.isfinite(r.rel_l2_mean_err) for r in whole)
+    cut = b.bsp_selftest_attn_unfinished(d, K, done, ws, diag)
+    for i, (w, c) in enumerate(zip(whole, cut)):
+        if i == 2 or (i == 1 and fp8_operands):                  # dK; dQ goes through the draws with FP8 operands
+            assert np.isnan(c.rel_l2_mean_err) and not np.isfinite(c.R) and c.verdict == b.FAILS
+        else:
+            assert bytes(w) == bytes(c)
+    again = b.bsp_selftest_attn_unfinished(d, K, 1 << 30, ws, diag)
+    assert [bytes(r) for r in again] == [bytes(r) for r in whole]
+    assert b.read_diag(diag)["status"] == 0
+
+
 @pytest.mark.parametrize("B,H,S,K", [(10, 15, 64, 9), (1, 1, 64, 37)])
 def test_mc_check_attention_draw_sets(b, B, H, S, K):
     """At least as many (key block, head) items as SMs: one set, several passes of an item in turn (10 x 15 heads,
