@@ -382,10 +382,20 @@ def test_mc_check_attention_cut_short_says_so(b, B, H, S, K, done, fp8_operands)
     assert b.read_diag(diag)["status"] == 0
 
 
-@pytest.mark.parametrize("B,H,S,K", [(10, 15, 64, 9), (1, 1, 64, 37)])
-def test_mc_check_attention_draw_sets(b, B, H, S, K):
+def _draw_sets(BH, S, K):
+    """How attn_draw_sets spreads K draws: (sets, passes of four draws per set)."""
+    passes = -(-K // 4)
+    sets = min(148 // (BH * -(-S // 128)), passes)
+    per = -(-passes // sets) if sets > 1 else passes
+    return -(-passes // per), per
+
+
+@pytest.mark.parametrize("B,H,S,K,sets,per", [(10, 15, 64, 9, 1, 3), (1, 1, 64, 37, 10, 1), (5, 10, 64, 21, 2, 3), (2, 8, 300, 61, 3, 6)])
+def test_mc_check_attention_draw_sets(b, B, H, S, K, sets, per):
     """At least as many (key block, head) items as SMs: one set, several passes of an item in turn (10 x 15 heads,
-    nine draws).  One item: ten sets of one pass each, the last of a single draw.  Against the plain oracle."""
+    nine draws).  One item: ten sets of one pass each, the last of a single draw.  50 and 48 items: sets of several passes,
+    the last pass of the last set with a single draw.  Against the plain oracle."""
+    assert _draw_sets(B * H, S, K) == (sets, per)
     inp = workloads.config3(B=B, H=H, S=S, D=64, K=K, seed=17)
     g = AttnGpu(b, inp, True)
     d = _attn_desc(b, g, inp, K, 4)
@@ -400,11 +410,13 @@ def test_mc_check_attention_draw_sets(b, B, H, S, K):
         assert np.isclose(getattr(res[2], f), getattr(want, f), rtol=1e-2), f      # as in the test above
 
 
-@pytest.mark.parametrize("B,H,S,K,causal", [(1, 2, 200, 9, 1), (2, 40, 256, 6, 1), (1, 1, 64, 4, 0), (1, 3, 300, 21, 0)])
-def test_mc_check_attention_fp8_draws_equal_single_backwards(b, B, H, S, K, causal):
-    """FP8 operands: the draws' sums of dQ and dK against one backward per draw.  160 items of two blocks: one set, two
-    passes; the others: sets of one or two passes, the last one partly filled.  The backward of a draw is the
+@pytest.mark.parametrize("B,H,S,K,causal,sets,per", [(1, 2, 200, 9, 1, 3, 1), (2, 40, 256, 6, 1, 1, 2), (1, 1, 64, 4, 0, 1, 1),
+                                                     (1, 3, 300, 21, 0, 6, 1), (1, 50, 64, 21, 1, 2, 3), (1, 16, 300, 61, 1, 3, 6)])
+def test_mc_check_attention_fp8_draws_equal_single_backwards(b, B, H, S, K, causal, sets, per):
+    """FP8 operands: the draws' sums of dQ and dK against one backward per draw.  160 items of two blocks: one set of two
+    passes; the others: sets of one pass and of several, the last one partly filled.  The backward of a draw is the
     same arithmetic in both, so what is left is FP32 sums of K terms (K 2^-24) and of the statistics: 1e-4."""
+    assert _draw_sets(B * H, S, K) == (sets, per)
     torch.manual_seed(S + K)
     BH, n, rows, c = B * H, B * H * S * 64, B * H * S, 0.125
     x = {nm: (torch.randn(n, device="cuda") * (1.0 if nm == "dO" else 0.5)).bfloat16() for nm in ("q", "k", "v", "dO")}
@@ -445,9 +457,6 @@ def test_mc_check_attention_fp8_draws_equal_single_backwards(b, B, H, S, K, caus
     full = b.bsp_mc_check_attn_workspace_bytes(desc, K)
     res = b.bsp_mc_check_attn(desc, K, b.workspace(full), diag)
     # the sets' own sums come last in the workspace: without room for them the draws stay in one set
-    passes = -(-K // 4)
-    sets = min(148 // (BH * -(-S // 128)), passes)
-    sets = -(-passes // -(-passes // sets)) if sets > 1 else 1
     small = full - (-(-16 * sets * n // 256) * 256 if sets > 1 else 0)
     again = b.bsp_mc_check_attn(desc, K, b.workspace(full)[:small], diag)
     assert b.read_diag(diag)["status"] == 0
@@ -458,6 +467,42 @@ def test_mc_check_attention_fp8_draws_equal_single_backwards(b, B, H, S, K, caus
         se2 = ((S2[i] - S1[i] ** 2 / K) / (K * (K - 1))).clamp(min=0).sum()
         assert np.isclose(r.rel_l2_mean_err, float(mean.norm() / ref[i].norm()), rtol=1e-4), (i, r.rel_l2_mean_err)
         assert np.isclose(r.R, float((mean ** 2).sum() / se2), rtol=1e-4), (i, r.R)
+
+
+def _e5m2(x):
+    """float64 to the nearest E5M2 value, saturating."""
+    a = x.abs()
+    step = torch.ldexp(torch.ones_like(a), torch.frexp(a)[1].clamp(min=-13) - 3)
+    return torch.copysign((torch.round(a / step) * step).clamp(max=57344.0), x)
+
+
+@pytest.mark.parametrize("B,H,S,causal", [(4, 4, 384, 0), (1, 3, 300, 1), (1, 2, 1000, 1)])
+def test_attention_fp8_backward_against_64_bits(b, B, H, S, causal):
+    """dQ and dK from the operands' codes, their scales, LSE and D, with every operation but the rounding of dS in float64.
+    What differs is which of two neighbouring codes a dS takes whose value lies within FP32 arithmetic of the middle:
+    with a relative error of 2^-20 of P (dP - D) (ex2.approx 2^-22, the rest the exponent's rounding), one in 2^16 (the
+    middles of a binade's four codes are at least an eighth of their value apart), each by up to a quarter: 1e-3 of the norm."""
+    torch.manual_seed(B + S)
+    BH, n, rows, c = B * H, B * H * S * 64, B * H * S, 0.125
+    q8 = {}
+    for nm in ("q", "k", "v", "dO"):
+        t = (torch.randn(n, device="cuda") * (1.0 if nm == "dO" else 0.125)).bfloat16()
+        xq, codes, amax, sc = torch.zeros_like(t), torch.zeros(n, dtype=torch.uint8, device="cuda"), torch.zeros(BH, device="cuda"), torch.zeros(BH, device="cuda")
+        b.bsp_attn_quantize(t, BH, S * 64, fp8.E5M2 if nm == "dO" else fp8.E4M3, xq, amax, sc, codes=codes)
+        q8[nm] = (xq, sc, codes)
+    f = b.attn_fp8(*(q8[nm][1] for nm in q8), 256.0, 1024.0, *(q8[nm][2] for nm in q8))
+    ops = [q8[nm][0] for nm in q8]
+    o, lse, D, dq, dk = (torch.zeros(m, device="cuda") for m in (n, rows, rows, n, n))
+    b.bsp_attn_fwd_stats(B, H, S, 64, causal, c, *ops[:3], o, lse, fp8=f)
+    b.bsp_attn_dterm(B, H, S, 64, ops[3], o, None, None, fp8.E4M3, 0, b.key(5, 3, b.STREAM_ATTN_D), 0, 1, D, do_scales=q8["dO"][1])
+    b.bsp_attn_bwd_dterm(B, H, S, 64, causal, c, *ops, lse, D, dq, dk, None, fp8=f)
+    val = {nm: (t.view(torch.float8_e5m2 if nm == "dO" else torch.float8_e4m3fn).double().view(BH, S, 64) / sc.double().view(BH, 1, 1))
+           for nm, (_, sc, t) in q8.items()}
+    P = torch.exp(c * val["q"] @ val["k"].mT - lse.double().view(BH, S, 1))
+    P = P.tril() if causal else P
+    dS = _e5m2(P * (val["dO"] @ val["v"].mT - D.double().view(BH, S, 1)) * 1024.0) / 1024.0
+    assert _rel(dq.cpu(), (c * dS @ val["k"]).cpu()) <= 1e-3
+    assert _rel(dk.cpu(), (c * dS.mT @ val["q"]).cpu()) <= 1e-3
 
 
 def _quantised_operands(b, inp):
