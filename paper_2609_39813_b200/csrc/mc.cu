@@ -33,7 +33,8 @@ __device__ __forceinline__ double warp_max_d(double v) {
 // z = err/se.  An element whose draws all coincide (no variance: the read is deterministic there,
 // e.g. every entry it touches already lies on the grid) is judged as a deterministic read: z = 0
 // when |err| <= det_tol |g*|, else +-infinity.  M2 below the resolution of the FP32 sums (1e-6 of
-// S2) counts as no variance.  Block partials in double, summed on the host in block order.
+// S2) counts as no variance.  Block partials in double: the checks sum them with mc_stats_sum_kernel, bsp_mc_stats on
+// the host.
 __global__ void __launch_bounds__(256)
 mc_stats_kernel(const float* g_ref, const float* g, const float* S2,
                 int64_t n, int K, int fresh, float det_tol, double* partials) {
@@ -136,7 +137,8 @@ int mc_stats_launch(const float* g_ref, const float* g, const float* S2, int64_t
   return BSP_OK;
 }
 
-// Sums a slot's block partials on the host, in block order, and fills the result of the use.
+// Sums records of partial statistics in order (the blocks' of bsp_mc_stats, the one of a check's slot) and fills the
+// result of the use.
 void mc_stats_finish(const double* host, int blocks, int64_t n, int K, int fresh, const bsp_verdict_rule_t* rule,
                      bsp_use_result_t* result) {
   if (!rule) rule = &kDefaultRule;

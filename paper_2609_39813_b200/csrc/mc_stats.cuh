@@ -20,9 +20,10 @@ constexpr size_t kStatSlotBytes = kStatSlotDoubles * sizeof(double);   // a mult
 int mc_stats_launch(const float* g_ref, const float* g, const float* S2, int64_t n, int K, int fresh,
                     const bsp_verdict_rule_t* rule, double* partials, cudaStream_t st, int* blocks_out);
 // Sums each of `count` consecutive slots over its blocks (in a fixed order) into out[slot][kStatFields].
-struct StatBlocks { int n[12]; };
+constexpr int kMaxPendingStats = 12;      // slots of a workspace; the last one takes the sums of the others
+struct StatBlocks { int n[kMaxPendingStats]; };
 int mc_stats_sum_slots(const double* slots, const StatBlocks& blocks, int count, double* out, cudaStream_t st);
-// Sums block partials on the host, in block order, and fills the result of the use; the
+// Sums `blocks` records of partial statistics in order and fills the result of the use; the
 // verdict follows `rule` (NULL: the default thresholds, see default_rule()).
 void mc_stats_finish(const double* host, int blocks, int64_t n, int K, int fresh, const bsp_verdict_rule_t* rule,
                      bsp_use_result_t* result);
@@ -30,7 +31,6 @@ const bsp_verdict_rule_t* default_rule();
 // A rule is usable when its thresholds are ordered: hold <= fail for both statistics, nothing negative.
 bool rule_valid(const bsp_verdict_rule_t* rule);
 
-constexpr int kMaxPendingStats = 12;      // slots of a workspace; the last one takes the sums of the others
 struct PendingStats {
   bsp_use_result_t* result[kMaxPendingStats];
   int blocks[kMaxPendingStats], K[kMaxPendingStats], fresh[kMaxPendingStats];
