@@ -21,7 +21,7 @@
  *   - device-detected conditions (non-finite inputs, saturated roundings, a bounded wait that
  *     ran out) are accumulated into the caller's device-resident bsp_diag_t, never trapped; the
  *     caller clears it (bsp_diag_clear) and reads it back after synchronising;
- *   - the same inputs give byte-identical outputs.  State the library keeps per process, none of
+ *   - the same inputs give byte-identical outputs (and the same workspace size, see bsp_mc_check_attn).  State the library keeps per process, none of
  *     which influences a result: the counters behind bsp_launch_count() and bsp_d2h_byte_count(), the record of which
  *     kernels already have their shared-memory limit raised on which device, and the fixed scratch
  *     array of bsp_norm_bwd_noalloc (a 20 MiB device array every GPU that loads the library holds).
@@ -522,9 +522,11 @@ int bsp_mc_check(const bsp_norm_linear_desc_t* op, int K, const bsp_verdict_rule
  * four draws per pass of the probabilities), so the statistics are not blurred by the rounding of
  * a full dS to the operand type, and no per-draw gradient is written.  dV does not read D: its
  * difference is exactly zero in every draw.
- * FP8-operand mode (fp8_operands = 1; p_scale, ds_scale as in bsp_attn_fp8_t) runs the rounded
- * backward once per draw: there dQ and dK pass through the nearest rounding of dS, which is not
- * linear in D, so their rows are marked `informational` and the verdict of the use is the row of D. */
+ * FP8-operand mode (fp8_operands = 1; p_scale, ds_scale as in bsp_attn_fp8_t) rounds dS and forms dQ
+ * and dK for every draw (the scores, dP and the probabilities once per four draws): there they pass
+ * through the nearest rounding of dS, which is not linear in D, so their rows are marked
+ * `informational` and the verdict of the use is the row of D.
+ * Sums over the draws that a bounded wait cut short are NaN, and so are their statistics. */
 typedef struct {
   int32_t B, H, S, Dh;
   int32_t causal;
@@ -543,6 +545,10 @@ typedef struct {
   float p_scale, ds_scale;   /* FP8-operand mode only */
 } bsp_attn_desc_t;
 
+/* The query includes partial sums for problems of few (key block, head) pairs, whose draws are spread over the
+ * SMs.  A workspace without room for them, 4 (BF16 operands: 2) arrays of at most 148 x 128 x 64 floats less, is
+ * taken as well: the draws of a pair are then summed one after the other, which takes longer, and the last bits of
+ * the statistics of dK (FP8 operands: and dQ) may differ.  Anything smaller is BSP_ERR_WORKSPACE. */
 size_t bsp_mc_check_attn_workspace_bytes(const bsp_attn_desc_t* op, int K);
 int bsp_mc_check_attn(const bsp_attn_desc_t* op, int K, const bsp_verdict_rule_t* rule,
                       bsp_use_result_t* results, int* n_results, void* ws, size_t ws_bytes,

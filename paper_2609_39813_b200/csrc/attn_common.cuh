@@ -157,8 +157,8 @@ int attn_dterm_impl(int B, int H, int S, int Dh, const void* dO, int dt, const f
 int attn_bwd_dterm_impl(int B, int H, int S, int Dh, int causal, float softmax_scale, const void* q, const void* k,
                         const void* v, const void* dO, int dt, const bsp_attn_fp8_t* f, const float* lse,
                         const float* dterm, float* dq, float* dk, float* dv, bsp_diag_t* diag, void* stream);
-// The draws of a fresh read go through the scores kDrawsPerPass at a time, and where (block, head) items are fewer than
-// the SMs they are spread over attn_draw_sets(BH, S, K) sets with sums of their own, [sets][BH * S * 64] per array,
+// The draws of a fresh read go through the scores kDrawsPerPass at a time, and where (block, head) items are at most half
+// as many as the SMs they are spread over attn_draw_sets(BH, S, K) sets with sums of their own, [sets][BH * S * 64] per array,
 // which attn_sum_sets adds in order into S1 and S2 (n floats each).
 constexpr int kDrawsPerPass = 4;
 int attn_draw_sets(int64_t BH, int S, int K);

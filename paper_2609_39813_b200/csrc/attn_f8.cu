@@ -20,13 +20,13 @@
 //
 // Measured at B H = 128, S = 2048, causal, 32 draws: both kernels 4.35 ms (a launch per pair of draws, with the
 // operands in tensor memory and eight softmax warps, 8.2; two operand buffers and reduce-adds 4.5), the whole
-// check 9.54 -> 6.15 ms.  Of a step's 4600 cycles the conversions take 1700 and the exponentials 1200, one after the
+// check 9.54 -> 6.08 ms.  Of a step's 4600 cycles the conversions take 1700 and the exponentials 1200, one after the
 // other in all warps (a start half a step apart does not last: a step's products need every warp's codes); 450
 // are a pass's end, the rest waits for barriers and tensor memory.
 //
 // Persistent CTA, one per SM, walking (block, head, set of draws) items, heaviest first.  A CTA takes the
-// draws of its set four at a time and adds to the sums in that order; where there are fewer (block, head)
-// items than SMs the draws are spread over several sets, each with sums of its own, which sum_sets_kernel
+// draws of its set four at a time and adds to the sums in that order; where there are at most half as many
+// (block, head) items as SMs the draws are spread over several sets, each with sums of its own, which sum_sets_kernel
 // adds in order, so the sums stay reproducible.  640 threads: warps 0..15 softmax and epilogue, warp 16
 // TMA, warp 17 MMA issue.  Every wait is bounded (the warps meet on mbarriers, never on a block barrier).
 #include <string.h>
@@ -574,8 +574,8 @@ int attn_f8_bwd(int BH, int S, int causal, float c, const bsp_attn_fp8_t* f, con
   return BSP_OK;
 }
 
-// Sets the K draws are spread over: as many as fill the SMs when there are fewer (block, head) items than that,
-// each of at least one pass.  (The partial sums then stay below 148 x 128 x 64 floats per array.)
+// Sets the K draws are spread over: as many whole sets of the (block, head) items as the SMs take in one round (so from
+// 75 items on one), each of at least one pass.  (The partial sums then stay below 148 x 128 x 64 floats per array.)
 int attn_draw_sets(int64_t BH, int S, int K) {
   const int64_t items = ((int64_t)S + AT_BLK - 1) / AT_BLK * BH;
   const int passes = (K + kF8ND - 1) / kF8ND;
